@@ -677,8 +677,12 @@ void launch_scan(ah_ctx *c, ScanKernel *k, const GenomeSet &gs, uint64_t n_tiles
     const uint32_t *tcont = gs.tile_contig, *troom = gs.tile_room;
     uint64_t wait_ns = c->scan_stall_first ? 20000ull : 2000000000ull;
     int stall = c->scan_stall_first ? 1 : 0;
+    // tiles a CTA claims at once: all claims go to one address (about one per nanosecond on a
+    // GB300; at one claim per 1/8 tile they bound the scan of cheap patterns: 435 us for 2 Gbp at
+    // k = 1), and 24 claims a CTA keep the tail short
+    uint32_t per_claim = (uint32_t)std::min<uint64_t>(8, std::max<uint64_t>(1, n_tiles / (grid * 24)));
     void *args[] = {&planes, &n_tiles,  &coff, &nc,        &keys,  &cap,   &c->d_counter,
-                    &pbits,  &c->d_err, &work, &tile_list, &tcont, &troom, &wait_ns, &stall};
+                    &pbits,  &c->d_err, &work, &tile_list, &tcont, &troom, &wait_ns, &stall, &per_claim};
     AH_CUDA(cudaLaunchKernel((const void *)k->fn, dim3((unsigned)grid), dim3(k->threads), args, k->smem, st));
 }
 
@@ -1497,19 +1501,18 @@ ah_status ah_create(int device, size_t mem_budget_bytes, ah_ctx **out)
     c->budget = mem_budget_bytes;
     ah_status st = guarded(c, [&] {
         AH_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device));
-        // default scan variant; AH_SCAN_TUNING="R,arith_pct,order,stages,warps[,min_blocks[,resident]]" overrides
+        // default scan variant; AH_SCAN_TUNING="R,arith_pct,order,stages[,min_blocks[,resident]]" overrides
         // it (profiling aid)
         if (const char *e = getenv("AH_SCAN_TUNING")) {
-            int R = 8, ap = 0, order = 1, S = 3, wpc = 4, mb = 1, res = 0;
-            if (sscanf(e, "%d,%d,%d,%d,%d,%d,%d", &R, &ap, &order, &S, &wpc, &mb, &res) >= 1 && (R == 4 || R == 8) &&
-                ap >= 0 && ap <= 100 && (order == 0 || order == 1) && S >= 2 && S <= 4 && wpc >= 1 && wpc <= 16 &&
-                mb >= 1 && mb <= 8 && res >= 0 && res <= 8) {
+            int R = 4, ap = 0, order = 0, S = 4, mb = 2, res = 0;
+            if (sscanf(e, "%d,%d,%d,%d,%d,%d", &R, &ap, &order, &S, &mb, &res) >= 1 && (R == 4 || R == 8) &&
+                ap >= 0 && ap <= 100 && (order == 0 || order == 1) && S >= 2 && S <= 6 && mb >= 1 && mb <= 8 &&
+                res >= 0 && res <= 8) {
                 c->tuning.resident = res;
                 c->tuning.R = R;
                 c->tuning.arith_pct = ap;
                 c->tuning.order = order;
                 c->tuning.stages = S;
-                c->tuning.warps = wpc;
                 c->tuning.min_blocks = mb;
             }
         }
@@ -2125,30 +2128,18 @@ ah_status ah_tune_scan(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uin
         uint64_t tiles = std::min<uint64_t>(gs.n_tiles, sample_tiles ? sample_tiles : 4096);
         require(tiles > 0, AH_ERR_ARG, "ah_tune_scan: empty genome set");
         // the sample must cover whole waves of the persistent grid to time it fairly
-        // register-capped variants (more resident warps) first: measured fastest on
-        // the 960-oligo pair; R = 8 uncapped for pattern sets that spill under the cap
+        // 8 warps per CTA at R = 4 (two or three CTAs per SM), 4 at R = 8
         std::vector<ScanTuning> cand;
-        const int shapes[][2] = {{16, 1}, {8, 2}, {4, 4}}; // warps per CTA, minimum CTAs per SM
+        const int shapes[][3] = {{4, 4, 2}, {4, 3, 2}, {4, 3, 3}, {8, 3, 3}, {8, 4, 2}}; // R, stages, minimum CTAs per SM
         for (const auto &sh : shapes)
-            for (int order : {0, 1})
-                for (int S : {3, 4}) {
-                    ScanTuning t;
-                    t.R = 4;
-                    t.order = order;
-                    t.stages = S;
-                    t.warps = sh[0];
-                    t.min_blocks = sh[1];
-                    cand.push_back(t);
-                }
-        for (int order : {0, 1}) {
-            ScanTuning t;
-            t.R = 8;
-            t.order = order;
-            t.stages = 3;
-            t.warps = 4;
-            t.min_blocks = 1;
-            cand.push_back(t);
-        }
+            for (int order : {0, 1}) {
+                ScanTuning t;
+                t.R = sh[0];
+                t.order = order;
+                t.stages = sh[1];
+                t.min_blocks = sh[2];
+                cand.push_back(t);
+            }
         cudaEvent_t e0 = get_event(c), e1 = get_event(c);
         // each launch group is tuned on its own (its kernel is compiled and run alone);
         // the result reports the slowest group's variant and the groups' summed time
@@ -2183,9 +2174,9 @@ ah_status ah_tune_scan(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uin
                 const double us = ms_min * 1e3 / (double)tiles;
                 if (getenv("AH_TUNE_VERBOSE"))
                     fprintf(stderr,
-                            "ah_tune_scan: patterns=%zu R=%d arith=%d order=%d stages=%d warps=%d regs=%d bps=%d  "
+                            "ah_tune_scan: patterns=%zu R=%d arith=%d order=%d stages=%d threads=%d regs=%d bps=%d  "
                             "%.4f us/tile\n",
-                            gp.size(), t.R, t.arith_pct, t.order, t.stages, t.warps, k->regs, k->blocks_per_sm, us);
+                            gp.size(), t.R, t.arith_pct, t.order, t.stages, k->threads, k->regs, k->blocks_per_sm, us);
                 if (us < best_us) {
                     best_us = us;
                     best = t;
@@ -2208,7 +2199,7 @@ ah_status ah_tune_scan(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uin
             best_out->min_blocks = worst.min_blocks;
             best_out->order = worst.order;
             best_out->stages = worst.stages;
-            best_out->warps_per_cta = worst.warps;
+            best_out->warps_per_cta = kTileW / (32 * worst.R);
             best_out->regs = worst_regs;
             best_out->us_per_tile = total_us;
             best_out->tiles = tiles;

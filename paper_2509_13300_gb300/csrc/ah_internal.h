@@ -106,10 +106,9 @@ void launch_hmm_score(const ah_amplicon *amps, const uint32_t *order, uint64_t n
 struct ScanTuning {
     int R = 4;            // 32-start words per thread (4 or 8: the loader reads 16-byte vectors at lane * R)
     int arith_pct = 0;    // share of full adders that form the sum with integer adds
-    int min_blocks = 1;   // __launch_bounds__ minimum blocks per SM (with warps: a register cap)
+    int min_blocks = 2;   // __launch_bounds__ minimum blocks per SM (a register cap: 128 at R = 4)
     int order = 0;        // 0: word-major, 1: pattern-major code order
-    int stages = 4;       // TMA stages per warp (2..4)
-    int warps = 16;       // warps per CTA (1..16); 16 warps = a 128-register cap
+    int stages = 4;       // tiles staged per CTA (2..6); a CTA has kTileW / (32 R) warps
     int resident = 0;     // CTAs launched per SM (0: as many as fit); fewer leave room for a
                           // kernel that runs beside the scan (the next set's packing)
 };

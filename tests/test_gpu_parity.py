@@ -219,6 +219,39 @@ def test_scan_wait_limit_reports_timeout_and_the_context_stays_usable(ctx):
     assert sites.tobytes() == oracle.scan(w.seq, w.contig_off, w.contig_genome, w.pairs).tobytes()
 
 
+@pytest.mark.parametrize("fwd,rev,k", [
+    ("ACGTTGCAAC", "GGTACCATTG", 1),            # network over a part of the positions
+    ("NNNNNN", "NNNACNNN", 0),                  # nothing, or two positions, to count
+    ("RYSWKMRYSW", "BDHVRYBDH", 2),             # no single-base position: no complements
+    ("ACGNBDHRYSWKAC", "TGCANNNNNNACGT", 2),  # complements beside single bases, N left out
+    ("ACGTACGTACGTACGTACGTACGTACGTACGT", "TTGACWSKMRYBDHANACGTACGGTACGATCA", 9),
+])
+@pytest.mark.parametrize("n_bases", [31, 32 * 1024 - 1, 32 * 1024 + 1, 5 * 32 * 1024, 300_007])
+def test_scan_filter_at_tile_edges(ctx, fwd, rev, k, n_bases):
+    """The scan's network counts only some positions and lets other starts through to the exact
+    count: sites equal the oracle's on sets around a tile's size, with runs of non-bases."""
+    rng = np.random.default_rng(n_bases + k)
+    seq = synth.random_bases(rng, n_bases, 0.5).copy()
+    for s0 in rng.integers(0, n_bases, 1 + n_bases // 2000):
+        seq[s0:s0 + int(rng.integers(1, 90))] = ord("N")
+    for i, L in ((0, len(fwd)), (1, len(rev))):  # planted sites, also at the very end
+        for at in [n_bases - L] + list(rng.integers(0, max(1, n_bases - L), 5)):
+            if 0 <= at <= n_bases - L:
+                oligo = synth._draw_oligo(rng, (fwd, rev)[i], int(rng.integers(0, k + 1)))
+                seq[at:at + L] = np.frombuffer((oligo if i == 0 else synth._revcomp(oligo)).encode(), np.uint8)
+    cuts = np.unique(rng.integers(1, n_bases, 4))
+    off = np.concatenate([[0], cuts, [n_bases]]).astype(np.uint64)
+    gen = np.zeros(len(off) - 1, np.uint32)
+    pairs = [synth.pcr_params(fwd, rev, k=k, min_len=20, max_len=400)]
+    want = oracle.scan(seq, off, gen, pairs)
+    sid = ctx.load(seq, off, gen)
+    try:
+        got = ctx.scan(sid, [ctx.ah_set_primers(fwd, rev, pairs[0])])
+    finally:
+        ctx.ah_unload_genomes(sid)
+    assert got.tobytes() == want.tobytes(), (len(got), len(want))
+
+
 def test_full_collection_workload_against_the_oracle(ctx):
     """The whole 100-genome collection workload (0.41 Gbp, 1,777 contigs, the
     960-oligo pair, k = 3, Tm threshold 50 C) through ah_run, against the oracle
