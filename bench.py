@@ -1659,7 +1659,7 @@ def bench_hmm(args):
     # the other kernel of each score on the same amplicons (AH_HMM_KERNEL), for comparison
     other = {}
     try:
-        for name, kern, fn, o in (("viterbi", "wave", ctx.hmm_score, out), ("forward", "rows", ctx.hmm_forward, out_f)):
+        for name, kern, fn, o in (("viterbi", "rows", ctx.hmm_score, out), ("forward", "rows", ctx.hmm_forward, out_f)):
             os.environ["AH_HMM_KERNEL"] = kern
             fn(sid, hid, dev_amps, n=len(amps), out=o, stream=stream)
             torch.cuda.synchronize()
@@ -1695,8 +1695,7 @@ def bench_hmm(args):
     err = np.abs(got[sample].astype(np.float64) - want)
     err_f = np.abs(got_f[sample].astype(np.float64) - want_f)
     clocks = clk.summary()
-    # FADD + FMNMX per cell of the recurrence (M 6, I 5, D 5); the block-per-group kernel
-    # that scores Viterbi executes 19 (its delete-chain scan evaluates D's terms twice)
+    # additions and maxima per cell of the recurrence (M 6, I 5, D 5; a three-input maximum counts as two)
     fp_ops_per_cell = 16
     fp32_peak = 152 * 128 * (clocks["sm_mhz"] or 2070.0) * 1e6
     achieved = cells / dt * fp_ops_per_cell
@@ -1718,8 +1717,8 @@ def bench_hmm(args):
                     "oracle_check": {"amplicons": len(sample),
                                      "max_abs_err_bits": float(err_f.max()) if len(err_f) else 0.0,
                                      "within_fp32_bound": bool((err_f <= tol_f).all())}},
-        "kernels": {"viterbi": "hmm_score_kernel (a block per group of amplicons, rows in lockstep)",
-                    "forward": "hmm_wave_kernel (one warp per amplicon, anti-diagonal steps)"},
+        "kernels": {"viterbi": "hmm_wave_kernel (a warp per stripe of an amplicon, anti-diagonal steps)",
+                    "forward": "hmm_wave_kernel on scaled odds"},
         "other_kernel": other,
         "cpu_baseline": {"value": cpu_cells / t_cpu / 1e9, "unit": "GCUPS", "cores": 1, "kind": "oracle",
                          "sample": f"{len(sample)} amplicons, fp64 Viterbi, {t_cpu:.1f} s"},

@@ -2825,11 +2825,22 @@ ah_status ah_hmm_build(ah_ctx *c, const char *seqs, const uint64_t *offsets, uin
         build_profile(seqs, offsets, n, p);
         require(p.m >= 1 && p.m + 1 <= kHmmMaxColumns, AH_ERR_ARG,
                 "ah_hmm_build: the reference must hold 1.." + std::to_string(kHmmMaxColumns - 1) + " letters");
-        p.d_t = (float *)dev_alloc(c, p.t.size() * sizeof(float));
-        p.d_e = (float *)dev_alloc(c, p.e.size() * sizeof(float));
-        AH_CUDA(cudaMemcpyAsync(p.d_t, p.t.data(), p.t.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-        AH_CUDA(cudaMemcpyAsync(p.d_e, p.e.data(), p.e.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-        AH_CUDA(cudaStreamSynchronize(c->stream));
+        std::vector<float> tables(p.t); // one device block: scores of moves and emissions, then both as odds
+        tables.insert(tables.end(), p.e.begin(), p.e.end());
+        const size_t n_t = p.t.size(), n_all = tables.size();
+        for (size_t i = 0; i < n_all; ++i)
+            tables.push_back((float)std::exp2((double)tables[i]));
+        p.d_t = (float *)dev_alloc(c, tables.size() * sizeof(float));
+        p.d_e = p.d_t + n_t;
+        p.d_t_odds = p.d_t + n_all;
+        p.d_e_odds = p.d_t_odds + n_t;
+        try {
+            AH_CUDA(cudaMemcpyAsync(p.d_t, tables.data(), tables.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
+            AH_CUDA(cudaStreamSynchronize(c->stream));
+        } catch (...) {
+            dev_free(c, p.d_t, 0);
+            throw;
+        }
         const uint32_t id = c->next_hmm++;
         c->hmms[id] = std::move(p);
         *hmm_id_out = id;
@@ -2905,11 +2916,25 @@ ah_status hmm_scores(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_ampli
         uint32_t *d_ord = (uint32_t *)scratch(c, "hmm_order", n * sizeof(uint32_t));
         AH_CUDA(cudaMemcpyAsync(d_ord, ord.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
         float *out = out_buf(c, "hmm_out", score_out, n);
-        if (hmm_use_wave(forward)) {
-            float *bnd = (float *)scratch(c, "hmm_bnd", hmm_scratch_bytes(n, (int)max_len, c->sms));
+        // the wavefront's boundary buffers (at most 1/16 of a memory budget): fewer blocks where
+        // there is no room for them, and without room for one block's the kernel that needs none
+        uint64_t blocks = hmm_use_wave() ? hmm_wave_blocks(n, p.m, (int)max_len, c->sms) : 0;
+        while (blocks > 1 && c->budget && hmm_scratch_bytes(blocks, p.m, (int)max_len) > c->budget / 16)
+            blocks /= 2;
+        void *bnd = nullptr;
+        while (blocks && !bnd && hmm_scratch_bytes(blocks, p.m, (int)max_len)) {
+            try {
+                bnd = scratch(c, "hmm_bnd", hmm_scratch_bytes(blocks, p.m, (int)max_len));
+            } catch (const Error &e) {
+                if (e.status != AH_ERR_BUDGET && e.status != AH_ERR_OOM)
+                    throw;
+                blocks /= 2;
+            }
+        }
+        if (blocks) {
             Stage sg(c, "hmm", st, 1);
-            launch_hmm_wave(a, d_ord, n, gs.planes, gs.contig_off, gs.n_contigs, p.d_t, p.d_e, p.m, (int)max_len,
-                            forward, bnd, out, c->d_err, c->sms, st);
+            launch_hmm_wave(a, d_ord, n, gs.planes, gs.contig_off, gs.n_contigs, p, (int)max_len, forward, bnd, blocks,
+                            out, c->d_err, c->sms, st);
         } else {
             Stage sg(c, "hmm", st, 1);
             launch_hmm_score(a, d_ord, n, gs.planes, gs.contig_off, gs.n_contigs, p.d_t, p.d_e, p.m, (int)max_len,
@@ -2958,8 +2983,7 @@ ah_status ah_hmm_free(ah_ctx *c, uint32_t hmm_id)
         auto it = c->hmms.find(hmm_id);
         require(it != c->hmms.end(), AH_ERR_ARG, "ah_hmm_free: unknown profile id");
         AH_CUDA(cudaStreamSynchronize(c->stream));
-        dev_free(c, it->second.d_t, 0);
-        dev_free(c, it->second.d_e, 0);
+        dev_free(c, it->second.d_t, 0); // the block of all four tables
         c->hmms.erase(it);
     });
 }

@@ -93,7 +93,8 @@ struct HmmProfile {
     int m = 0;
     uint64_t reference = 0; // index of the training sequence used as the reference
     std::vector<float> t, e;
-    float *d_t = nullptr, *d_e = nullptr;
+    float *d_t = nullptr, *d_e = nullptr;           // device: the scores
+    float *d_t_odds = nullptr, *d_e_odds = nullptr; // and 2^score, in the same block
 };
 void build_profile(const char *seqs, const uint64_t *off, uint64_t n, HmmProfile &p);
 // order: n indices into amps, amplicons of similar length next to each other;

@@ -16,31 +16,37 @@
 // bits against the uniform background: log2(p / (1/4)) for match emissions
 // (0 for an unknown letter), 0 for insert emissions, log2 p for moves.
 //
-// Scores (hmm_score_kernel): the glocal Viterbi log-odds score of each
-// amplicon's sequence (as ah_fetch returns it) against the profile, fp32, or
-// the glocal Forward score: the same recurrence with the maximum of the
-// predecessors replaced by log2(2^a + 2^b) (the log-sum semiring).
-// Two kernels compute the same recurrence.
+// Scores: the glocal Viterbi log-odds score of each amplicon's sequence (as
+// ah_fetch returns it) against the profile, fp32, or the glocal Forward score:
+// the same recurrence with the maximum of the predecessors replaced by
+// log2(2^a + 2^b) (the log-sum semiring).  Two kernels compute the recurrence.
 //
-// hmm_wave_kernel (the Forward scores' default): one warp per amplicon, no
-// block barriers.  The
-// profile's columns are cut into stripes of 32 * K; within a stripe lane l
-// owns K consecutive columns with their 13 scores in registers and, at step
-// s, computes row i = s - l (an anti-diagonal wavefront): M and I of its
-// columns from its own previous row, the delete chain along its K columns.
-// The left neighbour's last column arrives by one shuffle per state (its row
-// i from the previous step; its row i - 1 is kept from the step before).
-// Lane 0 takes column (stripe start - 1) from the previous stripe, whose
-// lane 31 wrote it per row to a per-warp boundary buffer in global memory;
-// the warp loads it 32 rows at a time (one row per lane, two blocks ahead of
-// use) and hands row i to lane 0 by shuffle at step i (row i is overwritten
-// at step i + 31, after its block was loaded).  A stripe
-// costs len + 32 steps, so the wavefront's fill and drain are 31 steps per
-// stripe.
+// hmm_wave_kernel (the default): a warp runs one stripe of 32 * K columns of one
+// amplicon; lane l owns K consecutive columns with their nine move scores in
+// registers and, at step s, computes row i = s - l (an anti-diagonal
+// wavefront): M and I of its columns from its own previous row, the delete
+// chain along its K columns.  The left neighbour's last column arrives by one
+// shuffle per state (its row i from the previous step; its row i - 1 is kept
+// from the step before); lane 0 takes it from the previous stripe, through a
+// buffer in global memory that is read 32 rows at a time, two blocks ahead.  The
+// stripes of a block's amplicons are one sequence of tasks dealt to its four
+// warps in turn, each stripe about 100 rows behind the one before it, so one
+// amplicon already fills four warps and a call's last amplicons leave no warp
+// idle for a whole amplicon.  Forward scores are computed as odds (sums and
+// products, no logarithms: the log-sum took an exp2 and a log2 per term, and
+// its roundings of scores of ~1,000 bits were the larger error) with a common
+// exponent per lane, brought up to date every fourth row.
+// Bound: issue slots, with latency next (three warps per scheduler by registers):
+// 143 instructions per step of 256 cells for Viterbi, 157 for Forward, issue 0.68
+// and 0.66.  K = 8 needs half the steps of K = 4 per profile; packed two-wide
+// fp32 instructions were measured no faster (they take two dispatch cycles, and
+// the packing moves come on top).  Measured on a GB300: Viterbi, 4,000 amplicons x
+// 1,461 columns 22.8 -> 6.3 ms (1.36 T cells/s); Forward, 5,000 x 460 11.3 -> 1.0 ms
+// (1.05 T cells/s); one amplicon of 1,461 letters 1,577 -> 500 us (Viterbi).
 //
-// hmm_score_kernel (the Viterbi scores' default; AH_HMM_KERNEL=rows or =wave
-// forces one kernel for both scores): a block scores a group of amplicons
-// of similar length in lockstep, rows = sequence letters: each thread owns K
+// hmm_score_kernel (where a memory budget has no room for the wavefront's
+// buffers, and AH_HMM_KERNEL=rows): a block scores a group of amplicons of
+// similar length in lockstep, rows = sequence letters: each thread owns K
 // consecutive profile columns with their 13 scores in registers; M and I of a
 // row depend only on the previous row (the left neighbour's values come by
 // shuffle, or through shared memory across warps); the delete chain
@@ -51,6 +57,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "ah_internal.h"
 #include "hmm.h"
@@ -488,204 +495,450 @@ bool launch_k(const ah_amplicon *amps, const uint32_t *order, uint64_t n, const 
     return true;
 }
 
-// Letter codes of amplicon `am` into seq, the warp's lanes in turn.
+// ---------------------------------------------------------------------------
+// The warp wavefront (see the head of this file).
+// ---------------------------------------------------------------------------
+constexpr int kWaveWarps = 4;       // warps per block: a pipeline over stripes
+constexpr int kWaveRing = 64 + 8;   // float4s per warp: 64 boundary rows, and one lane's columns at the end
+constexpr int kSeqPad = 64;         // letters of padding on either side of a warp's sequence in shared memory
+constexpr uint64_t kWaveScratchMax = 256ull << 20;
+constexpr uint64_t kWaveWaitNs = 2000000000ull; // bound of a wait on another warp's progress
+
+// The wavefront's two semirings.  Viterbi: scores in bits, (max, +).  Forward:
+// odds (2^score) with an exponent per lane, (+, x).  ext(a, t): a path
+// extended by a move; acc(s, a, t): the sum of s and a extended by t; acc3: the
+// sum of three extended paths.
+struct WaveMax {
+    static constexpr bool kScaled = false;
+    static constexpr float kZero = -INFINITY, kOne = 0.0f;
+    __device__ static __forceinline__ float ext(float a, float t) { return a + t; }
+    __device__ static __forceinline__ float acc(float s, float a, float t) { return fmaxf(s, a + t); }
+    __device__ static __forceinline__ float acc3(float a, float ta, float b, float tb, float c, float tc)
+    {
+        return fmaxf(fmaxf(a + ta, b + tb), c + tc); // one three-input maximum
+    }
+};
+struct WaveSum {
+    static constexpr bool kScaled = true;
+    static constexpr float kZero = 0.0f, kOne = 1.0f;
+    __device__ static __forceinline__ float ext(float a, float t) { return a * t; }
+    __device__ static __forceinline__ float acc(float s, float a, float t) { return fmaf(a, t, s); }
+    __device__ static __forceinline__ float acc3(float a, float ta, float b, float tb, float c, float tc)
+    {
+        return fmaf(c, tc, fmaf(b, tb, a * ta)); // (the last term may be the one that arrives late)
+    }
+};
+
+// Exponents of the scaled odds: a value is mantissa * 2^E with one E per lane.
+// Every four rows a lane's largest mantissa is brought to 2^kTop.  A row grows
+// it by at most 2^2 (an emission is at most 4, the moves into a cell sum to at
+// most 1 per state left), and what comes in from the left lane is at most
+// 2^kFar above the lane's own level (beyond that the lane takes the left one's
+// exponent), so it stays below 2^128; the smallest normal float lies 156 bits
+// below it.  Within a lane's eight columns a cell more than ~75 bits below the
+// largest adds nothing a float could hold to any later cell (the larger one
+// reaches the same cells by at most eight deletions or insertions, whose
+// probabilities are at least 1 / (training sequences + 3)), so what underflows
+// is no loss.
+constexpr int kTop = 30, kFar = 80, kRise = 24;
+constexpr int kNoMass = -(1 << 20); // exponent of a lane that holds only zeros
+__device__ __forceinline__ int level_of(float x) { return (int)(__float_as_uint(x) >> 23) - 127 - kTop; }
+__device__ __forceinline__ float power_of_two(int e) // 2^e for e <= 127; 0 below the normal range
+{
+    return e < -126 ? 0.0f : __uint_as_float((uint32_t)(e + 127) << 23);
+}
+
+// Letter codes of amplicon `am` into seq[0 .. len), the warp's lanes in turn, and
+// "unknown" on either side.
 __device__ void decode_letters_warp(const ah_amplicon &am, const uint32_t *__restrict__ planes,
                                     const uint64_t *__restrict__ contig_off, uint8_t *seq, int len, int lane)
 {
     const uint64_t base = contig_off[am.contig] + am.start;
     const bool rc = am.orient == 1;
-    for (int q = lane; q < len; q += 32) {
-        const uint64_t P = base + (rc ? (uint64_t)(len - 1 - q) : (uint64_t)q);
-        const uint64_t tt = P / kTileBases, r = P % kTileBases;
-        const int b = (int)(r / kTileW), j = (int)(r % kTileW);
-        const uint32_t *w = planes + tt * 4 * kTileWX + j;
+    for (int q = lane - kSeqPad; q < len + kSeqPad; q += 32) {
         int code = 4;
+        if (q >= 0 && q < len) {
+            const uint64_t P = base + (rc ? (uint64_t)(len - 1 - q) : (uint64_t)q);
+            const uint64_t tt = P / kTileBases, r = P % kTileBases;
+            const int b = (int)(r / kTileW), j = (int)(r % kTileW);
+            const uint32_t *w = planes + tt * 4 * kTileWX + j;
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
-            if ((__ldg(w + x * kTileWX) >> b) & 1u)
-                code = x;
-        if (code < 4 && rc)
-            code = 3 - code;
+            for (int x = 0; x < 4; ++x)
+                if ((__ldg(w + x * kTileWX) >> b) & 1u)
+                    code = x;
+            if (code < 4 && rc)
+                code = 3 - code;
+        }
         seq[q] = (uint8_t)code;
     }
 }
 
-constexpr int kWaveWarps = 4;        // warps (amplicons in flight) per block
-constexpr int kWaveBlocksPerSm = 8;  // grid: at most this many blocks per SM
-constexpr uint64_t kWaveScratchMax = 256ull << 20;
+// Waits (bounded) until *p >= need: another warp of the block has got that far.
+__device__ __forceinline__ bool wait_for(volatile uint64_t *p, uint64_t need)
+{
+    if (*p >= need)
+        return true;
+    uint64_t t0, t1;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    while (*p < need) {
+        __nanosleep(100);
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+        if (t1 - t0 > kWaveWaitNs)
+            return false;
+    }
+    return true;
+}
 
-// One warp per amplicon; lanes over the columns of a stripe, steps over
-// anti-diagonals (see the head of this file).  bnd_all: 3 * (max_len + 1)
-// floats per warp of the grid (M, I, D of the column left of the stripe, per
-// row).
+// A block scores the amplicons order[blockIdx.x + i * gridDim.x].  Their stripes
+// form one sequence of tasks (task = i * n_stripes + stripe), and warp w takes
+// the tasks with task % kWaveWarps == w, so the stripes of an amplicon run
+// behind one another and no warp waits for a whole amplicon.  A task hands its
+// last column on through one of its warp's two buffers in bnd_all (max_len + 1
+// float4s each: M, I, D and their exponent, per row): rows[w] = (task + 1) << 20
+// | rows written, and used[w] = task + 1 once the next warp has read all of a
+// task's rows (a buffer is reused two tasks later).
+// t, e: the profile's moves and emissions in the semiring's values (bits, or
+// odds).  Shared memory: the emissions of every column for letter codes 0..4;
+// per warp the boundary ring, the last row's states and the letters.
 template <class Op, int K>
-__global__ void __launch_bounds__(32 * kWaveWarps) hmm_wave_kernel(
+__global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kernel(
     const ah_amplicon *__restrict__ amps, const uint32_t *__restrict__ order, uint64_t n_amps,
     const uint32_t *__restrict__ planes, const uint64_t *__restrict__ contig_off, uint32_t n_contigs,
-    const float *__restrict__ t, const float *__restrict__ e, int m, int max_len, float *__restrict__ bnd_all,
+    const float *__restrict__ t, const float *__restrict__ e, int m, int max_len, float4 *bnd_all,
     float *__restrict__ score_out, int *__restrict__ err)
 {
-    extern __shared__ uint8_t wave_seq[]; // kWaveWarps x seq_stride letter codes
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int seq_stride = (max_len + 15) & ~15;
-    uint8_t *seq = wave_seq + warp * seq_stride;
-    const uint64_t slot = (uint64_t)blockIdx.x * kWaveWarps + warp;
-    float *bnd = bnd_all + slot * 3ull * (uint64_t)(max_len + 1);
     constexpr int span = 32 * K;
-    const int n_stripes = (m + 1 + span - 1) / span;
-    const float endM = t[m * 9 + kM * 3], endI = t[m * 9 + kI * 3], endD = t[m * 9 + kD * 3];
-    for (uint64_t q = slot; q < n_amps; q += (uint64_t)gridDim.x * kWaveWarps) {
-        const uint32_t idx = order[q];
-        const ah_amplicon am = amps[idx];
-        bool ok = am.contig < n_contigs && am.start <= am.end;
-        if (ok)
-            ok = (uint64_t)am.end <= contig_off[am.contig + 1] - contig_off[am.contig] &&
-                 am.end - am.start <= (uint32_t)max_len;
+    constexpr int kVec = K / 4; // float4s of a lane's emissions
+    static_assert(K % 4 == 0, "emissions are read as float4s");
+    extern __shared__ __align__(16) float4 wave_smem[];
+    __shared__ volatile uint64_t rows[kWaveWarps], used[kWaveWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_stripes = (m + span) / span;
+    const int letter_stride = n_stripes * kVec * 32; // float4s
+    float4 *emi = wave_smem;                         // [letter][stripe][vector][lane]
+    float4 *ring = wave_smem + 5 * letter_stride + warp * kWaveRing;
+    float4 *at_end = ring + 64; // the states of the lane of column m at the last row
+    const int seq_stride = ((max_len + 15) & ~15) + 2 * kSeqPad;
+    uint8_t *seq = reinterpret_cast<uint8_t *>(wave_smem + 5 * letter_stride + kWaveWarps * kWaveRing) + warp * seq_stride + kSeqPad;
+    for (int i = threadIdx.x; i < 5 * letter_stride; i += blockDim.x) {
+        const int l = i % 32, c = (i / 32) % kVec, sl = i / (32 * kVec); // sl: letter * n_stripes + stripe
+        const int letter = sl / n_stripes, j0 = (sl % n_stripes) * span + l * K + 4 * c;
+        auto at = [&](int j) { return letter < 4 && j >= 1 && j <= m ? e[j * 4 + letter] : Op::kOne; };
+        emi[i] = make_float4(at(j0), at(j0 + 1), at(j0 + 2), at(j0 + 3));
+    }
+    if (threadIdx.x < kWaveWarps)
+        rows[threadIdx.x] = used[threadIdx.x] = 0;
+    __syncthreads();
+    const int before = (warp + kWaveWarps - 1) % kWaveWarps; // the warp of the previous stripe
+    const uint64_t buffer = (uint64_t)(max_len + 1);
+    auto buffer_of = [&](int w, uint64_t task) {
+        return bnd_all + (((uint64_t)blockIdx.x * kWaveWarps + w) * 2 + (task / kWaveWarps & 1)) * buffer;
+    };
+    const uint64_t n_mine = (n_amps - blockIdx.x + gridDim.x - 1) / gridDim.x; // (gridDim.x <= n_amps)
+    const uint64_t n_tasks = n_mine * n_stripes;
+    bool failed = false; // a wait ran out: reported, and nothing more is waited for
+    uint64_t have = ~0ull; // the amplicon whose letters are in seq
+    int len = 0;
+    uint32_t idx = 0;
+    bool ok = false;
+    for (uint64_t task = warp; task < n_tasks; task += kWaveWarps) {
+        const uint64_t mine = task / n_stripes;
+        const int s = (int)(task % n_stripes);
+        const bool last_stripe = s + 1 == n_stripes;
+        if (mine != have) {
+            have = mine;
+            idx = order[blockIdx.x + mine * gridDim.x];
+            const ah_amplicon am = amps[idx];
+            ok = am.contig < n_contigs && am.start <= am.end;
+            if (ok)
+                ok = (uint64_t)am.end <= contig_off[am.contig + 1] - contig_off[am.contig] &&
+                     am.end - am.start <= (uint32_t)max_len;
+            len = ok ? (int)(am.end - am.start) : 0;
+            __syncwarp(); // the previous amplicon's letters are no longer read
+            if (ok)
+                decode_letters_warp(am, planes, contig_off, seq, len, lane);
+            __syncwarp();
+        }
         if (!ok) { // checked on the host; reported, not read
             if (lane == 0) {
-                atomicExch(err, kDevBounds);
-                score_out[idx] = kNeg;
+                if (s == 0) {
+                    atomicExch(err, kDevBounds);
+                    score_out[idx] = kNeg;
+                } else {
+                    used[before] = task;
+                }
             }
             continue;
         }
-        const int len = (int)(am.end - am.start);
-        __syncwarp(); // the previous amplicon's letters are no longer read
-        decode_letters_warp(am, planes, contig_off, seq, len, lane);
-        __syncwarp();
-        for (int s = 0; s < n_stripes; ++s) {
-            const int c0 = s * span + lane * K;
-            // scores of the moves into M_j (from j-1), into D_j (from j-1), into I_j (from j); M_j's emissions
-            float toM[K][3], toD[K][3], toI[K][3], em[K][4];
+        float4 *out_rows = buffer_of(warp, task);
+        const float4 *in_rows = buffer_of(before, task - 1); // (s > 0)
+        // the task that used this buffer before has been read
+        if (!last_stripe && task >= 2 * kWaveWarps && (task - 2 * kWaveWarps) % n_stripes + 1 != n_stripes && !failed &&
+            !wait_for(&used[warp], task - 2 * kWaveWarps + 1))
+            failed = true;
+        const int c0 = s * span + lane * K;
+        // the moves into M_j and D_j (from j - 1) and into I_j (from j), by state left
+        float toM[K][3], toI[K][3], toD[K][3];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int j = c0 + k;
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+                toM[k][x] = (j >= 1 && j <= m) ? t[(j - 1) * 9 + x * 3 + kM] : Op::kZero;
+                toD[k][x] = (j >= 1 && j <= m) ? t[(j - 1) * 9 + x * 3 + kD] : Op::kZero;
+                toI[k][x] = (j <= m) ? t[j * 9 + x * 3 + kI] : Op::kZero;
+            }
+        }
+        // this lane's columns at its previous row, and column c0 - 1 there
+        float pM[K], pI[K], pD[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            pM[k] = pI[k] = pD[k] = Op::kZero;
+        float lM = Op::kZero, lI = Op::kZero, lD = Op::kZero;
+        int E = kNoMass;
+        const int lane_m = (m - s * span) / K; // (last stripe) the lane of column m
+        const int steps = len + 1 + (last_stripe ? lane_m : 31);
+        // rows r0 + lane of the previous stripe's boundary, once they are written; each four rows
+        // (one group of steps of lane 0) at one exponent
+        auto boundary = [&](int r0) {
+            const int r = r0 + lane;
+            if (r0 <= len && !failed) {
+                if (!wait_for(&rows[before], task << 20 | (uint64_t)min(r0 + 32, len + 1)))
+                    failed = true;
+                __threadfence_block();
+            }
+            failed = __any_sync(0xffffffffu, failed);
+            float4 v = r <= len && !failed ? in_rows[r]
+                                           : make_float4(Op::kZero, Op::kZero, Op::kZero, __int_as_float(kNoMass));
+            if constexpr (Op::kScaled) {
+                const int x = __float_as_int(v.w);
+                int top = max(x, __shfl_xor_sync(0xffffffffu, x, 1));
+                top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
+                const float f = power_of_two(x - top);
+                v = make_float4(v.x * f, v.y * f, v.z * f, __int_as_float(top));
+            }
+            if (r0 <= len && r0 + 32 > len) { // that was the last of them
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence_block();
+                    used[before] = task;
+                }
+            }
+            return v;
+        };
+        // rows 0..31 in the ring, the next 32 in registers
+        float4 ahead;
+        if (s > 0) {
+            __syncwarp();
+            ring[lane] = boundary(0);
+            ahead = boundary(32);
+            __syncwarp();
+        }
+        const float4 *emi_s = emi + s * kVec * 32 + lane;
+        // emissions of the current row's letter, and the next row's letter (rows below 1 and
+        // above len: unknown)
+        float4 em[kVec];
+#pragma unroll
+        for (int c = 0; c < kVec; ++c)
+            em[c] = emi_s[4 * letter_stride + c * 32];
+        int x_next = seq[-lane];
+        float from_left = 1.0f; // 2^(left lane's exponent - this lane's)
+        auto scale_own = [&](float f) {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                const int j = c0 + k;
-#pragma unroll
-                for (int x = 0; x < 3; ++x) {
-                    toM[k][x] = (j >= 1 && j <= m) ? t[(j - 1) * 9 + x * 3 + 0] : kNeg;
-                    toD[k][x] = (j >= 1 && j <= m) ? t[(j - 1) * 9 + x * 3 + 2] : kNeg;
-                    toI[k][x] = (j <= m) ? t[j * 9 + x * 3 + 1] : kNeg;
-                }
-#pragma unroll
-                for (int l = 0; l < 4; ++l)
-                    em[k][l] = (j >= 1 && j <= m) ? e[j * 4 + l] : 0.0f;
+                pM[k] *= f;
+                pI[k] *= f;
+                pD[k] *= f;
             }
-            float pM[K], pI[K], pD[K]; // this lane's columns at its previous row
+            lM *= f;
+            lI *= f;
+            lD *= f;
+        };
+        // One step.  kFirst: the first 32 steps of a stripe, in which mass reaches each lane for the
+        // first time: exponents are compared in every step.  (Rows below 0: every state is zero,
+        // and so is what the recurrence makes of them; rows above len: unused.)
+        auto step = [&](int st, auto first) {
+            constexpr bool kFirst = decltype(first)::value;
+            // column c0 - 1 at this row: the left lane's latest row, or the previous stripe's boundary
+            float rM = __shfl_up_sync(0xffffffffu, pM[K - 1], 1);
+            float rI = __shfl_up_sync(0xffffffffu, pI[K - 1], 1);
+            float rD = __shfl_up_sync(0xffffffffu, pD[K - 1], 1);
+            int rE = kNoMass;
+            if constexpr (Op::kScaled && kFirst)
+                rE = __shfl_up_sync(0xffffffffu, E, 1);
+            if (lane == 0) {
+                rM = rI = rD = Op::kZero;
+                rE = kNoMass;
+                if (s > 0) {
+                    const float4 v = ring[st & 63];
+                    rM = v.x;
+                    rI = v.y;
+                    rD = v.z;
+                    rE = __float_as_int(v.w);
+                }
+            }
+            // the next row's emissions and the letter after it, for the next step
+            float4 em_next[kVec];
+#pragma unroll
+            for (int c = 0; c < kVec; ++c)
+                em_next[c] = emi_s[x_next * letter_stride + c * 32];
+            x_next = seq[st + 1 - lane];
+            if constexpr (Op::kScaled && kFirst) {
+                const float big = fmaxf(fmaxf(rM, rI), rD);
+                const int level = rE + level_of(big);
+                int d = rE - E;
+                if (level - E > kRise || d > kFar) {
+                    if (level > E && big > 0.0f) { // it outweighs the lane: the lane takes its level
+                        scale_own(power_of_two(max(E - level, -127)));
+                        E = level;
+                        d = rE - E;
+                    }
+                    rM = ldexpf(rM, d);
+                    rI = ldexpf(rI, d);
+                    rD = ldexpf(rD, d);
+                    from_left = 1.0f;
+                } else {
+                    from_left = power_of_two(d);
+                }
+            }
+            if constexpr (Op::kScaled) {
+                rM *= from_left;
+                rI *= from_left;
+                rD *= from_left;
+            }
+            float cM[K], cI[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const float4 v = em[k / 4];
+                const float ex = k % 4 == 0 ? v.x : k % 4 == 1 ? v.y : k % 4 == 2 ? v.z : v.w;
+                cM[k] = Op::ext(Op::acc3(k ? pM[k - 1] : lM, toM[k][kM], k ? pI[k - 1] : lI, toM[k][kI],
+                                         k ? pD[k - 1] : lD, toM[k][kD]),
+                                ex);
+                cI[k] = Op::acc3(pM[k], toI[k][kM], pI[k], toI[k][kI], pD[k], toI[k][kD]);
+            }
+            if constexpr (kFirst)
+                if (st == 0 && s == 0 && lane == 0) { // B = M_0 at row 0
+                    cM[0] = Op::kScaled ? power_of_two(kTop) : Op::kOne;
+                    E = Op::kScaled ? -kTop : E;
+                }
+            // the delete chain along the row
 #pragma unroll
             for (int k = 0; k < K; ++k)
-                pM[k] = pI[k] = pD[k] = kNeg;
-            float lpM = kNeg, lpI = kNeg, lpD = kNeg; // column c0 - 1 at the previous row
-            float oM = kNeg, oI = kNeg, oD = kNeg;    // this lane's last column at its latest row
-            const bool last_stripe = s + 1 == n_stripes;
-            // the previous stripe's boundary, 32 rows per block, row 32 b + lane in each lane:
-            // the block in use and the next one (loaded 32 steps before lane 0 needs it)
-            float bM, bI, bD, nM, nI, nD;
-            auto load_block = [&](int blk, float &M_, float &I_, float &D_) {
-                const int r = blk * 32 + lane;
-                M_ = I_ = D_ = kNeg;
-                if (s > 0 && r <= len) {
-                    M_ = bnd[3 * r];
-                    I_ = bnd[3 * r + 1];
-                    D_ = bnd[3 * r + 2];
-                }
-            };
-            load_block(0, bM, bI, bD);
-            load_block(1, nM, nI, nD);
-            for (int st = 0; st < len + 32; ++st) {
-                const int i = st - lane;
-                // column c0 - 1 at row i: the left lane's latest row, or the previous stripe's boundary
-                float rM = __shfl_up_sync(0xffffffffu, oM, 1);
-                float rI = __shfl_up_sync(0xffffffffu, oI, 1);
-                float rD = __shfl_up_sync(0xffffffffu, oD, 1);
-                if (s > 0) {
-                    const float gM = __shfl_sync(0xffffffffu, bM, st & 31);
-                    const float gI = __shfl_sync(0xffffffffu, bI, st & 31);
-                    const float gD = __shfl_sync(0xffffffffu, bD, st & 31);
-                    if (lane == 0) {
-                        rM = gM;
-                        rI = gI;
-                        rD = gD;
-                    }
-                    if ((st & 31) == 31) { // rows 32 b + 64 .. are not yet overwritten (row r at step r + 31)
-                        bM = nM;
-                        bI = nI;
-                        bD = nD;
-                        load_block((st >> 5) + 2, nM, nI, nD);
-                    }
-                } else if (lane == 0) {
-                    rM = rI = rD = kNeg;
-                }
-                if (i < 0 || i > len)
-                    continue;
-                float cM[K], cI[K], cD[K];
-                if (i == 0) { // B = M_0 at row 0; no letter consumed yet
+                pD[k] = Op::acc3(k ? cM[k - 1] : rM, toD[k][kM], k ? cI[k - 1] : rI, toD[k][kI], k ? pD[k - 1] : rD,
+                                 toD[k][kD]);
 #pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        cM[k] = (c0 + k == 0) ? 0.0f : kNeg;
-                        cI[k] = kNeg;
-                    }
-                } else {
-                    const int x = seq[i - 1];
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        const float qm = k ? pM[k - 1] : lpM, qi = k ? pI[k - 1] : lpI, qd = k ? pD[k - 1] : lpD;
-                        // (a select, not an indexed load: the emission scores stay in registers)
-                        const float ex =
-                            x == 0 ? em[k][0] : x == 1 ? em[k][1] : x == 2 ? em[k][2] : x == 3 ? em[k][3] : 0.0f;
-                        cM[k] = ex + Op::add(Op::add(qm + toM[k][kM], qi + toM[k][kI]), qd + toM[k][kD]);
-                        cI[k] = Op::add(Op::add(pM[k] + toI[k][kM], pI[k] + toI[k][kI]), pD[k] + toI[k][kD]);
-                    }
-                }
-                // the delete chain along the row
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const float lm = k ? cM[k - 1] : rM, li = k ? cI[k - 1] : rI, ld = k ? cD[k - 1] : rD;
-                    cD[k] = Op::add(Op::add(lm + toD[k][kM], li + toD[k][kI]), ld + toD[k][kD]);
-                }
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    pM[k] = cM[k];
-                    pI[k] = cI[k];
-                    pD[k] = cD[k];
-                }
-                lpM = rM;
-                lpI = rI;
-                lpD = rD;
-                oM = cM[K - 1];
-                oI = cI[K - 1];
-                oD = cD[K - 1];
-                if (lane == 31 && !last_stripe) {
-                    bnd[3 * i] = oM;
-                    bnd[3 * i + 1] = oI;
-                    bnd[3 * i + 2] = oD;
-                }
-                if (i == len && last_stripe)
-#pragma unroll
-                    for (int k = 0; k < K; ++k)
-                        if (c0 + k == m)
-                            score_out[idx] = Op::add(Op::add(cM[k] + endM, cI[k] + endI), cD[k] + endD);
+            for (int k = 0; k < K; ++k) {
+                pM[k] = cM[k];
+                pI[k] = cI[k];
             }
-            __syncwarp(); // the stripe's boundary is written before the next stripe reads it
+            lM = rM;
+            lI = rI;
+            lD = rD;
+#pragma unroll
+            for (int c = 0; c < kVec; ++c)
+                em[c] = em_next[c];
+            if (!last_stripe) {
+                if (lane == 31 && st >= 31 && st - 31 <= len)
+                    out_rows[st - 31] = make_float4(pM[K - 1], pI[K - 1], pD[K - 1], __int_as_float(E));
+            } else if (st + 1 == steps && lane == lane_m) { // row len: kept for the end state
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    at_end[k] = make_float4(pM[k], pI[k], pD[k], __int_as_float(E));
+            }
+        };
+        // after every fourth step (its last: st)
+        auto settle = [&](int st) {
+            if ((st & 31) == 31) {
+                if (!last_stripe && lane == 31) { // rows .. st - 31 are written
+                    __threadfence_block();
+                    rows[warp] = (task + 1) << 20 | (uint64_t)min(st - 30, len + 1);
+                }
+                if (s > 0) { // rows st + 1 .. st + 32 into the ring; the block after them
+                    ring[(st + 1 + lane) & 63] = ahead;
+                    ahead = boundary(st + 33);
+                    __syncwarp();
+                }
+            }
+            if constexpr (Op::kScaled) { // the lane's largest mantissa back to 2^kTop
+                float big[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    big[0] = fmaxf(big[0], pM[k]);
+                    big[1] = fmaxf(big[1], pI[k]);
+                    big[2] = fmaxf(big[2], pD[k]);
+                }
+                const float b = fmaxf(fmaxf(big[0], big[1]), big[2]);
+                const int up = b > 0.0f ? max(level_of(b), -126) : 0;
+                scale_own(power_of_two(-up));
+                E += up;
+                // the factor of what comes in during the next four steps
+                int rE = __shfl_up_sync(0xffffffffu, E, 1);
+                if (lane == 0)
+                    rE = s > 0 ? __float_as_int(ring[(st + 1) & 63].w) : kNoMass;
+                if (rE - E > kFar) {
+                    scale_own(power_of_two(max(E - rE, -127)));
+                    E = rE;
+                }
+                from_left = power_of_two(rE - E);
+            }
+        };
+        int st = 0;
+#pragma unroll 1
+        for (; st < 32 && st < steps; ++st) {
+            step(st, std::true_type());
+            if ((st & 3) == 3)
+                settle(st);
         }
+#pragma unroll 1
+        for (; st < steps; st += 4) { // (up to three steps more than needed)
+            step(st, std::false_type());
+            step(st + 1, std::false_type());
+            step(st + 2, std::false_type());
+            step(st + 3, std::false_type());
+            settle(st + 3);
+        }
+        if (!last_stripe) {
+            if (lane == 31) { // every row is written
+                __threadfence_block();
+                rows[warp] = (task + 1) << 20 | (uint64_t)(len + 1);
+            }
+        } else {
+            __syncwarp();
+            if (lane == 0) {
+                const float4 v = at_end[(m - s * span) % K];
+                const float endM = t[m * 9 + kM * 3], endI = t[m * 9 + kI * 3], endD = t[m * 9 + kD * 3];
+                float sum = Op::acc(Op::acc(Op::ext(v.x, endM), v.y, endI), v.z, endD);
+                if constexpr (Op::kScaled) {
+                    int x = 0;
+                    const float f = frexpf(sum, &x);
+                    sum = sum > 0.0f ? (float)((double)log2f(f) + (double)(x + __float_as_int(v.w))) : kNeg;
+                }
+                score_out[idx] = sum;
+            }
+        }
+        __syncwarp();
     }
+    if (__any_sync(0xffffffffu, failed) && lane == 0)
+        atomicExch(err, kDevTimeout);
 }
 
-uint64_t wave_blocks(uint64_t n, int max_len, int sms)
-{
-    const uint64_t per_block = (uint64_t)kWaveWarps * 3ull * (uint64_t)(max_len + 1) * sizeof(float);
-    uint64_t b = std::min<uint64_t>((n + kWaveWarps - 1) / kWaveWarps, (uint64_t)sms * kWaveBlocksPerSm);
-    b = std::min<uint64_t>(b, std::max<uint64_t>((uint64_t)sms, kWaveScratchMax / per_block));
-    return std::max<uint64_t>(b, 1);
-}
+// columns per lane: 4 holds up to 128 columns in one stripe; above that 8 halves the steps
+bool wave_narrow(int m) { return m + 1 <= 128; }
+int wave_stripes(int m) { return wave_narrow(m) ? 1 : (m + 256) / 256; }
+constexpr int kWaveBlocksPerSm = 4; // most blocks per SM (the register budgets of the kernels)
 
 template <class Op, int K>
 void launch_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n, const uint32_t *planes,
                  const uint64_t *contig_off, uint32_t n_contigs, const float *t, const float *e, int m, int max_len,
-                 float *bnd, float *out, int *err, int sms, cudaStream_t s)
+                 float4 *bnd, uint64_t blocks, float *out, int *err, int sms, cudaStream_t s)
 {
-    const size_t smem = (size_t)kWaveWarps * (size_t)((max_len + 15) & ~15);
-    AH_CUDA(cudaFuncSetAttribute(hmm_wave_kernel<Op, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)std::max<size_t>(smem, 1)));
-    const uint64_t blocks = wave_blocks(n, max_len, sms);
+    const size_t smem = (size_t)5 * wave_stripes(m) * 32 * K * sizeof(float) +
+                        (size_t)kWaveWarps * kWaveRing * sizeof(float4) +
+                        (size_t)kWaveWarps * (size_t)(((max_len + 15) & ~15) + 2 * kSeqPad);
+    AH_CUDA(cudaFuncSetAttribute(hmm_wave_kernel<Op, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 1;
+    AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hmm_wave_kernel<Op, K>, 32 * kWaveWarps, smem));
+    blocks = std::min<uint64_t>(blocks, (uint64_t)sms * (uint64_t)std::max(1, per_sm));
     hmm_wave_kernel<Op, K><<<(unsigned)blocks, 32 * kWaveWarps, smem, s>>>(amps, order, n, planes, contig_off,
                                                                            n_contigs, t, e, m, max_len, bnd, out, err);
     AH_CUDA(cudaGetLastError());
@@ -693,37 +946,45 @@ void launch_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n, con
 
 } // namespace
 
-size_t hmm_scratch_bytes(uint64_t n, int max_len, int sms)
+// One block per amplicon up to a full GPU; a profile of one stripe runs an amplicon per warp.
+uint64_t hmm_wave_blocks(uint64_t n, int m, int max_len, int sms)
 {
-    return wave_blocks(n, max_len, sms) * (uint64_t)kWaveWarps * 3ull * (uint64_t)(max_len + 1) * sizeof(float);
+    uint64_t b = std::min<uint64_t>(wave_stripes(m) == 1 ? (n + kWaveWarps - 1) / kWaveWarps : n,
+                                    (uint64_t)sms * kWaveBlocksPerSm);
+    const uint64_t per_block = hmm_scratch_bytes(1, m, max_len);
+    if (per_block)
+        b = std::min<uint64_t>(b, std::max<uint64_t>((uint64_t)sms, kWaveScratchMax / per_block));
+    return std::max<uint64_t>(b, 1);
 }
 
-bool hmm_use_wave(bool forward)
+size_t hmm_scratch_bytes(uint64_t blocks, int m, int max_len)
 {
-    // measured on 639 columns x 5,023 amplicons: Forward 108 GCUPS on the wavefront against 91 on
-    // the block kernel; Viterbi 310 against 457
+    return wave_stripes(m) == 1 ? 0 : blocks * kWaveWarps * 2ull * (uint64_t)(max_len + 1) * sizeof(float4);
+}
+
+bool hmm_use_wave()
+{
     const char *kern = getenv("AH_HMM_KERNEL");
-    if (kern && strcmp(kern, "rows") == 0)
-        return false;
-    if (kern && strcmp(kern, "wave") == 0)
-        return true;
-    return forward;
+    return !(kern && strcmp(kern, "rows") == 0);
 }
 
 void launch_hmm_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n, const uint32_t *planes,
-                     const uint64_t *contig_off, uint32_t n_contigs, const float *t, const float *e, int m,
-                     int max_len, bool forward, float *bnd, float *score_out, int *err, int sms, cudaStream_t s)
+                     const uint64_t *contig_off, uint32_t n_contigs, const HmmProfile &p, int max_len, bool forward,
+                     void *bnd, uint64_t blocks, float *score_out, int *err, int sms, cudaStream_t s)
 {
     if (n == 0)
         return;
-    if (m + 1 > kHmmMaxColumns)
+    if (p.m + 1 > kHmmMaxColumns)
         throw Error(AH_ERR_ARG, "ah_hmm_score: profile longer than " + std::to_string(kHmmMaxColumns) + " columns");
+    blocks = std::min<uint64_t>(blocks, n);
+    auto go = [&](auto *launch) {
+        launch(amps, order, n, planes, contig_off, n_contigs, forward ? p.d_t_odds : p.d_t,
+               forward ? p.d_e_odds : p.d_e, p.m, max_len, (float4 *)bnd, blocks, score_out, err, sms, s);
+    };
     if (forward)
-        launch_wave<LogSum, 4>(amps, order, n, planes, contig_off, n_contigs, t, e, m, max_len, bnd, score_out, err,
-                               sms, s);
+        wave_narrow(p.m) ? go(launch_wave<WaveSum, 4>) : go(launch_wave<WaveSum, 8>);
     else
-        launch_wave<MaxSum, 4>(amps, order, n, planes, contig_off, n_contigs, t, e, m, max_len, bnd, score_out, err,
-                               sms, s);
+        wave_narrow(p.m) ? go(launch_wave<WaveMax, 4>) : go(launch_wave<WaveMax, 8>);
 }
 
 void launch_hmm_score(const ah_amplicon *amps, const uint32_t *order, uint64_t n, const uint32_t *planes,

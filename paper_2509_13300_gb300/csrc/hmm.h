@@ -7,20 +7,21 @@
 
 namespace ah {
 
-// True when a score (Forward if `forward`, else Viterbi) runs on the warp
-// wavefront: by default the Forward scores; AH_HMM_KERNEL=wave or =rows forces
-// one kernel for both scores (a profiling aid).
-bool hmm_use_wave(bool forward);
+// False when AH_HMM_KERNEL=rows asks for the block-per-group kernel (a profiling aid).
+bool hmm_use_wave();
 
-// Device scratch of launch_hmm_wave in bytes: one stripe-boundary buffer of
-// 3 * (max_len + 1) floats per warp of its grid (at most 256 MB beyond one
-// block per SM).
-size_t hmm_scratch_bytes(uint64_t n, int max_len, int sms);
+// Blocks the wavefront takes for n amplicons of at most max_len letters, and the
+// device scratch of `blocks` of them in bytes: two stripe-boundary buffers of
+// max_len + 1 float4s per warp (none for a profile of one stripe; at most
+// 256 MB beyond one block per SM).
+uint64_t hmm_wave_blocks(uint64_t n, int m, int max_len, int sms);
+size_t hmm_scratch_bytes(uint64_t blocks, int m, int max_len);
 
 // The scores of n amplicons, as launch_hmm_score computes them, by the warp
-// wavefront; bnd holds hmm_scratch_bytes(n, max_len, sms) bytes.
+// wavefront in at most `blocks` blocks (any number from 1); bnd holds
+// hmm_scratch_bytes(blocks, m, max_len) bytes.
 void launch_hmm_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n, const uint32_t *planes,
-                     const uint64_t *contig_off, uint32_t n_contigs, const float *t, const float *e, int m,
-                     int max_len, bool forward, float *bnd, float *score_out, int *err, int sms, cudaStream_t s);
+                     const uint64_t *contig_off, uint32_t n_contigs, const HmmProfile &p, int max_len, bool forward,
+                     void *bnd, uint64_t blocks, float *score_out, int *err, int sms, cudaStream_t s);
 
 } // namespace ah

@@ -1245,3 +1245,49 @@ def test_profile_hmm_kernels_on_profiles_of_several_lengths(ctx, kernel, monkeyp
             assert (err_f <= tol_f).all(), (cut, kernel, err_f.max(), int(err_f.argmax()))
     finally:
         ctx.ah_unload_genomes(sid)
+
+
+@pytest.mark.parametrize("m,n", [(1, 3), (127, 9), (128, 1), (255, 700), (256, 5), (257, 13), (511, 40), (1100, 3)])
+def test_profile_hmm_wavefront_stripes_and_tasks(ctx, m, n):
+    """The wavefront at its stripes' edges (a narrow profile of at most 128 columns, stripes of
+    256: full, one column over), with fewer and more amplicons than blocks, from empty to longer
+    than the profile, and under a memory budget that leaves it few blocks' buffers: Viterbi and
+    Forward against the oracle in fp64."""
+    rng = np.random.default_rng(m * 1000 + n)
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    ref = acgt[rng.integers(0, 4, m)].tobytes().decode()
+    train = [ref, ref] + [synth._mutate(rng, ref, 0.03, 0.02) or "A" for _ in range(6)]
+    seqs = [synth._mutate(rng, ref, 0.05, 0.03) for _ in range(n)]
+    seqs[0] = ""
+    if n > 2:
+        seqs[1] = acgt[rng.integers(0, 4, 2 * m + 70)].tobytes().decode()  # unrelated and longer
+        seqs[2] = ref[m // 2:] + "N" + ref[:m // 3]
+    body = "".join(seqs) + "A"
+    seq = np.frombuffer(body.encode(), np.uint8).copy()
+    off = np.array([0, len(seq)], np.uint64)
+    amps = np.zeros(n, dtype=ah.AMPLICON_DTYPE)
+    ends = np.cumsum([len(x) for x in seqs])
+    amps["end"], amps["start"] = ends, ends - [len(x) for x in seqs]
+    ref_i, T, E = oracle.hmm_build(train)
+    some = np.unique(np.concatenate([np.arange(min(n, 6)), rng.integers(0, n, 6)]))
+    want = np.array([oracle.hmm_viterbi(T, E, seqs[i]) for i in some])
+    want_f = np.array([oracle.hmm_forward(T, E, seqs[i]) for i in some])
+    got = {}
+    with ah.Context(0, 12 << 20) as small:  # boundary buffers get at most 1/16 of it
+        for name, c in (("full", ctx), ("budget", small)):
+            sid = c.load(seq, off, np.zeros(1, np.uint32))
+            hid = c.hmm_build(train)
+            got[name] = c.hmm_score(sid, hid, amps), c.hmm_forward(sid, hid, amps)
+            c.hmm_free(hid)
+            c.ah_unload_genomes(sid)
+    # the bound of the parity test above: ten standard deviations of a walk of fp32 roundings
+    fin = ~np.isinf(T)
+    pmean = float(np.concatenate([np.abs(T[fin]), np.abs(E[1:]).ravel()]).mean())
+    N = np.array([len(seqs[i]) for i in some]) + len(T) - 1
+    for v, f in got.values():
+        tol = 10.0 * np.sqrt(N) * 2.0 ** -24 * (np.abs(want) + N * pmean) + 1e-4
+        assert (np.abs(v[some].astype(np.float64) - want) <= tol).all()
+        tol_f = 10.0 * np.sqrt(N) * (2.0 ** -24 * (np.abs(want_f) + N * pmean) + 4 * 2.0 ** -23) + 1e-4
+        assert (np.abs(f[some].astype(np.float64) - want_f) <= tol_f).all()
+    every = 1e-4 + 1e-5 * np.abs(got["full"][0])
+    assert (np.abs(got["full"][0] - got["budget"][0]) <= every).all()  # also the amplicons the oracle did not score
