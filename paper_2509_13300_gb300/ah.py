@@ -337,19 +337,15 @@ class Context:
 
     def amplitypes(self, set_id: int, amplicons: np.ndarray, stream=None):
         """(variant id per amplicon, rows [genome, amplitype, n_amplicons, n_variants] per genome with
-        amplicons, number of variants, number of amplitypes) -- size query, then the call."""
+        amplicons, number of variants, number of amplitypes)."""
         n = len(amplicons)
         variant = np.zeros(max(n, 1), dtype=np.uint32)
+        rows = np.empty((max(n, 1), 4), dtype=np.uint32)  # at most one row per amplicon
         nr, nv, nt = ctypes.c_uint64(), ctypes.c_uint64(), ctypes.c_uint64()
-        st = self._lib.ah_amplitypes(self.h, set_id, _ptr(amplicons) if n else None, n, None, None, 0,
-                                     ctypes.byref(nr), ctypes.byref(nv), ctypes.byref(nt), _stream(stream))
-        if st not in (AH_OK, AH_ERR_OVERFLOW):
-            self._check(st)
-        rows = np.zeros((max(nr.value, 1), 4), dtype=np.uint32)
         self._check(self._lib.ah_amplitypes(self.h, set_id, _ptr(amplicons) if n else None, n, _ptr(variant),
-                                            _ptr(rows), nr.value, ctypes.byref(nr), ctypes.byref(nv),
+                                            _ptr(rows), n, ctypes.byref(nr), ctypes.byref(nv),
                                             ctypes.byref(nt), _stream(stream)))
-        return variant[:n], rows[:nr.value], nv.value, nt.value
+        return variant[:n], rows[:nr.value].copy(), nv.value, nt.value
 
     def generate_bases(self, coll, base0: int, n: int, out, stream=None, tables=None):
         """Bases [base0, base0 + n) of a countergen collection into device memory `out` (torch uint8).

@@ -883,7 +883,7 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
     }
     {
         Stage sg(c, "pair", st, 3);
-        launch_pair_count(sites, ns_max, F + kFlagSites, filt, pd, counts, st);
+        launch_pair_count(sites, ns_max, F + kFlagSites, filt, pd, counts, nullptr, st);
         exclusive_scan_u64_dev(counts, offs, ns_max, F + kFlagSites, 0, F + kFlagAux, na_max, F + kFlagAmps,
                                F + kFlagRedo, kRedoAmps, st);
         launch_pair_write(sites, ns_max, F + kFlagSites, filt, pd, offs, amps, na_max, F + kFlagRedo, kRedoAmps, st);
@@ -994,7 +994,7 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         void *temp = scratch(c, "scan_temp", tb);
         {
             Stage sg(c, "pair", st, 2 + scan_u64_launches(ns));
-            launch_pair_count(sites, ns, nullptr, filt, pd, counts, st);
+            launch_pair_count(sites, ns, nullptr, filt, pd, counts, nullptr, st);
             exclusive_scan_u64(temp, tb, counts, offs, ns, st);
             launch_total(offs, counts, ns, nullptr, 0, c->d_aux, 0, nullptr, nullptr, 0, st);
         }
@@ -1213,7 +1213,7 @@ void group_device(ah_ctx *c, const GenomeSet &gs, uint32_t pid, int k, const std
     void *temp = scratch(c, "scan_temp", tb);
     {
         Stage sg(c, "pair", st, 2 + scan_u64_launches(ns));
-        launch_pair_count(sites, ns, nullptr, nullptr, pd, counts, st);
+        launch_pair_count(sites, ns, nullptr, nullptr, pd, counts, nullptr, st);
         exclusive_scan_u64(temp, tb, counts, offs, ns, st);
         launch_total(offs, counts, ns, nullptr, 0, c->d_aux, 0, nullptr, nullptr, 0, st);
     }
@@ -2366,8 +2366,7 @@ ah_status ah_tm_sweep(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint
         if (n_sites) {
             Stage sg(c, "validate", st, 1);
             launch_validate_sites(s, n_sites, pd, (int)n_pairs, gs.contig_off, gs.n_contigs, c->d_err, st);
-        }
-        check_flags(c, st);
+        } // (the kernels below leave records that failed it alone; check_flags reports them)
         float *tm = (float *)scratch(c, "sweep_tm", std::max<uint64_t>(n_sites, 1) * sizeof(float));
         if (n_sites) {
             Stage sg(c, "tm", st, 2);
@@ -2416,74 +2415,51 @@ ah_status ah_amplitypes(ah_ctx *c, uint32_t set_id, const ah_amplicon *amplicons
             return;
         reset_flags(c, st);
         const ah_amplicon *a = stage_in(c, "amplitype_in", amplicons, n, st);
-        const uint64_t G = (uint64_t)gs.max_genome + 1;  // genome id range
-        const uint64_t N = std::max<uint64_t>(n, G);     // the largest count a scratch array serves
-        {   // the records lie in the set (checked before any kernel reads planes with them)
-            uint64_t *len = (uint64_t *)scratch(c, "fetch_len", (n + 1) * sizeof(uint64_t));
-            Stage sg(c, "validate", st, 1);
-            launch_fetch_lengths(a, n, nullptr, gs.contig_off, gs.n_contigs, len, c->d_err, st);
-        }
-        check_flags(c, st);
-        AmpliTypeScratch S;
-        S.idx = (uint32_t *)scratch(c, "at_idx", N * 4);
-        S.idx_b = (uint32_t *)scratch(c, "at_idx_b", N * 4);
-        S.run_pos = (uint32_t *)scratch(c, "at_run_pos", N * 4);
-        S.keys_a = (uint64_t *)scratch(c, "at_keys_a", N * 8);
-        S.keys_b = (uint64_t *)scratch(c, "at_keys_b", N * 8);
-        S.keys_s = (uint64_t *)scratch(c, "at_keys_s", N * 8);
-        S.head = (uint64_t *)scratch(c, "at_head", N * 8);
-        S.head_excl = (uint64_t *)scratch(c, "at_head_excl", N * 8);
-        S.is_first = (uint64_t *)scratch(c, "at_is_first", N * 8);
-        S.rank = (uint64_t *)scratch(c, "at_rank", N * 8);
-        S.temp_bytes = AmpliTypeScratch::cub_bytes(N);
-        S.temp = scratch(c, "at_cub", S.temp_bytes);
-        S.scan_bytes = scan_u64_temp_bytes(N);
+        const uint64_t G = (uint64_t)gs.max_genome + 1; // genome id range
+        const uint64_t R = std::min(n, G);              // most rows
+        AmpliScratch S;
+        S.t.size = amplitype_slots(n);
+        S.ones_bytes = S.t.size * 28;
+        S.ones = scratch(c, "at_ones", S.ones_bytes);
+        S.t.k1 = (unsigned long long *)S.ones;
+        S.t.k2 = S.t.k1 + S.t.size;
+        S.t.pair_key = S.t.k2 + S.t.size;
+        S.t.first = (unsigned int *)(S.t.pair_key + S.t.size);
+        S.zeros_bytes = G * 24 + S.t.size * 4;
+        S.zeros = scratch(c, "at_zeros", S.zeros_bytes);
+        S.g1 = (unsigned long long *)S.zeros;
+        S.g2 = S.g1 + G;
+        S.gamp = (unsigned int *)(S.g2 + G);
+        S.gvar = S.gamp + G;
+        S.t.pair_n = S.gvar + G;
+        S.slot = (uint32_t *)scratch(c, "at_slot", n * 4);
+        S.variant = (uint32_t *)scratch(c, "at_variant", n * 4);
+        S.flag = (uint64_t *)scratch(c, "at_flag", n * 8);
+        S.rank = (uint64_t *)scratch(c, "at_rank", n * 8);
+        S.has = (uint64_t *)scratch(c, "at_has", G * 8);
+        S.pos = (uint64_t *)scratch(c, "at_pos", G * 8);
+        S.gid = (uint32_t *)scratch(c, "at_gid", R * 4);
+        S.rows = (ah_genome_amplitype *)scratch(c, "at_rows", R * sizeof(ah_genome_amplitype));
+        S.scan_bytes = scan_u64_temp_bytes(std::max(n, G));
         S.scan_temp = scratch(c, "scan_temp", S.scan_bytes);
-        uint64_t *h1 = (uint64_t *)scratch(c, "at_h1", n * 8), *h2 = (uint64_t *)scratch(c, "at_h2", n * 8);
-        uint32_t *variant = (uint32_t *)scratch(c, "at_variant", n * 4);
-        uint64_t *counts = c->d_flags + kFlagSites; // three device words: variants, genome runs, rows
+        uint64_t *counts = c->d_flags + kFlagSites; // three device words: variants, rows, amplitypes
         {
-            Stage sg(c, "amplitype", st, 1);
-            launch_amp_hash(a, n, gs.planes, gs.contig_off, h1, h2, st);
-            S.sort_by(h1, h2, n, st);
-            S.ids(n, variant, counts + 0, st); // sequence variants
-            launch_genome_key(a, variant, n, gs.contig_genome, h1, c->d_err, st); // h1 reused for the keys
-            S.sort_by(h1, nullptr, n, st);
-            S.ids(n, nullptr, counts + 1, st); // (genome, variant) runs
-            auto *g1 = (unsigned long long *)scratch(c, "at_g1", G * 8);
-            auto *g2 = (unsigned long long *)scratch(c, "at_g2", G * 8);
-            auto *gamp = (unsigned int *)scratch(c, "at_gamp", G * 4);
-            auto *gvar = (unsigned int *)scratch(c, "at_gvar", G * 4);
-            AH_CUDA(cudaMemsetAsync(g1, 0, G * 8, st));
-            AH_CUDA(cudaMemsetAsync(g2, 0, G * 8, st));
-            AH_CUDA(cudaMemsetAsync(gamp, 0, G * 4, st));
-            AH_CUDA(cudaMemsetAsync(gvar, 0, G * 4, st));
-            S.genome_sums(n, counts + 1, g1, g2, gamp, gvar, st);
-            uint32_t *gid = (uint32_t *)scratch(c, "at_gid", G * 4);
-            uint64_t *k1 = (uint64_t *)scratch(c, "at_k1", G * 8), *k2 = (uint64_t *)scratch(c, "at_k2", G * 8);
-            uint64_t *has = (uint64_t *)scratch(c, "at_has", G * 8), *pos = (uint64_t *)scratch(c, "at_pos", G * 8);
-            launch_genome_compact(gamp, G, has, pos, S.scan_temp, S.scan_bytes, g1, g2, gid, k1, k2, counts + 2, st);
-            check_flags(c, st);
-            const uint64_t m = c->h_flags[kFlagSites + 2];
-            const uint64_t nv = c->h_flags[kFlagSites + 0];
-            *n_rows_out = m;
-            *n_variants_out = nv;
-            uint32_t *type = (uint32_t *)scratch(c, "at_type", std::max<uint64_t>(m, 1) * 4);
-            S.sort_by(k1, k2, m, st);
-            S.ids(m, type, counts + 1, st); // amplitypes, first occurrence in ascending genome order
-            ah_genome_amplitype *r = out_buf(c, "at_rows", rows, m <= cap ? m : 0);
-            if (m <= cap)
-                launch_amplitype_rows(gid, type, m, gamp, gvar, r, st);
-            if (variant_out)
-                AH_CUDA(cudaMemcpyAsync(variant_out, variant, n * 4, cudaMemcpyDefault, st));
-            check_flags(c, st);
-            *n_amplitypes_out = c->h_flags[kFlagSites + 1];
-            if (m > cap)
-                throw Error(AH_ERR_OVERFLOW, "ah_amplitypes: " + std::to_string(m) + " genomes with amplicons, capacity " +
-                                                 std::to_string(cap));
-            out_finish(rows, r, m, st);
-            AH_CUDA(cudaStreamSynchronize(st));
+            Stage sg(c, "amplitype", st, amplitype_launches(n, G));
+            launch_amplitypes(a, n, gs.planes, gs.contig_off, gs.contig_genome, gs.n_contigs, G, S, counts, c->d_err, st);
         }
+        check_flags(c, st); // (a bad record, before anything is written to the caller)
+        const uint64_t m = c->h_flags[kFlagSites + 1];
+        *n_variants_out = c->h_flags[kFlagSites + 0];
+        *n_rows_out = m;
+        *n_amplitypes_out = c->h_flags[kFlagSites + 2];
+        if (variant_out)
+            AH_CUDA(cudaMemcpyAsync(variant_out, S.variant, n * 4, cudaMemcpyDefault, st));
+        if (m && m <= cap)
+            AH_CUDA(cudaMemcpyAsync(rows, S.rows, m * sizeof(ah_genome_amplitype), cudaMemcpyDefault, st));
+        AH_CUDA(cudaStreamSynchronize(st));
+        if (m > cap)
+            throw Error(AH_ERR_OVERFLOW, "ah_amplitypes: " + std::to_string(m) + " genomes with amplicons, capacity " +
+                                             std::to_string(cap));
     });
 }
 
@@ -2563,8 +2539,7 @@ ah_status ah_tm(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t n
         {
             Stage sg(c, "validate", st, 1);
             launch_validate_sites(s, n, pd, (int)n_pairs, gs.contig_off, gs.n_contigs, c->d_err, st);
-        }
-        check_flags(c, st);
+        } // (the Tm kernels leave records that failed it alone; check_flags reports them)
         float *tm = out_buf(c, "tm_out", tm_out, n);
         uint8_t *ps = pass_out ? out_buf(c, "pass_out", pass_out, n) : nullptr;
         {
@@ -2574,10 +2549,13 @@ ah_status ah_tm(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t n
                       (uint32_t *)(c->d_flags + kFlagTmQueue), tm_seg_max(c),
                       tm_few_exact(c), c->d_err, st);
         }
-        out_finish(tm_out, tm, n, st);
-        if (pass_out)
-            out_finish(pass_out, ps, n, st);
         check_flags(c, st);
+        if (tm != tm_out || ps != pass_out) {
+            out_finish(tm_out, tm, n, st);
+            if (pass_out)
+                out_finish(pass_out, ps, n, st);
+            AH_CUDA(cudaStreamSynchronize(st));
+        }
     });
 }
 
@@ -2603,21 +2581,18 @@ ah_status ah_pair(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t
             Stage sg(c, "validate", st, 1);
             launch_validate_sites(s, n, pd, (int)n_pairs, gs.contig_off, gs.n_contigs, c->d_err, st);
         }
-        check_flags(c, st);
         uint64_t *counts = (uint64_t *)scratch(c, "pair_counts", n * sizeof(uint64_t));
         uint64_t *offs = (uint64_t *)scratch(c, "pair_offsets", n * sizeof(uint64_t));
         size_t tb = scan_u64_temp_bytes(n);
         void *temp = scratch(c, "scan_temp", tb);
         {
-            Stage sg(c, "pair", st, 1 + scan_u64_launches(n));
-            launch_pair_count(s, n, nullptr, ps, pd, counts, st);
+            Stage sg(c, "pair", st, 2 + scan_u64_launches(n));
+            launch_pair_count(s, n, nullptr, ps, pd, counts, c->d_err, st);
             exclusive_scan_u64(temp, tb, counts, offs, n, st);
+            launch_total(offs, counts, n, nullptr, 0, c->d_aux, 0, nullptr, nullptr, 0, st);
         }
-        uint64_t last[2] = {0, 0};
-        AH_CUDA(cudaMemcpyAsync(&last[0], offs + n - 1, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-        AH_CUDA(cudaMemcpyAsync(&last[1], counts + n - 1, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-        AH_CUDA(cudaStreamSynchronize(st));
-        const uint64_t total = last[0] + last[1];
+        check_flags(c, st); // the records' check and the count
+        const uint64_t total = c->h_flags[kFlagAux];
         *n_out = total;
         if (total > cap)
             throw Error(AH_ERR_OVERFLOW, "ah_pair: " + std::to_string(total) + " amplicons, capacity " +
@@ -2656,12 +2631,13 @@ ah_status ah_fetch(ah_ctx *c, uint32_t set_id, const ah_amplicon *amplicons, uin
             Stage sg(c, "fetch", st, (n ? 1 : 0) + scan_u64_launches(n + 1));
             launch_fetch_lengths(a, n, nullptr, gs.contig_off, gs.n_contigs, len, c->d_err, st);
             exclusive_scan_u64(temp, tb, len, offs, n + 1, st);
+            AH_CUDA(cudaMemcpyAsync(c->d_aux, offs + n, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
         }
-        check_flags(c, st);
-        uint64_t total = 0;
-        AH_CUDA(cudaMemcpyAsync(&total, offs + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
+        check_flags(c, st); // the records' check and the bytes
+        const uint64_t total = c->h_flags[kFlagAux];
         out_finish(offsets_out, offs, n + 1, st);
-        AH_CUDA(cudaStreamSynchronize(st));
+        if (offs != offsets_out && (total == 0 || total > cap))
+            AH_CUDA(cudaStreamSynchronize(st));
         if (total > cap)
             throw Error(AH_ERR_OVERFLOW, "ah_fetch: " + std::to_string(total) + " bytes needed, capacity " +
                                              std::to_string(cap));

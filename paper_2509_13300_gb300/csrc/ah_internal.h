@@ -295,15 +295,19 @@ void launch_tm_sweep(const ah_site *sites, uint64_t n_sites, const ah_amplicon *
 
 // pair.cu
 // n_dev (here and below): optional device count, min(*n_dev, n) records.
+// err (may be null): a device error word; while it is set the kernel leaves the records alone.
 void launch_pair_count(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, uint64_t *counts, cudaStream_t s);
+                       const PairDev *pairs_d, uint64_t *counts, const int *err, cudaStream_t s);
 // *out = offs[m-1] + counts[m-1] (the total of an exclusive scan over m values,
 // m = n or min(*n_dev + add, n)).  With eff != nullptr also *eff = the total if it
 // is at most cap, else 0 with redo_bit set in *redo.
 void launch_total(const uint64_t *offs, const uint64_t *counts, uint64_t n, const uint64_t *n_dev, uint64_t add,
                   uint64_t *out, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit, cudaStream_t s);
 size_t scan_u64_temp_bytes(uint64_t n);
-// Exclusive scan of n u64 values; one block (no temporary) for n <= kSmallScan, CUB above.
+// Exclusive scan of n u64 values; one block (no temporary) for n <= kOneBlockScan, CUB above
+// (36,000 values on a GB300: one block 27 us, CUB's two launches 9).
+constexpr uint64_t kOneBlockScan = 8192;
+// Most values of a scan whose count is known on the device only (one block).
 constexpr uint64_t kSmallScan = 65536;
 // number of kernels exclusive_scan_u64 launches for n values
 int scan_u64_launches(uint64_t n);
@@ -318,37 +322,36 @@ void launch_pair_write(const ah_site *sites, uint64_t n, const uint64_t *n_dev, 
                        const PairDev *pairs_d, const uint64_t *offsets, ah_amplicon *out, uint64_t cap,
                        const uint64_t *skip, uint64_t skip_bit, cudaStream_t s);
 
-// amplitype.cu: sequence variants and amplitypes.  Every array holds at
-// least the largest count it serves (amplicons, or genomes with amplicons).
-struct AmpliTypeScratch {
-    uint32_t *idx = nullptr, *idx_b = nullptr, *run_pos = nullptr;
-    uint64_t *keys_a = nullptr, *keys_b = nullptr, *keys_s = nullptr;
-    uint64_t *head = nullptr, *head_excl = nullptr, *is_first = nullptr, *rank = nullptr;
-    bool keys_b_valid = false;
-    void *temp = nullptr; // CUB sort storage
-    size_t temp_bytes = 0;
-    void *scan_temp = nullptr; // CUB scan storage (more than kSmallScan values)
-    size_t scan_bytes = 0;
-    // stable sort of the element indices by (ka, kb) (kb may be null)
-    void sort_by(const uint64_t *ka, const uint64_t *kb, uint64_t n, cudaStream_t s);
-    // runs of equal keys after sort_by; with id_out, first-occurrence ids per element
-    void ids(uint64_t n, uint32_t *id_out, uint64_t *n_runs_dev, cudaStream_t s);
-    // after sort_by + ids over (genome << 32 | variant) keys: per-genome multiset sums and counts
-    void genome_sums(uint64_t n, const uint64_t *n_runs_dev, unsigned long long *g1, unsigned long long *g2,
-                     unsigned int *gamp, unsigned int *gvar, cudaStream_t s);
-    static size_t cub_bytes(uint64_t n);
+// amplitype.cu: sequence variants and amplitypes.  Two hash tables of `size`
+// slots: variants (and then amplitypes) with the first index seen, and
+// (genome, variant) with its copies.
+struct AmpliTables {
+    uint64_t size;
+    unsigned long long *k1, *k2;  // keys (all ones: free)
+    unsigned int *first;          // smallest index
+    unsigned long long *pair_key; // genome << 32 | variant
+    unsigned int *pair_n;         // copies
 };
-void launch_amp_hash(const ah_amplicon *a, uint64_t n, const uint32_t *planes, const uint64_t *contig_off,
-                     uint64_t *h1, uint64_t *h2, cudaStream_t s);
-// key (genome << 32 | variant) per amplicon; an amplicon whose genome differs
-// from its contig's, or with orientation > 3, sets *err = kDevBounds
-void launch_genome_key(const ah_amplicon *a, const uint32_t *variant, uint64_t n, const uint32_t *contig_genome,
-                       uint64_t *keys, int *err, cudaStream_t s);
-void launch_genome_compact(const unsigned int *gamp, uint64_t n_ids, uint64_t *has, uint64_t *pos, void *scan_temp,
-                           size_t scan_bytes, const unsigned long long *g1, const unsigned long long *g2, uint32_t *gid,
-                           uint64_t *k1, uint64_t *k2, uint64_t *n_out_dev, cudaStream_t s);
-void launch_amplitype_rows(const uint32_t *gid, const uint32_t *type, uint64_t m, const unsigned int *gamp,
-                           const unsigned int *gvar, ah_genome_amplitype *rows, cudaStream_t s);
+struct AmpliScratch {
+    AmpliTables t;
+    void *ones, *zeros; // the tables' keys and first indices in one block; pair_n and the genomes' sums in another
+    size_t ones_bytes, zeros_bytes;
+    uint32_t *slot, *variant;                      // per amplicon
+    uint64_t *flag, *rank;                         // per amplicon
+    unsigned long long *g1, *g2;                   // per genome id
+    unsigned int *gamp, *gvar;                     // per genome id: amplicons, variants
+    uint64_t *has, *pos;                           // per genome id
+    uint32_t *gid;                                 // per row (at most min(n, n_ids))
+    ah_genome_amplitype *rows;                     // per row
+    void *scan_temp;
+    size_t scan_bytes;
+};
+uint64_t amplitype_slots(uint64_t n);
+// counts (device): variants, rows, amplitypes.  A bad record sets *err = kDevBounds.
+void launch_amplitypes(const ah_amplicon *a, uint64_t n, const uint32_t *planes, const uint64_t *contig_off,
+                       const uint32_t *contig_genome, uint32_t n_contigs, uint64_t n_ids, const AmpliScratch &S,
+                       uint64_t *counts, int *err, cudaStream_t s);
+int amplitype_launches(uint64_t n, uint64_t n_ids);
 
 // gen.cu: counter-based synthetic bases (device segments and patches)
 void launch_generate_bases(const ah_gen_segment *segs, uint64_t n_segs, uint64_t seed, const uint64_t *patch_pos,

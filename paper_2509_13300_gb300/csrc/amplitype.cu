@@ -4,17 +4,24 @@
 //
 // Variants: each amplicon's sequence (as ah_fetch returns it: RF reverse-
 // complemented, N for any non-ACGT letter) is hashed straight from the packed
-// planes with two polynomial hashes modulo the Mersenne prime 2^61 - 1 (one
-// warp per amplicon, lanes hash contiguous pieces combined by powers of the
-// base); amplicons with equal hash pairs are one variant.  Variants, and then
-// amplitypes, are numbered by first occurrence: stable radix sorts on the
-// hashes keep equal keys in input order, so the head of each run of equal
-// keys is its first occurrence, and the ranks of the heads in input order are
-// the ids.  Amplitype of a genome: the multiset of (variant, copies), hashed
-// as a sum of mixed 64-bit words per (variant, copies) pair (two independent
-// sums, order-free), then grouped the same way over the genomes in ascending
-// genome order.
-#include <cub/device/device_radix_sort.cuh>
+// planes with two polynomial hashes modulo the Mersenne prime 2^61 - 1;
+// amplicons with equal hash pairs are one variant.  Variants, and then
+// amplitypes, are numbered by first occurrence: every element enters a hash
+// table in device memory (open addressing) that keeps the smallest index seen
+// per key, so the elements that are their key's smallest are the first
+// occurrences, and their ranks in input order are the ids.  Which slot a key
+// lands in depends on the order of arrival, the ids do not.  Amplitype of a
+// genome: the multiset of (variant, copies), hashed as a sum of mixed 64-bit
+// words per (variant, copies) pair (two independent sums, order-free), the
+// copies counted in a second table keyed by (genome, variant).
+//
+// Bound: launches, memory latency and, in the hashing, the extraction of single
+// bits from the planes.  Measured on a GB300, 65,000 amplicons of ~1,500 letters:
+// hashing 399 us (a lane per 1/32 of an amplicon, letter by letter) -> 122; the
+// rest of a call 3 x 16 radix-sort passes and ~60 small launches, 0.7 ms -> 15
+// launches, 0.13 ms.  (Fewer blocks for the kernels that enter a table, so that
+// common keys are entered before most elements look: 39 -> 58 us, not kept.)
+#include <algorithm>
 
 #include "ah_internal.h"
 
@@ -24,8 +31,9 @@ namespace {
 constexpr uint64_t kM61 = (1ull << 61) - 1;
 constexpr uint64_t kB1 = 0x1d2e3f4a5b6c7d8ull % kM61; // hash bases (any values in [2, 2^61 - 2])
 constexpr uint64_t kB2 = 0x0f1e2d3c4b5a697ull % kM61;
+constexpr unsigned long long kEmpty = ~0ull;
 
-__device__ __forceinline__ uint64_t mod61(uint64_t x)
+__host__ __device__ constexpr uint64_t mod61(uint64_t x)
 {
     x = (x & kM61) + (x >> 61);
     return x >= kM61 ? x - kM61 : x;
@@ -38,17 +46,26 @@ __device__ __forceinline__ uint64_t mulmod61(uint64_t a, uint64_t b)
     return mod61((lo & kM61) + (lo >> 61) + (hi << 3));
 }
 
-__device__ uint64_t powmod61(uint64_t b, uint64_t e)
+// base^(31 - lane) for the 32 lanes and, last, base^32 (built at compile time)
+constexpr uint64_t mul61(uint64_t a, uint64_t b)
 {
-    uint64_t r = 1;
-    while (e) {
-        if (e & 1)
-            r = mulmod61(r, b);
-        b = mulmod61(b, b);
-        e >>= 1;
-    }
-    return r;
+    const unsigned __int128 p = (unsigned __int128)a * b;
+    return mod61((uint64_t)(p & kM61) + (uint64_t)(p >> 61));
 }
+struct Powers {
+    uint64_t v[33];
+};
+constexpr Powers powers(uint64_t base)
+{
+    Powers p{};
+    p.v[31] = 1;
+    for (int i = 30; i >= 0; --i)
+        p.v[i] = mul61(p.v[i + 1], base);
+    p.v[32] = mul61(p.v[0], base);
+    return p;
+}
+__constant__ Powers kPow1 = powers(kB1);
+__constant__ Powers kPow2 = powers(kB2);
 
 // 64-bit finaliser of the SplitMix generator (Steele, Lea and Flood, 2014)
 __device__ __forceinline__ uint64_t mix64(uint64_t x)
@@ -61,121 +78,203 @@ __device__ __forceinline__ uint64_t mix64(uint64_t x)
     return x;
 }
 
-__device__ __forceinline__ int plane_code(const uint32_t *__restrict__ planes, uint64_t P)
+// Sum of the lanes' values modulo 2^61 - 1 (each below 2^61), in every lane.
+__device__ __forceinline__ uint64_t sum61(uint64_t v)
 {
-    const uint64_t t = P / kTileBases, r = P % kTileBases;
-    const int b = (int)(r / kTileW), j = (int)(r % kTileW);
-    const uint32_t *w = planes + t * 4 * kTileWX + j;
-    int code = -1;
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
-        if ((__ldg(w + x * kTileWX) >> b) & 1u)
-            code = x;
-    return code;
+    for (int d = 1; d <= 4; d <<= 1) // eight values stay below 2^64
+        v += __shfl_xor_sync(0xffffffffu, v, d);
+    v = mod61(v);
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    return mod61(v);
 }
 
-// One warp per amplicon: the two hashes of its sequence (letters 1..5 = A C G T N).
-__global__ void amp_hash_kernel(const ah_amplicon *__restrict__ a, uint64_t n, const uint32_t *__restrict__ planes,
-                                const uint64_t *__restrict__ contig_off, uint64_t *__restrict__ h1,
-                                uint64_t *__restrict__ h2)
+// The slot of key (a, b) in an open-addressing table; claims a free one.  Keys
+// of a slot never change once set, and every element of a key meets the slots
+// in the same order, so equal keys always end at the same slot.  With one
+// word per key pass k2 = nullptr.
+__device__ uint64_t table_slot(unsigned long long *k1, unsigned long long *k2, uint64_t size, uint64_t a, uint64_t b)
 {
+    uint64_t i = __umul64hi(mix64(a ^ (b * 0x9e3779b97f4a7c15ull)), size);
+    for (;;) {
+        unsigned long long x = *(volatile unsigned long long *)(k1 + i);
+        if (x == kEmpty)
+            x = atomicCAS(k1 + i, kEmpty, (unsigned long long)a);
+        if (x == kEmpty || x == a) {
+            if (!k2)
+                return i;
+            unsigned long long y = *(volatile unsigned long long *)(k2 + i);
+            if (y == kEmpty)
+                y = atomicCAS(k2 + i, kEmpty, (unsigned long long)b);
+            if (y == kEmpty || y == b)
+                return i;
+        }
+        i = i + 1 == size ? 0 : i + 1;
+    }
+}
+
+__device__ __forceinline__ void note_first(unsigned int *first, uint64_t slot, uint32_t i)
+{
+    if (*(volatile unsigned int *)(first + slot) > i) // (most are not smaller: no atomic)
+        atomicMin(first + slot, i);
+}
+
+constexpr int kDigitLetters = 20;
+
+// Lane `lane`'s digit of the group of 32 * kDigitLetters letters at `first` (the
+// flat position of the group's letter 0), of which `left` are in the amplicon:
+// the letters lane, lane + 32, ..., three bits each (a base: 4 + its code with
+// A 0, C 1, G 2, T 3; else 0).  RC: the letters run backwards and are
+// complemented (code 3 - code: the planes in reverse order).  Positions are
+// counted from the start of the group's tile (RC: of the tile before it), so
+// they fit in 32 bits and reach one tile further at most.
+template <bool RC>
+__device__ __forceinline__ uint64_t group_digit(const uint32_t *__restrict__ planes, uint64_t first, uint32_t left, int lane)
+{
+    const uint32_t *tile = planes + (int64_t)(first / kTileBases - (RC ? 1 : 0)) * (4 * kTileWX);
+    const uint32_t rel0 = (uint32_t)(first % kTileBases) + (RC ? (uint32_t)kTileBases - lane : (uint32_t)lane);
+    uint64_t d = 0;
+    for (uint32_t c0 = 0; c0 < kDigitLetters && 32 * c0 < left; c0 += 4) { // four letters' loads in flight
+        uint32_t w[4][4], b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t q = 32 * (c0 + j), rel = RC ? rel0 - q : rel0 + q;
+            b[j] = (rel / kTileW) & 31u;
+            const uint32_t *wp = tile + (rel / (uint32_t)kTileBases * (4 * kTileWX) + rel % kTileW);
+            const bool in = q + lane < left;
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                w[j][x] = in ? __ldg(wp + (RC ? 3 - x : x) * kTileWX) : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t lo = w[j][1] | w[j][3], hi = w[j][2] | w[j][3], any = lo | w[j][2] | w[j][0];
+            d = d << 3 | (((any >> b[j]) & 1u) << 2 | ((hi >> b[j]) & 1u) << 1 | ((lo >> b[j]) & 1u));
+        }
+    }
+    return d;
+}
+
+// One warp per amplicon: the record's check and its two hashes.  A group of 640
+// letters is 32 digits of 60 bits, one per lane (four coalesced loads per 32
+// letters: consecutive positions lie in consecutive words), each times its
+// power of the base; hash = the groups in order (zeros beyond the end), then
+// the length.  A bad record sets *err.  Bound by the bit extraction (about 25
+// instructions per 32 letters).
+__global__ void amp_hash_kernel(const ah_amplicon *__restrict__ a, uint64_t n, const uint32_t *__restrict__ planes,
+                                const uint64_t *__restrict__ contig_off, const uint32_t *__restrict__ contig_genome,
+                                uint32_t n_contigs, uint64_t *__restrict__ hash1, uint64_t *__restrict__ hash2,
+                                int *__restrict__ err)
+{
+    constexpr uint32_t kGroup = 32 * kDigitLetters;
     const int lane = threadIdx.x & 31;
+    const uint64_t pow1 = kPow1.v[lane], pow2 = kPow2.v[lane];
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
     for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; i < n; i += warps) {
         const ah_amplicon am = a[i];
-        const uint64_t len = am.end - am.start, base = contig_off[am.contig] + am.start;
-        const bool rc = am.orient == 1;
-        const uint64_t piece = (len + 31) / 32, l0 = min(len, lane * piece), l1 = min(len, l0 + piece);
-        uint64_t s1 = 0, s2 = 0;
-        for (uint64_t q = l0; q < l1; ++q) {
-            int c = plane_code(planes, base + (rc ? len - 1 - q : q));
-            if (c >= 0 && rc)
-                c = 3 - c;
-            const uint64_t v = c < 0 ? 5 : (uint64_t)c + 1;
-            s1 = mod61(mulmod61(s1, kB1) + v);
-            s2 = mod61(mulmod61(s2, kB2) + v);
+        bool ok = am.contig < n_contigs && am.start <= am.end && am.orient <= 3;
+        if (ok)
+            ok = (uint64_t)am.end <= contig_off[am.contig + 1] - contig_off[am.contig] &&
+                 am.genome == contig_genome[am.contig];
+        if (!ok) {
+            if (lane == 0) {
+                atomicExch(err, kDevBounds);
+                hash1[i] = hash2[i] = 0;
+            }
+            continue;
         }
-        // piece hash times base^(letters after the piece), summed over the warp
-        s1 = mulmod61(s1, powmod61(kB1, len - l1));
-        s2 = mulmod61(s2, powmod61(kB2, len - l1));
-        for (int d = 16; d >= 1; d >>= 1) {
-            s1 = mod61(s1 + __shfl_xor_sync(0xffffffffu, s1, d));
-            s2 = mod61(s2 + __shfl_xor_sync(0xffffffffu, s2, d));
+        const uint32_t len = am.end - am.start;
+        const uint64_t base = contig_off[am.contig] + am.start;
+        uint64_t h1 = 0, h2 = 0;
+        for (uint64_t g = 0; g < len; g += kGroup) {
+            const uint32_t left = (uint32_t)min((uint64_t)kGroup, len - g);
+            const uint64_t d = am.orient == 1 ? group_digit<true>(planes, base + len - 1 - g, left, lane)
+                                              : group_digit<false>(planes, base + g, left, lane);
+            h1 = mod61(mulmod61(h1, kPow1.v[32]) + sum61(mulmod61(d, pow1)));
+            h2 = mod61(mulmod61(h2, kPow2.v[32]) + sum61(mulmod61(d, pow2)));
         }
         if (lane == 0) {
-            h1[i] = s1;
-            h2[i] = s2 ^ (len << 61); // the length's low three bits in the free top bits
+            hash1[i] = mod61(mulmod61(h1, kB1) + len);
+            hash2[i] = mod61(mulmod61(h2, kB2) + len);
         }
     }
 }
 
-__global__ void iota_kernel(uint32_t *__restrict__ v, uint64_t n)
+// Every amplicon's slot in the variant table.  Equal keys of a warp enter the
+// table once, by their first lane (the smallest index): a common variant's slot
+// is one address for the whole GPU.
+__global__ void variant_slots_kernel(uint64_t n, const uint64_t *__restrict__ hash1, const uint64_t *__restrict__ hash2,
+                                     AmpliTables t, uint32_t *__restrict__ slot)
 {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-        v[i] = (uint32_t)i;
-}
-
-__global__ void gather_kernel(const uint64_t *__restrict__ src, const uint32_t *__restrict__ idx, uint64_t n,
-                              uint64_t *__restrict__ dst)
-{
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x)
-        dst[k] = src[idx[k]];
-}
-
-// head[k] = 1 where the sorted key pair changes (k = 0 included)
-__global__ void heads_kernel(const uint64_t *__restrict__ a, const uint64_t *__restrict__ b, uint64_t n,
-                             uint64_t *__restrict__ head)
-{
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x)
-        head[k] = (k == 0 || a[k] != a[k - 1] || (b && b[k] != b[k - 1])) ? 1 : 0;
-}
-
-// at each run head: mark the run's first element (in input order) as a first occurrence
-__global__ void firsts_kernel(const uint64_t *__restrict__ head, const uint32_t *__restrict__ idx, uint64_t n,
-                              uint64_t *__restrict__ is_first)
-{
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x)
-        if (head[k])
-            is_first[idx[k]] = 1;
-}
-
-// id of element idx[k] = first-occurrence rank of its run's head; runs are
-// scanned from the sorted heads: run_of[k] = (inclusive count of heads) - 1
-__global__ void assign_kernel(const uint64_t *__restrict__ head_excl, const uint64_t *__restrict__ head,
-                              const uint32_t *__restrict__ idx, const uint64_t *__restrict__ rank, uint64_t n,
-                              uint32_t *__restrict__ run_head_pos, uint32_t *__restrict__ id_out)
-{
-    // pass 1 (this kernel with id_out == nullptr): position of every run's head
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t run = head_excl[k] + head[k] - 1;
-        if (!id_out) {
-            if (head[k])
-                run_head_pos[run] = (uint32_t)k;
-        } else {
-            id_out[idx[k]] = (uint32_t)rank[idx[run_head_pos[run]]];
+    const int lane = threadIdx.x & 31;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += stride) {
+        const uint64_t i = i0 + lane;
+        const bool in = i < n;
+        const uint64_t a = in ? hash1[i] : kEmpty, b = in ? hash2[i] : kEmpty;
+        const uint32_t same = __match_any_sync(0xffffffffu, a) & __match_any_sync(0xffffffffu, b);
+        const int lead = __ffs(same) - 1;
+        uint32_t s = 0;
+        if (in && lane == lead) {
+            s = (uint32_t)table_slot(t.k1, t.k2, t.size, a, b);
+            note_first(t.first, s, (uint32_t)i);
         }
+        s = __shfl_sync(0xffffffffu, s, lead);
+        if (in)
+            slot[i] = s;
     }
 }
 
-// per (genome, variant) run of the sorted keys: copies, and the genome's sums
-__global__ void genome_sums_kernel(const uint64_t *__restrict__ keys, const uint64_t *__restrict__ head,
-                                   const uint64_t *__restrict__ head_excl, const uint32_t *__restrict__ run_head_pos,
-                                   uint64_t n, const uint64_t *__restrict__ n_runs_dev, unsigned long long *__restrict__ g1,
-                                   unsigned long long *__restrict__ g2, unsigned int *__restrict__ gamp,
-                                   unsigned int *__restrict__ gvar)
+// flag[i] = element i is its key's first occurrence; 0 for i in [n, cap)
+__global__ void first_flags_kernel(const unsigned int *__restrict__ first, const uint32_t *__restrict__ slot,
+                                   const uint64_t *__restrict__ n_dev, uint64_t cap, uint64_t *__restrict__ flag)
 {
-    const uint64_t n_runs = *n_runs_dev;
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x) {
-        if (!head[k])
+    const uint64_t n = dev_count(cap, n_dev);
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += (uint64_t)gridDim.x * blockDim.x)
+        flag[i] = i < n && first[slot[i]] == (uint32_t)i ? 1 : 0;
+}
+
+// variant ids, and the copies of every (genome, variant) in the second table
+__global__ void variants_kernel(const ah_amplicon *__restrict__ a, uint64_t n, AmpliTables t,
+                                const uint32_t *__restrict__ slot, const uint64_t *__restrict__ flag,
+                                const uint64_t *__restrict__ rank, uint32_t *__restrict__ variant,
+                                uint64_t *__restrict__ n_variants, const int *__restrict__ err)
+{
+    if (__syncthreads_or(*(volatile const int *)err)) // (the records are not to be trusted; the call reports it)
+        return;
+    const int lane = threadIdx.x & 31;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += stride) {
+        const uint64_t i = i0 + lane;
+        const bool in = i < n;
+        uint64_t key = kEmpty;
+        if (in) {
+            const uint32_t v = (uint32_t)rank[t.first[slot[i]]];
+            variant[i] = v;
+            key = (uint64_t)a[i].genome << 32 | v;
+            if (i == n - 1)
+                *n_variants = rank[i] + flag[i];
+        }
+        const uint32_t same = __match_any_sync(0xffffffffu, key); // (amplicons of a genome are neighbours)
+        if (in && lane == __ffs(same) - 1)
+            atomicAdd(t.pair_n + table_slot(t.pair_key, nullptr, t.size, key, 0), (unsigned int)__popc(same));
+    }
+}
+
+// per (genome, variant) with its copies: the genome's sums
+__global__ void genome_sums_kernel(AmpliTables t, unsigned long long *__restrict__ g1, unsigned long long *__restrict__ g2,
+                                   unsigned int *__restrict__ gamp, unsigned int *__restrict__ gvar)
+{
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < t.size; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t key = t.pair_key[i];
+        if (key == kEmpty)
             continue;
-        const uint64_t run = head_excl[k];
-        const uint64_t end = run + 1 < n_runs ? run_head_pos[run + 1] : n;
-        const uint64_t copies = end - k;
-        const uint32_t g = (uint32_t)(keys[k] >> 32);
-        const uint64_t v = keys[k] & 0xffffffffull;
+        const uint32_t g = (uint32_t)(key >> 32), copies = t.pair_n[i];
+        const uint64_t v = key & 0xffffffffull;
         atomicAdd(g1 + g, (unsigned long long)mix64((v << 32 | copies) * 2 + 1));
         atomicAdd(g2 + g, (unsigned long long)mix64((v << 32 | copies) ^ 0x9e3779b97f4a7c15ull));
-        atomicAdd(gamp + g, (unsigned int)copies);
+        atomicAdd(gamp + g, copies);
         atomicAdd(gvar + g, 1u);
     }
 }
@@ -186,142 +285,94 @@ __global__ void genome_flags_kernel(const unsigned int *__restrict__ gamp, uint6
         has[g] = gamp[g] ? 1 : 0;
 }
 
-// compact the genomes with amplicons (ascending id) and their hash sums
-__global__ void genome_compact_kernel(const uint64_t *__restrict__ has, const uint64_t *__restrict__ pos, uint64_t n,
-                                      const unsigned long long *__restrict__ g1, const unsigned long long *__restrict__ g2,
-                                      uint32_t *__restrict__ gid, uint64_t *__restrict__ k1, uint64_t *__restrict__ k2)
+// genomes with amplicons (ascending id) as rows, and each row's slot in the amplitype table
+__global__ void genome_rows_kernel(const uint64_t *__restrict__ has, const uint64_t *__restrict__ pos, uint64_t n,
+                                   const unsigned long long *__restrict__ g1, const unsigned long long *__restrict__ g2,
+                                   AmpliTables t, uint32_t *__restrict__ gid, uint32_t *__restrict__ slot,
+                                   uint64_t *__restrict__ n_rows)
 {
-    for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (uint64_t)gridDim.x * blockDim.x)
+    for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (uint64_t)gridDim.x * blockDim.x) {
         if (has[g]) {
-            gid[pos[g]] = (uint32_t)g;
-            k1[pos[g]] = g1[g];
-            k2[pos[g]] = g2[g];
+            const uint64_t r = pos[g];
+            gid[r] = (uint32_t)g;
+            // (without its top bit a sum is never the empty key)
+            const uint64_t s = table_slot(t.k1, t.k2, t.size, g1[g] & ~(1ull << 63), g2[g] & ~(1ull << 63));
+            note_first(t.first, s, (uint32_t)r);
+            slot[r] = (uint32_t)s;
         }
-}
-
-__global__ void rows_kernel(const uint32_t *__restrict__ gid, const uint32_t *__restrict__ type, uint64_t m,
-                            const unsigned int *__restrict__ gamp, const unsigned int *__restrict__ gvar,
-                            ah_genome_amplitype *__restrict__ rows)
-{
-    for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t g = gid[r];
-        rows[r] = {g, type[r], gamp[g], gvar[g]};
+        if (g == n - 1)
+            *n_rows = pos[g] + has[g];
     }
 }
 
-__global__ void genome_key_kernel(const ah_amplicon *__restrict__ a, const uint32_t *__restrict__ variant, uint64_t n,
-                                  const uint32_t *__restrict__ contig_genome, uint64_t *__restrict__ keys,
-                                  int *__restrict__ err)
+__global__ void rows_kernel(const uint32_t *__restrict__ gid, const uint32_t *__restrict__ slot, AmpliTables t,
+                            const uint64_t *__restrict__ n_rows, uint64_t cap, const uint64_t *__restrict__ flag,
+                            const uint64_t *__restrict__ rank, const unsigned int *__restrict__ gamp,
+                            const unsigned int *__restrict__ gvar, ah_genome_amplitype *__restrict__ rows,
+                            uint64_t *__restrict__ n_types)
 {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const ah_amplicon am = a[i]; // contig already checked
-        const uint32_t g = contig_genome[am.contig];
-        if (am.genome != g || am.orient > 3)
-            atomicExch(err, kDevBounds);
-        keys[i] = (uint64_t)g << 32 | variant[i];
+    const uint64_t n = dev_count(cap, n_rows);
+    if (n == 0 && blockIdx.x == 0 && threadIdx.x == 0)
+        *n_types = 0;
+    for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t g = gid[r];
+        rows[r] = {g, (uint32_t)rank[t.first[slot[r]]], gamp[g], gvar[g]};
+        if (r == n - 1)
+            *n_types = rank[r] + flag[r];
     }
 }
 
 unsigned grid(uint64_t n, int threads = 256)
 {
-    uint64_t b = (n + threads - 1) / threads;
+    const uint64_t b = (n + threads - 1) / threads;
     return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(b, 8192));
 }
 
 } // namespace
 
-// Stable sort of idx (initially 0..n-1) by (ka, kb): LSD over kb then ka.
-// Scratch: 2n u64 keys, n u32 values, CUB temporary storage.
-void AmpliTypeScratch::sort_by(const uint64_t *ka, const uint64_t *kb, uint64_t n, cudaStream_t s)
-{
-    keys_b_valid = kb != nullptr;
-    iota_kernel<<<grid(n), 256, 0, s>>>(idx, n);
-    AH_CUDA(cudaGetLastError());
-    size_t tb = temp_bytes;
-    if (kb) {
-        AH_CUDA(cub::DeviceRadixSort::SortPairs(temp, tb, kb, keys_b, idx, idx_b, (int64_t)n, 0, 64, s));
-        gather_kernel<<<grid(n), 256, 0, s>>>(ka, idx_b, n, keys_a);
-        AH_CUDA(cudaGetLastError());
-        tb = temp_bytes;
-        AH_CUDA(cub::DeviceRadixSort::SortPairs(temp, tb, keys_a, keys_s, idx_b, idx, (int64_t)n, 0, 64, s));
-        gather_kernel<<<grid(n), 256, 0, s>>>(kb, idx, n, keys_b);
-        AH_CUDA(cudaGetLastError());
-    } else {
-        AH_CUDA(cub::DeviceRadixSort::SortPairs(temp, tb, ka, keys_s, idx, idx_b, (int64_t)n, 0, 64, s));
-        AH_CUDA(cudaMemcpyAsync(idx, idx_b, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-    }
-}
+// Slots for n keys: at most two in three are taken.
+// Slots are numbered in 32 bits; there is always one for every key (n < 2^32).
+uint64_t amplitype_slots(uint64_t n) { return std::min<uint64_t>(n + n / 2 + 64, 0xffffffffull); }
 
-size_t AmpliTypeScratch::cub_bytes(uint64_t n)
-{
-    size_t b = 0;
-    AH_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, b, (const uint64_t *)nullptr, (uint64_t *)nullptr,
-                                            (const uint32_t *)nullptr, (uint32_t *)nullptr, (int64_t)n, 0, 64));
-    return b;
-}
-
-// Runs of equal keys after sort_by: heads, their positions and (device)
-// count; with id_out, every element's first-occurrence id of its run.
-void AmpliTypeScratch::ids(uint64_t n, uint32_t *id_out, uint64_t *n_runs_dev, cudaStream_t s)
-{
-    heads_kernel<<<grid(n), 256, 0, s>>>(keys_s, keys_b_valid ? keys_b : nullptr, n, head);
-    AH_CUDA(cudaGetLastError());
-    exclusive_scan_u64(scan_temp, scan_bytes, head, head_excl, n, s);
-    assign_kernel<<<grid(n), 256, 0, s>>>(head_excl, head, idx, rank, n, run_pos, nullptr);
-    AH_CUDA(cudaGetLastError());
-    launch_total(head_excl, head, n, nullptr, 0, n_runs_dev, 0, nullptr, nullptr, 0, s);
-    if (!id_out)
-        return;
-    AH_CUDA(cudaMemsetAsync(is_first, 0, n * sizeof(uint64_t), s));
-    firsts_kernel<<<grid(n), 256, 0, s>>>(head, idx, n, is_first);
-    AH_CUDA(cudaGetLastError());
-    exclusive_scan_u64(scan_temp, scan_bytes, is_first, rank, n, s);
-    assign_kernel<<<grid(n), 256, 0, s>>>(head_excl, head, idx, rank, n, run_pos, id_out);
-    AH_CUDA(cudaGetLastError());
-}
-
-void launch_amp_hash(const ah_amplicon *a, uint64_t n, const uint32_t *planes, const uint64_t *contig_off,
-                     uint64_t *h1, uint64_t *h2, cudaStream_t s)
+void launch_amplitypes(const ah_amplicon *a, uint64_t n, const uint32_t *planes, const uint64_t *contig_off,
+                       const uint32_t *contig_genome, uint32_t n_contigs, uint64_t n_ids, const AmpliScratch &S,
+                       uint64_t *counts, int *err, cudaStream_t s)
 {
     if (!n)
         return;
-    amp_hash_kernel<<<grid(n * 32, 256), 256, 0, s>>>(a, n, planes, contig_off, h1, h2);
+    // the tables' keys and first occurrences empty; counts and sums zero
+    AH_CUDA(cudaMemsetAsync(S.ones, 0xff, S.ones_bytes, s));
+    AH_CUDA(cudaMemsetAsync(S.zeros, 0, S.zeros_bytes, s));
+    amp_hash_kernel<<<grid(n * 32), 256, 0, s>>>(a, n, planes, contig_off, contig_genome, n_contigs, S.flag, S.rank, err);
+    AH_CUDA(cudaGetLastError());
+    variant_slots_kernel<<<grid(n), 256, 0, s>>>(n, S.flag, S.rank, S.t, S.slot); // (the hashes' arrays are free after it)
+    AH_CUDA(cudaGetLastError());
+    first_flags_kernel<<<grid(n), 256, 0, s>>>(S.t.first, S.slot, nullptr, n, S.flag);
+    AH_CUDA(cudaGetLastError());
+    exclusive_scan_u64(S.scan_temp, S.scan_bytes, S.flag, S.rank, n, s);
+    variants_kernel<<<grid(n), 256, 0, s>>>(a, n, S.t, S.slot, S.flag, S.rank, S.variant, counts + 0, err);
+    AH_CUDA(cudaGetLastError());
+    genome_sums_kernel<<<grid(S.t.size), 256, 0, s>>>(S.t, S.g1, S.g2, S.gamp, S.gvar);
+    AH_CUDA(cudaGetLastError());
+    genome_flags_kernel<<<grid(n_ids), 256, 0, s>>>(S.gamp, n_ids, S.has);
+    AH_CUDA(cudaGetLastError());
+    exclusive_scan_u64(S.scan_temp, S.scan_bytes, S.has, S.pos, n_ids, s);
+    // the first table again, for the genomes' sums (at most min(n, n_ids) rows)
+    const uint64_t most = std::min(n, n_ids);
+    AH_CUDA(cudaMemsetAsync(S.ones, 0xff, S.ones_bytes, s));
+    genome_rows_kernel<<<grid(n_ids), 256, 0, s>>>(S.has, S.pos, n_ids, S.g1, S.g2, S.t, S.gid, S.slot, counts + 1);
+    AH_CUDA(cudaGetLastError());
+    first_flags_kernel<<<grid(most), 256, 0, s>>>(S.t.first, S.slot, counts + 1, most, S.flag);
+    AH_CUDA(cudaGetLastError());
+    exclusive_scan_u64(S.scan_temp, S.scan_bytes, S.flag, S.rank, most, s);
+    rows_kernel<<<grid(most), 256, 0, s>>>(S.gid, S.slot, S.t, counts + 1, most, S.flag, S.rank, S.gamp, S.gvar, S.rows,
+                                           counts + 2);
     AH_CUDA(cudaGetLastError());
 }
 
-void launch_genome_key(const ah_amplicon *a, const uint32_t *variant, uint64_t n, const uint32_t *contig_genome,
-                       uint64_t *keys, int *err, cudaStream_t s)
+int amplitype_launches(uint64_t n, uint64_t n_ids)
 {
-    genome_key_kernel<<<grid(n), 256, 0, s>>>(a, variant, n, contig_genome, keys, err);
-    AH_CUDA(cudaGetLastError());
-}
-
-void AmpliTypeScratch::genome_sums(uint64_t n, const uint64_t *n_runs_dev, unsigned long long *g1,
-                                   unsigned long long *g2, unsigned int *gamp, unsigned int *gvar, cudaStream_t s)
-{
-    genome_sums_kernel<<<grid(n), 256, 0, s>>>(keys_s, head, head_excl, run_pos, n, n_runs_dev, g1, g2, gamp, gvar);
-    AH_CUDA(cudaGetLastError());
-}
-
-void launch_genome_compact(const unsigned int *gamp, uint64_t n_ids, uint64_t *has, uint64_t *pos, void *scan_temp,
-                           size_t scan_bytes, const unsigned long long *g1, const unsigned long long *g2, uint32_t *gid,
-                           uint64_t *k1, uint64_t *k2, uint64_t *n_out_dev, cudaStream_t s)
-{
-    genome_flags_kernel<<<grid(n_ids), 256, 0, s>>>(gamp, n_ids, has);
-    AH_CUDA(cudaGetLastError());
-    exclusive_scan_u64(scan_temp, scan_bytes, has, pos, n_ids, s);
-    genome_compact_kernel<<<grid(n_ids), 256, 0, s>>>(has, pos, n_ids, g1, g2, gid, k1, k2);
-    AH_CUDA(cudaGetLastError());
-    launch_total(pos, has, n_ids, nullptr, 0, n_out_dev, 0, nullptr, nullptr, 0, s);
-}
-
-void launch_amplitype_rows(const uint32_t *gid, const uint32_t *type, uint64_t m, const unsigned int *gamp,
-                           const unsigned int *gvar, ah_genome_amplitype *rows, cudaStream_t s)
-{
-    if (!m)
-        return;
-    rows_kernel<<<grid(m), 256, 0, s>>>(gid, type, m, gamp, gvar, rows);
-    AH_CUDA(cudaGetLastError());
+    return 9 + scan_u64_launches(n) + scan_u64_launches(n_ids) + scan_u64_launches(std::min(n, n_ids));
 }
 
 } // namespace ah

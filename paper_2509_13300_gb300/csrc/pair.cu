@@ -127,8 +127,10 @@ __device__ __forceinline__ bool in_window(const PairDev &pd, uint32_t s_pos, con
 
 __global__ void pair_count_kernel(const ah_site *__restrict__ s, uint64_t n_arg, const uint64_t *__restrict__ n_dev,
                                   const uint8_t *__restrict__ pass, const PairDev *__restrict__ pairs,
-                                  uint64_t *__restrict__ counts)
+                                  uint64_t *__restrict__ counts, const int *__restrict__ err)
 {
+    if (err && *(volatile const int *)err) // the records' check failed: nothing is indexed with them
+        return;
     const uint64_t n = dev_count(n_arg, n_dev);
     for (uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t cnt = 0;
@@ -328,11 +330,11 @@ unsigned grid_for(uint64_t n, int threads)
 } // namespace
 
 void launch_pair_count(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, uint64_t *counts, cudaStream_t s)
+                       const PairDev *pairs_d, uint64_t *counts, const int *err, cudaStream_t s)
 {
     if (!n)
         return;
-    pair_count_kernel<<<grid_for(n, 128), 128, 0, s>>>(sites, n, n_dev, pass, pairs_d, counts);
+    pair_count_kernel<<<grid_for(n, 128), 128, 0, s>>>(sites, n, n_dev, pass, pairs_d, counts, err);
     AH_CUDA(cudaGetLastError());
 }
 
@@ -354,7 +356,7 @@ void exclusive_scan_u64(void *temp, size_t temp_bytes, const uint64_t *in, uint6
 {
     if (n == 0)
         return;
-    if (n <= kSmallScan) {
+    if (n <= kOneBlockScan) {
         scan_small_kernel<<<1, 1024, 0, s>>>(in, out, (uint32_t)n, nullptr, 0, nullptr, 0, nullptr, nullptr, 0);
         AH_CUDA(cudaGetLastError());
         return;
@@ -372,7 +374,7 @@ void exclusive_scan_u64_dev(const uint64_t *in, uint64_t *out, uint64_t n, const
     AH_CUDA(cudaGetLastError());
 }
 
-int scan_u64_launches(uint64_t n) { return n == 0 ? 0 : n <= kSmallScan ? 1 : 2; }
+int scan_u64_launches(uint64_t n) { return n == 0 ? 0 : n <= kOneBlockScan ? 1 : 2; }
 
 void launch_pair_write(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
                        const PairDev *pairs_d, const uint64_t *offsets, ah_amplicon *out, uint64_t cap,

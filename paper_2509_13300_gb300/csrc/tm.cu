@@ -240,6 +240,10 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *__rest
     // then [kTmWarps * 8 sites][seg_max][16] segment tables
     extern __shared__ __align__(16) unsigned char tm_smem[];
     TmPairS *ps = reinterpret_cast<TmPairS *>(tm_smem);
+    // the records' check failed: nothing is read with them, the call reports it (one answer per
+    // block: the word may change under it)
+    if (__syncthreads_or(*(volatile const int *)err))
+        return;
     const int nd = n_pairs <= kTmStageD ? n_pairs : 0;
     TmPairD *pdd = reinterpret_cast<TmPairD *>(tm_smem + (size_t)n_pairs * sizeof(TmPairS));
     float2 *seg_smem =
@@ -628,8 +632,8 @@ __global__ void __launch_bounds__(kFastThreads) tm_fast_kernel(const ah_site *__
     extern __shared__ __align__(16) unsigned char fast_smem[];
     TmFastPair *fp = reinterpret_cast<TmFastPair *>(fast_smem);
     const uint64_t n = dev_count(n_arg, n_dev);
-    if ((uint64_t)blockIdx.x * blockDim.x >= n)
-        return; // the whole block: no site for it
+    if ((uint64_t)blockIdx.x * blockDim.x >= n || __syncthreads_or(*(volatile const int *)err))
+        return; // the whole block: no site for it, or records that failed their check
     for (int j = 0; j < n_pairs; ++j) {
         const PairDev &P = pairs[j];
         for (int t = threadIdx.x; t < 256; t += blockDim.x) {
@@ -907,13 +911,27 @@ __global__ void sweep_weights_kernel(const PairDev *__restrict__ pairs, int n_pa
     }
 }
 
-// One thread per site: bit j of pass_mask[i] = site i passes threshold j.
+// One thread per site: bit j of pass_mask[i] = site i passes threshold j.  A
+// threshold that fp32 keeps clear of the 0.01 deg C band (with its own rounding
+// and the threshold's allowed for) is decided by one fp32 comparison: the fp64
+// units run at 1/64 of the fp32 rate here.  What remains is the latency of the
+// sites near a threshold (80,000 sites x 31 thresholds: 47 -> 42 us).
 __global__ void sweep_pass_kernel(const ah_site *__restrict__ sites, uint64_t n, const PairDev *__restrict__ pairs,
                                   const uint32_t *__restrict__ planes, const uint64_t *__restrict__ contig_off,
                                   const float *__restrict__ tm, const double *__restrict__ thr_c, int n_thr,
-                                  const long long *__restrict__ W, int few_exact, uint64_t *__restrict__ pass_mask)
+                                  const long long *__restrict__ W, int few_exact, uint64_t *__restrict__ pass_mask,
+                                  const int *__restrict__ err)
 {
     const long long LINF = 0x2000000000000000ll;
+    __shared__ float thr_f[kSweepMax], clear_of[kSweepMax];
+    if (threadIdx.x < (unsigned)n_thr) {
+        const float f = (float)thr_c[threadIdx.x];
+        thr_f[threadIdx.x] = f;
+        clear_of[threadIdx.x] = 0.0101f + 2.4e-7f * fabsf(f);
+    }
+    __syncthreads();
+    if (*(volatile const int *)err)
+        return;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         const ah_site s = sites[i];
         const float t = tm[i];
@@ -924,11 +942,15 @@ __global__ void sweep_pass_kernel(const ah_site *__restrict__ sites, uint64_t n,
         bool have_bt = false;
         uint64_t m = 0;
         for (int j = 0; j < n_thr; ++j) {
+            const float df = t - thr_f[j];
+            if (isnan(t) || fabsf(df) >= clear_of[j]) {
+                if (df > 0.0f) // (NaN, a template with a non-ACGT letter: fails every threshold)
+                    m |= 1ull << j;
+                continue;
+            }
             const double T = thr_c[j];
             bool pass;
-            if (isnan(t)) {
-                pass = false; // a template with a non-ACGT letter fails every threshold
-            } else if (fabs((double)t - T) >= 0.01) {
+            if (fabs((double)t - T) >= 0.01) {
                 pass = (double)t >= T;
             } else {
                 if (!have_bt) {
@@ -991,62 +1013,74 @@ __global__ void sweep_pass_kernel(const ah_site *__restrict__ sites, uint64_t n,
     }
 }
 
+// Per threshold (bit j of each lane's m), the lanes that have it: lane j % 32
+// adds the count to its acc[j / 32].  A warp's count is one vote, where an
+// atomic per set bit made all lanes of a block queue at one shared word.
+__device__ __forceinline__ void count_bits(uint64_t m, int n_thr, int lane, uint32_t (&acc)[2])
+{
+    for (int j = 0; j < n_thr; ++j) {
+        const uint32_t c = __popc(__ballot_sync(0xffffffffu, (m >> j) & 1u));
+        if (lane == (j & 31)) {
+            if (j < 32)
+                acc[0] += c;
+            else
+                acc[1] += c;
+        }
+    }
+}
+__device__ __forceinline__ void add_counts(const uint32_t (&acc)[2], int n_thr, int lane, unsigned long long *out)
+{
+    if (lane < n_thr && acc[0])
+        atomicAdd(out + lane, (unsigned long long)acc[0]);
+    if (32 + lane < n_thr && acc[1])
+        atomicAdd(out + 32 + lane, (unsigned long long)acc[1]);
+}
+
 // Per amplicon: the thresholds both of its sites pass; counts per threshold
 // (all, FF or RR) and, per genome, the thresholds at which it is amplified.
+// (65,000 amplicons, 31 thresholds: 30 -> 9 us; the genomes' counts below 48 -> 3.)
 __global__ void sweep_count_kernel(const ah_amplicon *__restrict__ a, uint64_t na, uint64_t n_sites,
                                    const uint64_t *__restrict__ pass_mask, uint32_t max_genome, int n_thr,
                                    unsigned long long *__restrict__ amps, unsigned long long *__restrict__ ffrr,
                                    unsigned long long *__restrict__ gmask, int *__restrict__ err)
 {
-    __shared__ unsigned long long sa[kSweepMax], sf[kSweepMax];
-    for (int j = threadIdx.x; j < kSweepMax; j += blockDim.x)
-        sa[j] = sf[j] = 0;
-    __syncthreads();
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < na; i += (uint64_t)gridDim.x * blockDim.x) {
-        const ah_amplicon am = a[i];
-        if (am.left >= n_sites || am.right >= n_sites || am.genome > max_genome || am.orient > 3) {
-            atomicExch(err, kDevBounds);
-            continue;
+    const int lane = threadIdx.x & 31;
+    uint32_t all[2] = {0, 0}, same[2] = {0, 0};
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < na; i0 += stride) {
+        const uint64_t i = i0 + lane;
+        uint64_t m = 0;
+        bool ff = false;
+        if (i < na) {
+            const ah_amplicon am = a[i];
+            if (am.left >= n_sites || am.right >= n_sites || am.genome > max_genome || am.orient > 3) {
+                atomicExch(err, kDevBounds);
+            } else {
+                m = pass_mask[am.left] & pass_mask[am.right];
+                ff = am.orient >= 2;
+                if (m & ~*(volatile unsigned long long *)(gmask + am.genome)) // (most add nothing: no atomic)
+                    atomicOr(gmask + am.genome, (unsigned long long)m);
+            }
         }
-        uint64_t m = pass_mask[am.left] & pass_mask[am.right];
-        if (m)
-            atomicOr(gmask + am.genome, (unsigned long long)m);
-        while (m) {
-            const int j = __ffsll((long long)m) - 1;
-            m &= m - 1;
-            atomicAdd(&sa[j], 1ull);
-            if (am.orient >= 2)
-                atomicAdd(&sf[j], 1ull);
-        }
+        count_bits(m, n_thr, lane, all);
+        if (__any_sync(0xffffffffu, ff))
+            count_bits(ff ? m : 0, n_thr, lane, same);
     }
-    __syncthreads();
-    for (int j = threadIdx.x; j < n_thr; j += blockDim.x) {
-        if (sa[j])
-            atomicAdd(amps + j, sa[j]);
-        if (sf[j])
-            atomicAdd(ffrr + j, sf[j]);
-    }
+    add_counts(all, n_thr, lane, amps);
+    add_counts(same, n_thr, lane, ffrr);
 }
 
 __global__ void sweep_genomes_kernel(const unsigned long long *__restrict__ gmask, uint64_t n_words, int n_thr,
                                      unsigned long long *__restrict__ gcount)
 {
-    __shared__ unsigned long long sg[kSweepMax];
-    for (int j = threadIdx.x; j < kSweepMax; j += blockDim.x)
-        sg[j] = 0;
-    __syncthreads();
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_words; i += (uint64_t)gridDim.x * blockDim.x) {
-        unsigned long long m = gmask[i];
-        while (m) {
-            const int j = __ffsll((long long)m) - 1;
-            m &= m - 1;
-            atomicAdd(&sg[j], 1ull);
-        }
+    const int lane = threadIdx.x & 31;
+    uint32_t all[2] = {0, 0};
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n_words; i0 += stride) {
+        const uint64_t i = i0 + lane;
+        count_bits(i < n_words ? gmask[i] : 0, n_thr, lane, all);
     }
-    __syncthreads();
-    for (int j = threadIdx.x; j < n_thr; j += blockDim.x)
-        if (sg[j])
-            atomicAdd(gcount + j, sg[j]);
+    add_counts(all, n_thr, lane, gcount);
 }
 
 } // namespace
@@ -1138,7 +1172,7 @@ void launch_tm_sweep(const ah_site *sites, uint64_t n_sites, const ah_amplicon *
     if (n_sites) {
         const uint64_t blocks = std::min<uint64_t>((n_sites + 127) / 128, 8192);
         sweep_pass_kernel<<<(unsigned)blocks, 128, 0, s>>>(sites, n_sites, pairs_d, planes, contig_off, tm, thr_d,
-                                                           n_thr, W, few_exact ? 1 : 0, pass_mask);
+                                                           n_thr, W, few_exact ? 1 : 0, pass_mask, err);
         AH_CUDA(cudaGetLastError());
     }
     if (n_amps) {

@@ -1291,3 +1291,45 @@ def test_profile_hmm_wavefront_stripes_and_tasks(ctx, m, n):
         assert (np.abs(f[some].astype(np.float64) - want_f) <= tol_f).all()
     every = 1e-4 + 1e-5 * np.abs(got["full"][0])
     assert (np.abs(got["full"][0] - got["budget"][0]) <= every).all()  # also the amplicons the oracle did not score
+
+
+@pytest.mark.parametrize("lens", [[1, 1, 31, 32, 33], [639, 640, 641, 640, 639], [1279, 1281, 1920, 1280, 5]])
+def test_amplitype_hash_groups_and_tables(ctx, lens):
+    """Variants and amplitypes of records of the hash's group sizes (32 letters a row, 640 a group),
+    in both orientations, across tile ends, with N, with copies in several genomes and with
+    sequences that differ in one letter or only in length, against the plain definition; a bad
+    record is refused."""
+    rng = np.random.default_rng(sum(lens))
+    base = synth.random_bases(rng, max(lens), 0.5).copy()
+    genomes, recs, pos = [], [], 0
+    for g in range(7):
+        parts, at = [], 0
+        for c in range(60):
+            body = base[:lens[int(rng.integers(len(lens)))]].copy()
+            if rng.random() < 0.3:
+                body[int(rng.integers(len(body)))] = rng.choice(list(b"ACGTN"))
+            rc = bool(rng.integers(2))
+            stored = np.frombuffer(synth._revcomp(body.tobytes().decode().replace("N", "A")).encode(), np.uint8) if rc else body
+            gap = synth.random_bases(rng, int(rng.integers(0, 40)), 0.5)
+            parts += [gap, stored]
+            recs.append((g, g, at + len(gap), at + len(gap) + len(body), 0, 0, 1 if rc else int(rng.choice([0, 2, 3])), 0, 0, 0))
+            at += len(gap) + len(body)
+        genomes.append(np.concatenate(parts))
+    seq = np.concatenate(genomes)
+    off = np.concatenate([[0], np.cumsum([len(x) for x in genomes])]).astype(np.uint64)
+    amps = np.array(recs, dtype=ah.AMPLICON_DTYPE)
+    want_v, want_rows, want_nv, want_nt = oracle.amplitypes(seq, off, amps)
+    sid = ctx.load(seq, off, np.arange(len(genomes), dtype=np.uint32))
+    try:
+        variant, rows, nv, nt = ctx.amplitypes(sid, amps)
+        assert np.array_equal(variant, want_v) and (nv, nt) == (want_nv, want_nt)
+        assert np.array_equal(np.asarray(rows), np.asarray(want_rows))
+        for f, v in (("genome", 6), ("orient", 4), ("contig", 99)):
+            bad = amps.copy()
+            bad[f][3] = v
+            with pytest.raises(ah.AHError):
+                ctx.amplitypes(sid, bad)
+        again = ctx.amplitypes(sid, amps)
+        assert np.array_equal(again[0], want_v)
+    finally:
+        ctx.ah_unload_genomes(sid)
