@@ -1755,11 +1755,40 @@ static ah_status load_impl(ah_ctx *c, const uint8_t *seq, uint64_t n_bases, cons
         require(!two || !reversed, AH_ERR_ARG, "ah_load_genomes_2bit: no reversed form");
         require(!two || !dev_seq || reinterpret_cast<uintptr_t>(seq) % 16 == 0, AH_ERR_ARG,
                 "ah_load_genomes_2bit: device codes must be 16-byte aligned");
-        // the packing first (it reads no contig table), then the tables' copies
+        auto queue_tables = [&] {
+            HostSpan hs_tables(c, "host.load.tables");
+            // the tables through a mapped pinned slot, read by one copy kernel; the
+            // per-tile contig table is built here by a merge walk over tiles and contigs
+            ah_ctx::PinSlot &sl = pin_slot(c, table_bytes);
+            memcpy(sl.p, contig_off, ob);
+            memcpy(sl.p + ob, contig_genome, gb);
+            {
+                // tile t: the last contig starting at or before t * kTileBases, and
+                // the room from the tile's first position to that contig's end
+                uint32_t *tc = (uint32_t *)(sl.p + ob + gb);
+                uint32_t *room = tc + (gs->n_tiles + 1);
+                uint32_t ci = 0;
+                for (uint64_t t = 0; t <= gs->n_tiles; ++t) {
+                    const uint64_t P = t * kTileBases;
+                    while (ci + 1 < n_contigs && contig_off[ci + 1] <= P)
+                        ++ci;
+                    tc[t] = ci;
+                    const uint64_t end = n_contigs ? contig_off[ci + 1] : 0;
+                    room[t] = end > P ? (uint32_t)std::min<uint64_t>(end - P, 0xffffffffull) : 0u;
+                }
+            }
+            Stage sg(c, "tables", st, 1);
+            launch_copy_words((const uint32_t *)sl.dp, (uint32_t *)gs->contig_off, table_bytes / 4, st);
+            AH_CUDA(cudaEventRecord(sl.ev, st));
+        };
+        // the packing first (it reads no contig table), then the tables' copies; a reversed
+        // packing reads the tables
+        if (reversed)
+            queue_tables();
         std::vector<void *> temp; // freed once the packing is done (reversed loads)
         if (gs->n_tiles && reversed) {
             HostSpan hs_pack(c, "host.load.pack");
-            // decoy: the input on the device, reversed contig by contig, then packed
+            // decoy: the input on the device, packed with every contig mirrored
             const uint8_t *src = seq;
             if (!dev_seq) {
                 uint8_t *d = (uint8_t *)dev_alloc(c, n_bases);
@@ -1767,51 +1796,38 @@ static ah_status load_impl(ah_ctx *c, const uint8_t *seq, uint64_t n_bases, cons
                 AH_CUDA(cudaMemcpyAsync(d, seq, n_bases, cudaMemcpyHostToDevice, st));
                 src = d;
             }
-            uint8_t *dst = (uint8_t *)dev_alloc(c, n_bases);
-            temp.push_back(dst);
-            const uint64_t kStretch = 1ull << 16;
-            std::vector<RevChunk> ch;
-            ch.reserve(n_bases / kStretch + n_contigs);
-            for (uint32_t i = 0; i < n_contigs; ++i) {
-                const uint64_t o = contig_off[i], len = contig_off[i + 1] - o;
-                for (uint64_t q = 0; q < len; q += kStretch)
-                    ch.push_back({o + q, 2 * o + len - 1, std::min(kStretch, len - q)});
-            }
-            RevChunk *ch_d = (RevChunk *)dev_alloc(c, std::max<size_t>(ch.size(), 1) * sizeof(RevChunk));
-            temp.push_back(ch_d);
-            AH_CUDA(cudaMemcpyAsync(ch_d, ch.data(), ch.size() * sizeof(RevChunk), cudaMemcpyHostToDevice, st));
-            Stage sg(c, "pack", st, 2);
-            launch_reverse_contigs(src, dst, ch_d, ch.size(), st);
-            launch_pack(dst, 0, n_bases, n_bases, gs->planes, 0, gs->n_tiles, c->d_err, st);
+            Stage sg(c, "pack", st, 1);
+            launch_pack_reversed(src, n_bases, gs->planes, gs->n_tiles, gs->contig_off, gs->tile_contig, c->d_err, st);
         } else if (gs->n_tiles && two) {
             HostSpan hs_pack(c, "host.load.pack");
             // the no-base runs on the device, owned by the set (another load in flight on
             // another stream must not overwrite them while this packing reads them),
-            // followed by each tile's first run that ends after the tile's start (a
-            // merge walk here, so the packing searches nothing); through a pinned
-            // slot, like the contig tables
-            const uint64_t run_bytes = two->n_gaps * 16, tab_bytes = (gs->n_tiles + 1) * 4;
+            // followed by the range of runs each tile meets (a merge walk here, so the
+            // packing searches nothing); through a pinned slot, like the contig tables
+            const uint64_t run_bytes = two->n_gaps * 16, tab_bytes = gs->n_tiles * 8;
             gs->gaps_bytes = std::max<uint64_t>(run_bytes + tab_bytes, 16);
             gs->gaps = (uint64_t *)dev_alloc(c, gs->gaps_bytes);
             uint64_t *gaps_d = gs->gaps;
-            const uint32_t *tile_gap_d = reinterpret_cast<const uint32_t *>(gs->gaps + 2 * two->n_gaps);
+            const uint2 *tile_gap_d = reinterpret_cast<const uint2 *>(gs->gaps + 2 * two->n_gaps);
             {
                 ah_ctx::PinSlot &gsl = pin_slot(c, run_bytes + tab_bytes);
                 memcpy(gsl.p, two->gaps, run_bytes);
-                uint32_t *tg = reinterpret_cast<uint32_t *>(gsl.p + run_bytes);
-                uint64_t gi = 0;
-                for (uint64_t t = 0; t <= gs->n_tiles; ++t) {
+                uint2 *tg = reinterpret_cast<uint2 *>(gsl.p + run_bytes);
+                uint64_t gi = 0, ge = 0; // the first run ending after the tile's start, the first starting past its reach
+                for (uint64_t t = 0; t < gs->n_tiles; ++t) {
                     const uint64_t p0 = t * kTileBases;
                     while (gi < two->n_gaps && two->gaps[2 * gi] + two->gaps[2 * gi + 1] <= p0)
                         ++gi;
-                    tg[t] = (uint32_t)gi;
+                    while (ge < two->n_gaps && two->gaps[2 * ge] < p0 + kTileBases + 32)
+                        ++ge;
+                    tg[t] = make_uint2((uint32_t)gi, (uint32_t)std::max(gi, ge));
                 }
                 launch_copy_words((const uint32_t *)gsl.dp, (uint32_t *)gaps_d, (run_bytes + tab_bytes) / 4, st);
                 AH_CUDA(cudaEventRecord(gsl.ev, st));
             }
             if (dev_seq) {
                 Stage sg(c, "pack", st, 1);
-                launch_pack2(seq, 0, n_bases, n_bases, gaps_d, two->n_gaps, tile_gap_d, gs->planes, 0, gs->n_tiles,
+                launch_pack2(seq, 0, n_bases, n_bases, gaps_d, tile_gap_d, gs->planes, 0, gs->n_tiles,
                              st);
             } else {
                 // host codes: tile-aligned chunks through two staging buffers (the whole
@@ -1839,7 +1855,7 @@ static ah_status load_impl(ah_ctx *c, const uint8_t *seq, uint64_t n_bases, cons
                     AH_CUDA(cudaStreamWaitEvent(st, c->ev_copied[b], 0));
                     {
                         Stage sg(c, "pack", st, 1);
-                        launch_pack2(stage[b], b0, b1 - b0, n_bases, gaps_d, two->n_gaps, tile_gap_d, gs->planes, t0,
+                        launch_pack2(stage[b], b0, b1 - b0, n_bases, gaps_d, tile_gap_d, gs->planes, t0,
                                      t1, st);
                     }
                     AH_CUDA(cudaEventRecord(c->ev_packed[b], st));
@@ -1887,32 +1903,8 @@ static ah_status load_impl(ah_ctx *c, const uint8_t *seq, uint64_t n_bases, cons
                 AH_CUDA(cudaEventRecord(c->ev_last_copy, c->copy_stream));
             }
         }
-        {
-            HostSpan hs_tables(c, "host.load.tables");
-            // the tables through a mapped pinned slot, read by one copy kernel; the
-            // per-tile contig table is built here by a merge walk over tiles and contigs
-            ah_ctx::PinSlot &sl = pin_slot(c, table_bytes);
-            memcpy(sl.p, contig_off, ob);
-            memcpy(sl.p + ob, contig_genome, gb);
-            {
-                // tile t: the last contig starting at or before t * kTileBases, and
-                // the room from the tile's first position to that contig's end
-                uint32_t *tc = (uint32_t *)(sl.p + ob + gb);
-                uint32_t *room = tc + (gs->n_tiles + 1);
-                uint32_t ci = 0;
-                for (uint64_t t = 0; t <= gs->n_tiles; ++t) {
-                    const uint64_t P = t * kTileBases;
-                    while (ci + 1 < n_contigs && contig_off[ci + 1] <= P)
-                        ++ci;
-                    tc[t] = ci;
-                    const uint64_t end = n_contigs ? contig_off[ci + 1] : 0;
-                    room[t] = end > P ? (uint32_t)std::min<uint64_t>(end - P, 0xffffffffull) : 0u;
-                }
-            }
-            Stage sg(c, "tables", st, 1);
-            launch_copy_words((const uint32_t *)sl.dp, (uint32_t *)gs->contig_off, table_bytes / 4, st);
-            AH_CUDA(cudaEventRecord(sl.ev, st));
-        }
+        if (!reversed)
+            queue_tables();
         if (c->set_events.empty()) {
             cudaEvent_t e;
             AH_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));

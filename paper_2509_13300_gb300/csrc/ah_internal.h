@@ -176,19 +176,14 @@ void launch_copy_words(const uint32_t *src, uint32_t *dst, uint64_t n_words, cud
 // 2 (p % 4) of byte p / 4) whose first byte holds position base0 (a tile
 // boundary) and that hold n_avail positions; gaps (device, n_gaps (start,
 // length) pairs, sorted, disjoint) and positions >= n_bases are no base;
-// tile_gap (device, one per tile + 1): the index of the first gap that ends
-// after the tile's first position.  codes must be 16-byte aligned.
+// tile_gap (device, one per tile): the gaps [x, y) that meet the tile or its 32
+// extension positions.  codes must be 16-byte aligned.
 void launch_pack2(const uint8_t *codes, uint64_t base0, uint64_t n_avail, uint64_t n_bases, const uint64_t *gaps,
-                  uint64_t n_gaps, const uint32_t *tile_gap, uint32_t *planes, uint64_t t0, uint64_t t1,
-                  cudaStream_t s);
-// One stretch of a contig-wise reversal: dst[k] = src[mirror - k] for k in
-// [start, start + len) (mirror = 2 * contig start + contig length - 1).
-struct RevChunk {
-    uint64_t start, mirror;
-    uint64_t len;
-};
-void launch_reverse_contigs(const uint8_t *src, uint8_t *dst, const RevChunk *chunks, uint64_t n_chunks,
-                            cudaStream_t s);
+                  const uint2 *tile_gap, uint32_t *planes, uint64_t t0, uint64_t t1, cudaStream_t s);
+// Pack a whole set with every contig reversed: position P of contig [o, e) holds
+// the base at o + e - 1 - P of seq (contig_off, tile_contig: the set's device tables).
+void launch_pack_reversed(const uint8_t *seq, uint64_t n_bases, uint32_t *planes, uint64_t n_tiles,
+                          const uint64_t *contig_off, const uint32_t *tile_contig, int *err, cudaStream_t s);
 void launch_unpack_check(const uint32_t *planes, uint64_t n_tiles, uint8_t *codes, uint64_t n_bases,
                          cudaStream_t s);
 

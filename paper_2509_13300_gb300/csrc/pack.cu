@@ -28,6 +28,16 @@
 // split between the logic and the multiply pipes (shifts by constants are
 // multiplies by run-time powers of two) so that the kernel is bound by HBM:
 // 1 byte read and 0.516 bytes written per base.
+//
+// Input at any address, and contigs packed reversed (decoy sets): the tile's
+// bytes are copied from the 16-byte boundary below their first, so the staged
+// tile is shifted by 0..15 bytes (the same for every tile), and a row word is two
+// staged words and a funnel shift; a reversed tile that lies in one contig is
+// the contig's mirrored stretch staged as it is, read backwards with the bytes
+// of each word reversed.  Tiles with a contig end inside (reversed) or at the
+// end of the input are gathered word by word.  Measured on a GB300: a reversed set
+// of 0.1 Gbp 233 us for a reversal pass and 41 for the packing -> 52 us; 4.6 Mbp at
+// an odd address 11.5 -> 8 us (byte loads before).
 #include <algorithm>
 #include <cstdlib>
 
@@ -220,13 +230,73 @@ __device__ __forceinline__ void pack_columns(const Row &rowf, int ci, uint32_t *
     }
 }
 
-__global__ void __launch_bounds__(kPackThreads, 6) pack_kernel(const uint8_t *__restrict__ seq, uint64_t seq_base,
+// Four bytes from any address, as aligned words.
+__device__ __forceinline__ uint32_t load4(const uint8_t *a)
+{
+    const uintptr_t u = reinterpret_cast<uintptr_t>(a);
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(u & ~(uintptr_t)3);
+    const uint32_t sh = (uint32_t)(u & 3u) * 8u;
+    const uint32_t lo = __ldg(w), hi = sh ? __ldg(w + 1) : 0u;
+    return __funnelshift_r(lo, hi, sh);
+}
+
+// What the input is to the packer: at a 16-byte boundary, at any address, or a
+// set whose contigs are packed reversed (at any address; position P of contig
+// [o, e) takes byte o + e - 1 - P).
+enum PackInput { kAligned, kShifted, kReversed };
+
+// A tile at the end of the input, or (reversed) with a contig end, into the
+// staging buffer: word by word, byte by byte where a word holds such an end;
+// zero past the end.
+template <int In>
+__device__ __forceinline__ void gather_tile(const uint8_t *__restrict__ seq, uint64_t seq_base, uint64_t lim, uint64_t p0,
+                                         const uint64_t *__restrict__ contig_off, uint32_t c, uint32_t *rows)
+{
+    constexpr uint32_t kWords = ((uint32_t)kTileBases + 32) / 4;
+    for (uint32_t w = threadIdx.x; w < kWords; w += blockDim.x) {
+        const uint64_t pos = p0 + 4ull * w;
+        uint32_t v = 0;
+        if (In == kReversed) {
+            if (pos < lim) {
+                while (contig_off[c + 1] <= pos)
+                    ++c;
+                if (pos + 4 <= contig_off[c + 1]) {
+                    v = __byte_perm(load4(seq + (contig_off[c] + contig_off[c + 1] - 4 - pos)), 0, 0x0123);
+                } else {
+                    uint32_t cc = c;
+                    for (int q = 0; q < 4 && pos + q < lim; ++q) {
+                        while (contig_off[cc + 1] <= pos + q)
+                            ++cc;
+                        v |= (uint32_t)seq[contig_off[cc] + contig_off[cc + 1] - 1 - (pos + q)] << (8 * q);
+                    }
+                }
+            }
+            rows[kWords - 1 - w] = __byte_perm(v, 0, 0x0123); // where a mirrored tile has it
+        } else {
+            if (pos >= seq_base && pos + 4 <= lim) {
+                v = load4(seq + (pos - seq_base));
+            } else {
+                for (int q = 0; q < 4; ++q)
+                    if (pos + q >= seq_base && pos + q < lim)
+                        v |= (uint32_t)seq[pos + q - seq_base] << (8 * q);
+            }
+            rows[w] = v;
+        }
+    }
+}
+
+// (five blocks per SM for shifted input: the second word and the shift do not fit in 40 registers)
+template <int In>
+__global__ void __launch_bounds__(kPackThreads, In == kAligned ? 6 : 5) pack_kernel(const uint8_t *__restrict__ seq, uint64_t seq_base,
                                                             uint64_t seq_len, uint64_t n_bases,
                                                             uint32_t *__restrict__ planes, uint64_t t0, uint64_t t1,
-                                                            int tma_ok, uint32_t one, int *__restrict__ err)
+                                                            const uint64_t *__restrict__ contig_off,
+                                                            const uint32_t *__restrict__ tile_contig, uint32_t one,
+                                                            int *__restrict__ err)
 {
     extern __shared__ __align__(128) uint32_t smem[]; // two staged tiles
     __shared__ __align__(8) uint64_t bar[2];
+    constexpr uint32_t kNeed = (uint32_t)kTileBases + 32; // the tile and the next one's head
     const uint64_t lim = n_bases < seq_base + seq_len ? n_bases : seq_base + seq_len;
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar[0])) : "memory");
@@ -234,20 +304,32 @@ __global__ void __launch_bounds__(kPackThreads, 6) pack_kernel(const uint8_t *__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    // a tile goes through TMA when all of its bytes (and the next tile's head) are present and aligned
+    // a tile goes through TMA when all of its bytes (and the next tile's head) are present
+    // (reversed: and in one contig)
     auto full = [&](uint64_t t) {
         const uint64_t p0 = t * kTileBases;
-        return tma_ok && p0 >= seq_base && p0 + kTileBases + 32 <= lim;
+        if (In == kReversed)
+            return p0 + kNeed <= contig_off[tile_contig[t] + 1];
+        return p0 >= seq_base && p0 + kNeed <= lim;
+    };
+    // the first source byte of a full tile
+    auto source = [&](uint64_t t) {
+        const uint64_t p0 = t * kTileBases;
+        if (In == kReversed) {
+            const uint32_t c = tile_contig[t];
+            return seq + (contig_off[c] + contig_off[c + 1] - (p0 + kNeed));
+        }
+        return seq + (p0 - seq_base);
     };
     auto issue = [&](uint64_t t, int sb) {
-        const uint64_t p0 = t * kTileBases;
         uint32_t *rows = smem + sb * kBufWords;
+        const uint8_t *src = source(t);
+        const uint32_t shift = In == kAligned ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(src) & 15u);
+        const uint32_t bytes = (kNeed + shift + 15u) & ~15u; // (both ends stay in their 16-byte granules)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar[sb])),
-                     "r"((uint32_t)(kTileBases + 32))
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar[sb])), "r"(bytes)
                      : "memory");
-        tma_load(rows, seq + (p0 - seq_base), (uint32_t)kTileBases, &bar[sb]);
-        tma_load(rows + 32 * kRowWords, seq + (p0 + kTileBases - seq_base), 32u, &bar[sb]);
+        tma_load(rows, src - shift, bytes, &bar[sb]);
     };
     uint32_t phase0 = 0, phase1 = 0;
     const uint64_t first = t0 + blockIdx.x;
@@ -262,7 +344,10 @@ __global__ void __launch_bounds__(kPackThreads, 6) pack_kernel(const uint8_t *__
         if (threadIdx.x == 0 && next < t1 && full(next))
             issue(next, sb ^ 1);
         const uint64_t p0 = t * kTileBases;
+        uint32_t shift = 0; // of the staged tile, in bytes
         if (full(t)) {
+            if (In != kAligned)
+                shift = (uint32_t)(reinterpret_cast<uintptr_t>(source(t)) & 15u);
             const bool ok = mbar_wait(&bar[sb], sb ? phase1 : phase0);
             if (sb)
                 phase1 ^= 1;
@@ -277,22 +362,21 @@ __global__ void __launch_bounds__(kPackThreads, 6) pack_kernel(const uint8_t *__
                 return;
             }
         } else {
-            // tail or unaligned tile: byte loads with bounds, zero past the end
-            for (int w = threadIdx.x; w < kBufWords; w += blockDim.x) {
-                const int r = w / kRowWords, cw = w % kRowWords;
-                uint32_t v = 0;
-                if (r < 32 || cw < 8) {
-                    const uint64_t pos = p0 + (uint64_t)r * kTileW + 4ull * cw;
-                    for (int q = 0; q < 4; ++q)
-                        if (pos + q >= seq_base && pos + q < lim)
-                            v |= (uint32_t)seq[pos + q - seq_base] << (8 * q);
-                }
-                rows[w] = v;
-            }
+            gather_tile<In>(seq, seq_base, lim, p0, contig_off, In == kReversed ? tile_contig[t] : 0u, rows);
             __syncthreads();
         }
         const int ci = threadIdx.x;
-        pack_columns([&](int r) { return rows[r * kRowWords + ci]; }, ci, planes + t * 4 * kTileWX, one);
+        const uint32_t *staged = rows + shift / 4;
+        const uint32_t sh = (shift & 3u) * 8u;
+        if constexpr (In == kAligned)
+            pack_columns([&](int r) { return rows[r * kRowWords + ci]; }, ci, planes + t * 4 * kTileWX, one);
+        else
+            pack_columns([&](int r) {
+                const uint32_t *w = In == kReversed ? staged + (kNeed / 4 - 1 - r * kRowWords - ci)
+                                                    : staged + (r * kRowWords + ci);
+                const uint32_t v = __funnelshift_r(w[0], w[1], sh);
+                return In == kReversed ? __byte_perm(v, 0, 0x0123) : v;
+            }, ci, planes + t * 4 * kTileWX, one);
         __syncthreads(); // this buffer is refilled two tiles from now
     }
 }
@@ -305,139 +389,152 @@ __global__ void __launch_bounds__(kPackThreads, 6) pack_kernel(const uint8_t *__
 // planes 0).  One block per tile: the tile's 8 KB of codes and the next
 // tile's first 8 bytes (the extension row) are loaded into shared memory with
 // coalesced 16-byte loads; thread ci builds the plane words of columns
-// 4 ci .. 4 ci + 3, for which row b holds exactly byte ci of the row.  Four
-// rows at a time: the rows' bytes form one 32-bit word, and each column's low
-// and high code bits are gathered into a nibble by one carry-free multiply.
-// A tile that a gap or the end of the data touches marks its no-base
-// positions in a shared bitmap first; tile_gap[t] (built at load by a merge
-// walk) is the first gap that ends after tile t's start.
+// 4 ci .. 4 ci + 3, for which row b holds exactly byte ci of the row: a 32 x 8
+// bit matrix, transposed in registers by three rounds of masked exchanges.  The
+// no-base runs of a tile (tile_gap, built at load by a merge walk) become masks
+// per column: the rows of column j that a run [a, b) covers are consecutive.
+// Bound: HBM (0.25 B read + 0.516 B written per base), then the latency of one
+// tile (its loads, a barrier, the matrix).  Measured, 1.5 Gbp with 0.1 % of no-base
+// runs on a GB300: 416 us with persistent blocks, a serial search of the tile's
+// runs and a bitmap read back row by row -> 266 us (4.3 TB/s).  (Packing pieces of a
+// host set while later pieces cross the link gains nothing: the copies stand
+// still for as long as the packing runs.)
 // ---------------------------------------------------------------------------
 constexpr int kCodeRowBytes = kTileW / 4;                  // 256 bytes of codes per row
 constexpr int kCodeWords = (32 * kCodeRowBytes + 16) / 4;  // the tile + the extension row (16 bytes read)
-constexpr int kInvWords = (kTileBases + 32) / 32;          // no-base bitmap of the tile + extension row
+constexpr int kFewGaps = 16;                               // runs of a tile turned into masks by every thread
 
-// bits 0, 8, 16, 24 of v (each 0 or 1) -> bits 0..3
-__device__ __forceinline__ uint32_t gather4(uint32_t v) { return (v * 0x10204080u) >> 28; }
+// The rows b of column j (bit b) whose position b * kTileW + j lies in [a, e).
+__device__ __forceinline__ uint32_t rows_of(uint32_t a, uint32_t e, uint32_t j)
+{
+    const uint32_t r0 = a > j ? (a - j + kTileW - 1) / kTileW : 0u; // first row at or above a
+    const uint32_t r1 = e > j ? (e - j + kTileW - 1) / kTileW : 0u; // first row at or above e
+    const uint32_t lo = r0 >= 32 ? 0xffffffffu : (1u << r0) - 1u, hi = r1 >= 32 ? 0xffffffffu : (1u << r1) - 1u;
+    return hi & ~lo;
+}
 
-__global__ void __launch_bounds__(kPackThreads) pack2_kernel(const uint8_t *__restrict__ codes, uint64_t base0,
-                                                             uint64_t n_avail, uint64_t n_bases,
-                                                             const uint64_t *__restrict__ gaps, uint64_t n_gaps,
-                                                             const uint32_t *__restrict__ tile_gap,
-                                                             uint32_t *__restrict__ planes, uint64_t t0, uint64_t t1)
+__global__ void __launch_bounds__(kPackThreads, 8) pack2_kernel(const uint8_t *__restrict__ codes, uint64_t base0,
+                                                                uint64_t n_avail, uint64_t n_bases,
+                                                                const ulonglong2 *__restrict__ gaps,
+                                                                const uint2 *__restrict__ tile_gap,
+                                                                uint32_t *__restrict__ planes, uint64_t t0)
 {
     __shared__ __align__(16) uint32_t cw[kCodeWords];
-    __shared__ uint32_t inv[kInvWords];
+    __shared__ uint2 run[kFewGaps + 1];             // the tile's runs, relative to its start
+    __shared__ __align__(16) uint32_t none[kTileW]; // many runs: per column, the rows that are no base
+    __shared__ uint32_t none_head;                  // ... and of the extension row's 32 positions
     const int ci = threadIdx.x;
     const uint64_t avail_end = base0 + n_avail < n_bases ? base0 + n_avail : n_bases; // bases present here
-    for (uint64_t t = t0 + blockIdx.x; t < t1; t += gridDim.x) {
-        const uint64_t p0 = t * kTileBases, pe = p0 + kTileBases + 32; // the tile and its extension row
-        // codes: bytes (p0 - base0) / 4 .. + 8208 of `codes`; zero past the available bytes
-        const uint64_t cb0 = (p0 - base0) / 4;
-        const uint64_t bytes_avail = (avail_end > p0 ? (avail_end - p0 + 3) / 4 : 0);
-        if (bytes_avail >= (uint64_t)kCodeWords * 4) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(codes + cb0);
-            for (int w = ci; w < kCodeWords / 4; w += blockDim.x)
-                reinterpret_cast<uint4 *>(cw)[w] = __ldg(src + w);
-        } else {
-            for (int w = ci; w < kCodeWords; w += blockDim.x) {
-                uint32_t v = 0;
-                for (int q = 0; q < 4; ++q)
-                    if ((uint64_t)(4 * w + q) < bytes_avail)
-                        v |= (uint32_t)codes[cb0 + 4 * w + q] << (8 * q);
-                cw[w] = v;
-            }
+    const uint64_t t = t0 + blockIdx.x;
+    const uint64_t p0 = t * kTileBases;
+    constexpr uint32_t kEnd = (uint32_t)kTileBases + 32; // the tile and its extension row
+    const uint2 tg = __ldg(tile_gap + t);                // its runs: gaps[tg.x .. tg.y)
+    // codes: bytes (p0 - base0) / 4 .. + 8208 of `codes`; zero past the available bytes
+    const uint64_t cb0 = (p0 - base0) / 4;
+    const uint64_t bytes_avail = (avail_end > p0 ? (avail_end - p0 + 3) / 4 : 0);
+    if (bytes_avail >= (uint64_t)kCodeWords * 4) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(codes + cb0);
+        for (int w = ci; w < kCodeWords / 4; w += kPackThreads)
+            reinterpret_cast<uint4 *>(cw)[w] = __ldg(src + w);
+    } else {
+        for (int w = ci; w < kCodeWords; w += kPackThreads) {
+            uint32_t v = 0;
+            for (int q = 0; q < 4; ++q)
+                if ((uint64_t)(4 * w + q) < bytes_avail)
+                    v |= (uint32_t)codes[cb0 + 4 * w + q] << (8 * q);
+            cw[w] = v;
         }
-        // no-base positions: gaps that meet [p0, pe), and everything at or past avail_end;
-        // the tile's first gap ending after p0 comes from the table built at load
-        const uint64_t first_gap = tile_gap[t];
-        const bool marked = (first_gap < n_gaps && gaps[2 * first_gap] < pe) || avail_end < pe;
+    }
+    const uint32_t listed = tg.y - tg.x;
+    const bool few = listed <= kFewGaps;
+    const bool cut = avail_end < p0 + kEnd; // everything at or past avail_end is no base
+    auto clipped = [&](uint32_t g) {        // run g of the tile, relative to p0
+        const ulonglong2 x = __ldg(gaps + tg.x + g);
+        auto rel = [&](uint64_t p) { return p <= p0 ? 0u : p - p0 < kEnd ? (uint32_t)(p - p0) : kEnd; };
+        return make_uint2(rel(x.x), rel(x.x + x.y));
+    };
+    if (few) {
+        if ((uint32_t)ci < listed)
+            run[ci] = clipped(ci);
+        if (cut && ci == 0)
+            run[listed] = make_uint2((uint32_t)(avail_end > p0 ? avail_end - p0 : 0ull), kEnd);
+    } else { // mark every position of every run, a run per warp
+        for (int w = ci; w < kTileW; w += kPackThreads)
+            none[w] = 0u;
+        if (ci == 0)
+            none_head = 0u;
         __syncthreads();
-        if (marked) {
-            for (int w = ci; w < kInvWords; w += blockDim.x)
-                inv[w] = 0u;
-            __syncthreads();
-            auto mark = [&](uint64_t a, uint64_t b) { // positions [a, b) of the tile, relative to p0
-                const uint64_t w0 = a >> 5, w1 = (b - 1) >> 5;
-                for (uint64_t w = w0 + ci; w <= w1; w += blockDim.x) {
-                    const uint64_t x0 = a > 32 * w ? a - 32 * w : 0, x1 = b < 32 * w + 32 ? b - 32 * w : 32;
-                    const uint32_t m = (x1 - x0 >= 32 ? 0xffffffffu : ((1u << (x1 - x0)) - 1u)) << x0;
-                    atomicOr(&inv[w], m);
-                }
-            };
-            for (uint64_t g = first_gap; g < n_gaps && gaps[2 * g] < pe; ++g) {
-                const uint64_t e = gaps[2 * g] + gaps[2 * g + 1];
-                if (e <= p0) // (only out-of-order runs end before the tile: never index with them)
-                    continue;
-                const uint64_t a = gaps[2 * g] > p0 ? gaps[2 * g] - p0 : 0;
-                const uint64_t b = (e < pe ? e : pe) - p0;
-                if (b > a)
-                    mark(a, b);
-            }
-            if (avail_end < pe)
-                mark(avail_end > p0 ? avail_end - p0 : 0, pe - p0);
+        for (uint32_t g = ci / 32; g < listed + (cut ? 1u : 0u); g += kPackThreads / 32) {
+            const uint2 r = g < listed ? clipped(g) : make_uint2((uint32_t)(avail_end > p0 ? avail_end - p0 : 0ull), kEnd);
+            for (uint32_t x = r.x + ci % 32; x < r.y; x += 32)
+                if (x < kTileBases)
+                    atomicOr(&none[x % kTileW], 1u << (x / kTileW));
+                else
+                    atomicOr(&none_head, 1u << (x - kTileBases));
         }
-        __syncthreads();
-        const uint8_t *cbytes = reinterpret_cast<const uint8_t *>(cw);
-        uint32_t lo[4] = {0, 0, 0, 0}, hi[4] = {0, 0, 0, 0};
+    }
+    __syncthreads();
+    const int j0 = 4 * ci;
+    const uint8_t *cbytes = reinterpret_cast<const uint8_t *>(cw);
+    // x[r], byte q = the codes of row r + 8 q (4 columns, 2 bits each) ...
+    uint32_t x[8];
 #pragma unroll
-        for (int rb = 0; rb < 8; ++rb) {
-            const uint32_t x = (uint32_t)cbytes[(4 * rb + 0) * kCodeRowBytes + ci] |
-                               ((uint32_t)cbytes[(4 * rb + 1) * kCodeRowBytes + ci] << 8) |
-                               ((uint32_t)cbytes[(4 * rb + 2) * kCodeRowBytes + ci] << 16) |
-                               ((uint32_t)cbytes[(4 * rb + 3) * kCodeRowBytes + ci] << 24);
+    for (int r = 0; r < 8; ++r) {
+        const uint32_t b0 = cbytes[r * kCodeRowBytes + ci], b1 = cbytes[(r + 8) * kCodeRowBytes + ci],
+                       b2 = cbytes[(r + 16) * kCodeRowBytes + ci], b3 = cbytes[(r + 24) * kCodeRowBytes + ci];
+        x[r] = __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
+    }
+    // ... transposed as an 8 x 8 bit matrix in every byte: x[k], bit 8 q + r = bit k of that row's codes
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int sft = 1 << i;
+        const uint32_t m = i == 0 ? 0x55555555u : i == 1 ? 0x33333333u : 0x0f0f0f0fu;
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            if (!(r & sft)) {
+                const uint32_t u = x[r], v = x[r | sft];
+                x[r] = (u & m) | ((v << sft) & ~m);
+                x[r | sft] = ((u >> sft) & m) | (v & ~m);
+            }
+    }
+    // the rows that are no base, per column (bit k of head: position k of this thread's part of the extension row)
+    uint32_t bad[4] = {0, 0, 0, 0}, head = 0;
+    if (few) {
+        for (uint32_t g = 0; g < listed + (cut ? 1u : 0u); ++g) {
+            const uint2 r = run[g];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                lo[k] |= gather4((x >> (2 * k)) & 0x01010101u) << (4 * rb);
-                hi[k] |= gather4((x >> (2 * k + 1)) & 0x01010101u) << (4 * rb);
+                bad[k] |= rows_of(r.x, r.y, j0 + k);
+                const uint32_t h = (uint32_t)kTileBases + j0 + k;
+                head |= (h >= r.x && h < r.y ? 1u : 0u) << k;
             }
         }
-        uint32_t val[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-        if (marked) {
-#pragma unroll 4
-            for (int b = 0; b < 32; ++b) {
-                const uint32_t nib = (inv[b * (kTileW / 32) + (ci >> 3)] >> (4 * (ci & 7))) & 0xFu;
+    } else {
+        const uint4 v = *reinterpret_cast<const uint4 *>(none + j0);
+        bad[0] = v.x;
+        bad[1] = v.y;
+        bad[2] = v.z;
+        bad[3] = v.w;
+        head = j0 < kTileExt ? none_head >> j0 : 0u;
+    }
+    uint32_t *dst = planes + t * 4 * kTileWX;
+    const uint32_t hb = j0 < kTileExt ? (uint32_t)cbytes[32 * kCodeRowBytes + ci] : 0u;
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    val[k] &= ~(((nib >> k) & 1u) << b);
-            }
-        }
-        uint4 pa, pc, pg, pt;
-        uint32_t *A = &pa.x, *C = &pc.x, *G = &pg.x, *T = &pt.x;
+    for (int pl = 0; pl < 4; ++pl) { // A 00, C 01, G 10, T 11
+        uint4 w;
+        uint32_t *W = &w.x;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            A[k] = val[k] & ~hi[k] & ~lo[k];
-            C[k] = val[k] & ~hi[k] & lo[k];
-            G[k] = val[k] & hi[k] & ~lo[k];
-            T[k] = val[k] & hi[k] & lo[k];
-        }
-        uint32_t *dst = planes + t * 4 * kTileWX;
-        const int j0 = 4 * ci;
-        *reinterpret_cast<uint4 *>(dst + 0 * kTileWX + j0) = pa;
-        *reinterpret_cast<uint4 *>(dst + 1 * kTileWX + j0) = pc;
-        *reinterpret_cast<uint4 *>(dst + 2 * kTileWX + j0) = pg;
-        *reinterpret_cast<uint4 *>(dst + 3 * kTileWX + j0) = pt;
-        if (j0 < kTileExt) {
-            // extension words: row b + 1 of the same column, bit 31 from the next tile's head
-            const uint32_t hb = cbytes[32 * kCodeRowBytes + ci];
-            uint32_t hv = 0xFu;
-            if (marked)
-                hv = ~(inv[kTileBases / 32 + (ci >> 3)] >> (4 * (ci & 7))) & 0xFu;
-            uint4 ea, ec, eg, et;
-            uint32_t *EA = &ea.x, *EC = &ec.x, *EG = &eg.x, *ET = &et.x;
+        for (int k = 0; k < 4; ++k)
+            W[k] = ~bad[k] & (pl & 1 ? x[2 * k] : ~x[2 * k]) & (pl & 2 ? x[2 * k + 1] : ~x[2 * k + 1]);
+        *reinterpret_cast<uint4 *>(dst + pl * kTileWX + j0) = w;
+        if (j0 < kTileExt) { // extension words: row b + 1 of the same column, bit 31 from the next tile's head
+            uint4 ew;
+            uint32_t *EW = &ew.x;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t code = (hb >> (2 * k)) & 3u, v = (hv >> k) & 1u;
-                EA[k] = (A[k] >> 1) | ((v & (code == 0)) << 31);
-                EC[k] = (C[k] >> 1) | ((v & (code == 1)) << 31);
-                EG[k] = (G[k] >> 1) | ((v & (code == 2)) << 31);
-                ET[k] = (T[k] >> 1) | ((v & (code == 3)) << 31);
-            }
-            *reinterpret_cast<uint4 *>(dst + 0 * kTileWX + kTileW + j0) = ea;
-            *reinterpret_cast<uint4 *>(dst + 1 * kTileWX + kTileW + j0) = ec;
-            *reinterpret_cast<uint4 *>(dst + 2 * kTileWX + kTileW + j0) = eg;
-            *reinterpret_cast<uint4 *>(dst + 3 * kTileWX + kTileW + j0) = et;
+            for (int k = 0; k < 4; ++k)
+                EW[k] = (W[k] >> 1) | ((((hb >> (2 * k)) & 3u) == (uint32_t)pl && !(head >> k & 1u) ? 1u : 0u) << 31);
+            *reinterpret_cast<uint4 *>(dst + pl * kTileWX + kTileW + j0) = ew;
         }
-        __syncthreads(); // the shared buffers are refilled for the next tile
     }
 }
 
@@ -472,23 +569,16 @@ __global__ void copy_words_kernel(const uint32_t *__restrict__ src, uint32_t *__
 } // namespace
 
 void launch_pack2(const uint8_t *codes, uint64_t base0, uint64_t n_avail, uint64_t n_bases, const uint64_t *gaps,
-                  uint64_t n_gaps, const uint32_t *tile_gap, uint32_t *planes, uint64_t t0, uint64_t t1,
-                  cudaStream_t s)
+                  const uint2 *tile_gap, uint32_t *planes, uint64_t t0, uint64_t t1, cudaStream_t s)
 {
     if (t1 <= t0)
         return;
     if (reinterpret_cast<uintptr_t>(codes) % 16 != 0 || base0 % kTileBases != 0)
         throw Error(AH_ERR_ARG, "2-bit codes must start 16-byte aligned at a tile boundary");
-    static int cached_dev = -1, sms = 148;
-    int dev = 0;
-    AH_CUDA(cudaGetDevice(&dev));
-    if (dev != cached_dev) {
-        AH_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        cached_dev = dev;
-    }
-    const uint64_t blocks = std::min<uint64_t>(t1 - t0, (uint64_t)sms * 8);
-    pack2_kernel<<<(unsigned)blocks, kPackThreads, 0, s>>>(codes, base0, n_avail, n_bases, gaps, n_gaps, tile_gap,
-                                                           planes, t0, t1);
+    // one block per tile (blocks end as tiles are done, as in launch_pack)
+    pack2_kernel<<<(unsigned)(t1 - t0), kPackThreads, 0, s>>>(codes, base0, n_avail, n_bases,
+                                                              reinterpret_cast<const ulonglong2 *>(gaps), tile_gap,
+                                                              planes, t0);
     AH_CUDA(cudaGetLastError());
 }
 
@@ -501,12 +591,14 @@ void launch_copy_words(const uint32_t *src, uint32_t *dst, uint64_t n_words, cud
     AH_CUDA(cudaGetLastError());
 }
 
-void launch_pack(const uint8_t *seq, uint64_t seq_base, uint64_t seq_len, uint64_t n_bases, uint32_t *planes,
-                 uint64_t t0, uint64_t t1, int *err, cudaStream_t s)
+namespace {
+template <int In>
+void launch_pack_as(const uint8_t *seq, uint64_t seq_base, uint64_t seq_len, uint64_t n_bases, uint32_t *planes,
+                    uint64_t t0, uint64_t t1, const uint64_t *contig_off, const uint32_t *tile_contig, int *err,
+                    cudaStream_t s)
 {
-    if (t1 <= t0)
-        return;
     static_assert(kTileW % 128 == 0 && kTileExt == 32, "pack layout");
+    static_assert(kBufWords * 4 >= kTileBases + 32 + 32, "a staged tile with its shift");
     const size_t smem = 2ull * kBufWords * sizeof(uint32_t); // two staged tiles (67.6 KB)
     // grid size and the shared-memory opt-in, once per device
     static int cached_dev = -1, sms = 148, per_sm = 1;
@@ -514,8 +606,8 @@ void launch_pack(const uint8_t *seq, uint64_t seq_base, uint64_t seq_len, uint64
     AH_CUDA(cudaGetDevice(&dev));
     if (dev != cached_dev) {
         AH_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        AH_CUDA(cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pack_kernel, kPackThreads, smem));
+        AH_CUDA(cudaFuncSetAttribute(pack_kernel<In>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pack_kernel<In>, kPackThreads, smem));
         // one block per tile: blocks end as tiles are done, so kernels that run
         // beside the packing (a run's later stages) get SMs as they free up;
         // AH_PACK_BLOCKS=n keeps n persistent blocks per SM instead (profiling aid)
@@ -539,37 +631,29 @@ void launch_pack(const uint8_t *seq, uint64_t seq_base, uint64_t seq_len, uint64
     size_t smem_launch = blocks >= t1 - t0 ? smem / 2 : smem;
     if (const char *e = getenv("AH_PACK_SMEM_KB"))
         smem_launch = std::min(smem, std::max(blocks >= t1 - t0 ? smem / 2 : smem, (size_t)atoi(e) * 1024));
-    const int tma_ok = ((reinterpret_cast<uintptr_t>(seq) - seq_base) % 16 == 0) ? 1 : 0;
-    pack_kernel<<<(unsigned)blocks, kPackThreads, smem_launch, s>>>(seq, seq_base, seq_len, n_bases, planes, t0, t1,
-                                                                    tma_ok, 1u, err);
+    pack_kernel<In><<<(unsigned)blocks, kPackThreads, smem_launch, s>>>(seq, seq_base, seq_len, n_bases, planes, t0,
+                                                                        t1, contig_off, tile_contig, 1u, err);
     AH_CUDA(cudaGetLastError());
 }
-
-namespace {
-
-// Contig-wise reversal of the ASCII input (decoy genomes): one block per
-// stretch; consecutive threads read consecutive (descending) source bytes.
-__global__ void reverse_contigs_kernel(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst,
-                                       const RevChunk *__restrict__ chunks)
-{
-    const RevChunk c = chunks[blockIdx.x];
-    for (uint64_t i = threadIdx.x; i < c.len; i += blockDim.x) {
-        const uint64_t k = c.start + i;
-        dst[k] = src[c.mirror - k];
-    }
-}
-
 } // namespace
 
-void launch_reverse_contigs(const uint8_t *src, uint8_t *dst, const RevChunk *chunks, uint64_t n_chunks,
-                            cudaStream_t s)
+void launch_pack(const uint8_t *seq, uint64_t seq_base, uint64_t seq_len, uint64_t n_bases, uint32_t *planes,
+                 uint64_t t0, uint64_t t1, int *err, cudaStream_t s)
 {
-    if (n_chunks == 0)
+    if (t1 <= t0)
         return;
-    if (n_chunks > 0x7fffffffull)
-        throw Error(AH_ERR_ARG, "reversal: too many stretches");
-    reverse_contigs_kernel<<<(unsigned)n_chunks, 256, 0, s>>>(src, dst, chunks);
-    AH_CUDA(cudaGetLastError());
+    // (tiles start 32 KB apart, so all of an input's tiles are shifted alike)
+    if ((reinterpret_cast<uintptr_t>(seq) - seq_base) % 16 == 0)
+        launch_pack_as<kAligned>(seq, seq_base, seq_len, n_bases, planes, t0, t1, nullptr, nullptr, err, s);
+    else
+        launch_pack_as<kShifted>(seq, seq_base, seq_len, n_bases, planes, t0, t1, nullptr, nullptr, err, s);
+}
+
+void launch_pack_reversed(const uint8_t *seq, uint64_t n_bases, uint32_t *planes, uint64_t n_tiles,
+                          const uint64_t *contig_off, const uint32_t *tile_contig, int *err, cudaStream_t s)
+{
+    if (n_tiles)
+        launch_pack_as<kReversed>(seq, 0, n_bases, n_bases, planes, 0, n_tiles, contig_off, tile_contig, err, s);
 }
 
 void launch_unpack_check(const uint32_t *planes, uint64_t n_tiles, uint8_t *codes, uint64_t n_bases, cudaStream_t s)

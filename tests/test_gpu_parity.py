@@ -1333,3 +1333,67 @@ def test_amplitype_hash_groups_and_tables(ctx, lens):
         assert np.array_equal(again[0], want_v)
     finally:
         ctx.ah_unload_genomes(sid)
+
+
+@pytest.mark.parametrize("offset", [0, 1, 3, 4, 7, 8, 13, 15])
+@pytest.mark.parametrize("reversed_", [False, True])
+def test_packing_at_any_address_and_mirrored(ctx, offset, reversed_):
+    """Device input at every kind of misalignment, forward and with its contigs reversed: the
+    letters of every contig (sets ending inside, at and just past a tile; contigs from one letter
+    to several tiles; letters of either case, N and other bytes) come back as the oracle gives them."""
+    import torch
+    rng = np.random.default_rng(offset)
+    T = 32 * 1024
+    for n in (5, T - 1, T, T + 33, 4 * T + 17):
+        seq = synth.random_bases(rng, n, 0.5).copy()
+        at = rng.integers(0, n, 1 + n // 500)
+        seq[at] = rng.integers(0, 256, len(at), dtype=np.uint8)
+        low = rng.random(n) < 0.2
+        seq[low & (seq >= 65) & (seq <= 90)] += 32
+        cuts = np.unique(rng.integers(1, n, 6)) if n > 10 else np.array([2])
+        off = np.concatenate([[0], cuts, cuts[-1:], [n]]).astype(np.uint64)  # one empty contig
+        gen = np.zeros(len(off) - 1, np.uint32)
+        buf = torch.zeros(n + 64, dtype=torch.uint8, device="cuda")
+        buf[:] = ord("C")  # neighbours of the input are bases
+        buf[offset:offset + n] = torch.from_numpy(seq).cuda()
+        torch.cuda.synchronize()
+        amps = np.zeros(len(off) - 1, dtype=ah.AMPLICON_DTYPE)
+        amps["contig"] = np.arange(len(amps))
+        amps["end"] = np.diff(off.astype(np.int64))
+        want, _ = oracle.fetch(oracle.reverse_contigs(seq, off) if reversed_ else seq, off, amps)
+        sid = ctx.ah_load_genomes(buf[offset:], n, off, gen, reversed=reversed_)
+        try:
+            got, _ = ctx.fetch(sid, amps)
+        finally:
+            ctx.ah_unload_genomes(sid)
+        assert got == want, n
+
+
+@pytest.mark.parametrize("per_tile", [0, 1, 15, 16, 17, 900])
+def test_2bit_packing_with_few_and_many_no_base_runs(ctx, per_tile):
+    """2-bit loads whose tiles meet few no-base runs (masks per column) and many (marked position by
+    position), runs across tile ends, over whole tiles and at the set's end: the letters come back."""
+    import torch
+    rng = np.random.default_rng(per_tile)
+    T = 32 * 1024
+    for n in (70, T - 3, 4 * T + 40):
+        seq = synth.random_bases(rng, n, 0.5).copy()
+        for t in range(0, n, T):
+            for s0 in rng.integers(t, min(n, t + T), per_tile):
+                seq[s0:s0 + int(rng.integers(1, 12))] = ord("N")
+        if n > 2 * T:
+            seq[T - 5:T + 40] = ord("N")      # across a tile end and its extension row
+            seq[2 * T - 1:3 * T + 1] = ord("N")  # a whole tile
+            seq[n - 9:] = ord("N")
+        codes, gaps = ah.encode_2bit(seq)
+        off = np.array([0, n], np.uint64)
+        amps = np.zeros(1, dtype=ah.AMPLICON_DTYPE)
+        amps["end"] = n
+        for c in (codes, torch.from_numpy(codes).cuda()):
+            torch.cuda.synchronize()
+            sid = ctx.ah_load_genomes_2bit(c, n, gaps, off, np.zeros(1, np.uint32))
+            try:
+                got, _ = ctx.fetch(sid, amps)
+            finally:
+                ctx.ah_unload_genomes(sid)
+            assert got == seq.tobytes(), n
