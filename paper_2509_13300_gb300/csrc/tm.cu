@@ -589,301 +589,524 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *__rest
 // ---------------------------------------------------------------------------
 // Thread-per-site Tm (the path taken when every pair has few_exact).  The same
 // maximum as tm_kernel -- Dinkelbach iteration on the key-position shortest
-// path, fp32 -- but one thread carries all four states of one site: each
-// state keeps its path cost and the path's dH and dS sums, so the argmin
-// oligo's terms come out of the forward pass without a backtrack.  Between
-// two keys that are not adjacent the segment's table is separable (the stack
-// out of key k0 depends only on the base at k0, the stack into key k1 only on
-// the base at k1, the fixed stretch between them on neither), so one argmin
-// over the four predecessors serves all four successors.  A warp gathers its
-// 32 sites' windows together: per site, four coalesced 32-word loads (one per
-// plane) and four ballots give the window's bases as 32-bit columns.  Sites
-// whose maximum lies within 0.01 deg C of tm_min are deferred to tm_kernel
-// (which decides them exactly); everything else is written here.
+// path, fp32 -- but one thread carries all states of one site: each state keeps
+// its path cost and the path's dH and dS sums, so the argmin oligo's terms come
+// out of the forward pass without a backtrack.  Between two keys that are not
+// adjacent the segment's table is separable (the stack out of key k0 depends
+// only on the base at k0, the stack into key k1 only on the base at k1, the
+// fixed stretch between them on neither), so one argmin over the predecessors
+// serves all successors.  Sites whose maximum lies within 0.01 deg C of tm_min are
+// deferred to tm_kernel (which decides them exactly); everything else is
+// written here.
+//
+// A block takes up to kFastBatch sites at a time.  Gather: a warp fetches a
+// site's window with one 16-byte load per lane (8 lanes per plane, 4 words each,
+// from the 16-byte boundary below the window) and four ballots; each lane unpacks
+// its own site's ballots into 2-bit template codes.  Sort: the block lists its
+// sites by primer and its warps claim 32 of one primer at a time: a primer's path
+// is a list of steps (its keys, and the table offsets of the bases each allows)
+// that all lanes follow together, so no branch diverges and bases outside a set
+// are not visited; steps between sets of one or two bases, all but the few with
+// three or four, run without a test.  (Sites in canonical order mix both primers
+// in every warp.)  Bound: issue slots.  Measured on a GB300, 3.3 M sites of three
+// pairs: 727 us with sites in order, four loads per site and all 16 transitions ->
+// 419 us; 0.94 M sites of two pairs 243 -> 145 us.
 // ---------------------------------------------------------------------------
-constexpr int kFastThreads = 128;
+constexpr int kFastThreads = 256;
+constexpr int kFastBatch = 1024;                        // sites of a block between two barriers, at most
+constexpr int kFastClasses = 2 * AH_MAX_PAIRS_PER_SCAN; // pair * 2 + primer
+constexpr int kFastChunks = kFastBatch / 32 + kFastClasses; // groups of 32 sites of one class, at most
+static_assert(kFastClasses == 32, "one lane per class");
 
-// Per pair in shared memory: stacks as (1000 dH, dS) indexed [template bases
-// (t0, t1)][oligo bases (o0, o1)], so the 16 entries of one template pair are
-// contiguous; terminal pairs [oligo base][template base]; per primer its keys,
-// masks, length and C + salt entropy.
+// One step of a primer's path, from key k0 to the next key k1.  Sets of one or two
+// bases at both: byte offsets of the stack table's rows for the two bases x at k0
+// and y at k1, in ascending order (a single base stands twice).
+struct TmStep {
+    uint8_t sh0, sh1;     // 2 k0, 2 (k1 - 1): the template pairs (k0, k0 + 1) and (k1 - 1, k1)
+    uint8_t n0, n1;       // bases at k0 and at k1
+    uint16_t off[4];      // k1 = k0 + 1: [2 x + y]; else out of k0 [x], then into k1 [2 + y]
+    uint8_t list0, list1; // the bases, ascending, 2 bits each
+    uint8_t fixed;        // the fixed bases at k0 + 1 and (<< 2) k1 - 1
+    uint8_t kind;         // 1: k1 > k0 + 1, 2: a set of three or four bases at either key
+};
+static_assert(sizeof(TmStep) == 16, "a step is one 16-byte load");
+
+struct TmFastPrimer {
+    TmStep step[AH_MAX_PRIMER_LEN - 1];
+    uint64_t has[4]; // bit 2 q: the base is in position q's set
+    uint64_t first;  // the lowest base of each set
+    uint32_t fixes;  // bit q: positions q and q + 1 lie between two keys
+    int n_step, L;
+    int nF, listF, nL, listL; // the sets at both ends
+    float cst;                // C + salt entropy
+    int pad[2];
+};
+// Per pair: stacks as (1000 dH, dS), a row per oligo pair o0 + 4 o1, indexed by the
+// template pair t0 + 4 t1: lanes that read one row at their own template pairs meet
+// no bank twice (a row per template pair puts all lanes of such a read into one
+// bank: 234 us on the 0.94 M sites).  Terminal pairs [oligo base][template base].
 struct TmFastPair {
     float2 st[256];
     float2 tm[16];
-    uint8_t mask[2][AH_MAX_PRIMER_LEN];
-    uint8_t key[2][AH_MAX_PRIMER_LEN];
-    int L[2], nkey[2];
-    float cst[2];
-    float tm_min_f, tm_shift_f;
+    TmFastPrimer pr[2];
+    float tm_min_f, tm_shift_f, pad[2];
 };
-static_assert(sizeof(TmFastPair) % 8 == 0, "TmFastPair keeps 8-byte alignment");
+static_assert(sizeof(TmFastPair) % 16 == 0 && offsetof(TmFastPair, pr) % 16 == 0 && sizeof(TmFastPrimer) % 16 == 0,
+              "steps keep 16-byte alignment");
 
-__global__ void __launch_bounds__(kFastThreads) tm_fast_kernel(const ah_site *__restrict__ sites, uint64_t n_arg,
-                                                               const uint64_t *__restrict__ n_dev,
-                                                               const PairDev *__restrict__ pairs, int n_pairs,
-                                                               const uint32_t *__restrict__ planes,
-                                                               const uint64_t *__restrict__ contig_off,
-                                                               float *__restrict__ tm_out,
-                                                               uint8_t *__restrict__ pass_out,
-                                                               uint32_t *__restrict__ defer,
-                                                               unsigned long long *__restrict__ defer_n,
-                                                               int *__restrict__ err)
+// One warp builds a primer's steps: lane q holds position q.
+__device__ __forceinline__ void tm_fast_primer(TmFastPrimer &F, const PairDev &P, int x, int lane)
+{
+    const int L = P.L[x];
+    const uint32_t m = lane < L ? P.mask[x][lane] : 0u;
+    const bool key = lane < L && (lane == 0 || lane == L - 1 || __popc(m) > 1);
+    const uint32_t keys = __ballot_sync(0xffffffffu, key), below = keys & ((1u << lane) - 1u);
+    const uint32_t fixed = __ballot_sync(0xffffffffu, lane < L && !key);
+    uint32_t list = 0; // ascending, 2 bits each
+    for (int b = 3; b >= 0; --b)
+        if (m >> b & 1u)
+            list = list << 2 | (uint32_t)b;
+    const int k0 = below ? 31 - __clz(below) : 0;
+    const int cnt = __popc(m);
+    const uint32_t list0 = __shfl_sync(0xffffffffu, list, k0);
+    const int cnt0 = __shfl_sync(0xffffffffu, cnt, k0);
+    const uint32_t fa = __shfl_sync(0xffffffffu, list, (k0 + 1) & 31) & 3u;
+    const uint32_t fb = __shfl_sync(0xffffffffu, list, (lane - 1) & 31) & 3u;
+    if (key && lane > 0) {
+        TmStep s{};
+        s.sh0 = (uint8_t)(2 * k0);
+        s.sh1 = (uint8_t)(2 * (lane - 1));
+        s.n0 = (uint8_t)cnt0;
+        s.n1 = (uint8_t)cnt;
+        s.list0 = (uint8_t)list0;
+        s.list1 = (uint8_t)list;
+        s.fixed = (uint8_t)(fa | fb << 2);
+        const bool apart = lane > k0 + 1;
+        s.kind = (uint8_t)((apart ? 1 : 0) | (cnt0 > 2 || cnt > 2 ? 2 : 0));
+        const uint32_t a0 = list0 & 3u, a1 = cnt0 > 1 ? list0 >> 2 & 3u : a0;
+        const uint32_t c0 = list & 3u, c1 = cnt > 1 ? list >> 2 & 3u : c0;
+        s.off[0] = (uint16_t)(128 * (apart ? a0 + 4 * fa : a0 + 4 * c0));
+        s.off[1] = (uint16_t)(128 * (apart ? a1 + 4 * fa : a0 + 4 * c1));
+        s.off[2] = (uint16_t)(128 * (apart ? fb + 4 * c0 : a1 + 4 * c0));
+        s.off[3] = (uint16_t)(128 * (apart ? fb + 4 * c1 : a1 + 4 * c1));
+        F.step[__popc(below) - 1] = s;
+    }
+    uint64_t bits = lane < L ? (uint64_t)(list & 3u) << (2 * lane) : 0ull;
+    const uint32_t flo = __reduce_or_sync(0xffffffffu, (uint32_t)bits), fhi = __reduce_or_sync(0xffffffffu, (uint32_t)(bits >> 32));
+    for (int b = 0; b < 4; ++b) {
+        bits = (uint64_t)(m >> b & 1u) << (2 * lane);
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)bits), hi = __reduce_or_sync(0xffffffffu, (uint32_t)(bits >> 32));
+        if (lane == b)
+            F.has[b] = (uint64_t)hi << 32 | lo;
+    }
+    if (lane == 0) {
+        F.first = (uint64_t)fhi << 32 | flo;
+        F.fixes = fixed & fixed >> 1;
+        F.n_step = __popc(keys) - 1;
+        F.L = L;
+        F.nF = cnt;
+        F.listF = (int)list;
+        F.cst = (float)(P.sconst + (P.saltcorr == 5 ? 0.368 * (double)(L - 1) * P.log_na : 0.0));
+    }
+    if (lane == L - 1) {
+        F.nL = cnt;
+        F.listL = (int)list;
+    }
+}
+
+// 8 x 8 bit transpose: bit c of byte r -> bit r of byte c
+__device__ __forceinline__ uint64_t transpose8(uint64_t x)
+{
+    uint64_t t = (x ^ (x >> 7)) & 0x00AA00AA00AA00AAull;
+    x ^= t ^ (t << 7);
+    t = (x ^ (x >> 14)) & 0x0000CCCC0000CCCCull;
+    x ^= t ^ (t << 14);
+    t = (x ^ (x >> 28)) & 0x00000000F0F0F0F0ull;
+    return x ^ t ^ (t << 28);
+}
+
+__global__ void __launch_bounds__(kFastThreads, 4) tm_fast_kernel(const ah_site *__restrict__ sites, uint64_t n_arg,
+                                                                  const uint64_t *__restrict__ n_dev,
+                                                                  const PairDev *__restrict__ pairs, int n_pairs,
+                                                                  const uint32_t *__restrict__ planes,
+                                                                  const uint64_t *__restrict__ contig_off,
+                                                                  float *__restrict__ tm_out,
+                                                                  uint8_t *__restrict__ pass_out,
+                                                                  uint32_t *__restrict__ defer,
+                                                                  unsigned long long *__restrict__ defer_n,
+                                                                  int *__restrict__ err)
 {
     extern __shared__ __align__(16) unsigned char fast_smem[];
     TmFastPair *fp = reinterpret_cast<TmFastPair *>(fast_smem);
+    __shared__ uint64_t win[kFastThreads];                 // byte offset of a window's 16-byte boundary in the A plane
+    __shared__ uint32_t win_last[kFastThreads];            // byte offset of its last 16-byte group from there
+    __shared__ uint32_t win_bit[kFastThreads];             // the bit of its row
+    __shared__ uint4 got[kFastThreads];                    // its ballots: bit 8 x + g of word j = plane x at word 4 g + j
+    __shared__ uint64_t codes[kFastBatch];                 // template codes of the batch's sites, 2 bits each
+    __shared__ uint16_t list[kFastChunks * 32];            // its sites by class, each class padded to 32
+    __shared__ uint32_t cnt[kFastClasses], first[kFastClasses]; // sites of a class; its first entry in list
+    __shared__ uint8_t chunk_class[kFastChunks];
+    __shared__ int n_chunks, next_chunk;
     const uint64_t n = dev_count(n_arg, n_dev);
     if ((uint64_t)blockIdx.x * blockDim.x >= n || __syncthreads_or(*(volatile const int *)err))
         return; // the whole block: no site for it, or records that failed their check
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = 0; j < n_pairs; ++j) {
         const PairDev &P = pairs[j];
         for (int t = threadIdx.x; t < 256; t += blockDim.x) {
             const int o0 = t >> 6, o1 = (t >> 4) & 3, t0 = (t >> 2) & 3, t1 = t & 3; // PairDev index order
-            fp[j].st[((t0 * 4 + t1) * 4 + o0) * 4 + o1] = make_float2(1000.f * P.stack_dH[t], P.stack_dS[t]);
+            fp[j].st[((o1 * 4 + o0) * 4 + t1) * 4 + t0] = make_float2(1000.f * P.stack_dH[t], P.stack_dS[t]);
         }
         if (threadIdx.x < 16)
             fp[j].tm[threadIdx.x] = make_float2(1000.f * P.term_dH[threadIdx.x], P.term_dS[threadIdx.x]);
-        if (threadIdx.x < 2 * AH_MAX_PRIMER_LEN) {
-            (&fp[j].mask[0][0])[threadIdx.x] = (&P.mask[0][0])[threadIdx.x];
-            (&fp[j].key[0][0])[threadIdx.x] = (&P.key[0][0])[threadIdx.x];
-        }
-        if (threadIdx.x < 2) {
-            const int x = threadIdx.x;
-            fp[j].L[x] = P.L[x];
-            fp[j].nkey[x] = P.nkey[x];
-            fp[j].cst[x] = (float)(P.sconst + (P.saltcorr == 5 ? 0.368 * (double)(P.L[x] - 1) * P.log_na : 0.0));
-        }
         if (threadIdx.x == 0) {
             fp[j].tm_min_f = P.tm_min_f;
             fp[j].tm_shift_f = (float)P.tm_shift;
         }
     }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
+    for (int c = warp; c < 2 * n_pairs; c += kFastThreads / 32)
+        tm_fast_primer(fp[c >> 1].pr[c & 1], pairs[c >> 1], c & 1, lane);
     const float INF = INFINITY;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    // whole warps take 32 consecutive sites, so the window gather below is uniform
-    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += stride) {
-        const uint64_t i = i0 + lane;
-        const bool live = i < n;
-        ah_site s{};
-        if (live)
-            s = sites[i];
-        const bool bad_rec = live && (s.pair >= n_pairs || s.primer > 1 || s.strand > 1);
-        if (bad_rec)
-            atomicExch(err, kDevBounds);
-        const bool act = live && !bad_rec;
-        const TmFastPair &sp = fp[act ? s.pair : 0];
-        const int pr = act ? s.primer : 0;
-        const int L = sp.L[pr];
-        // window of the site: tile word offset and bit row of its first position
-        uint64_t wofs = 0;
-        int brow = 0;
-        if (act) {
-            const uint64_t P = contig_off[s.contig] + s.pos;
-            const uint64_t t = P / kTileBases, r = P % kTileBases;
-            brow = (int)(r / kTileW);
-            wofs = t * 4 * kTileWX + (r % kTileW);
-        }
-        // columns of the window's bases (bit q = base at position P + q is A / C / G / T),
-        // eight sites at a time: their 32 loads are all in flight before the ballots
-        uint32_t cA = 0, cC = 0, cG = 0, cT = 0;
-        const uint32_t actm = __ballot_sync(0xffffffffu, act);
-        for (int k0 = 0; k0 < 32; k0 += 8) {
-            if (!((actm >> k0) & 0xffu))
+    constexpr uint32_t kNone = ~0u;
+    // an equal share per block (the blocks that start: one per 256 sites, at most the grid), in equal batches
+    const uint64_t blocks = min((uint64_t)gridDim.x, (n + kFastThreads - 1) / kFastThreads);
+    const uint64_t share = (n + blocks - 1) / blocks;
+    const uint64_t lo = min(n, blockIdx.x * share), hi = min(n, lo + share);
+    const uint64_t rounds = (share + kFastBatch - 1) / kFastBatch;
+    const uint32_t batch = (uint32_t)((share + rounds - 1) / rounds + 31) & ~31u;
+    for (uint64_t b0 = lo; b0 < hi; b0 += batch) {
+        const uint32_t here = (uint32_t)min((uint64_t)batch, hi - b0);
+        __syncthreads(); // the tables; the previous batch's lists are no longer read
+        if (threadIdx.x < kFastClasses)
+            cnt[threadIdx.x] = 0;
+        __syncthreads();
+        uint32_t slot[kFastBatch / kFastThreads]; // class << 16 | rank in it, of this lane's sites; kNone
+#pragma unroll
+        for (int r = 0; r < kFastBatch / kFastThreads; ++r) {
+            const uint32_t local = r * kFastThreads + threadIdx.x;
+            slot[r] = kNone;
+            if (r * kFastThreads + 32 * warp >= here) // the whole warp
                 continue;
-            uint32_t wv[8][4];
-            int bk[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint64_t wk = __shfl_sync(0xffffffffu, wofs, k0 + j);
-                bk[j] = __shfl_sync(0xffffffffu, brow, k0 + j);
-                const int Lk = __shfl_sync(0xffffffffu, L, k0 + j);
-                // the window's L positions only (the sectors past them are not read)
-                const bool on = ((actm >> (k0 + j)) & 1u) && lane < Lk;
-                const uint32_t *w = planes + wk + lane; // position P_k + lane (the tile's extension covers 32 more)
-#pragma unroll
-                for (int x = 0; x < 4; ++x)
-                    wv[j][x] = on ? __ldg(w + x * kTileWX) : 0u;
+            // ---- gather
+            const uint64_t i = b0 + local;
+            const bool live = local < here;
+            ah_site s{};
+            if (live)
+                s = sites[i];
+            const bool bad_rec = live && (s.pair >= n_pairs || s.primer > 1 || s.strand > 1);
+            if (bad_rec)
+                atomicExch(err, kDevBounds);
+            const bool act = live && !bad_rec;
+            const int L = act ? fp[s.pair].pr[s.primer].L : 1;
+            uint64_t base = 0; // byte offset of the window's 16-byte boundary in the A plane
+            uint32_t o = 0, row = 0;
+            if (act) {
+                const uint64_t P = contig_off[s.contig] + s.pos;
+                const uint32_t w = (uint32_t)(P % kTileBases);
+                o = w & 3u;
+                row = w / kTileW;
+                base = 4 * (P / kTileBases * (4 * kTileWX) + (w & (kTileW - 4)));
             }
+            const uint32_t last = min(o + (uint32_t)L, 32u) - 1u; // last word, from the boundary, of its 8 groups
+            __syncwarp();
+            win[threadIdx.x] = base;
+            win_last[threadIdx.x] = 16u * (last >> 2);
+            win_bit[threadIdx.x] = 1u << row;
+            __syncwarp();
+            const uint32_t actm = __ballot_sync(0xffffffffu, act);
+            const uint32_t g16 = 16u * (lane & 7);
+            const char *pl = reinterpret_cast<const char *>(planes + (lane >> 3) * kTileWX);
+            for (int k0 = 0; k0 < 32; k0 += 8) { // eight sites' loads in flight
+                if (!((actm >> k0) & 0xffu))
+                    continue;
+                uint4 w[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t a = __ballot_sync(0xffffffffu, (wv[j][0] >> bk[j]) & 1u);
-                const uint32_t c = __ballot_sync(0xffffffffu, (wv[j][1] >> bk[j]) & 1u);
-                const uint32_t g = __ballot_sync(0xffffffffu, (wv[j][2] >> bk[j]) & 1u);
-                const uint32_t tt = __ballot_sync(0xffffffffu, (wv[j][3] >> bk[j]) & 1u);
-                if (lane == k0 + j) {
-                    cA = a;
-                    cC = c;
-                    cG = g;
-                    cT = tt;
+                for (int j = 0; j < 8; ++j) { // (lanes past the window read its last group again: no other sector)
+                    const int k = 32 * warp + k0 + j;
+                    w[j] = __ldg(reinterpret_cast<const uint4 *>(pl + win[k] + min(g16, win_last[k])));
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint32_t bit = win_bit[32 * warp + k0 + j];
+                    const uint32_t v0 = __ballot_sync(0xffffffffu, w[j].x & bit);
+                    const uint32_t v1 = __ballot_sync(0xffffffffu, w[j].y & bit);
+                    const uint32_t v2 = __ballot_sync(0xffffffffu, w[j].z & bit);
+                    const uint32_t v3 = __ballot_sync(0xffffffffu, w[j].w & bit);
+                    if (lane == k0 + j)
+                        got[threadIdx.x] = make_uint4(v0, v1, v2, v3);
                 }
             }
-        }
-        if (!act) {
-            if (bad_rec) {
+            // ---- this lane's site: template codes, opposite each primer position (A 0, C 1, G 2, T 3)
+            int cls = -1;
+            if (act) {
+                uint32_t extra[4] = {0, 0, 0, 0}; // words 32 .. 34 of a long window that starts off the boundary, per plane
+                if (o + L > 32) {
+                    const uint32_t *p = planes + (base >> 2) + 32;
+#pragma unroll
+                    for (int x = 0; x < 4; ++x)
+#pragma unroll
+                        for (int j = 0; j < 3; ++j)
+                            if (32u + j < o + L)
+                                extra[x] |= ((__ldg(p + x * kTileWX + j) >> row) & 1u) << j;
+                }
+                // words outside [o, o + L) cleared; every position has exactly one plane set, or the window is bad
+                const uint4 b4 = got[threadIdx.x];
+                const uint32_t B[4] = {b4.x, b4.y, b4.z, b4.w};
+                int set = __popc(extra[0] | extra[1] | extra[2] | extra[3]);
+                uint64_t rows = 0; // byte 2 j + h: bit g = bit h of the code at word 4 g + j
+#pragma unroll
+                for (uint32_t j = 0; j < 4; ++j) {
+                    // groups whose word 4 g + j is at most `last`: all before last's, and its own up to last
+                    uint32_t keep = (1u << ((last >> 2) + (j <= (last & 3u)))) - 1u;
+                    if (j < o)
+                        keep &= ~1u;
+                    const uint32_t v = B[j] & keep * 0x01010101u;
+                    set += __popc(v);
+                    const uint32_t lo8 = ((v >> 8) | (v >> 24)) & 0xffu, hi8 = ((v >> 16) | (v >> 24)) & 0xffu;
+                    rows |= (uint64_t)(lo8 | hi8 << 8) << (16 * j);
+                }
+                uint64_t code = transpose8(rows) >> (2 * o);
+                if (o) { // (o = 0: nothing past word 31)
+                    const uint64_t elo = extra[1] | extra[3], ehi = extra[2] | extra[3];
+#pragma unroll
+                    for (int j = 0; j < 3; ++j)
+                        code |= ((elo >> j & 1u) | (ehi >> j & 1u) << 1) << (2 * (32 + j) - 2 * o) % 64;
+                }
+                if (s.strand == 0) { // the complement of the window base at q
+                    code = ~code;
+                } else { // the window base at L - 1 - q
+                    code = __brevll(code) >> (64 - 2 * L);
+                    code = (code >> 1 & 0x5555555555555555ull) | (code & 0x5555555555555555ull) << 1;
+                }
+                codes[local] = code;
+                if (set == L)
+                    cls = s.pair * 2 + s.primer;
+            }
+            if (live && cls < 0) { // a letter other than A, C, G, T, or a record outside its bounds
                 tm_out[i] = NAN;
                 if (pass_out)
                     pass_out[i] = 0;
             }
-            continue;
+            // its rank in its class
+            const uint32_t same = __match_any_sync(0xffffffffu, cls);
+            uint32_t at = 0;
+            if (cls >= 0 && lane == __ffs(same) - 1)
+                at = atomicAdd(&cnt[cls], (uint32_t)__popc(same));
+            at = __shfl_sync(0xffffffffu, at, __ffs(same) - 1) + __popc(same & ((1u << lane) - 1u));
+            if (cls >= 0)
+                slot[r] = (uint32_t)cls << 16 | at;
         }
-        const uint32_t lm = L >= 32 ? 0xffffffffu : ((1u << L) - 1u);
-        const bool bad = (~(cA | cC | cG | cT) & lm) != 0u; // a letter other than A, C, G, T
-        // template base opposite primer position q, 2 bits as (hi << 1) | lo with
-        // A 0, C 1, G 2, T 3: '+' the complement of the window base at q, '-' the
-        // window base at L - 1 - q
-        uint32_t blo, bhi;
-        if (s.strand == 0) {
-            blo = ~(cC | cT) & lm;
-            bhi = ~(cG | cT) & lm;
-        } else {
-            blo = __brev(cC | cT) >> (32 - L);
-            bhi = __brev(cG | cT) >> (32 - L);
-        }
-        if (bad) {
-            tm_out[i] = NAN;
-            if (pass_out)
-                pass_out[i] = 0;
-            continue;
-        }
-        auto bt = [&](int q) { return (int)(((blo >> q) & 1u) | (((bhi >> q) & 1u) << 1)); };
-        const uint8_t *key = sp.key[pr];
-        const uint8_t *mask = sp.mask[pr];
-        const int nk = sp.nkey[pr];
-        const int b0 = bt(0), bL = bt(L - 1);
-        const float cst = sp.cst[pr];
-        // What does not depend on lam, once per site.  The fixed stretches
-        // between keys that are not adjacent are the same for every oligo: they
-        // add one constant to every path, move no argmin, and join H and S at
-        // the end.  The start is an achieved ratio, that of one oligo: at each
-        // position the base pairing with the template where the mask allows it,
-        // else the mask's first base.  Each pass then either confirms the ratio
-        // (no oligo beats it by more than 1e-4 K) or moves to a better one.
-        float SH = 0.f, SE = 0.f;
-        for (int si = 0; si + 1 < nk; ++si) {
-            const int k0 = key[si], k1 = key[si + 1];
-            for (int q = k0 + 2; q < k1; ++q) {
-                const float2 v2 =
-                    sp.st[(bt(q - 1) * 4 + bt(q)) * 16 + (__ffs(mask[q - 1]) - 1) * 4 + (__ffs(mask[q]) - 1)];
-                SH += v2.x;
-                SE += v2.y;
+        // ---- the batch's sites by class
+        __syncthreads();
+        if (warp == 0) {
+            const uint32_t chunks = (cnt[lane] + 31) / 32;
+            uint32_t incl = chunks;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d)
+                    incl += y;
+            }
+            first[lane] = (incl - chunks) * 32;
+            for (uint32_t c = incl - chunks; c < incl; ++c)
+                chunk_class[c] = (uint8_t)lane;
+            if (lane == 31) {
+                n_chunks = (int)incl;
+                next_chunk = 0;
             }
         }
-        float lam;
-        {
-            auto pick = [&](int q) {
-                const int pairing = 3 - bt(q);
-                return ((mask[q] >> pairing) & 1) ? pairing : __ffs(mask[q]) - 1;
-            };
-            int o0 = pick(0);
-            float2 t = sp.tm[o0 * 4 + b0];
-            float H0 = t.x, S0 = t.y;
-            for (int q = 1; q < L; ++q) {
-                const int o1 = pick(q);
-                const float2 v2 = sp.st[(bt(q - 1) * 4 + bt(q)) * 16 + o0 * 4 + o1];
-                H0 += v2.x;
-                S0 += v2.y;
-                o0 = o1;
-            }
-            t = sp.tm[o0 * 4 + bL];
-            lam = (H0 + t.x) / (S0 + t.y + cst);
-        }
-        for (int it = 0; it < 64; ++it) {
-            // forward pass at lam: per state y (oligo base at the current key) the
-            // cheapest path cost 1000 dH - lam dS and that path's 1000 dH and dS
-            // (fixed stretches left out)
-            float c[4], h[4], e[4];
+        __syncthreads();
 #pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const float2 t = sp.tm[y * 4 + b0];
-                const bool ok = (mask[0] >> y) & 1;
-                c[y] = ok ? fmaf(-lam, t.y, t.x) : INF;
-                h[y] = t.x;
-                e[y] = t.y;
-            }
-            for (int si = 0; si + 1 < nk; ++si) {
-                const int k0 = key[si], k1 = key[si + 1];
-                const int m1 = mask[k1];
-                float nc[4], nh[4], ne[4];
-                if (k1 == k0 + 1) {
-                    const float2 *E = &sp.st[(bt(k0) * 4 + bt(k1)) * 16]; // E[o0 * 4 + o1]
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        float best = INF, bh = 0.f, be = 0.f;
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) {
-                            const float2 v2 = E[x * 4 + y];
-                            const float v = c[x] + fmaf(-lam, v2.y, v2.x);
-                            if (v < best) {
-                                best = v;
-                                bh = h[x] + v2.x;
-                                be = e[x] + v2.y;
-                            }
-                        }
-                        const bool ok = (m1 >> y) & 1;
-                        nc[y] = ok ? best : INF;
-                        nh[y] = bh;
-                        ne[y] = be;
-                    }
-                } else {
-                    // the stack out of k0 into the fixed base after it: one argmin over
-                    // the bases at k0, shared by every y; then the stack into k1
-                    const int fa = __ffs(mask[k0 + 1]) - 1, fb = __ffs(mask[k1 - 1]) - 1;
-                    const float2 *EA = &sp.st[(bt(k0) * 4 + bt(k0 + 1)) * 16 + fa]; // EA[o0 * 4]
-                    float best = INF, bh = 0.f, be = 0.f;
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const float2 v2 = EA[x * 4];
-                        const float v = c[x] + fmaf(-lam, v2.y, v2.x);
-                        if (v < best) {
-                            best = v;
-                            bh = h[x] + v2.x;
-                            be = e[x] + v2.y;
-                        }
-                    }
-                    const float2 *EB = &sp.st[(bt(k1 - 1) * 4 + bt(k1)) * 16 + fb * 4]; // EB[o1]
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        const float2 v2 = EB[y];
-                        const bool ok = ((m1 >> y) & 1) && best < INF;
-                        nc[y] = ok ? best + fmaf(-lam, v2.y, v2.x) : INF;
-                        nh[y] = bh + v2.x;
-                        ne[y] = be + v2.y;
+        for (int r = 0; r < kFastBatch / kFastThreads; ++r)
+            if (slot[r] != kNone)
+                list[first[slot[r] >> 16] + (slot[r] & 0xffffu)] = (uint16_t)(r * kFastThreads + threadIdx.x);
+        __syncthreads();
+        // ---- 32 sites of one primer per warp
+        for (;;) {
+            int ch = 0;
+            if (lane == 0)
+                ch = atomicAdd(&next_chunk, 1);
+            ch = __shfl_sync(0xffffffffu, ch, 0);
+            if (ch >= n_chunks)
+                break;
+            const int c = chunk_class[ch];
+            const TmFastPair &sp = fp[c >> 1];
+            const TmFastPrimer &F = sp.pr[c & 1];
+            if ((uint32_t)(ch * 32 + lane) >= first[c] + cnt[c])
+                continue; // padding
+            const uint32_t local = list[ch * 32 + lane];
+            const uint64_t code = codes[local];
+            const char *st = reinterpret_cast<const char *>(sp.st);
+            // the stack table's column of the template pair at shift sh
+            auto column = [&](uint32_t sh) { return st + (((uint32_t)(code >> sh) & 15u) << 3); };
+            auto entry = [](const char *E, uint32_t off) { return *reinterpret_cast<const float2 *>(E + off); };
+            const int L = F.L, n_step = F.n_step;
+            const float2 *tF = sp.tm + ((uint32_t)code & 3u), *tL = sp.tm + ((uint32_t)(code >> (2 * (L - 1))) & 3u);
+            const float cst = F.cst;
+            // What does not depend on lam, once per site.  The fixed stretches
+            // between keys that are not adjacent are the same for every oligo: they
+            // add one constant to every path, move no argmin, and join H and S at
+            // the end.  The start is an achieved ratio, that of one oligo: at each
+            // position the base pairing with the template where the set allows it,
+            // else the set's lowest base (for about nine sites in ten the best oligo).
+            // Each pass then either confirms the ratio (no oligo beats it by more
+            // than 1e-4 K) or moves to a better one.
+            float SH = 0.f, SE = 0.f, lam;
+            {
+                const uint64_t pairing = ~code, one = 0x5555555555555555ull, plo = pairing & one, phi = pairing >> 1 & one;
+                const uint64_t in = (F.has[0] & ~(plo | phi)) | (F.has[1] & plo & ~phi) | (F.has[2] & phi & ~plo) |
+                                    (F.has[3] & plo & phi);
+                const uint64_t m = in | in << 1, oligo = (pairing & m) | (F.first & ~m);
+                float2 t = tF[((uint32_t)oligo & 3u) * 4];
+                float H0 = t.x, S0 = t.y;
+                const uint32_t fixes = F.fixes;
+                for (int q = 0; q + 1 < L; ++q) {
+                    const float2 v = entry(column(2 * q), ((uint32_t)(oligo >> (2 * q)) & 15u) << 7);
+                    H0 += v.x;
+                    S0 += v.y;
+                    if (fixes >> q & 1u) {
+                        SH += v.x;
+                        SE += v.y;
                     }
                 }
+                t = tL[((uint32_t)(oligo >> (2 * (L - 1))) & 3u) * 4];
+                lam = (H0 + t.x) / (S0 + t.y + cst);
+            }
+            for (int it = 0; it < 64; ++it) {
+                // forward pass at lam: per base of the current key's set (ascending) the
+                // cheapest path cost 1000 dH - lam dS and that path's 1000 dH and dS
+                // (fixed stretches left out)
+                float cc[4], h[4], e[4];
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
-                    c[y] = nc[y];
-                    h[y] = nh[y];
-                    e[y] = ne[y];
+                    cc[y] = INF;
+                    h[y] = e[y] = 0.f;
+                    if (y < F.nF) {
+                        const float2 t = tF[(F.listF >> (2 * y) & 3) * 4];
+                        cc[y] = fmaf(-lam, t.y, t.x);
+                        h[y] = t.x;
+                        e[y] = t.y;
+                    }
                 }
-            }
-            // the 3' terminal pair, then the argmin end state (ties: the lowest base)
-            float best = INF, H = 0.f, S = 0.f;
+                for (int si = 0; si < n_step; ++si) {
+                    const uint4 d4 = *reinterpret_cast<const uint4 *>(&F.step[si]);
+                    const uint32_t sh0 = d4.x & 63u, sh1 = d4.x >> 8 & 63u;
+                    const uint32_t off0 = d4.y & 0xffffu, off1 = d4.y >> 16, off2 = d4.z & 0xffffu, off3 = d4.z >> 16;
+                    const uint32_t kind = d4.w >> 24, apart = kind & 1u;
+                    if (kind < 2u) {
+                        if (!apart) {
+                            const char *E = column(sh0);
+                            const float2 e00 = entry(E, off0), e01 = entry(E, off1), e10 = entry(E, off2), e11 = entry(E, off3);
+                            const float v00 = cc[0] + fmaf(-lam, e00.y, e00.x), v10 = cc[1] + fmaf(-lam, e10.y, e10.x);
+                            const float v01 = cc[0] + fmaf(-lam, e01.y, e01.x), v11 = cc[1] + fmaf(-lam, e11.y, e11.x);
+                            const bool p0 = v10 < v00, p1 = v11 < v01;
+                            const float h0 = h[0], h1 = h[1], s0 = e[0], s1 = e[1];
+                            cc[0] = p0 ? v10 : v00;
+                            cc[1] = p1 ? v11 : v01;
+                            h[0] = (p0 ? h1 : h0) + (p0 ? e10.x : e00.x);
+                            h[1] = (p1 ? h1 : h0) + (p1 ? e11.x : e01.x);
+                            e[0] = (p0 ? s1 : s0) + (p0 ? e10.y : e00.y);
+                            e[1] = (p1 ? s1 : s0) + (p1 ? e11.y : e01.y);
+                        } else {
+                            // the stack out of k0 into the fixed base after it: one argmin over
+                            // the bases at k0, shared by every y; then the stack into k1
+                            const char *EA = column(sh0), *EB = column(sh1);
+                            const float2 a0 = entry(EA, off0), a1 = entry(EA, off1), q0 = entry(EB, off2), q1 = entry(EB, off3);
+                            const float v0 = cc[0] + fmaf(-lam, a0.y, a0.x), v1 = cc[1] + fmaf(-lam, a1.y, a1.x);
+                            const bool p = v1 < v0;
+                            const float best = p ? v1 : v0;
+                            const float bh = (p ? h[1] : h[0]) + (p ? a1.x : a0.x);
+                            const float be = (p ? e[1] : e[0]) + (p ? a1.y : a0.y);
+                            cc[0] = best + fmaf(-lam, q0.y, q0.x);
+                            cc[1] = best + fmaf(-lam, q1.y, q1.x);
+                            h[0] = bh + q0.x;
+                            h[1] = bh + q1.x;
+                            e[0] = be + q0.y;
+                            e[1] = be + q1.y;
+                        }
+                        continue;
+                    }
+                    const uint32_t n0 = d4.x >> 16 & 255u, n1 = d4.x >> 24;
+                    const uint32_t list0 = d4.w & 255u, list1 = d4.w >> 8 & 255u;
+                    const uint32_t fa = d4.w >> 16 & 3u, fb = d4.w >> 18 & 3u;
+                    float nc[4], nh[4], ne[4];
+                    const char *EA = column(sh0), *EB = column(sh1);
+                    float ab = INF, ah = 0.f, ae = 0.f; // keys apart: the argmin over x
+                    if (apart) {
 #pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const float2 t = sp.tm[y * 4 + bL];
-                const float v = c[y] < INF ? c[y] + fmaf(-lam, t.y, t.x) : INF;
-                if (v < best) {
-                    best = v;
-                    H = h[y] + t.x;
-                    S = e[y] + t.y;
+                        for (uint32_t x = 0; x < 4; ++x)
+                            if (x < n0) {
+                                const float2 v2 = entry(EA, 128 * ((list0 >> (2 * x) & 3u) + 4 * fa));
+                                const float v = cc[x] + fmaf(-lam, v2.y, v2.x);
+                                if (v < ab) {
+                                    ab = v;
+                                    ah = h[x] + v2.x;
+                                    ae = e[x] + v2.y;
+                                }
+                            }
+                    }
+#pragma unroll
+                    for (uint32_t y = 0; y < 4; ++y) {
+                        nc[y] = INF;
+                        nh[y] = ne[y] = 0.f;
+                        if (y < n1) {
+                            const uint32_t by = list1 >> (2 * y) & 3u;
+                            if (apart) {
+                                const float2 v2 = entry(EB, 128 * (fb + 4 * by));
+                                nc[y] = ab + fmaf(-lam, v2.y, v2.x);
+                                nh[y] = ah + v2.x;
+                                ne[y] = ae + v2.y;
+                            } else {
+#pragma unroll
+                                for (uint32_t x = 0; x < 4; ++x)
+                                    if (x < n0) {
+                                        const float2 v2 = entry(EA, 128 * ((list0 >> (2 * x) & 3u) + 4 * by));
+                                        const float v = cc[x] + fmaf(-lam, v2.y, v2.x);
+                                        if (v < nc[y]) {
+                                            nc[y] = v;
+                                            nh[y] = h[x] + v2.x;
+                                            ne[y] = e[x] + v2.y;
+                                        }
+                                    }
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) {
+                        cc[y] = nc[y];
+                        h[y] = nh[y];
+                        e[y] = ne[y];
+                    }
                 }
+                // the 3' terminal pair, then the argmin end state (ties: the lowest base)
+                float best = INF, H = 0.f, S = 0.f;
+#pragma unroll
+                for (int y = 0; y < 4; ++y)
+                    if (y < F.nL) {
+                        const float2 t = tL[(F.listL >> (2 * y) & 3) * 4];
+                        const float v = cc[y] + fmaf(-lam, t.y, t.x);
+                        if (v < best) {
+                            best = v;
+                            H = h[y] + t.x;
+                            S = e[y] + t.y;
+                        }
+                    }
+                const float r = (H + SH) / (S + SE + cst);
+                // stop when the ratio no longer improves by more than 1e-4 K (as tm_kernel)
+                if (!(r > lam + 1e-4f))
+                    break;
+                lam = r;
             }
-            const float r = (H + SH) / (S + SE + cst);
-            // stop when the ratio no longer improves by more than 1e-4 K (as tm_kernel)
-            if (!(r > lam + 1e-4f))
-                break;
-            lam = r;
+            const float tm32 = lam - 273.15f + sp.tm_shift_f;
+            const uint64_t io = b0 + local;
+            if (pass_out && fabsf(tm32 - sp.tm_min_f) < 0.01f) {
+                defer[atomicAdd(defer_n, 1ull)] = (uint32_t)io; // decided exactly by tm_kernel
+                continue;
+            }
+            tm_out[io] = tm32;
+            if (pass_out)
+                pass_out[io] = tm32 >= sp.tm_min_f;
         }
-        const float tm32 = lam - 273.15f + sp.tm_shift_f;
-        if (pass_out && fabsf(tm32 - sp.tm_min_f) < 0.01f) {
-            defer[atomicAdd(defer_n, 1ull)] = (uint32_t)i; // decided exactly by tm_kernel
-            continue;
-        }
-        tm_out[i] = tm32;
-        if (pass_out)
-            pass_out[i] = tm32 >= sp.tm_min_f;
     }
 }
 
@@ -1093,7 +1316,7 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
         return;
     if (seg_max < 1 || seg_max > AH_MAX_PRIMER_LEN - 1)
         throw Error(AH_ERR_ARG, "Tm: segment count outside 1..31");
-    static int cached_dev = -1, sms = 148, fast_bps = 1, tm_bps = 1;
+    static int cached_dev = -1, sms = 148, tm_bps = 1, fast_blocks[AH_MAX_PAIRS_PER_SCAN + 1];
     int dev = 0;
     AH_CUDA(cudaGetDevice(&dev));
     const size_t smem = (size_t)n_pairs * sizeof(TmPairS) + (size_t)(n_pairs <= kTmStageD ? n_pairs : 0) * sizeof(TmPairD) +
@@ -1106,28 +1329,32 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
         AH_CUDA(cudaFuncSetAttribute(tm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         const int most_fast = AH_MAX_PAIRS_PER_SCAN * (int)sizeof(TmFastPair);
         AH_CUDA(cudaFuncSetAttribute(tm_fast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most_fast));
-        AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fast_bps, tm_fast_kernel, kFastThreads, most_fast));
+        for (int j = 1; j <= AH_MAX_PAIRS_PER_SCAN; ++j) {
+            AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fast_blocks[j], tm_fast_kernel, kFastThreads,
+                                                                  j * sizeof(TmFastPair)));
+            fast_blocks[j] = std::max(1, fast_blocks[j]);
+        }
         AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tm_bps, tm_kernel, 32 * kTmWarps, most));
-        fast_bps = std::max(1, fast_bps);
         tm_bps = std::max(1, tm_bps);
         // AH_TM_FAST_BLOCKS=n: at most n blocks of the thread-per-site kernel per SM (profiling aid)
         if (const char *e = getenv("AH_TM_FAST_BLOCKS"))
             if (atoi(e) > 0)
-                fast_bps = std::min(fast_bps, atoi(e));
+                for (int &b : fast_blocks)
+                    b = std::min(b, atoi(e));
         cached_dev = dev;
     }
     // queue length, finished blocks, deferred sites
     AH_CUDA(cudaMemsetAsync(queue_n, 0, 2 * sizeof(uint64_t), s));
     // Few sites (a latency-bound launch): the four-lane kernel alone finishes first
     // (measured on GB300 for 6,253 sites: 33 us, against 36 + 27 us for the two
-    // kernels below); many sites: one thread per site (3.5x the four-lane rate on
+    // kernels below); many sites: one thread per site (6x the four-lane rate on
     // 3.2 M sites).
     constexpr uint64_t kFastMinSites = 32768;
     if (few_exact && n >= kFastMinSites) {
         // every site in one thread; those near tm_min go to the four-lane kernel below
         uint32_t *defer = queue + n;
         unsigned long long *defer_n = reinterpret_cast<unsigned long long *>(queue_n) + 1;
-        const uint64_t fb = std::min<uint64_t>((n + kFastThreads - 1) / kFastThreads, (uint64_t)sms * fast_bps);
+        const uint64_t fb = std::min<uint64_t>((n + kFastThreads - 1) / kFastThreads, (uint64_t)sms * fast_blocks[n_pairs]);
         tm_fast_kernel<<<(unsigned)fb, kFastThreads, fast_smem, s>>>(sites, n, n_dev, pairs_d, n_pairs, planes,
                                                                       contig_off, tm_out, pass_out, defer, defer_n,
                                                                       err);

@@ -1397,3 +1397,41 @@ def test_2bit_packing_with_few_and_many_no_base_runs(ctx, per_tile):
             finally:
                 ctx.ah_unload_genomes(sid)
             assert got == seq.tobytes(), n
+
+
+@pytest.mark.parametrize("lengths,codes,n_sites", [([(32, 29)], ("RN", "BDHV"), 32768), ([(30, 31)], ("", "NNY"), 33001),
+                                                   ([(12 + j, 27 - j) for j in range(16)], ("YW", "VK"), 60001)])
+def test_thread_per_site_tm_over_window_offsets_and_primer_mixes(ctx, lengths, codes, n_sites):
+    """Caller's sites at every offset of a window in its 16-byte groups and rows, across tile ends, on windows with
+    other letters, for primers up to 32 long and sets of one to four bases, up to 16 pairs mixed at random: the
+    maxima within 0.01 C of the oracle's (the bound of the entry point), NaN and pass flags the same."""
+    rng = np.random.default_rng(n_sites)
+    n = 5 * 32768 + 77
+    seq = synth.random_bases(rng, n, 0.5).copy()
+    seq[rng.integers(0, n, 60)] = ord("N")
+    off = np.array([0, 40_001, 40_100, n], np.uint64)
+    pairs = [synth.pcr_params(synth.random_primer(rng, lf, codes[0]), synth.random_primer(rng, lr, codes[1]), k=3,
+                              min_len=30, max_len=900, tm_min=20.0) for lf, lr in lengths]
+    sites = np.zeros(n_sites, dtype=ah.SITE_DTYPE)
+    sites["contig"] = rng.choice(3, n_sites, p=[0.3, 0.1, 0.6])
+    sites["pair"] = rng.integers(0, len(pairs), n_sites)
+    sites["primer"] = rng.integers(0, 2, n_sites)
+    sites["strand"] = rng.integers(0, 2, n_sites)
+    size = np.diff(off.astype(np.int64))[sites["contig"]]
+    sites["pos"] = rng.random(n_sites) * (size - 32 + 1)
+    sid = ctx.load(seq, off, np.zeros(3, np.uint32))
+    try:
+        pids = [ctx.ah_set_primers(p["fwd"], p["rev"], p) for p in pairs]
+        want, _ = oracle.tm(seq, off, sites, pairs)
+        med = float(np.nanmedian(want))
+        pairs = [dict(p, tm_min=med) for p in pairs]
+        want, passed = oracle.tm(seq, off, sites, pairs)
+        pids = [ctx.ah_set_primers(p["fwd"], p["rev"], p) for p in pairs]
+        tm, ps = ctx.tm(sid, pids, sites)
+    finally:
+        ctx.ah_unload_genomes(sid)
+    nan = np.isnan(want)
+    assert 0 < nan.sum() < n_sites // 4 and 0.2 < passed.mean() < 0.8
+    assert np.array_equal(np.isnan(tm), nan)
+    assert np.abs(tm[~nan].astype(np.float64) - want[~nan]).max() <= TM_TOL
+    assert np.array_equal(ps, passed)
