@@ -886,11 +886,11 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
         launch_pair_count(sites, ns_max, F + kFlagSites, filt, pd, counts, nullptr, st);
         exclusive_scan_u64_dev(counts, offs, ns_max, F + kFlagSites, 0, F + kFlagAux, na_max, F + kFlagAmps,
                                F + kFlagRedo, kRedoAmps, st);
-        launch_pair_write(sites, ns_max, F + kFlagSites, filt, pd, offs, amps, na_max, F + kFlagRedo, kRedoAmps, st);
+        launch_pair_write(sites, ns_max, F + kFlagSites, filt, pd, offs, amps, len, na_max, F + kFlagRedo, kRedoAmps,
+                          st);
     }
     {
-        Stage sg(c, "fetch", st, 3);
-        launch_fetch_lengths(amps, na_max, F + kFlagAmps, gs.contig_off, gs.n_contigs, len, c->d_err, st);
+        Stage sg(c, "fetch", st, 2);
         exclusive_scan_u64_dev(len, qoff, na_max + 1, F + kFlagAmps, 1, F + kFlagAux, nq_max, F + kFlagSeq,
                                F + kFlagRedo, kRedoSeq, st);
         launch_fetch(amps, na_max, F + kFlagAmps, qoff, gs.planes, gs.contig_off, seq, F + kFlagRedo, kRedoSeq, st);
@@ -1006,7 +1006,7 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         qoff = direct_or_scratch(c, "run_qoff", o->seq_offsets, o->seq_offsets ? o->amplicons_cap + 1 : 0, na + 1);
         if (na) {
             Stage sg(c, "pair", st, 1);
-            launch_pair_write(sites, ns, nullptr, filt, pd, offs, amps, na, nullptr, 0, st);
+            launch_pair_write(sites, ns, nullptr, filt, pd, offs, amps, nullptr, na, nullptr, 0, st);
         }
         uint64_t *len = (uint64_t *)scratch(c, "fetch_len", (na + 1) * sizeof(uint64_t));
         size_t tb2 = scan_u64_temp_bytes(na + 1);
@@ -1014,7 +1014,7 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         {
             Stage sg(c, "fetch", st, (na ? 1 : 0) + scan_u64_launches(na + 1));
             AH_CUDA(cudaMemsetAsync(len + na, 0, sizeof(uint64_t), st));
-            launch_fetch_lengths(amps, na, nullptr, gs.contig_off, gs.n_contigs, len, c->d_err, st);
+            launch_fetch_lengths(amps, na, gs.contig_off, gs.n_contigs, len, c->d_err, st);
             exclusive_scan_u64(temp2, tb2, len, qoff, na + 1, st);
             AH_CUDA(cudaMemcpyAsync(c->d_aux, qoff + na, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
         }
@@ -1222,7 +1222,7 @@ void group_device(ah_ctx *c, const GenomeSet &gs, uint32_t pid, int k, const std
     ah_amplicon *amps = (ah_amplicon *)scratch(c, "serve_amps", std::max<uint64_t>(na, 1) * sizeof(ah_amplicon));
     if (na) {
         Stage sg(c, "pair", st, 1);
-        launch_pair_write(sites, ns, nullptr, nullptr, pd, offs, amps, na, nullptr, 0, st);
+        launch_pair_write(sites, ns, nullptr, nullptr, pd, offs, amps, nullptr, na, nullptr, 0, st);
     }
     // staging layout: sites, amplicons, pass flags
     const size_t sb = ns * sizeof(ah_site), ab = na * sizeof(ah_amplicon);
@@ -2594,7 +2594,7 @@ ah_status ah_pair(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t
         ah_amplicon *dst = out_buf(c, "amp_out", out, total);
         {
             Stage sg(c, "pair", st, 1);
-            launch_pair_write(s, n, nullptr, ps, pd, offs, dst, total, nullptr, 0, st);
+            launch_pair_write(s, n, nullptr, ps, pd, offs, dst, nullptr, total, nullptr, 0, st);
         }
         out_finish(out, dst, total, st);
         AH_CUDA(cudaStreamSynchronize(st));
@@ -2621,7 +2621,7 @@ ah_status ah_fetch(ah_ctx *c, uint32_t set_id, const ah_amplicon *amplicons, uin
         void *temp = scratch(c, "scan_temp", tb);
         {
             Stage sg(c, "fetch", st, (n ? 1 : 0) + scan_u64_launches(n + 1));
-            launch_fetch_lengths(a, n, nullptr, gs.contig_off, gs.n_contigs, len, c->d_err, st);
+            launch_fetch_lengths(a, n, gs.contig_off, gs.n_contigs, len, c->d_err, st);
             exclusive_scan_u64(temp, tb, len, offs, n + 1, st);
             AH_CUDA(cudaMemcpyAsync(c->d_aux, offs + n, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
         }

@@ -226,7 +226,35 @@ constexpr uint64_t kRedoSites = 1, kRedoAmps = 2, kRedoSeq = 4;
 // Count of a kernel that may read it on the device: min(*n_dev, n), or n.
 __device__ __forceinline__ uint64_t dev_count(uint64_t n, const uint64_t *n_dev)
 {
-    return n_dev ? (*n_dev < n ? *n_dev : n) : n;
+    return n_dev ? min(*(const volatile uint64_t *)n_dev, n) : n;
+}
+
+// The kernels after a scan form a chain of short launches, each of which needs all
+// of its predecessor.  They are launched so that a kernel's blocks start while its
+// predecessor drains (launch_chained) and wait, with chain_wait, before they read
+// or write anything that another kernel of the chain touches.  Every block of such
+// a kernel waits, so a kernel that is complete has all earlier ones complete.  What
+// the chain hands on is read with plain loads (no const __restrict__, no __ldg: it
+// is not constant over the kernel's lifetime).  Measured on a GB300, one 4.8 Mbp
+// genome at k = 2 from its scan's end to the last kernel's: ten launches, 57 us
+// -> seven chained ones, 37.
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    AH_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
 }
 
 struct PairDev;
@@ -270,7 +298,7 @@ struct PairDev {
 // within 0.01 C of tm_min to the four-lane kernel, whose last block evaluates
 // the exhaustive queue; else the four-lane kernel takes every site and a
 // second kernel works off the queue, a block per site.
-// n_dev: optional device count (min(*n_dev, n) sites).
+// n_dev: optional device count (min(*n_dev, n) sites); queue_n is then zero already.
 void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const PairDev *pairs_d, int n_pairs, const uint32_t *planes,
                const uint64_t *contig_off, float *tm_out, uint8_t *pass_out, uint32_t *queue, uint32_t *queue_n,
                int seg_max, bool few_exact, int *err, cudaStream_t s);
@@ -307,14 +335,17 @@ constexpr uint64_t kSmallScan = 65536;
 // number of kernels exclusive_scan_u64 launches for n values
 int scan_u64_launches(uint64_t n);
 void exclusive_scan_u64(void *temp, size_t temp_bytes, const uint64_t *in, uint64_t *out, uint64_t n, cudaStream_t s);
-// One-block exclusive scan of min(*n_dev + add, n) values (n <= kSmallScan);
+// One-block exclusive scan of min(*n_dev + add, n) values (n <= kSmallScan), the
+// last `add` of them zero whatever `in` holds there;
 // with tot also their sum, and with eff the capacity check of launch_total.
 void exclusive_scan_u64_dev(const uint64_t *in, uint64_t *out, uint64_t n, const uint64_t *n_dev, uint64_t add,
                             uint64_t *tot, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit,
                             cudaStream_t s);
 // skip: optional device word; the kernel writes nothing when (*skip & skip_bit) != 0.
+// len (may be null): the amplicons' lengths as launch_fetch_lengths gives them, for sites
+// that a scan found.
 void launch_pair_write(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, const uint64_t *offsets, ah_amplicon *out, uint64_t cap,
+                       const PairDev *pairs_d, const uint64_t *offsets, ah_amplicon *out, uint64_t *len, uint64_t cap,
                        const uint64_t *skip, uint64_t skip_bit, cudaStream_t s);
 
 // amplitype.cu: sequence variants and amplitypes.  Two hash tables of `size`
@@ -355,9 +386,8 @@ void launch_generate_bases(const ah_gen_segment *segs, uint64_t n_segs, uint64_t
 
 // fetch.cu
 // lengths of the amplicons; a record outside its contig sets *err = kDevBounds (length 0)
-// With n_dev the kernel also writes len[count] = 0 (the scan's closing entry).
-void launch_fetch_lengths(const ah_amplicon *a, uint64_t n, const uint64_t *n_dev, const uint64_t *contig_off,
-                          uint32_t n_contigs, uint64_t *len, int *err, cudaStream_t s);
+void launch_fetch_lengths(const ah_amplicon *a, uint64_t n, const uint64_t *contig_off, uint32_t n_contigs,
+                          uint64_t *len, int *err, cudaStream_t s);
 void launch_fetch(const ah_amplicon *a, uint64_t n, const uint64_t *n_dev, const uint64_t *offsets,
                   const uint32_t *planes, const uint64_t *contig_off, char *out, const uint64_t *skip,
                   uint64_t skip_bit, cudaStream_t s);

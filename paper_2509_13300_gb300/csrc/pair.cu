@@ -33,7 +33,7 @@ __device__ __forceinline__ bool site_less(const ah_site &m, uint32_t pair, uint3
 // the last gap.  Candidates usually sit right after the group, so this takes
 // one or two dependent loads where a plain binary search over all sites takes
 // log2(n).
-__device__ uint64_t lower_bound_pos(const ah_site *__restrict__ s, uint64_t lo, uint64_t n, uint32_t pair,
+__device__ uint64_t lower_bound_pos(const ah_site *s, uint64_t lo, uint64_t n, uint32_t pair,
                                     uint32_t contig, uint64_t t)
 {
     uint64_t step = 1, hi = lo;
@@ -63,7 +63,7 @@ struct Group {
     bool valid;
 };
 
-__device__ Group make_group(const ah_site *__restrict__ s, uint64_t n, const uint8_t *__restrict__ pass,
+__device__ Group make_group(const ah_site *s, uint64_t n, const uint8_t *pass,
                             const PairDev *__restrict__ pairs, uint64_t a)
 {
     Group g;
@@ -125,10 +125,11 @@ __device__ __forceinline__ bool in_window(const PairDev &pd, uint32_t s_pos, con
     return r.pos >= s_pos && len >= pd.min_len && len <= pd.max_len;
 }
 
-__global__ void pair_count_kernel(const ah_site *__restrict__ s, uint64_t n_arg, const uint64_t *__restrict__ n_dev,
-                                  const uint8_t *__restrict__ pass, const PairDev *__restrict__ pairs,
-                                  uint64_t *__restrict__ counts, const int *__restrict__ err)
+__global__ void pair_count_kernel(const ah_site *s, uint64_t n_arg, const uint64_t *n_dev, const uint8_t *pass,
+                                  const PairDev *__restrict__ pairs, uint64_t *counts, const int *err)
 {
+    chain_start();
+    chain_wait();
     if (err && *(volatile const int *)err) // the records' check failed: nothing is indexed with them
         return;
     const uint64_t n = dev_count(n_arg, n_dev);
@@ -155,12 +156,13 @@ __global__ void pair_count_kernel(const ah_site *__restrict__ s, uint64_t n_arg,
 
 __device__ __forceinline__ int orient_of(int x, int y) { return (x == 0 && y == 1) ? 0 : (x == 1 && y == 0) ? 1 : (x == 0 ? 2 : 3); }
 
-__global__ void pair_write_kernel(const ah_site *__restrict__ s, uint64_t n_arg, const uint64_t *__restrict__ n_dev,
-                                  const uint8_t *__restrict__ pass, const PairDev *__restrict__ pairs,
-                                  const uint64_t *__restrict__ offsets, ah_amplicon *__restrict__ out, uint64_t cap,
-                                  const uint64_t *__restrict__ skip, uint64_t skip_bit)
+__global__ void pair_write_kernel(const ah_site *s, uint64_t n_arg, const uint64_t *n_dev, const uint8_t *pass,
+                                  const PairDev *__restrict__ pairs, const uint64_t *offsets, ah_amplicon *out,
+                                  uint64_t *len, uint64_t cap, const uint64_t *skip, uint64_t skip_bit)
 {
-    if (skip && (*skip & skip_bit))
+    chain_start();
+    chain_wait();
+    if (skip && (*(const volatile uint64_t *)skip & skip_bit))
         return;
     const uint64_t n = dev_count(n_arg, n_dev);
     for (uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (uint64_t)gridDim.x * blockDim.x) {
@@ -219,6 +221,8 @@ __global__ void pair_write_kernel(const ah_site *__restrict__ s, uint64_t n_arg,
                 am.pair = sa.pair;
                 am.pad0 = am.pad1 = 0;
                 out[o] = am;
+                if (len) // of sites from a scan: both ends lie in the contig
+                    len[o] = bend - sa.pos;
             }
             ++o;
             cur[best] = advance(best, cur[best] + 1);
@@ -226,10 +230,12 @@ __global__ void pair_write_kernel(const ah_site *__restrict__ s, uint64_t n_arg,
     }
 }
 
-__global__ void total_kernel(const uint64_t *__restrict__ offs, const uint64_t *__restrict__ counts, uint64_t n_arg,
-                             const uint64_t *__restrict__ n_dev, uint64_t add, uint64_t *__restrict__ out,
-                             uint64_t cap, uint64_t *__restrict__ eff, uint64_t *__restrict__ redo, uint64_t redo_bit)
+__global__ void total_kernel(const uint64_t *offs, const uint64_t *counts, uint64_t n_arg, const uint64_t *n_dev,
+                             uint64_t add, uint64_t *out, uint64_t cap, uint64_t *eff, uint64_t *redo,
+                             uint64_t redo_bit)
 {
+    chain_start();
+    chain_wait();
     const uint64_t n = n_dev ? min(*n_dev + add, n_arg) : n_arg;
     const uint64_t t = n ? offs[n - 1] + counts[n - 1] : 0;
     *out = t;
@@ -246,16 +252,17 @@ __global__ void total_kernel(const uint64_t *__restrict__ offs, const uint64_t *
 // one shared pass scan the 1024 thread sums, and the results leave through
 // shared memory as coalesced stores.  With tot it also writes the sum of all
 // m values; with eff, *eff = that sum if it is at most cap, else 0 with
-// redo_bit set in *redo.
-__global__ void __launch_bounds__(1024) scan_small_kernel(const uint64_t *__restrict__ in, uint64_t *__restrict__ out,
-                                                          uint32_t n_arg, const uint64_t *__restrict__ n_dev,
-                                                          uint64_t add, uint64_t *__restrict__ tot, uint64_t cap,
-                                                          uint64_t *__restrict__ eff, uint64_t *__restrict__ redo,
+// redo_bit set in *redo.  The last `add` values count as zero (not read).
+__global__ void __launch_bounds__(1024) scan_small_kernel(const uint64_t *in, uint64_t *out, uint32_t n_arg,
+                                                          const uint64_t *n_dev, uint64_t add, uint64_t *tot,
+                                                          uint64_t cap, uint64_t *eff, uint64_t *redo,
                                                           uint64_t redo_bit)
 {
+    chain_start();
+    chain_wait();
     __shared__ uint64_t buf[4096];
     __shared__ uint64_t wsum[32];
-    const uint32_t n = n_dev ? (uint32_t)min(*n_dev + add, (uint64_t)n_arg) : n_arg;
+    const uint32_t n = n_dev ? (uint32_t)min(*(const volatile uint64_t *)n_dev + add, (uint64_t)n_arg) : n_arg;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint64_t carry = 0;
     for (uint32_t base = 0; base < n; base += 4096) {
@@ -263,7 +270,7 @@ __global__ void __launch_bounds__(1024) scan_small_kernel(const uint64_t *__rest
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const uint32_t i = base + tid + 1024u * u;
-            v[u] = i < n ? in[i] : 0;
+            v[u] = i + add < n ? in[i] : 0;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -334,15 +341,14 @@ void launch_pair_count(const ah_site *sites, uint64_t n, const uint64_t *n_dev, 
 {
     if (!n)
         return;
-    pair_count_kernel<<<grid_for(n, 128), 128, 0, s>>>(sites, n, n_dev, pass, pairs_d, counts, err);
-    AH_CUDA(cudaGetLastError());
+    launch_chained(pair_count_kernel, grid_for(n, 128), 128, 0, s, sites, n, n_dev, pass, pairs_d,
+                   counts, err);
 }
 
 void launch_total(const uint64_t *offs, const uint64_t *counts, uint64_t n, const uint64_t *n_dev, uint64_t add,
                   uint64_t *out, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit, cudaStream_t s)
 {
-    total_kernel<<<1, 1, 0, s>>>(offs, counts, n, n_dev, add, out, cap, eff, redo, redo_bit);
-    AH_CUDA(cudaGetLastError());
+    launch_chained(total_kernel, 1, 1, 0, s, offs, counts, n, n_dev, add, out, cap, eff, redo, redo_bit);
 }
 
 size_t scan_u64_temp_bytes(uint64_t n)
@@ -357,8 +363,8 @@ void exclusive_scan_u64(void *temp, size_t temp_bytes, const uint64_t *in, uint6
     if (n == 0)
         return;
     if (n <= kOneBlockScan) {
-        scan_small_kernel<<<1, 1024, 0, s>>>(in, out, (uint32_t)n, nullptr, 0, nullptr, 0, nullptr, nullptr, 0);
-        AH_CUDA(cudaGetLastError());
+        launch_chained(scan_small_kernel, 1, 1024, 0, s, in, out, (uint32_t)n, nullptr, 0, nullptr, 0, nullptr, nullptr,
+                       0);
         return;
     }
     AH_CUDA(cub::DeviceScan::ExclusiveSum(temp, temp_bytes, in, out, (int64_t)n, s));
@@ -370,21 +376,20 @@ void exclusive_scan_u64_dev(const uint64_t *in, uint64_t *out, uint64_t n, const
 {
     if (n == 0 || n > kSmallScan)
         throw Error(AH_ERR_ARG, "device-count scan: size outside 1..65536");
-    scan_small_kernel<<<1, 1024, 0, s>>>(in, out, (uint32_t)n, n_dev, add, tot, cap, eff, redo, redo_bit);
-    AH_CUDA(cudaGetLastError());
+    launch_chained(scan_small_kernel, 1, 1024, 0, s, in, out, (uint32_t)n, n_dev, add, tot, cap, eff, redo,
+                   redo_bit);
 }
 
 int scan_u64_launches(uint64_t n) { return n == 0 ? 0 : n <= kOneBlockScan ? 1 : 2; }
 
 void launch_pair_write(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, const uint64_t *offsets, ah_amplicon *out, uint64_t cap,
+                       const PairDev *pairs_d, const uint64_t *offsets, ah_amplicon *out, uint64_t *len, uint64_t cap,
                        const uint64_t *skip, uint64_t skip_bit, cudaStream_t s)
 {
     if (!n)
         return;
-    pair_write_kernel<<<grid_for(n, 128), 128, 0, s>>>(sites, n, n_dev, pass, pairs_d, offsets, out, cap, skip,
-                                                       skip_bit);
-    AH_CUDA(cudaGetLastError());
+    launch_chained(pair_write_kernel, grid_for(n, 128), 128, 0, s, sites, n, n_dev, pass, pairs_d,
+                   offsets, out, len, cap, skip, skip_bit);
 }
 
 } // namespace ah

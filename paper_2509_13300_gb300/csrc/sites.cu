@@ -135,14 +135,15 @@ template <> struct Vec16<uint64_t> {
 // the contig offsets when stage_contigs.
 template <typename K>
 __global__ void __launch_bounds__(32 * kRankWarps)
-    rank_sort_decode_kernel(const uint64_t *__restrict__ keys, uint64_t n_arg, const uint64_t *__restrict__ n_dev,
-                            int pbits, const uint64_t *__restrict__ contig_off, uint32_t n_contigs,
-                            bool stage_contigs, const uint32_t *__restrict__ contig_genome, ah_site *__restrict__ out,
-                            uint64_t *__restrict__ n_out, uint64_t *__restrict__ redo)
+    rank_sort_decode_kernel(const uint64_t *keys, uint64_t n_arg, const uint64_t *n_dev, int pbits, const uint64_t *__restrict__ contig_off, uint32_t n_contigs,
+                            bool stage_contigs, const uint32_t *__restrict__ contig_genome, ah_site *out, uint64_t *n_out,
+                            uint64_t *redo)
 {
+    chain_start();
+    chain_wait();
     using VT = Vec16<K>;
     constexpr int V = VT::V;
-    const uint64_t n64 = n_dev ? *n_dev : n_arg;
+    const uint64_t n64 = n_dev ? *(const volatile uint64_t *)n_dev : n_arg;
     if (n64 > n_arg) { // device count above the launch's size: the host redoes this step
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             *n_out = 0;
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(32 * kRankWarps)
 #pragma unroll
     for (int j = 0; j < kRankQ; ++j) {
         const uint32_t i = q0 + lane + 32u * j;
-        qkey[j] = i < n ? __ldg(keys + i) : 0;
+        qkey[j] = i < n ? keys[i] : 0;
     }
     // stage every key (sort bits only): two keys per 16-byte load, eight loads in flight per thread
     {
@@ -178,7 +179,7 @@ __global__ void __launch_bounds__(32 * kRankWarps)
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const uint32_t p = b + u * blockDim.x;
-                x[u] = p < pairs ? __ldg(k2 + p) : make_ulonglong2(~0ull, ~0ull);
+                x[u] = p < pairs ? k2[p] : make_ulonglong2(~0ull, ~0ull);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(32 * kRankWarps)
             }
         }
         for (uint32_t i = 2 * pairs + threadIdx.x; i < nv * V; i += blockDim.x)
-            cand[i] = i < n ? (K)(__ldg(keys + i) >> 8) : (K)~(K)0; // odd tail and padding (never below a key)
+            cand[i] = i < n ? (K)(keys[i] >> 8) : (K)~(K)0; // odd tail and padding (never below a key)
     }
     if (stage_contigs) { // n_contigs + 1 <= kRankStageContigs: at most 8 vector loads per thread, all in flight
         const uint32_t m = n_contigs + 1, m2 = m / 2;
@@ -292,9 +293,8 @@ void run_rank_sort(const uint64_t *keys, uint64_t n, const uint64_t *n_dev, int 
         attr_dev = dev;
     }
     const unsigned blocks = (unsigned)((n + 32 * kRankQ - 1) / (32 * kRankQ));
-    rank_sort_decode_kernel<K><<<blocks, 32 * kRankWarps, smem, s>>>(keys, n, n_dev, pbits, contig_off, n_contigs,
-                                                                      stage, contig_genome, out, n_out, redo);
-    AH_CUDA(cudaGetLastError());
+    launch_chained(rank_sort_decode_kernel<K>, blocks, 32 * kRankWarps, smem, s, keys, n, n_dev,
+                   pbits, contig_off, n_contigs, stage, contig_genome, out, n_out, redo);
 }
 
 } // namespace

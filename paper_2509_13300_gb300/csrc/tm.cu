@@ -218,21 +218,20 @@ __device__ __forceinline__ long long fix_weight(double dH, double dS, double thr
     return __double2ll_rn((1000.0 * dH - thr * dS) * kFix);
 }
 constexpr int kTmStageD = 4;
+constexpr unsigned kTmEarlyBlocks = 152;
 
 // Four lanes per site: lane y of a group holds the DP state "oligo base at
 // the current key position = y".  Each step takes the four predecessor costs
 // by shuffles and keeps the best predecessor (2 bits per key), so the argmin
 // oligo is recovered by a backtrack across the group's lanes; its dH, dS are
 // then summed by the four lanes together.  Eight sites per warp.
-__global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *__restrict__ sites, uint64_t n_arg,
-                                                           const uint64_t *__restrict__ n_dev,
+__global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites, uint64_t n_arg, const uint64_t *n_dev,
                                                            const PairDev *__restrict__ pairs, int n_pairs,
                                                            const uint32_t *__restrict__ planes,
                                                            const uint64_t *__restrict__ contig_off,
-                                                           float *__restrict__ tm_out, uint8_t *__restrict__ pass_out,
-                                                           uint32_t *__restrict__ queue, uint32_t *__restrict__ queue_n,
-                                                           int seg_max, int last_block_exact, int *__restrict__ err,
-                                                           const uint32_t *__restrict__ idx_list)
+                                                           float *tm_out, uint8_t *pass_out, uint32_t *queue,
+                                                           uint32_t *queue_n, int seg_max, int last_block_exact,
+                                                           int *err, const uint32_t *idx_list)
 {
     static_assert(32 * kTmWarps == kExactThreads, "the last block evaluates queued sites with exact_site");
     __shared__ int8_t bts[kTmWarps][8][AH_MAX_PRIMER_LEN];
@@ -240,16 +239,19 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *__rest
     // then [kTmWarps * 8 sites][seg_max][16] segment tables
     extern __shared__ __align__(16) unsigned char tm_smem[];
     TmPairS *ps = reinterpret_cast<TmPairS *>(tm_smem);
-    // the records' check failed: nothing is read with them, the call reports it (one answer per
-    // block: the word may change under it)
-    if (__syncthreads_or(*(volatile const int *)err))
-        return;
+    chain_start();
+    // The first blocks of a launch lay out the tables (which no kernel of the chain writes)
+    // while its predecessor runs; the others, and the list form's, learn first whether they
+    // have a site.
+    const bool early = !idx_list && blockIdx.x < kTmEarlyBlocks;
+    if (!early)
+        chain_wait();
     const int nd = n_pairs <= kTmStageD ? n_pairs : 0;
     TmPairD *pdd = reinterpret_cast<TmPairD *>(tm_smem + (size_t)n_pairs * sizeof(TmPairS));
     float2 *seg_smem =
         reinterpret_cast<float2 *>(tm_smem + (size_t)n_pairs * sizeof(TmPairS) + (size_t)nd * sizeof(TmPairD));
     // a block with no site of the list skips the tables (it still counts itself below)
-    const bool has_work = (uint64_t)blockIdx.x * kTmWarps * 8 < dev_count(n_arg, n_dev);
+    const bool has_work = early || (uint64_t)blockIdx.x * kTmWarps * 8 < dev_count(n_arg, n_dev);
     for (int j = 0; has_work && j < n_pairs; ++j) {
         const PairDev &P = pairs[j];
         for (int t = threadIdx.x; t < 256; t += blockDim.x)
@@ -271,7 +273,12 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *__rest
                 pdd[j].tm[threadIdx.x] = fix_weight(P.term_dH_d[threadIdx.x], P.term_dS_d[threadIdx.x], P.thr);
         }
     }
-    __syncthreads();
+    if (early)
+        chain_wait();
+    // the records' check failed: nothing is read with them, the call reports it (one answer per
+    // block: the word may change under it)
+    if (__syncthreads_or(*(volatile const int *)err))
+        return;
     const uint64_t n = dev_count(n_arg, n_dev);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, y = lane & 3, g0 = lane & ~3;
@@ -403,7 +410,7 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *__rest
         float dm = sm + ((amask >> m & 1u) ? tL.y : 0.f);
         dm = group_reduce(dm, [](float a, float b) { return a > b ? a : b; });
         const bool dink = run && dm + cst < 0.f;
-        float lam = 0.f;
+        float lam = 320.f; // any start gives an oligo; near annealing temperatures mostly the best one
         for (int it = 0; it < 64; ++it) {
             // min over oligos of 1000 dH - lam dS, with the best predecessor at every key
             float c = (dink && (amask & 1u)) ? 1000.f * t0.x - lam * t0.y : INF;
@@ -1344,7 +1351,8 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
         cached_dev = dev;
     }
     // queue length, finished blocks, deferred sites
-    AH_CUDA(cudaMemsetAsync(queue_n, 0, 2 * sizeof(uint64_t), s));
+    if (!n_dev)
+        AH_CUDA(cudaMemsetAsync(queue_n, 0, 2 * sizeof(uint64_t), s));
     // Few sites (a latency-bound launch): the four-lane kernel alone finishes first
     // (measured on GB300 for 6,253 sites: 33 us, against 36 + 27 us for the two
     // kernels below); many sites: one thread per site (6x the four-lane rate on
@@ -1361,20 +1369,18 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
         AH_CUDA(cudaGetLastError());
         // deferred sites (few; their count stays on the device): a persistent grid
         const uint64_t tb = std::min<uint64_t>((n + 8 * kTmWarps - 1) / (8 * kTmWarps), (uint64_t)sms * tm_bps);
-        tm_kernel<<<(unsigned)tb, 32 * kTmWarps, smem, s>>>(sites, n, reinterpret_cast<const uint64_t *>(defer_n),
-                                                            pairs_d, n_pairs, planes, contig_off, tm_out, pass_out,
-                                                            queue, queue_n, seg_max, 1, err, defer);
-        AH_CUDA(cudaGetLastError());
+        launch_chained(tm_kernel, (unsigned)tb, 32 * kTmWarps, smem, s, sites, n,
+                       reinterpret_cast<const uint64_t *>(defer_n), pairs_d, n_pairs, planes, contig_off, tm_out, pass_out,
+                       queue, queue_n, seg_max, 1, err, defer);
         return;
     }
     const uint64_t per_block = 8ull * kTmWarps; // sites per block per pass
     uint64_t blocks = (n + per_block - 1) / per_block;
     if (blocks > 65535)
         blocks = 65535;
-    tm_kernel<<<(unsigned)blocks, 32 * kTmWarps, smem, s>>>(sites, n, n_dev, pairs_d, n_pairs, planes, contig_off,
-                                                            tm_out, pass_out, queue, queue_n, seg_max,
-                                                            few_exact ? 1 : 0, err, nullptr);
-    AH_CUDA(cudaGetLastError());
+    launch_chained(tm_kernel, (unsigned)blocks, 32 * kTmWarps, smem, s, sites, n, n_dev, pairs_d,
+                   n_pairs, planes, contig_off, tm_out, pass_out, queue, queue_n, seg_max, few_exact ? 1 : 0, err,
+                   nullptr);
     if (few_exact)
         return;
     tm_exact_kernel<<<(unsigned)sms, kExactThreads, 0, s>>>(sites, pairs_d, planes, contig_off, queue, queue_n,
