@@ -125,9 +125,9 @@ __device__ uint64_t oligo_number(const uint8_t *qm, int L, int o)
 // the Tm and the pass flag.  bt and wmax are the block's shared scratch.
 constexpr int kExactThreads = 128; // fp64-bound: a block of 128 already keeps the SM's fp64 units busy
 
-__device__ void exact_site(const ah_site *__restrict__ sites, const PairDev *__restrict__ pairs,
-                           const uint32_t *__restrict__ planes, const uint64_t *__restrict__ contig_off, uint32_t i,
-                           float *__restrict__ tm_out, uint8_t *__restrict__ pass_out, int8_t *bt, double *wmax)
+__device__ void exact_site(const ah_site *sites, const PairDev *__restrict__ pairs, const uint32_t *__restrict__ planes,
+                           const uint64_t *__restrict__ contig_off, uint32_t i, float *tm_out, uint8_t *pass_out,
+                           int8_t *bt, double *wmax)
 {
     const ah_site s = sites[i];
     const PairDev &pd = pairs[s.pair];
@@ -191,20 +191,29 @@ __global__ void __launch_bounds__(kExactThreads) tm_exact_kernel(const ah_site *
 // Per-pair constants of the fp32 path, staged in shared memory by every
 // block (the shortest-path steps read them in dependent chains).
 struct TmPairS {
-    float2 st[256]; // (dH, dS) of each stack
-    float2 tm[16];  // (dH, dS) of each terminal pair
-    uint8_t mask[2][AH_MAX_PRIMER_LEN];
-    uint8_t key[2][AH_MAX_PRIMER_LEN];
+    float2 st[256]; // (dH, dS) of each stack, [oligo pair o0 + 4 o1][template pair t0 + 4 t1]
+    float2 tm[16];  // of each terminal pair, [oligo base][template base]
+    uint64_t first[2];      // lowest base of each position's set, 2 bits each
+    uint32_t allowed[2][4]; // per base, bit i: it is in key i's set
+    uint8_t key[2][AH_MAX_PRIMER_LEN]; // key positions (both ends and every degenerate one), ascending
     int L[2], nkey[2];
+    float cst[2]; // C + salt entropy
+    float tm_min_f, tm_shift_f;
 };
 static_assert(sizeof(TmPairS) % 16 == 0, "TmPairS keeps 16-byte alignment");
+
+// The entry of a table indexed like PairDev's, o0 o1 t0 t1, in the order of TmPairS.
+__device__ __forceinline__ int staged_stack(int t)
+{
+    return ((t >> 4 & 3) * 4 + (t >> 6)) * 16 + (t & 3) * 4 + (t >> 2 & 3);
+}
 
 // The weights 1000 dH - thr dS of every table entry at the pair's threshold
 // thr, for the near-threshold sign test: computed in fp64 from the fp64
 // table, then held as fixed point (units of 2^-30 cal/mol, int64) so that
 // every path sum is exact; staged for up to kTmStageD pairs.
 struct TmPairD {
-    long long st[256];
+    long long st[256]; // in the order of TmPairS
     long long tm[16];
 };
 constexpr double kFix = 1073741824.0; // 2^30: fixed-point scale of the sign test
@@ -218,23 +227,122 @@ __device__ __forceinline__ long long fix_weight(double dH, double dS, double thr
     return __double2ll_rn((1000.0 * dH - thr * dS) * kFix);
 }
 constexpr int kTmStageD = 4;
-constexpr unsigned kTmEarlyBlocks = 152;
+constexpr unsigned kTmEarlyBlocks = 304; // two per SM
+
+// 8 x 8 bit transpose: bit c of byte r -> bit r of byte c
+__device__ __forceinline__ uint64_t transpose8(uint64_t x)
+{
+    uint64_t t = (x ^ (x >> 7)) & 0x00AA00AA00AA00AAull;
+    x ^= t ^ (t << 7);
+    t = (x ^ (x >> 14)) & 0x0000CCCC0000CCCCull;
+    x ^= t ^ (t << 14);
+    t = (x ^ (x >> 28)) & 0x00000000F0F0F0F0ull;
+    return x ^ t ^ (t << 28);
+}
+
+// A site's window in the planes, for a warp that fetches it with one 16-byte load per
+// lane: 8 lanes per plane, 4 words each, from the 16-byte boundary below the window.
+struct Window {
+    uint64_t base;   // byte offset of that boundary in the A plane
+    uint32_t o, row; // words from there to the window; the bit of its row
+    uint32_t last;   // its last word, from the boundary (at most 31)
+};
+
+__device__ __forceinline__ Window window_at(uint64_t P, int L)
+{
+    const uint32_t w = (uint32_t)(P % kTileBases);
+    Window d;
+    d.base = 4 * (P / kTileBases * (4 * kTileWX) + (w & (kTileW - 4)));
+    d.o = w & 3u;
+    d.row = w / kTileW;
+    d.last = min(d.o + (uint32_t)L, 32u) - 1u;
+    return d;
+}
+
+// The load of a lane: plane lane / 8, words 4 (lane % 8) .. + 3.  Lanes past the window
+// read its last group again (no other sector).
+__device__ __forceinline__ uint4 window_load(const uint32_t *planes, int lane, uint64_t base, uint32_t last_group)
+{
+    const char *p = reinterpret_cast<const char *>(planes + (lane >> 3) * kTileWX);
+    return __ldg(reinterpret_cast<const uint4 *>(p + base + min(16u * (lane & 7), last_group)));
+}
+
+// Template codes opposite each primer position (A 0, C 1, G 2, T 3), 2 bits each, from
+// the four ballots of a window's row: bit 8 x + g of B[j] = plane x at word 4 g + j.
+// ok: every position holds one of the four letters.
+__device__ __forceinline__ uint64_t window_codes(const uint32_t *planes, const Window &d, int L, int strand,
+                                                 const uint32_t (&B)[4], bool *ok)
+{
+    uint32_t extra[4] = {0, 0, 0, 0}; // words 32 .. 34 of a long window that starts off the boundary, per plane
+    if (d.o + L > 32) {
+        const uint32_t *p = planes + (d.base >> 2) + 32;
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+                if (32u + j < d.o + L)
+                    extra[x] |= ((__ldg(p + x * kTileWX + j) >> d.row) & 1u) << j;
+    }
+    // words outside [o, o + L) cleared; every position has exactly one plane set, or the window is bad
+    int set = __popc(extra[0] | extra[1] | extra[2] | extra[3]);
+    uint64_t rows = 0; // byte 2 j + h: bit g = bit h of the code at word 4 g + j
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+        // groups whose word 4 g + j is at most `last`: all before last's, and its own up to last
+        uint32_t keep = (1u << ((d.last >> 2) + (j <= (d.last & 3u)))) - 1u;
+        if (j < d.o)
+            keep &= ~1u;
+        const uint32_t v = B[j] & keep * 0x01010101u;
+        set += __popc(v);
+        const uint32_t lo8 = ((v >> 8) | (v >> 24)) & 0xffu, hi8 = ((v >> 16) | (v >> 24)) & 0xffu;
+        rows |= (uint64_t)(lo8 | hi8 << 8) << (16 * j);
+    }
+    uint64_t code = transpose8(rows) >> (2 * d.o);
+    if (d.o) { // (o = 0: nothing past word 31)
+        const uint64_t elo = extra[1] | extra[3], ehi = extra[2] | extra[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            code |= ((elo >> j & 1u) | (ehi >> j & 1u) << 1) << (2 * (32 + j) - 2 * d.o) % 64;
+    }
+    *ok = set == L;
+    if (strand == 0) // the complement of the window base at q
+        return ~code;
+    code = __brevll(code) >> (64 - 2 * L); // the window base at L - 1 - q
+    return (code >> 1 & 0x5555555555555555ull) | (code & 0x5555555555555555ull) << 1;
+}
 
 // Four lanes per site: lane y of a group holds the DP state "oligo base at
 // the current key position = y".  Each step takes the four predecessor costs
 // by shuffles and keeps the best predecessor (2 bits per key), so the argmin
 // oligo is recovered by a backtrack across the group's lanes; its dH, dS are
-// then summed by the four lanes together.  Eight sites per warp.
+// then summed by the four lanes together.  (Carrying dH and dS of the best
+// predecessor along takes two more dependent shuffles per step: 3,650 cycles per
+// pass of nine steps instead of 2,520.)  Eight sites per warp, their windows
+// fetched together (one 16-byte load per lane and site).
+//
+// kFew (tables under which only the rare ambiguous sites need the exhaustive
+// evaluation, all duplexes having dS + C < 0): a block evaluates its own sites'.
+// Else the largest denominator decides whether the iteration applies, and the
+// sites for the exhaustive evaluation go to a queue.
+//
+// Bound: latency (a few sites per warp, dependent loads and shuffles).  Cycles on
+// a GB300 for 20 sites, from the wait for the predecessor: 24,000 with the error
+// word, the count and the records read one after the other, a window position per
+// load, template bases in shared memory, a backtrack per pass and a last block
+// that looks for queued sites -> 12,500.
+template <bool kFew>
 __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites, uint64_t n_arg, const uint64_t *n_dev,
                                                            const PairDev *__restrict__ pairs, int n_pairs,
                                                            const uint32_t *__restrict__ planes,
                                                            const uint64_t *__restrict__ contig_off,
                                                            float *tm_out, uint8_t *pass_out, uint32_t *queue,
-                                                           uint32_t *queue_n, int seg_max, int last_block_exact,
-                                                           int *err, const uint32_t *idx_list)
+                                                           uint32_t *queue_n, int seg_max, int *err,
+                                                           const uint32_t *idx_list)
 {
-    static_assert(32 * kTmWarps == kExactThreads, "the last block evaluates queued sites with exact_site");
-    __shared__ int8_t bts[kTmWarps][8][AH_MAX_PRIMER_LEN];
+    static_assert(32 * kTmWarps == kExactThreads, "a block evaluates its ambiguous sites with exact_site");
+    __shared__ uint32_t xq[8 * kTmWarps], xn; // kFew: ambiguous sites of a round
+    __shared__ int8_t xbt[AH_MAX_PRIMER_LEN];
+    __shared__ double xmax[kTmWarps];
     // dynamic: [n_pairs] TmPairS, [n_pairs <= kTmStageD ? n_pairs : 0] TmPairD,
     // then [kTmWarps * 8 sites][seg_max][16] segment tables
     extern __shared__ __align__(16) unsigned char tm_smem[];
@@ -250,199 +358,217 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
     TmPairD *pdd = reinterpret_cast<TmPairD *>(tm_smem + (size_t)n_pairs * sizeof(TmPairS));
     float2 *seg_smem =
         reinterpret_cast<float2 *>(tm_smem + (size_t)n_pairs * sizeof(TmPairS) + (size_t)nd * sizeof(TmPairD));
-    // a block with no site of the list skips the tables (it still counts itself below)
-    const bool has_work = early || (uint64_t)blockIdx.x * kTmWarps * 8 < dev_count(n_arg, n_dev);
-    for (int j = 0; has_work && j < n_pairs; ++j) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (!early && (uint64_t)blockIdx.x * kTmWarps * 8 >= dev_count(n_arg, n_dev))
+        return;
+    for (int j = 0; j < n_pairs; ++j) {
         const PairDev &P = pairs[j];
         for (int t = threadIdx.x; t < 256; t += blockDim.x)
-            ps[j].st[t] = make_float2(P.stack_dH[t], P.stack_dS[t]);
+            ps[j].st[staged_stack(t)] = make_float2(P.stack_dH[t], P.stack_dS[t]);
         if (threadIdx.x < 16)
             ps[j].tm[threadIdx.x] = make_float2(P.term_dH[threadIdx.x], P.term_dS[threadIdx.x]);
-        if (threadIdx.x < 2 * AH_MAX_PRIMER_LEN) {
-            (&ps[j].mask[0][0])[threadIdx.x] = (&P.mask[0][0])[threadIdx.x];
-            (&ps[j].key[0][0])[threadIdx.x] = (&P.key[0][0])[threadIdx.x];
-        }
-        if (threadIdx.x < 2) {
-            ps[j].L[threadIdx.x] = P.L[threadIdx.x];
-            ps[j].nkey[threadIdx.x] = P.nkey[threadIdx.x];
+        if (threadIdx.x == 0) {
+            ps[j].tm_min_f = P.tm_min_f;
+            ps[j].tm_shift_f = (float)P.tm_shift;
         }
         if (j < nd) {
             for (int t = threadIdx.x; t < 256; t += blockDim.x)
-                pdd[j].st[t] = fix_weight(P.stack_dH_d[t], P.stack_dS_d[t], P.thr);
+                pdd[j].st[staged_stack(t)] = fix_weight(P.stack_dH_d[t], P.stack_dS_d[t], P.thr);
             if (threadIdx.x < 16)
                 pdd[j].tm[threadIdx.x] = fix_weight(P.term_dH_d[threadIdx.x], P.term_dS_d[threadIdx.x], P.thr);
         }
     }
+    for (int c = warp; c < 2 * n_pairs; c += kTmWarps) { // a warp per primer, lane q position q
+        const PairDev &P = pairs[c >> 1];
+        TmPairS &sp = ps[c >> 1];
+        const int x = c & 1, L = P.L[x];
+        const uint32_t m = lane < L ? P.mask[x][lane] : 0u;
+        const bool key = lane < L && (lane == 0 || lane == L - 1 || __popc(m) > 1);
+        const uint32_t keys = __ballot_sync(0xffffffffu, key);
+        const int at = __popc(keys & ((1u << lane) - 1u));
+        uint32_t allowed[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            allowed[b] = __reduce_or_sync(0xffffffffu, key ? (m >> b & 1u) << at : 0u);
+        if (key)
+            sp.key[x][at] = (uint8_t)lane;
+        const uint64_t low = lane < L ? (uint64_t)(__ffs(m) - 1) << (2 * lane) : 0ull;
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)low);
+        const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(low >> 32));
+        if (lane == 0) {
+            sp.first[x] = (uint64_t)hi << 32 | lo;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                sp.allowed[x][b] = allowed[b];
+            sp.L[x] = L;
+            sp.nkey[x] = __popc(keys);
+            sp.cst[x] = (float)(P.sconst + (P.saltcorr == 5 ? 0.368 * (double)(L - 1) * P.log_na : 0.0));
+        }
+    }
     if (early)
         chain_wait();
-    // the records' check failed: nothing is read with them, the call reports it (one answer per
-    // block: the word may change under it)
-    if (__syncthreads_or(*(volatile const int *)err))
-        return;
-    const uint64_t n = dev_count(n_arg, n_dev);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, y = lane & 3, g0 = lane & ~3;
-    int8_t *bt = bts[warp][g];
+    // The error word, the count and the first record (below n_arg, so in its buffer) as loads
+    // that wait for none of the others.  With the word set nothing is read with the records, the
+    // call reports it (one answer per block: the word may change under it).
+    const int bad_word = *(volatile const int *)err;
+    const uint64_t n = dev_count(n_arg, n_dev);
+    uint64_t first_block = (uint64_t)blockIdx.x * kTmWarps * 8;
+    ah_site s0{};
+    if (!idx_list && first_block + warp * 8 + g < n_arg)
+        s0 = sites[first_block + warp * 8 + g];
+    if (__syncthreads_or(bad_word))
+        return;
     const float INF = INFINITY;
-    const uint64_t groups = (uint64_t)gridDim.x * kTmWarps * 8;
-    for (uint64_t base = ((uint64_t)blockIdx.x * kTmWarps + warp) * 8; base < n; base += groups) {
+    const uint64_t step = (uint64_t)gridDim.x * kTmWarps * 8;
+    for (uint64_t base0 = first_block; base0 < n; base0 += step) { // all warps of the block together
+        const uint64_t base = base0 + warp * 8;
         const bool live = base + g < n;
         // with idx_list, the sites taken are sites[idx_list[0 .. n)]
         const uint64_t i = live && idx_list ? (uint64_t)idx_list[base + g] : base + g;
         ah_site s{};
         if (live)
-            s = sites[i];
+            s = !idx_list && base0 == first_block ? s0 : sites[i];
         const bool bad_rec = live && (s.pair >= n_pairs || s.primer > 1 || s.strand > 1);
         if (bad_rec && y == 0)
             atomicExch(err, kDevBounds);
         const bool act = live && !bad_rec;
-        const PairDev &pd = pairs[act ? s.pair : 0];
-        const TmPairS &sp = ps[act ? s.pair : 0];
-        const int L = act ? sp.L[s.primer] : 2;
-        const uint8_t *mask = sp.mask[act ? s.primer : 0];
-        // template base opposite each primer position; every entry the DP reads
-        // is written (0..3), also for groups without a live site.  All of a lane's
-        // plane words are requested before any is used (one memory latency).
-        bool bad = false;
-        if (act) {
-            const uint64_t P = contig_off[s.contig] + s.pos;
-            uint32_t w[8][4];
-            int bitpos[8];
+        const int pi = act ? s.pair : 0, x1 = act ? s.primer : 0;
+        const PairDev &pd = pairs[pi];
+        const TmPairS &sp = ps[pi];
+        const int L = sp.L[x1];
+        // the group's window (without a live site: the first of the planes, unused)
+        Window d{};
+        if (act)
+            d = window_at(contig_off[s.contig] + s.pos, L);
+        uint32_t B[4] = {0, 0, 0, 0};
+        {
+            uint4 w[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                w[j] = window_load(planes, lane, __shfl_sync(0xffffffffu, d.base, 4 * j),
+                                   4u * (__shfl_sync(0xffffffffu, d.last, 4 * j) & ~3u));
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const int q = min(y + 4 * j, L - 1); // past the primer: a repeat of its last position, unused
-                const uint64_t Pq = P + (s.strand == 0 ? q : L - 1 - q);
-                const uint64_t t = Pq / kTileBases, r = Pq % kTileBases;
-                bitpos[j] = (int)(r / kTileW);
-                const uint32_t *wp = planes + t * 4 * kTileWX + (r % kTileW);
-#pragma unroll
-                for (int x = 0; x < 4; ++x)
-                    w[j][x] = __ldg(wp + x * kTileWX);
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int q = y + 4 * j;
-                if (q < L) {
-                    int c = -1;
-#pragma unroll
-                    for (int x = 0; x < 4; ++x)
-                        if ((w[j][x] >> bitpos[j]) & 1u)
-                            c = x;
-                    bad |= c < 0;
-                    bt[q] = (int8_t)(c < 0 ? 0 : (s.strand == 0 ? 3 - c : c));
+                const uint32_t bit = 1u << __shfl_sync(0xffffffffu, d.row, 4 * j);
+                const uint32_t v0 = __ballot_sync(0xffffffffu, w[j].x & bit);
+                const uint32_t v1 = __ballot_sync(0xffffffffu, w[j].y & bit);
+                const uint32_t v2 = __ballot_sync(0xffffffffu, w[j].z & bit);
+                const uint32_t v3 = __ballot_sync(0xffffffffu, w[j].w & bit);
+                if (g == j) {
+                    B[0] = v0;
+                    B[1] = v1;
+                    B[2] = v2;
+                    B[3] = v3;
                 }
             }
-        } else {
-            for (int q = y; q < L; q += 4)
-                bt[q] = 0;
         }
-        __syncwarp();
-        bad = __shfl_sync(0xffffffffu, (int)bad, g0) | __shfl_sync(0xffffffffu, (int)bad, g0 + 1) |
-              __shfl_sync(0xffffffffu, (int)bad, g0 + 2) | __shfl_sync(0xffffffffu, (int)bad, g0 + 3);
-        const bool run = act && !bad;
-        const float cst =
-            act ? (float)(pd.sconst + (pd.saltcorr == 5 ? 0.368 * (double)(L - 1) * pd.log_na : 0.0)) : -1.f;
+        bool ok = false;
+        uint64_t code = 0;
+        if (act)
+            code = window_codes(planes, d, L, s.strand, B, &ok);
+        const bool bad = !ok, run = act && ok;
+        const float cst = sp.cst[x1];
         // Steps at key positions only (primer positions 0 and L-1 and every
         // degenerate one): between two keys the oligo bases are fixed, so all
         // stacks from key i to key i+1 form a 4x4 table of (dH, dS) sums
         // indexed by the bases at the two keys, E[i][a * 4 + b].  Lane y fills
         // column y of the site's tables once; every pass below reads them.
-        const int m = act ? sp.nkey[s.primer] - 1 : 0; // segments
-        const uint8_t *key = sp.key[act ? s.primer : 0];
+        const uint8_t *key = sp.key[x1];
+        const uint64_t first = sp.first[x1];
+        const int m = run ? sp.nkey[x1] - 1 : 0; // segments
+        // Shuffles need all 32 lanes, but the groups' segment counts differ: every
+        // segment loop runs to the warp's largest count mw and each group only
+        // updates its state while si < m.
+        const int mw = (int)__reduce_max_sync(0xffffffffu, (uint32_t)m);
+        auto oligo2 = [&](int q) { return (int)(first >> (2 * q)) & 15; }; // fixed bases at q and q + 1
+        auto templ2 = [&](int q) { return (int)(code >> (2 * q)) & 15; };  // template bases at q and q + 1
         float2 *E = seg_smem + (size_t)(warp * 8 + g) * seg_max * 16;
-        if (run) {
-            for (int si = 0; si < m; ++si) {
-                const int k0 = key[si], k1 = key[si + 1];
-                if (k1 == k0 + 1) {
+        for (int sb = 0; sb < mw; sb += 4) {
+            // the stacks between two fixed bases: lane y sums those of segment sb + y
+            float cH = 0.f, cS = 0.f;
+            if (sb + y < m) {
+                const int k1 = key[sb + y + 1];
+#pragma unroll 4
+                for (int q = key[sb + y] + 1; q < k1 - 1; ++q) {
+                    const float2 e = sp.st[oligo2(q) * 16 + templ2(q)];
+                    cH += e.x;
+                    cS += e.y;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float uH = __shfl_sync(0xffffffffu, cH, g0 + u), uS = __shfl_sync(0xffffffffu, cS, g0 + u);
+                const int si = sb + u;
+                if (si < m) {
+                    const int k0 = key[si], k1 = key[si + 1], p0 = templ2(k0);
+                    const bool apart = k1 > k0 + 1; // else one stack from x to y
+                    const int fa = oligo2(k0 + 1) & 3, fb = oligo2(k1 - 1) & 3;
+                    const float2 eq = sp.st[(fb + 4 * y) * 16 + templ2(k1 - 1)]; // into key k1, base y
+                    const float qH = apart ? eq.x + uH : 0.f, qS = apart ? eq.y + uS : 0.f;
+                    const int to = apart ? fa : y;
+#pragma unroll
                     for (int x = 0; x < 4; ++x) {
-                        E[si * 16 + x * 4 + y] = sp.st[((x * 4 + y) * 4 + bt[k0]) * 4 + bt[k1]];
-                    }
-                } else {
-                    float cH = 0.f, cS = 0.f; // stacks between two fixed bases
-                    for (int q = k0 + 2; q < k1; ++q) {
-                        const int a0 = __ffs(mask[q - 1]) - 1, b0 = __ffs(mask[q]) - 1;
-                        const float2 e = sp.st[((a0 * 4 + b0) * 4 + bt[q - 1]) * 4 + bt[q]];
-                        cH += e.x;
-                        cS += e.y;
-                    }
-                    const int fa = __ffs(mask[k0 + 1]) - 1, fb = __ffs(mask[k1 - 1]) - 1;
-                    const float2 eq = sp.st[((fb * 4 + y) * 4 + bt[k1 - 1]) * 4 + bt[k1]]; // into key k1, base y
-                    const float qH = eq.x + cH, qS = eq.y + cS;
-                    for (int x = 0; x < 4; ++x) {
-                        const float2 ep = sp.st[((x * 4 + fa) * 4 + bt[k0]) * 4 + bt[k0 + 1]]; // out of key k0, base x
+                        const float2 ep = sp.st[(x + 4 * to) * 16 + p0]; // out of key k0, base x
                         E[si * 16 + x * 4 + y] = make_float2(ep.x + qH, ep.y + qS);
                     }
                 }
             }
         }
-        __syncwarp();
         // bit i: base y is allowed at key i; this lane's terminal terms at both ends
-        uint32_t amask = 0;
-        float2 t0 = make_float2(0.f, 0.f), tL = make_float2(0.f, 0.f);
-        if (run) {
-            for (int si = 0; si <= m; ++si)
-                amask |= (uint32_t)(mask[key[si]] >> y & 1) << si;
-            t0 = sp.tm[y * 4 + bt[0]];
-            tL = sp.tm[y * 4 + bt[L - 1]];
-        }
-        // Shuffles need all 32 lanes, but the groups' segment counts differ: every
-        // segment loop runs to the warp's largest count mw and each group only
-        // updates its state while si < m.
-        int mw = run ? m : 0;
-        for (int d = 16; d >= 1; d >>= 1)
-            mw = max(mw, __shfl_xor_sync(0xffffffffu, mw, d));
-        // largest denominator over oligos (max-path of dS)
-        float sm = (amask & 1u) ? t0.y : -INF;
-        for (int si = 0; si < mw; ++si) {
-            const bool in = run && si < m;
-            float best = -INF;
+        const uint32_t amask = run ? sp.allowed[x1][y] : 0u;
+        const int tF = (int)code & 3, tE = (int)(code >> (2 * (L - 1))) & 3;
+        const float2 t0 = run ? sp.tm[y * 4 + tF] : make_float2(0.f, 0.f);
+        const float2 tL = run ? sp.tm[y * 4 + tE] : make_float2(0.f, 0.f);
+        __syncwarp(); // the group's tables
+        bool dink = run;
+        if (!kFew) { // largest denominator over oligos (max-path of dS)
+            float sm = (amask & 1u) ? t0.y : -INF;
+            for (int si = 0; si < mw; ++si) {
+                const bool in = run && si < m;
+                float best = -INF;
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const float cx = __shfl_sync(0xffffffffu, sm, g0 + x);
-                if (in) {
-                    const float v = cx + E[si * 16 + x * 4 + y].y;
-                    best = v > best ? v : best;
+                for (int x = 0; x < 4; ++x) {
+                    const float cx = __shfl_sync(0xffffffffu, sm, g0 + x);
+                    if (in) {
+                        const float v = cx + E[si * 16 + x * 4 + y].y;
+                        best = v > best ? v : best;
+                    }
                 }
+                if (in)
+                    sm = (amask >> (si + 1) & 1u) ? best : -INF;
             }
-            if (in)
-                sm = (amask >> (si + 1) & 1u) ? best : -INF;
+            float dm = sm + ((amask >> m & 1u) ? tL.y : 0.f);
+            dm = group_reduce(dm, [](float a, float b) { return a > b ? a : b; });
+            dink = run && dm + cst < 0.f;
         }
-        float dm = sm + ((amask >> m & 1u) ? tL.y : 0.f);
-        dm = group_reduce(dm, [](float a, float b) { return a > b ? a : b; });
-        const bool dink = run && dm + cst < 0.f;
         float lam = 320.f; // any start gives an oligo; near annealing temperatures mostly the best one
         for (int it = 0; it < 64; ++it) {
             // min over oligos of 1000 dH - lam dS, with the best predecessor at every key
-            float c = (dink && (amask & 1u)) ? 1000.f * t0.x - lam * t0.y : INF;
+            float c = (dink && (amask & 1u)) ? fmaf(-lam, t0.y, 1000.f * t0.x) : INF;
             uint64_t pred = 0;
             for (int si = 0; si < mw; ++si) {
-                const bool in = dink && si < m;
-                float best = INF;
-                int arg = 0;
+                float v[4]; // (past its own segments a group reads entries that it then leaves alone)
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
-                    const float cx = __shfl_sync(0xffffffffu, c, g0 + x);
-                    if (in) {
-                        const float2 e = E[si * 16 + x * 4 + y];
-                        const float v = cx + fmaf(-lam, e.y, 1000.f * e.x);
-                        if (v < best) {
-                            best = v;
-                            arg = x;
-                        }
-                    }
+                    const float2 e = E[si * 16 + x * 4 + y];
+                    v[x] = __shfl_sync(0xffffffffu, c, g0 + x) + fmaf(-lam, e.y, 1000.f * e.x);
                 }
-                if (in) {
-                    c = (amask >> (si + 1) & 1u) ? best : INF;
+                const bool b1 = v[1] < v[0], b3 = v[3] < v[2]; // ties: the lowest base
+                const float lo = b1 ? v[1] : v[0], hi = b3 ? v[3] : v[2];
+                const bool bh = hi < lo;
+                const uint32_t arg = bh ? (b3 ? 3u : 2u) : (b1 ? 1u : 0u);
+                if (si < m) {
+                    c = dink && (amask >> (si + 1) & 1u) ? (bh ? hi : lo) : INF;
                     pred |= (uint64_t)arg << (2 * si);
                 }
             }
-            float fin = dink ? c + 1000.f * tL.x - lam * tL.y : INF;
-            if (!(c < INF))
-                fin = INF;
+            const float fin = dink && c < INF ? c + fmaf(-lam, tL.y, 1000.f * tL.x) : INF;
             // argmin over the group's four end states (ties: lowest base)
             const float fmin = group_reduce(fin, [](float a, float b) { return a < b ? a : b; });
             const unsigned hit = __ballot_sync(0xffffffffu, fin == fmin) >> g0 & 0xFu;
             int cur = hit ? __ffs(hit) - 1 : 0;
+            const int last = cur;
             // backtrack the bases at the keys: ks[i] = base at key i (2 bits each)
             uint64_t ks = (uint64_t)cur << (2 * m);
             for (int si = mw - 1; si >= 0; --si) {
@@ -456,17 +582,15 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
             float H = 0.f, S = 0.f;
             if (dink)
                 for (int si = y; si < m; si += 4) {
-                    const int a0 = (int)(ks >> (2 * si) & 3u), b0 = (int)(ks >> (2 * (si + 1)) & 3u);
-                    const float2 e = E[si * 16 + a0 * 4 + b0];
+                    const float2 e = E[si * 16 + (int)(ks >> (2 * si) & 3u) * 4 + (int)(ks >> (2 * (si + 1)) & 3u)];
                     H += e.x;
                     S += e.y;
                 }
             H = group_reduce(H, [](float a, float b) { return a + b; });
             S = group_reduce(S, [](float a, float b) { return a + b; });
             // terminal terms of the chosen end bases: held by the lanes of those bases
-            const int o0 = (int)(ks & 3u), oL = (int)(ks >> (2 * m) & 3u);
-            H += __shfl_sync(0xffffffffu, t0.x, g0 + o0) + __shfl_sync(0xffffffffu, tL.x, g0 + oL);
-            S += __shfl_sync(0xffffffffu, t0.y, g0 + o0) + __shfl_sync(0xffffffffu, tL.y, g0 + oL);
+            H += __shfl_sync(0xffffffffu, t0.x, g0 + cur) + __shfl_sync(0xffffffffu, tL.x, g0 + last);
+            S += __shfl_sync(0xffffffffu, t0.y, g0 + cur) + __shfl_sync(0xffffffffu, tL.y, g0 + last);
             const float r = 1000.f * H / (S + cst);
             // Warp-uniform loop: stop when no group still improves by more than
             // 1e-4 K.  In fp32 two oligos of nearly equal ratio could otherwise
@@ -478,9 +602,9 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
             if (!__any_sync(0xffffffffu, more))
                 break;
         }
-        const float tm32 = lam - 273.15f + (act ? (float)pd.tm_shift : 0.f);
+        const float tm32 = lam - 273.15f + sp.tm_shift_f;
         // near the threshold: the sign of min F at lam = thr, in fp64 (file comment)
-        const bool near = dink && pass_out && fabsf(tm32 - pd.tm_min_f) < 0.01f;
+        const bool near = dink && pass_out && fabsf(tm32 - sp.tm_min_f) < 0.01f;
         int decided = -1; // 1 pass, 0 fail, -1 undecided
         if (__any_sync(0xffffffffu, near)) {
             // Same key segments, exact fixed-point weights at lam = thr.  First every
@@ -488,10 +612,13 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
             // fp32 tables, no longer needed), then the dependent chain over the segments.
             const long long LINF = 0x2000000000000000ll; // above any path sum, no overflow when added to
             long long *W = reinterpret_cast<long long *>(E); // W[si * 16 + x * 4 + y], 8 bytes per float2 slot
-            const bool staged = act && s.pair < nd;
-            const TmPairD &sd = pdd[staged ? s.pair : 0];
-            auto stW = [&](int idx) {
-                return staged ? sd.st[idx] : fix_weight(pd.stack_dH_d[idx], pd.stack_dS_d[idx], pd.thr);
+            const bool staged = pi < nd;
+            const TmPairD &sd = pdd[staged ? pi : 0];
+            auto stW = [&](int o2, int t2) { // oligo and template pairs, as in TmPairS
+                if (staged)
+                    return sd.st[o2 * 16 + t2];
+                const int idx = (((o2 & 3) * 4 + (o2 >> 2)) * 4 + (t2 & 3)) * 4 + (t2 >> 2);
+                return fix_weight(pd.stack_dH_d[idx], pd.stack_dS_d[idx], pd.thr);
             };
             auto tmW = [&](int idx) {
                 return staged ? sd.tm[idx] : fix_weight(pd.term_dH_d[idx], pd.term_dS_d[idx], pd.thr);
@@ -499,25 +626,23 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
             __syncwarp();
             if (near) {
                 for (int si = 0; si < m; ++si) {
-                    const int k0 = key[si], k1 = key[si + 1];
+                    const int k0 = key[si], k1 = key[si + 1], p0 = templ2(k0);
                     if (k1 == k0 + 1) {
                         for (int x = 0; x < 4; ++x)
-                            W[si * 16 + x * 4 + y] = stW(((x * 4 + y) * 4 + bt[k0]) * 4 + bt[k1]);
+                            W[si * 16 + x * 4 + y] = stW(x + 4 * y, p0);
                     } else {
                         long long cw = 0; // the fixed stretch and the step into key k1 with base y
-                        for (int q = k0 + 2; q < k1; ++q) {
-                            const int a0 = __ffs(mask[q - 1]) - 1, b0 = __ffs(mask[q]) - 1;
-                            cw += stW(((a0 * 4 + b0) * 4 + bt[q - 1]) * 4 + bt[q]);
-                        }
-                        const int fa = __ffs(mask[k0 + 1]) - 1, fb = __ffs(mask[k1 - 1]) - 1;
-                        cw += stW(((fb * 4 + y) * 4 + bt[k1 - 1]) * 4 + bt[k1]);
+                        for (int q = k0 + 1; q < k1 - 1; ++q)
+                            cw += stW(oligo2(q), templ2(q));
+                        const int fa = oligo2(k0 + 1) & 3, fb = oligo2(k1 - 1) & 3;
+                        cw += stW(fb + 4 * y, templ2(k1 - 1));
                         for (int x = 0; x < 4; ++x)
-                            W[si * 16 + x * 4 + y] = stW(((x * 4 + fa) * 4 + bt[k0]) * 4 + bt[k0 + 1]) + cw;
+                            W[si * 16 + x * 4 + y] = stW(x + 4 * fa, p0) + cw;
                     }
                 }
             }
             __syncwarp();
-            long long cd = (near && (amask & 1u)) ? tmW(y * 4 + bt[0]) : LINF;
+            long long cd = (near && (amask & 1u)) ? tmW(y * 4 + tF) : LINF;
             for (int si = 0; si < mw; ++si) {
                 const bool in = near && si < m;
                 long long best = LINF;
@@ -532,7 +657,7 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
                 if (in)
                     cd = (amask >> (si + 1) & 1u) ? best : LINF;
             }
-            long long fin = cd < LINF ? cd + tmW(y * 4 + bt[L - 1]) : LINF;
+            long long fin = cd < LINF ? cd + tmW(y * 4 + tE) : LINF;
             long long o1 = __shfl_xor_sync(0xffffffffu, fin, 1);
             fin = o1 < fin ? o1 : fin;
             o1 = __shfl_xor_sync(0xffffffffu, fin, 2);
@@ -544,23 +669,23 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
                 decided = F < -kFixMargin ? 1 : (F > kFixMargin ? 0 : -1);
             }
         }
-        // sites decided the reference way (see the file comment) go to a queue, worked
-        // off below by the last block or by tm_exact_kernel, a whole block per site
+        // sites decided the reference way (see the file comment): kFew by this block below,
+        // else by tm_exact_kernel, a whole block per site
         const bool exact = run && (!dink || (near && decided < 0));
-        if (exact && y == 0)
+        if (!kFew && exact && y == 0)
             queue[atomicAdd(queue_n, 1u)] = (uint32_t)i;
         if (y == 0 && act) {
             float tm = NAN;
             uint8_t pass = 0;
             if (!bad) {
-                tm = tm32; // replaced by the exact evaluation for queued sites
-                pass = tm32 >= pd.tm_min_f;
+                tm = tm32; // replaced by the exact evaluation for the sites it decides
+                pass = tm32 >= sp.tm_min_f;
                 if (decided >= 0) { // the exact decision; the fp32 value (within 1e-3) made consistent with it
                     pass = (uint8_t)decided;
-                    if (decided && tm < pd.tm_min_f)
-                        tm = pd.tm_min_f;
-                    if (!decided && tm >= pd.tm_min_f)
-                        tm = nextafterf(pd.tm_min_f, -INFINITY);
+                    if (decided && tm < sp.tm_min_f)
+                        tm = sp.tm_min_f;
+                    if (!decided && tm >= sp.tm_min_f)
+                        tm = nextafterf(sp.tm_min_f, -INFINITY);
                 }
             }
             tm_out[i] = tm;
@@ -572,23 +697,16 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
                 pass_out[i] = 0;
         }
         __syncwarp();
-    }
-    // Tables under which only the rare ambiguous sites queue: the last block to
-    // finish evaluates them (no second launch).  queue_n[1] counts finished blocks.
-    if (last_block_exact) {
-        __shared__ int is_last;
-        __threadfence(); // this block's queue entries and results before its count
-        __syncthreads();
-        if (threadIdx.x == 0)
-            is_last = atomicAdd(queue_n + 1, 1u) == gridDim.x - 1;
-        __syncthreads();
-        if (is_last) {
-            __threadfence();
-            const uint32_t nq = *(volatile const uint32_t *)queue_n;
-            double *wmax = reinterpret_cast<double *>(seg_smem); // the segment tables are free now
-            int8_t *bt0 = &bts[0][0][0];
-            for (uint32_t e = 0; e < nq; ++e)
-                exact_site(sites, pairs, planes, contig_off, queue[e], tm_out, pass_out, bt0, wmax);
+        if (kFew && __syncthreads_or(exact)) {
+            if (threadIdx.x == 0)
+                xn = 0;
+            __syncthreads();
+            if (exact && y == 0)
+                xq[atomicAdd(&xn, 1u)] = (uint32_t)i;
+            __syncthreads();
+            const uint32_t nx = xn;
+            for (uint32_t k = 0; k < nx; ++k)
+                exact_site(sites, pairs, planes, contig_off, xq[k], tm_out, pass_out, xbt, xmax);
         }
     }
 }
@@ -721,17 +839,6 @@ __device__ __forceinline__ void tm_fast_primer(TmFastPrimer &F, const PairDev &P
     }
 }
 
-// 8 x 8 bit transpose: bit c of byte r -> bit r of byte c
-__device__ __forceinline__ uint64_t transpose8(uint64_t x)
-{
-    uint64_t t = (x ^ (x >> 7)) & 0x00AA00AA00AA00AAull;
-    x ^= t ^ (t << 7);
-    t = (x ^ (x >> 14)) & 0x0000CCCC0000CCCCull;
-    x ^= t ^ (t << 14);
-    t = (x ^ (x >> 28)) & 0x00000000F0F0F0F0ull;
-    return x ^ t ^ (t << 28);
-}
-
 __global__ void __launch_bounds__(kFastThreads, 4) tm_fast_kernel(const ah_site *__restrict__ sites, uint64_t n_arg,
                                                                   const uint64_t *__restrict__ n_dev,
                                                                   const PairDev *__restrict__ pairs, int n_pairs,
@@ -805,32 +912,23 @@ __global__ void __launch_bounds__(kFastThreads, 4) tm_fast_kernel(const ah_site 
                 atomicExch(err, kDevBounds);
             const bool act = live && !bad_rec;
             const int L = act ? fp[s.pair].pr[s.primer].L : 1;
-            uint64_t base = 0; // byte offset of the window's 16-byte boundary in the A plane
-            uint32_t o = 0, row = 0;
-            if (act) {
-                const uint64_t P = contig_off[s.contig] + s.pos;
-                const uint32_t w = (uint32_t)(P % kTileBases);
-                o = w & 3u;
-                row = w / kTileW;
-                base = 4 * (P / kTileBases * (4 * kTileWX) + (w & (kTileW - 4)));
-            }
-            const uint32_t last = min(o + (uint32_t)L, 32u) - 1u; // last word, from the boundary, of its 8 groups
+            Window d{};
+            if (act)
+                d = window_at(contig_off[s.contig] + s.pos, L);
             __syncwarp();
-            win[threadIdx.x] = base;
-            win_last[threadIdx.x] = 16u * (last >> 2);
-            win_bit[threadIdx.x] = 1u << row;
+            win[threadIdx.x] = d.base;
+            win_last[threadIdx.x] = 4u * (d.last & ~3u);
+            win_bit[threadIdx.x] = 1u << d.row;
             __syncwarp();
             const uint32_t actm = __ballot_sync(0xffffffffu, act);
-            const uint32_t g16 = 16u * (lane & 7);
-            const char *pl = reinterpret_cast<const char *>(planes + (lane >> 3) * kTileWX);
             for (int k0 = 0; k0 < 32; k0 += 8) { // eight sites' loads in flight
                 if (!((actm >> k0) & 0xffu))
                     continue;
                 uint4 w[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) { // (lanes past the window read its last group again: no other sector)
+                for (int j = 0; j < 8; ++j) {
                     const int k = 32 * warp + k0 + j;
-                    w[j] = __ldg(reinterpret_cast<const uint4 *>(pl + win[k] + min(g16, win_last[k])));
+                    w[j] = window_load(planes, lane, win[k], win_last[k]);
                 }
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
@@ -843,50 +941,14 @@ __global__ void __launch_bounds__(kFastThreads, 4) tm_fast_kernel(const ah_site 
                         got[threadIdx.x] = make_uint4(v0, v1, v2, v3);
                 }
             }
-            // ---- this lane's site: template codes, opposite each primer position (A 0, C 1, G 2, T 3)
+            // ---- this lane's site
             int cls = -1;
             if (act) {
-                uint32_t extra[4] = {0, 0, 0, 0}; // words 32 .. 34 of a long window that starts off the boundary, per plane
-                if (o + L > 32) {
-                    const uint32_t *p = planes + (base >> 2) + 32;
-#pragma unroll
-                    for (int x = 0; x < 4; ++x)
-#pragma unroll
-                        for (int j = 0; j < 3; ++j)
-                            if (32u + j < o + L)
-                                extra[x] |= ((__ldg(p + x * kTileWX + j) >> row) & 1u) << j;
-                }
-                // words outside [o, o + L) cleared; every position has exactly one plane set, or the window is bad
                 const uint4 b4 = got[threadIdx.x];
                 const uint32_t B[4] = {b4.x, b4.y, b4.z, b4.w};
-                int set = __popc(extra[0] | extra[1] | extra[2] | extra[3]);
-                uint64_t rows = 0; // byte 2 j + h: bit g = bit h of the code at word 4 g + j
-#pragma unroll
-                for (uint32_t j = 0; j < 4; ++j) {
-                    // groups whose word 4 g + j is at most `last`: all before last's, and its own up to last
-                    uint32_t keep = (1u << ((last >> 2) + (j <= (last & 3u)))) - 1u;
-                    if (j < o)
-                        keep &= ~1u;
-                    const uint32_t v = B[j] & keep * 0x01010101u;
-                    set += __popc(v);
-                    const uint32_t lo8 = ((v >> 8) | (v >> 24)) & 0xffu, hi8 = ((v >> 16) | (v >> 24)) & 0xffu;
-                    rows |= (uint64_t)(lo8 | hi8 << 8) << (16 * j);
-                }
-                uint64_t code = transpose8(rows) >> (2 * o);
-                if (o) { // (o = 0: nothing past word 31)
-                    const uint64_t elo = extra[1] | extra[3], ehi = extra[2] | extra[3];
-#pragma unroll
-                    for (int j = 0; j < 3; ++j)
-                        code |= ((elo >> j & 1u) | (ehi >> j & 1u) << 1) << (2 * (32 + j) - 2 * o) % 64;
-                }
-                if (s.strand == 0) { // the complement of the window base at q
-                    code = ~code;
-                } else { // the window base at L - 1 - q
-                    code = __brevll(code) >> (64 - 2 * L);
-                    code = (code >> 1 & 0x5555555555555555ull) | (code & 0x5555555555555555ull) << 1;
-                }
-                codes[local] = code;
-                if (set == L)
+                bool ok;
+                codes[local] = window_codes(planes, d, L, s.strand, B, &ok);
+                if (ok)
                     cls = s.pair * 2 + s.primer;
             }
             if (live && cls < 0) { // a letter other than A, C, G, T, or a record outside its bounds
@@ -1333,7 +1395,8 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
         AH_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const int most = AH_MAX_PAIRS_PER_SCAN * (int)sizeof(TmPairS) + kTmStageD * (int)sizeof(TmPairD) +
                          kTmWarps * 8 * (AH_MAX_PRIMER_LEN - 1) * 16 * (int)sizeof(float2);
-        AH_CUDA(cudaFuncSetAttribute(tm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        AH_CUDA(cudaFuncSetAttribute(tm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        AH_CUDA(cudaFuncSetAttribute(tm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         const int most_fast = AH_MAX_PAIRS_PER_SCAN * (int)sizeof(TmFastPair);
         AH_CUDA(cudaFuncSetAttribute(tm_fast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most_fast));
         for (int j = 1; j <= AH_MAX_PAIRS_PER_SCAN; ++j) {
@@ -1341,7 +1404,7 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
                                                                   j * sizeof(TmFastPair)));
             fast_blocks[j] = std::max(1, fast_blocks[j]);
         }
-        AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tm_bps, tm_kernel, 32 * kTmWarps, most));
+        AH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tm_bps, tm_kernel<true>, 32 * kTmWarps, most));
         tm_bps = std::max(1, tm_bps);
         // AH_TM_FAST_BLOCKS=n: at most n blocks of the thread-per-site kernel per SM (profiling aid)
         if (const char *e = getenv("AH_TM_FAST_BLOCKS"))
@@ -1350,15 +1413,15 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
                     b = std::min(b, atoi(e));
         cached_dev = dev;
     }
-    // queue length, finished blocks, deferred sites
-    if (!n_dev)
+    constexpr uint64_t kFastMinSites = 24576;
+    const bool fast = few_exact && n >= kFastMinSites;
+    if (!n_dev && (fast || !few_exact)) // queue length, deferred sites
         AH_CUDA(cudaMemsetAsync(queue_n, 0, 2 * sizeof(uint64_t), s));
-    // Few sites (a latency-bound launch): the four-lane kernel alone finishes first
-    // (measured on GB300 for 6,253 sites: 33 us, against 36 + 27 us for the two
-    // kernels below); many sites: one thread per site (6x the four-lane rate on
-    // 3.2 M sites).
-    constexpr uint64_t kFastMinSites = 32768;
-    if (few_exact && n >= kFastMinSites) {
+    // Few sites (a latency-bound launch): the four-lane kernel alone finishes first; many
+    // sites: one thread per site (6x the four-lane rate on 3.2 M sites).  On a GB300:
+    // 16,384 sites 22 us against 15 + 14 for the two kernels below (2 when no site is
+    // deferred), 24,000 sites 25 against 15 + 14, 32,767 sites 44 against 15 + 14.
+    if (fast) {
         // every site in one thread; those near tm_min go to the four-lane kernel below
         uint32_t *defer = queue + n;
         unsigned long long *defer_n = reinterpret_cast<unsigned long long *>(queue_n) + 1;
@@ -1369,18 +1432,17 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
         AH_CUDA(cudaGetLastError());
         // deferred sites (few; their count stays on the device): a persistent grid
         const uint64_t tb = std::min<uint64_t>((n + 8 * kTmWarps - 1) / (8 * kTmWarps), (uint64_t)sms * tm_bps);
-        launch_chained(tm_kernel, (unsigned)tb, 32 * kTmWarps, smem, s, sites, n,
+        launch_chained(tm_kernel<true>, (unsigned)tb, 32 * kTmWarps, smem, s, sites, n,
                        reinterpret_cast<const uint64_t *>(defer_n), pairs_d, n_pairs, planes, contig_off, tm_out, pass_out,
-                       queue, queue_n, seg_max, 1, err, defer);
+                       queue, queue_n, seg_max, err, defer);
         return;
     }
     const uint64_t per_block = 8ull * kTmWarps; // sites per block per pass
     uint64_t blocks = (n + per_block - 1) / per_block;
     if (blocks > 65535)
         blocks = 65535;
-    launch_chained(tm_kernel, (unsigned)blocks, 32 * kTmWarps, smem, s, sites, n, n_dev, pairs_d,
-                   n_pairs, planes, contig_off, tm_out, pass_out, queue, queue_n, seg_max, few_exact ? 1 : 0, err,
-                   nullptr);
+    launch_chained(few_exact ? tm_kernel<true> : tm_kernel<false>, (unsigned)blocks, 32 * kTmWarps, smem, s, sites, n,
+                   n_dev, pairs_d, n_pairs, planes, contig_off, tm_out, pass_out, queue, queue_n, seg_max, err, nullptr);
     if (few_exact)
         return;
     tm_exact_kernel<<<(unsigned)sms, kExactThreads, 0, s>>>(sites, pairs_d, planes, contig_off, queue, queue_n,
