@@ -886,8 +886,8 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
         launch_pair_count(sites, ns_max, F + kFlagSites, filt, pd, counts, nullptr, st);
         exclusive_scan_u64_dev(counts, offs, ns_max, F + kFlagSites, 0, F + kFlagAux, na_max, F + kFlagAmps,
                                F + kFlagRedo, kRedoAmps, st);
-        launch_pair_write(sites, ns_max, F + kFlagSites, filt, pd, offs, amps, len, na_max, F + kFlagRedo, kRedoAmps,
-                          st);
+        launch_pair_write(sites, ns_max, F + kFlagSites, filt, pd, counts, offs, amps, len, na_max, F + kFlagRedo,
+                          kRedoAmps, st);
     }
     {
         Stage sg(c, "fetch", st, 2);
@@ -1006,7 +1006,7 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         qoff = direct_or_scratch(c, "run_qoff", o->seq_offsets, o->seq_offsets ? o->amplicons_cap + 1 : 0, na + 1);
         if (na) {
             Stage sg(c, "pair", st, 1);
-            launch_pair_write(sites, ns, nullptr, filt, pd, offs, amps, nullptr, na, nullptr, 0, st);
+            launch_pair_write(sites, ns, nullptr, filt, pd, counts, offs, amps, nullptr, na, nullptr, 0, st);
         }
         uint64_t *len = (uint64_t *)scratch(c, "fetch_len", (na + 1) * sizeof(uint64_t));
         size_t tb2 = scan_u64_temp_bytes(na + 1);
@@ -1222,7 +1222,7 @@ void group_device(ah_ctx *c, const GenomeSet &gs, uint32_t pid, int k, const std
     ah_amplicon *amps = (ah_amplicon *)scratch(c, "serve_amps", std::max<uint64_t>(na, 1) * sizeof(ah_amplicon));
     if (na) {
         Stage sg(c, "pair", st, 1);
-        launch_pair_write(sites, ns, nullptr, nullptr, pd, offs, amps, nullptr, na, nullptr, 0, st);
+        launch_pair_write(sites, ns, nullptr, nullptr, pd, counts, offs, amps, nullptr, na, nullptr, 0, st);
     }
     // staging layout: sites, amplicons, pass flags
     const size_t sb = ns * sizeof(ah_site), ab = na * sizeof(ah_amplicon);
@@ -2594,7 +2594,7 @@ ah_status ah_pair(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t
         ah_amplicon *dst = out_buf(c, "amp_out", out, total);
         {
             Stage sg(c, "pair", st, 1);
-            launch_pair_write(s, n, nullptr, ps, pd, offs, dst, nullptr, total, nullptr, 0, st);
+            launch_pair_write(s, n, nullptr, ps, pd, counts, offs, dst, nullptr, total, nullptr, 0, st);
         }
         out_finish(out, dst, total, st);
         AH_CUDA(cudaStreamSynchronize(st));

@@ -342,11 +342,12 @@ void exclusive_scan_u64_dev(const uint64_t *in, uint64_t *out, uint64_t n, const
                             uint64_t *tot, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit,
                             cudaStream_t s);
 // skip: optional device word; the kernel writes nothing when (*skip & skip_bit) != 0.
+// counts, offsets: launch_pair_count's results and their exclusive scan.
 // len (may be null): the amplicons' lengths as launch_fetch_lengths gives them, for sites
 // that a scan found.
 void launch_pair_write(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, const uint64_t *offsets, ah_amplicon *out, uint64_t *len, uint64_t cap,
-                       const uint64_t *skip, uint64_t skip_bit, cudaStream_t s);
+                       const PairDev *pairs_d, const uint64_t *counts, const uint64_t *offsets, ah_amplicon *out,
+                       uint64_t *len, uint64_t cap, const uint64_t *skip, uint64_t skip_bit, cudaStream_t s);
 
 // amplitype.cu: sequence variants and amplitypes.  Two hash tables of `size`
 // slots: variants (and then amplitypes) with the first index seen, and

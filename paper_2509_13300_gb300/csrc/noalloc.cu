@@ -167,7 +167,7 @@ extern "C" ah_status ah_pair_noalloc(const int32_t *pair_windows, uint32_t n_pai
         if (total > cap)
             return AH_ERR_OVERFLOW;
         if (total) {
-            ah::launch_pair_write(sites, n, nullptr, pass, pd, offs, out, nullptr, total, nullptr, 0, st);
+            ah::launch_pair_write(sites, n, nullptr, pass, pd, counts, offs, out, nullptr, total, nullptr, 0, st);
             AH_CUDA(cudaStreamSynchronize(st));
         }
     } catch (const ah::Error &e) {

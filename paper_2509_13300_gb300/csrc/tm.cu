@@ -624,37 +624,40 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
                 return staged ? sd.tm[idx] : fix_weight(pd.term_dH_d[idx], pd.term_dS_d[idx], pd.thr);
             };
             __syncwarp();
-            if (near) {
-                for (int si = 0; si < m; ++si) {
-                    const int k0 = key[si], k1 = key[si + 1], p0 = templ2(k0);
-                    if (k1 == k0 + 1) {
-                        for (int x = 0; x < 4; ++x)
-                            W[si * 16 + x * 4 + y] = stW(x + 4 * y, p0);
-                    } else {
-                        long long cw = 0; // the fixed stretch and the step into key k1 with base y
-                        for (int q = k0 + 1; q < k1 - 1; ++q)
-                            cw += stW(oligo2(q), templ2(q));
+            for (int sb = 0; sb < mw; sb += 4) { // as the fp32 tables above
+                long long cw = 0;
+                if (near && sb + y < m) {
+                    const int k1 = key[sb + y + 1];
+                    for (int q = key[sb + y] + 1; q < k1 - 1; ++q)
+                        cw += stW(oligo2(q), templ2(q));
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const long long uw = __shfl_sync(0xffffffffu, cw, g0 + u);
+                    const int si = sb + u;
+                    if (near && si < m) {
+                        const int k0 = key[si], k1 = key[si + 1], p0 = templ2(k0);
+                        const bool apart = k1 > k0 + 1;
                         const int fa = oligo2(k0 + 1) & 3, fb = oligo2(k1 - 1) & 3;
-                        cw += stW(fb + 4 * y, templ2(k1 - 1));
+                        const long long into = apart ? stW(fb + 4 * y, templ2(k1 - 1)) + uw : 0;
+                        const int to = apart ? fa : y;
+#pragma unroll
                         for (int x = 0; x < 4; ++x)
-                            W[si * 16 + x * 4 + y] = stW(x + 4 * fa, p0) + cw;
+                            W[si * 16 + x * 4 + y] = stW(x + 4 * to, p0) + into;
                     }
                 }
             }
             __syncwarp();
             long long cd = (near && (amask & 1u)) ? tmW(y * 4 + tF) : LINF;
             for (int si = 0; si < mw; ++si) {
-                const bool in = near && si < m;
                 long long best = LINF;
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
                     const long long cx = __shfl_sync(0xffffffffu, cd, g0 + x);
-                    if (in) {
-                        const long long v = cx + W[si * 16 + x * 4 + y];
-                        best = v < best ? v : best;
-                    }
+                    const long long v = cx < LINF ? cx + W[si * 16 + x * 4 + y] : LINF;
+                    best = v < best ? v : best;
                 }
-                if (in)
+                if (near && si < m)
                     cd = (amask >> (si + 1) & 1u) ? best : LINF;
             }
             long long fin = cd < LINF ? cd + tmW(y * 4 + tE) : LINF;
