@@ -776,7 +776,7 @@ void sort_decode(ah_ctx *c, const GenomeSet &gs, uint32_t n_pairs, const uint64_
     const int end_bit = 10 + pbits + bit_length(n_pairs - 1);
     if (count <= kSmallSort) { // one launch: rank sort and decode
         Stage sg(c, "sort", st, 1);
-        launch_rank_sort_decode(keys, count, nullptr, end_bit - 8 <= 32, pbits, gs.contig_off, gs.n_contigs,
+        launch_rank_sort_decode(keys, count, nullptr, end_bit, pbits, gs.contig_off, gs.n_contigs,
                                 gs.contig_genome, dst, nullptr, nullptr, st);
         return;
     }
@@ -873,7 +873,7 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
         AH_CUDA(cudaEventRecord(scan_done, st));
     {
         Stage sg(c, "sort", st, 1);
-        launch_rank_sort_decode(keys, ns_max, F + kFlagCounter, end_bit - 8 <= 32, pbits, gs.contig_off,
+        launch_rank_sort_decode(keys, ns_max, F + kFlagCounter, end_bit, pbits, gs.contig_off,
                                 gs.n_contigs, gs.contig_genome, sites, F + kFlagSites, F + kFlagRedo, st);
     }
     {

@@ -198,9 +198,9 @@ void launch_decode_keys(const uint64_t *keys, uint64_t n, int pbits, const uint6
 // (one-synchronisation path): the count is *n_dev and n is the largest count
 // the launch was sized for; above it the kernel writes *n_out = 0, sets
 // kRedoSites in *redo and sorts nothing.  Otherwise *n_out = the count.
-// key32: the sort bits [8, end_bit) fit in 32 bits.
+// end_bit: bits of the largest key.
 constexpr uint64_t kSmallSort = 16384;
-void launch_rank_sort_decode(const uint64_t *keys, uint64_t n, const uint64_t *n_dev, bool key32, int pbits,
+void launch_rank_sort_decode(const uint64_t *keys, uint64_t n, const uint64_t *n_dev, int end_bit, int pbits,
                              const uint64_t *contig_off, uint32_t n_contigs, const uint32_t *contig_genome,
                              ah_site *out, uint64_t *n_out, uint64_t *redo, cudaStream_t s);
 

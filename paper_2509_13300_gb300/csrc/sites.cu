@@ -102,215 +102,182 @@ void launch_decode_keys(const uint64_t *keys, uint64_t n, int pbits, const uint6
 // ---------------------------------------------------------------------------
 // Small-count path: rank sort.  Site keys are distinct in their bits
 // [8, end_bit) -- (pair, flat position, primer, strand) names one site -- so
-// a key's place in canonical order is the number of keys below it.  A block
-// of kRankWarps warps takes 32 * kRankQ keys ("queries", kRankQ per lane);
-// each of its warps counts, for every query, the smaller keys in one
-// kRankWarps-th of the whole key array staged in shared memory; warp 0 adds
-// the partial counts, decodes its keys and writes each record at its rank.
-// n^2 compares spread over the whole GPU in one launch: a few microseconds
-// for thousands of sites, where a one-block radix sort or a series of
-// device-wide sort launches takes tens.
+// a key's place in canonical order is the number of keys below it.  Every block
+// sorts all keys into kRankBuckets ranges of equal width in shared memory (count,
+// scan, scatter; up to 1,024 keys stay one range), then ranks its own share of
+// them, a warp per key against the keys of its range, decodes them and writes each
+// record at its rank: no block waits for another, one launch.
+// Bound: latency (the count and the scatter are one shared-memory atomic per key
+// and thread).  Measured on a GB300, against the former n^2 compares of all keys
+// over the GPU: 6,000 sites @A@; 10,000 sites of 33 sort bits @B@; 20 sites @C@.
+// (All keys in one range: every key is compared with all, a third of the former
+// compares' instructions.)
 // ---------------------------------------------------------------------------
 namespace ah {
 namespace {
 
-constexpr int kRankWarps = 8;
-constexpr int kRankQ = 2;
+constexpr int kRankThreads = 512;
+constexpr int kRankKeys = 16;    // keys of a thread held in registers; more are read twice
+constexpr int kRankBuckets = 1024;
 constexpr uint32_t kRankStageContigs = 4096; // contig offset tables up to this size are staged in shared memory
 
-template <typename K> struct Vec16;
-template <> struct Vec16<uint32_t> {
-    using T = uint4;
-    static constexpr int V = 4;
-    __device__ static void get(const T &x, uint32_t (&e)[4]) { e[0] = x.x; e[1] = x.y; e[2] = x.z; e[3] = x.w; }
-};
-template <> struct Vec16<uint64_t> {
-    using T = ulonglong2;
-    static constexpr int V = 2;
-    __device__ static void get(const T &x, uint64_t (&e)[2]) { e[0] = x.x; e[1] = x.y; }
-};
-
-// K: uint32_t when the sort bits [8, end_bit) fit in 32 bits, else uint64_t.
-// Shared memory: the keys (rounded up to 16 bytes), the partial counts, and
-// the contig offsets when stage_contigs.
-template <typename K>
-__global__ void __launch_bounds__(32 * kRankWarps)
-    rank_sort_decode_kernel(const uint64_t *keys, uint64_t n_arg, const uint64_t *n_dev, int pbits, const uint64_t *__restrict__ contig_off, uint32_t n_contigs,
-                            bool stage_contigs, const uint32_t *__restrict__ contig_genome, ah_site *out, uint64_t *n_out,
-                            uint64_t *redo)
+// Shared memory: the keys by range, then the contig offsets when stage_contigs.
+__global__ void __launch_bounds__(kRankThreads, 2)
+    rank_sort_decode_kernel(const uint64_t *keys, uint64_t n_arg, const uint64_t *n_dev, int shift, int pbits,
+                            const uint64_t *__restrict__ contig_off, uint32_t n_contigs, bool stage_contigs,
+                            const uint32_t *__restrict__ contig_genome, ah_site *out, uint64_t *n_out, uint64_t *redo)
 {
+    extern __shared__ __align__(16) uint64_t rank_smem[];
+    __shared__ uint32_t end[kRankBuckets]; // keys of a range; then where it ends in cand
+    __shared__ uint32_t wsum[kRankThreads / 32];
+    __shared__ uint64_t query[kRankThreads];
+    __shared__ uint32_t rank[kRankThreads];
+    uint64_t *cand = rank_smem, *coff = rank_smem + n_arg;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     chain_start();
+    if (stage_contigs) // (no kernel of the chain writes them)
+        for (uint32_t i = tid; i <= n_contigs; i += kRankThreads)
+            coff[i] = __ldg(contig_off + i);
+    for (int i = tid; i < kRankBuckets; i += kRankThreads)
+        end[i] = 0;
     chain_wait();
-    using VT = Vec16<K>;
-    constexpr int V = VT::V;
     const uint64_t n64 = n_dev ? *(const volatile uint64_t *)n_dev : n_arg;
     if (n64 > n_arg) { // device count above the launch's size: the host redoes this step
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (blockIdx.x == 0 && tid == 0) {
             *n_out = 0;
             atomicOr((unsigned long long *)redo, (unsigned long long)kRedoSites);
         }
         return;
     }
     const uint32_t n = (uint32_t)n64;
-    if (n_out && blockIdx.x == 0 && threadIdx.x == 0)
+    if (n_out && blockIdx.x == 0 && tid == 0)
         *n_out = n;
-    const uint32_t q0 = blockIdx.x * 32u * kRankQ;
+    const uint32_t share = (n + gridDim.x - 1) / gridDim.x, q0 = blockIdx.x * share;
     if (q0 >= n)
         return;
-    extern __shared__ __align__(16) unsigned char rank_smem[];
-    const uint32_t nv = (n + V - 1) / V;
-    K *cand = reinterpret_cast<K *>(rank_smem);
-    uint32_t *part = reinterpret_cast<uint32_t *>(rank_smem + (size_t)nv * 16);
-    uint64_t *coff = reinterpret_cast<uint64_t *>(rank_smem + (size_t)nv * 16 + kRankWarps * 32 * kRankQ * 4);
-    // the block's own queries, full keys, loaded first so their latency overlaps the staging
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint64_t qkey[kRankQ];
+    const uint32_t q1 = min(n, q0 + share);
+    if ((uint32_t)tid < q1 - q0) // the block's first queries
+        query[tid] = keys[q0 + tid];
+    const bool flat = n <= kRankBuckets; // few keys: one range
+    if (flat) {
+        for (uint32_t i = tid; i < n; i += kRankThreads)
+            cand[i] = keys[i];
+    } else {
+        // count
+        uint64_t k[kRankKeys];
 #pragma unroll
-    for (int j = 0; j < kRankQ; ++j) {
-        const uint32_t i = q0 + lane + 32u * j;
-        qkey[j] = i < n ? keys[i] : 0;
-    }
-    // stage every key (sort bits only): two keys per 16-byte load, eight loads in flight per thread
-    {
-        const uint32_t pairs = n / 2; // keys is 16-byte aligned (a scratch allocation)
-        const ulonglong2 *k2 = reinterpret_cast<const ulonglong2 *>(keys);
-        for (uint32_t b = threadIdx.x; b < pairs; b += 8 * blockDim.x) {
-            ulonglong2 x[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t p = b + u * blockDim.x;
-                x[u] = p < pairs ? k2[p] : make_ulonglong2(~0ull, ~0ull);
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t p = b + u * blockDim.x;
-                if (p < pairs) {
-                    cand[2 * p] = (K)(x[u].x >> 8);
-                    cand[2 * p + 1] = (K)(x[u].y >> 8);
-                }
-            }
+        for (int u = 0; u < kRankKeys; ++u) {
+            const uint32_t i = tid + u * kRankThreads;
+            k[u] = i < n ? keys[i] : 0;
         }
-        for (uint32_t i = 2 * pairs + threadIdx.x; i < nv * V; i += blockDim.x)
-            cand[i] = i < n ? (K)(keys[i] >> 8) : (K)~(K)0; // odd tail and padding (never below a key)
-    }
-    if (stage_contigs) { // n_contigs + 1 <= kRankStageContigs: at most 8 vector loads per thread, all in flight
-        const uint32_t m = n_contigs + 1, m2 = m / 2;
-        const ulonglong2 *c2 = reinterpret_cast<const ulonglong2 *>(contig_off); // 16-byte aligned (checked on the host)
-        ulonglong2 x[8];
+        __syncthreads();
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const uint32_t p = threadIdx.x + u * blockDim.x;
-            if (p < m2)
-                x[u] = __ldg(c2 + p);
-        }
+        for (int u = 0; u < kRankKeys; ++u)
+            if (tid + u * kRankThreads < n)
+                atomicAdd(&end[k[u] >> shift], 1u);
+        for (uint32_t i = tid + kRankKeys * kRankThreads; i < n; i += kRankThreads)
+            atomicAdd(&end[keys[i] >> shift], 1u);
+        __syncthreads();
+        // exclusive scan: each thread its kRankBuckets / kRankThreads = 2 ranges
+        static_assert(kRankBuckets == 2 * kRankThreads, "two ranges per thread");
+        const uint32_t c0 = end[2 * tid], c1 = end[2 * tid + 1];
+        uint32_t incl = c0 + c1;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const uint32_t p = threadIdx.x + u * blockDim.x;
-            if (p < m2) {
-                coff[2 * p] = x[u].x;
-                coff[2 * p + 1] = x[u].y;
-            }
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d)
+                incl += y;
         }
-        if ((m & 1) && threadIdx.x == 0)
-            coff[m - 1] = __ldg(contig_off + m - 1);
+        if (lane == 31)
+            wsum[warp] = incl;
+        __syncthreads();
+        uint32_t before = incl - c0 - c1;
+        for (int w = 0; w < warp; ++w)
+            before += wsum[w];
+        end[2 * tid] = before;
+        end[2 * tid + 1] = before + c0;
+        __syncthreads();
+        // scatter: `end` moves from a range's start to its end
+#pragma unroll
+        for (int u = 0; u < kRankKeys; ++u)
+            if (tid + u * kRankThreads < n)
+                cand[atomicAdd(&end[k[u] >> shift], 1u)] = k[u];
+        for (uint32_t i = tid + kRankKeys * kRankThreads; i < n; i += kRankThreads) {
+            const uint64_t key = keys[i];
+            cand[atomicAdd(&end[key >> shift], 1u)] = key;
+        }
     }
     __syncthreads();
-    K q[kRankQ];
-    uint32_t r[kRankQ];
-#pragma unroll
-    for (int j = 0; j < kRankQ; ++j) {
-        q[j] = (K)(qkey[j] >> 8);
-        r[j] = 0;
-    }
-    const uint32_t v0 = (uint32_t)((uint64_t)nv * w / kRankWarps);
-    const uint32_t v1 = (uint32_t)((uint64_t)nv * (w + 1) / kRankWarps);
-    const typename VT::T *cv = reinterpret_cast<const typename VT::T *>(cand);
-#pragma unroll 4
-    for (uint32_t v = v0; v < v1; ++v) {
-        K e[V];
-        VT::get(cv[v], e);
-#pragma unroll
-        for (int t = 0; t < V; ++t)
-#pragma unroll
-            for (int j = 0; j < kRankQ; ++j)
-                r[j] += e[t] < q[j] ? 1u : 0u;
-    }
-#pragma unroll
-    for (int j = 0; j < kRankQ; ++j)
-        part[w * 32 * kRankQ + lane + 32 * j] = r[j];
-    __syncthreads();
-    if (w != 0)
-        return;
-    const uint64_t *co = stage_contigs ? coff : contig_off;
-#pragma unroll
-    for (int j = 0; j < kRankQ; ++j) {
-        const uint32_t i = q0 + lane + 32u * j;
-        if (i >= n)
-            break;
-        uint32_t rank = 0;
-#pragma unroll
-        for (int ww = 0; ww < kRankWarps; ++ww)
-            rank += part[ww * 32 * kRankQ + lane + 32 * j];
-        const uint64_t key = qkey[j];
-        const uint64_t pp = key >> 10;
-        const uint64_t P = pp & ((1ull << pbits) - 1);
-        uint32_t lo = 0, hi = n_contigs;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (co[mid] <= P)
-                lo = mid;
-            else
-                hi = mid;
+    // the block's keys, kRankThreads at a time
+    for (uint32_t qb = q0; qb < q1; qb += kRankThreads) {
+        const uint32_t m = min(q1 - qb, (uint32_t)kRankThreads);
+        if (qb > q0) { // (the first ones are there)
+            __syncthreads();
+            if ((uint32_t)tid < m)
+                query[tid] = keys[qb + tid];
+            __syncthreads();
         }
-        ah_site s;
-        s.genome = __ldg(contig_genome + lo);
-        s.contig = lo;
-        s.pos = (uint32_t)(P - co[lo]);
-        s.primer = (uint8_t)((key >> 9) & 1);
-        s.strand = (uint8_t)((key >> 8) & 1);
-        s.mm = (uint8_t)(key & 0xff);
-        s.pair = (uint8_t)(pp >> pbits);
-        out[rank] = s;
+        for (uint32_t j = warp; j < m; j += kRankThreads / 32) {
+            const uint64_t key = query[j];
+            const uint32_t b = (uint32_t)(key >> shift);
+            const uint32_t first = flat || !b ? 0u : end[b - 1], last = flat ? n : end[b];
+            uint32_t below = 0;
+            for (uint32_t i = first + lane; i < last; i += 32)
+                below += cand[i] < key ? 1u : 0u;
+            below = __reduce_add_sync(0xffffffffu, below);
+            if (lane == 0)
+                rank[j] = first + below;
+        }
+        __syncthreads();
+        if ((uint32_t)tid < m) {
+            const uint64_t key = query[tid], pp = key >> 10;
+            const uint64_t P = pp & ((1ull << pbits) - 1);
+            const uint64_t *co = stage_contigs ? coff : contig_off;
+            uint32_t lo = 0, hi = n_contigs;
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (co[mid] <= P)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            ah_site s;
+            s.genome = __ldg(contig_genome + lo);
+            s.contig = lo;
+            s.pos = (uint32_t)(P - co[lo]);
+            s.primer = (uint8_t)((key >> 9) & 1);
+            s.strand = (uint8_t)((key >> 8) & 1);
+            s.mm = (uint8_t)(key & 0xff);
+            s.pair = (uint8_t)(pp >> pbits);
+            out[rank[tid]] = s;
+        }
     }
-}
-
-template <typename K>
-void run_rank_sort(const uint64_t *keys, uint64_t n, const uint64_t *n_dev, int pbits, const uint64_t *contig_off,
-                   uint32_t n_contigs, const uint32_t *contig_genome, ah_site *out, uint64_t *n_out, uint64_t *redo,
-                   cudaStream_t s)
-{
-    // staging reads the offsets with 16-byte loads, 8 per thread of 256
-    const bool stage = n_contigs + 1 <= kRankStageContigs && reinterpret_cast<uintptr_t>(contig_off) % 16 == 0;
-    const size_t smem = (size_t)((n + Vec16<K>::V - 1) / Vec16<K>::V) * 16 + kRankWarps * 32 * kRankQ * 4 +
-                        (stage ? (size_t)(n_contigs + 1) * 8 : 0);
-    static int attr_dev = -1; // one instance per key type: opt in to the largest size once per device
-    int dev = 0;
-    AH_CUDA(cudaGetDevice(&dev));
-    if (dev != attr_dev) {
-        const size_t most = kSmallSort * sizeof(K) + kRankWarps * 32 * kRankQ * 4 + kRankStageContigs * 8;
-        AH_CUDA(cudaFuncSetAttribute(rank_sort_decode_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)most));
-        attr_dev = dev;
-    }
-    const unsigned blocks = (unsigned)((n + 32 * kRankQ - 1) / (32 * kRankQ));
-    launch_chained(rank_sort_decode_kernel<K>, blocks, 32 * kRankWarps, smem, s, keys, n, n_dev,
-                   pbits, contig_off, n_contigs, stage, contig_genome, out, n_out, redo);
 }
 
 } // namespace
 
-void launch_rank_sort_decode(const uint64_t *keys, uint64_t n, const uint64_t *n_dev, bool key32, int pbits,
+void launch_rank_sort_decode(const uint64_t *keys, uint64_t n, const uint64_t *n_dev, int end_bit, int pbits,
                              const uint64_t *contig_off, uint32_t n_contigs, const uint32_t *contig_genome,
                              ah_site *out, uint64_t *n_out, uint64_t *redo, cudaStream_t s)
 {
     if (n == 0 || n > kSmallSort)
         throw Error(AH_ERR_ARG, "rank sort: count outside 1..16384");
-    if (reinterpret_cast<uintptr_t>(keys) % 16 != 0)
-        throw Error(AH_ERR_ARG, "rank sort: keys not 16-byte aligned");
-    if (key32)
-        run_rank_sort<uint32_t>(keys, n, n_dev, pbits, contig_off, n_contigs, contig_genome, out, n_out, redo, s);
-    else
-        run_rank_sort<uint64_t>(keys, n, n_dev, pbits, contig_off, n_contigs, contig_genome, out, n_out, redo, s);
+    const bool stage = n_contigs + 1 <= kRankStageContigs;
+    const size_t smem = (n + (stage ? n_contigs + 1 : 0)) * sizeof(uint64_t);
+    static int attr_dev = -1, sms = 148; // opt in to the largest size once per device
+    int dev = 0;
+    AH_CUDA(cudaGetDevice(&dev));
+    if (dev != attr_dev) {
+        AH_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        AH_CUDA(cudaFuncSetAttribute(rank_sort_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)((kSmallSort + kRankStageContigs) * sizeof(uint64_t))));
+        attr_dev = dev;
+    }
+    // a block per SM, but at least a key per warp
+    const unsigned blocks = (unsigned)std::min<uint64_t>((uint64_t)sms, (n + kRankThreads / 32 - 1) / (kRankThreads / 32));
+    const int shift = end_bit > 10 + 8 ? end_bit - 10 : 8; // kRankBuckets ranges of the bits below end_bit
+    launch_chained(rank_sort_decode_kernel, blocks, kRankThreads, smem, s, keys, n, n_dev, shift, pbits, contig_off,
+                   n_contigs, stage, contig_genome, out, n_out, redo);
 }
 
 } // namespace ah

@@ -228,6 +228,9 @@ __device__ __forceinline__ long long fix_weight(double dH, double dS, double thr
 }
 constexpr int kTmStageD = 4;
 constexpr unsigned kTmEarlyBlocks = 304; // two per SM
+// Entries from one site's segment tables to the next: four more than the tables, so that the
+// eight sites of a warp, which read the same entry of their tables, meet different banks.
+__host__ __device__ constexpr int tm_group_stride(int seg_max) { return seg_max * 16 + 4; }
 
 // 8 x 8 bit transpose: bit c of byte r -> bit r of byte c
 __device__ __forceinline__ uint64_t transpose8(uint64_t x)
@@ -344,7 +347,7 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
     __shared__ int8_t xbt[AH_MAX_PRIMER_LEN];
     __shared__ double xmax[kTmWarps];
     // dynamic: [n_pairs] TmPairS, [n_pairs <= kTmStageD ? n_pairs : 0] TmPairD,
-    // then [kTmWarps * 8 sites][seg_max][16] segment tables
+    // then per site of the block its [seg_max][16] segment tables, tm_group_stride apart
     extern __shared__ __align__(16) unsigned char tm_smem[];
     TmPairS *ps = reinterpret_cast<TmPairS *>(tm_smem);
     chain_start();
@@ -483,7 +486,7 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
         const int mw = (int)__reduce_max_sync(0xffffffffu, (uint32_t)m);
         auto oligo2 = [&](int q) { return (int)(first >> (2 * q)) & 15; }; // fixed bases at q and q + 1
         auto templ2 = [&](int q) { return (int)(code >> (2 * q)) & 15; };  // template bases at q and q + 1
-        float2 *E = seg_smem + (size_t)(warp * 8 + g) * seg_max * 16;
+        float2 *E = seg_smem + (warp * 8 + g) * tm_group_stride(seg_max);
         for (int sb = 0; sb < mw; sb += 4) {
             // the stacks between two fixed bases: lane y sums those of segment sb + y
             float cH = 0.f, cS = 0.f;
@@ -1392,12 +1395,12 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
     int dev = 0;
     AH_CUDA(cudaGetDevice(&dev));
     const size_t smem = (size_t)n_pairs * sizeof(TmPairS) + (size_t)(n_pairs <= kTmStageD ? n_pairs : 0) * sizeof(TmPairD) +
-                        (size_t)kTmWarps * 8 * seg_max * 16 * sizeof(float2);
+                        kTmWarps * 8 * tm_group_stride(seg_max) * sizeof(float2);
     const size_t fast_smem = (size_t)n_pairs * sizeof(TmFastPair);
     if (dev != cached_dev) {
         AH_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const int most = AH_MAX_PAIRS_PER_SCAN * (int)sizeof(TmPairS) + kTmStageD * (int)sizeof(TmPairD) +
-                         kTmWarps * 8 * (AH_MAX_PRIMER_LEN - 1) * 16 * (int)sizeof(float2);
+                         kTmWarps * 8 * tm_group_stride(AH_MAX_PRIMER_LEN - 1) * (int)sizeof(float2);
         AH_CUDA(cudaFuncSetAttribute(tm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         AH_CUDA(cudaFuncSetAttribute(tm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         const int most_fast = AH_MAX_PAIRS_PER_SCAN * (int)sizeof(TmFastPair);

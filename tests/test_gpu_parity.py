@@ -1435,3 +1435,36 @@ def test_thread_per_site_tm_over_window_offsets_and_primer_mixes(ctx, lengths, c
     assert np.array_equal(np.isnan(tm), nan)
     assert np.abs(tm[~nan].astype(np.float64) - want[~nan]).max() <= TM_TOL
     assert np.array_equal(ps, passed)
+
+
+@pytest.mark.parametrize("n_sites", [1, 31, 513, 8192, 8193, 16384])
+@pytest.mark.parametrize("spread", [False, True])
+def test_rank_sort_ranges(ctx, n_sites, spread):
+    """Small runs sort their sites in 1,024 ranges of the key space: counts at the edges of what a thread holds in
+    registers and of the path, hits spread over the set or in a few adjacent ranges, in canonical order."""
+    rng = np.random.default_rng(n_sites)
+    fwd, rev = "ACGTTGCAAGCT", "GGATCCATTCAG"
+    n = 30_000_000 if spread else 16384 * 24 + 4096
+    seq = np.full(n, ord("T"), np.uint8)
+    at = np.sort(rng.choice(n // 24 - 2, n_sites, replace=False)) * 24 + 3
+    words = [np.frombuffer(w.encode(), np.uint8) for w in (fwd, oracle_reverse_complement(fwd), rev,
+                                                           oracle_reverse_complement(rev))]
+    for p, w in zip(at, rng.integers(0, 4, n_sites)):
+        seq[p:p + 12] = words[w]
+    off = np.unique(np.r_[0, rng.integers(1, n, 5) // 24 * 24, n]).astype(np.uint64)
+    gen = np.arange(len(off) - 1, dtype=np.uint32)
+    pair = synth.pcr_params(fwd, rev, k=0, min_len=30, max_len=200)
+    want = oracle.scan(seq, off, gen, [pair])
+    sid = ctx.load(seq, off, gen)
+    try:
+        pid = ctx.ah_set_primers(fwd, rev, pair)
+        got = ctx.scan(sid, [pid])
+        run = ctx.run(sid, [pid])
+    finally:
+        ctx.ah_unload_genomes(sid)
+    assert len(want) == n_sites
+    assert got.tobytes() == want.tobytes() and run["sites"].tobytes() == want.tobytes()
+
+
+def oracle_reverse_complement(s):
+    return s[::-1].translate(str.maketrans("ACGT", "TGCA"))
