@@ -226,6 +226,8 @@ __device__ __forceinline__ long long fix_weight(double dH, double dS, double thr
 {
     return __double2ll_rn((1000.0 * dH - thr * dS) * kFix);
 }
+// Out of line: the tables of more than kTmStageD pairs, rarely read.
+__device__ __noinline__ long long far_weight(double dH, double dS, double thr) { return fix_weight(dH, dS, thr); }
 constexpr int kTmStageD = 4;
 constexpr unsigned kTmEarlyBlocks = 304; // two per SM
 // Entries from one site's segment tables to the next: four more than the tables, so that the
@@ -499,7 +501,7 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
                     cS += e.y;
                 }
             }
-#pragma unroll
+#pragma unroll 1
             for (int u = 0; u < 4; ++u) {
                 const float uH = __shfl_sync(0xffffffffu, cH, g0 + u), uS = __shfl_sync(0xffffffffu, cS, g0 + u);
                 const int si = sb + u;
@@ -621,20 +623,23 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
                 if (staged)
                     return sd.st[o2 * 16 + t2];
                 const int idx = (((o2 & 3) * 4 + (o2 >> 2)) * 4 + (t2 & 3)) * 4 + (t2 >> 2);
-                return fix_weight(pd.stack_dH_d[idx], pd.stack_dS_d[idx], pd.thr);
+                return far_weight(pd.stack_dH_d[idx], pd.stack_dS_d[idx], pd.thr);
             };
             auto tmW = [&](int idx) {
-                return staged ? sd.tm[idx] : fix_weight(pd.term_dH_d[idx], pd.term_dS_d[idx], pd.thr);
+                return staged ? sd.tm[idx] : far_weight(pd.term_dH_d[idx], pd.term_dS_d[idx], pd.thr);
             };
             __syncwarp();
-            for (int sb = 0; sb < mw; sb += 4) { // as the fp32 tables above
+            // (as the fp32 tables above; loops left rolled: a warp comes here once, and fetching
+            // unrolled code cost more than running it, 14,000 cycles against 5,000)
+            for (int sb = 0; sb < mw; sb += 4) {
                 long long cw = 0;
                 if (near && sb + y < m) {
                     const int k1 = key[sb + y + 1];
+#pragma unroll 1
                     for (int q = key[sb + y] + 1; q < k1 - 1; ++q)
                         cw += stW(oligo2(q), templ2(q));
                 }
-#pragma unroll
+#pragma unroll 1
                 for (int u = 0; u < 4; ++u) {
                     const long long uw = __shfl_sync(0xffffffffu, cw, g0 + u);
                     const int si = sb + u;
@@ -644,7 +649,7 @@ __global__ void __launch_bounds__(32 * kTmWarps) tm_kernel(const ah_site *sites,
                         const int fa = oligo2(k0 + 1) & 3, fb = oligo2(k1 - 1) & 3;
                         const long long into = apart ? stW(fb + 4 * y, templ2(k1 - 1)) + uw : 0;
                         const int to = apart ? fa : y;
-#pragma unroll
+#pragma unroll 1
                         for (int x = 0; x < 4; ++x)
                             W[si * 16 + x * 4 + y] = stW(x + 4 * to, p0) + into;
                     }
