@@ -71,6 +71,7 @@ struct ah_ctx {
     const PairDev *pairdev_d = nullptr;
     uint64_t pairs_version = 1;        // bumped whenever a registered pair changes
     ScanTuning tuning;                          // default tuning
+    bool tuning_given = false;                  // the default comes from AH_SCAN_TUNING
     std::map<std::string, ScanTuning> tuned;    // autotuned, per pattern-set signature
     uint64_t key_cap = 1 << 20;
     // one-synchronisation run: sizes of its scratch outputs, grown from the
@@ -657,10 +658,25 @@ std::string signature(const std::vector<ScanPattern> &pats)
     return k;
 }
 
-const ScanTuning &tuning_for(ah_ctx *c, const std::vector<ScanPattern> &pats)
+// The scan variant of a launch group: a tuned or overridden one, else the default.  One pair at
+// k <= 1 has a network so short that the waits for a tile and the visits take their share:
+// three CTAs per SM (80 registers, three tiles each) hide more of them than two of 128
+// registers.  Measured on a GB300, 1 Gbp, one pair, two -> three CTAs: k = 0 99 -> 91 us and
+// 103 -> 93; k = 1 132 -> 125, 130 -> 125, 130 -> 123, 129 -> 122, 136 -> 137, 136 -> 137;
+// k = 2 180 -> 178, 177 -> 178; two pairs at k = 1 198 -> 201; k = 3 of one 960-oligo pair over
+// 0.41 Gbp 88 -> 102.
+ScanTuning tuning_for(ah_ctx *c, const std::vector<ScanPattern> &pats)
 {
     auto it = c->tuned.find(signature(pats));
-    return it != c->tuned.end() ? it->second : c->tuning;
+    if (it != c->tuned.end())
+        return it->second;
+    ScanTuning t = c->tuning;
+    if (!c->tuning_given && pats.size() == 4 &&
+        std::all_of(pats.begin(), pats.end(), [](const ScanPattern &p) { return p.k <= 1; })) {
+        t.min_blocks = 3;
+        t.stages = 3;
+    }
+    return t;
 }
 
 // Launch the generated scan kernel over tiles [0, n_tiles) of a set.
@@ -1514,6 +1530,7 @@ ah_status ah_create(int device, size_t mem_budget_bytes, ah_ctx **out)
                 c->tuning.order = order;
                 c->tuning.stages = S;
                 c->tuning.min_blocks = mb;
+                c->tuning_given = true;
             }
         }
         AH_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
