@@ -842,6 +842,7 @@ template <class T> bool deliver(T *user, uint64_t cap, const T *dev, uint64_t co
 // synchronisation per data-dependent size, any size.
 // ---------------------------------------------------------------------------
 enum FastResult { kFastDone, kFastKeys, kFastRescan };
+constexpr uint64_t kFastAmps = 65535; // most amplicons of the one-synchronisation form
 
 // Queue the one-synchronisation form; scan_done (optional) is recorded right
 // after the scan.  The flag block is copied to the host after the last kernel.
@@ -860,7 +861,7 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
         ns_max = std::min<uint64_t>(ns_max, o->sites_cap);
     const bool amps_direct = o->amplicons_cap && is_device_ptr(c, o->amplicons) &&
                              (!o->seq_offsets || is_device_ptr(c, o->seq_offsets));
-    const uint64_t na_max = std::min<uint64_t>(amps_direct ? o->amplicons_cap : c->fast_amps, kSmallScan - 1);
+    const uint64_t na_max = std::min<uint64_t>(amps_direct ? o->amplicons_cap : c->fast_amps, kFastAmps);
     const bool seq_direct = o->seq_cap && is_device_ptr(c, o->seq);
     const uint64_t nq_max = seq_direct ? o->seq_cap : c->fast_seq;
 
@@ -869,12 +870,9 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
     float *tm = sites_direct && o->tm ? o->tm : (float *)scratch(c, "run_tm", ns_max * sizeof(float));
     uint8_t *pass = sites_direct && o->pass ? o->pass : (uint8_t *)scratch(c, "run_pass", ns_max);
     uint32_t *queue = (uint32_t *)scratch(c, "tm_queue", 2 * ns_max * sizeof(uint32_t));
-    uint64_t *counts = (uint64_t *)scratch(c, "pair_counts", ns_max * sizeof(uint64_t));
-    uint64_t *offs = (uint64_t *)scratch(c, "pair_offsets", ns_max * sizeof(uint64_t));
     ah_amplicon *amps = amps_direct ? o->amplicons : (ah_amplicon *)scratch(c, "run_amps", na_max * sizeof(ah_amplicon));
     uint64_t *qoff = amps_direct && o->seq_offsets ? o->seq_offsets
                                                    : (uint64_t *)scratch(c, "run_qoff", (na_max + 1) * sizeof(uint64_t));
-    uint64_t *len = (uint64_t *)scratch(c, "fetch_len", (na_max + 1) * sizeof(uint64_t));
     char *seq = seq_direct ? o->seq : (char *)scratch(c, "run_seq", nq_max);
     const uint8_t *filt = o->tm_filter ? pass : nullptr;
 
@@ -898,17 +896,12 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
                   (uint32_t *)(F + kFlagTmQueue), tm_seg_max(c), tm_few_exact(c), c->d_err, st);
     }
     {
-        Stage sg(c, "pair", st, 3);
-        launch_pair_count(sites, ns_max, F + kFlagSites, filt, pd, counts, nullptr, st);
-        exclusive_scan_u64_dev(counts, offs, ns_max, F + kFlagSites, 0, F + kFlagAux, na_max, F + kFlagAmps,
-                               F + kFlagRedo, kRedoAmps, st);
-        launch_pair_write(sites, ns_max, F + kFlagSites, filt, pd, counts, offs, amps, len, na_max, F + kFlagRedo,
-                          kRedoAmps, st);
+        Stage sg(c, "pair", st, 1);
+        launch_pair_run(sites, ns_max, F + kFlagSites, filt, pd, amps, qoff, na_max, nq_max, F + kFlagAmps,
+                        F + kFlagSeq, F + kFlagRedo, st);
     }
     {
-        Stage sg(c, "fetch", st, 2);
-        exclusive_scan_u64_dev(len, qoff, na_max + 1, F + kFlagAmps, 1, F + kFlagAux, nq_max, F + kFlagSeq,
-                               F + kFlagRedo, kRedoSeq, st);
+        Stage sg(c, "fetch", st, 1);
         launch_fetch(amps, na_max, F + kFlagAmps, qoff, gs.planes, gs.contig_off, seq, F + kFlagRedo, kRedoSeq, st);
     }
     AH_CUDA(cudaMemcpyAsync(c->h_flags, c->d_flags, kFlagWords * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
@@ -1010,9 +1003,9 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         void *temp = scratch(c, "scan_temp", tb);
         {
             Stage sg(c, "pair", st, 2 + scan_u64_launches(ns));
-            launch_pair_count(sites, ns, nullptr, filt, pd, counts, nullptr, st);
+            launch_pair_count(sites, ns, filt, pd, counts, nullptr, st);
             exclusive_scan_u64(temp, tb, counts, offs, ns, st);
-            launch_total(offs, counts, ns, nullptr, 0, c->d_aux, 0, nullptr, nullptr, 0, st);
+            launch_total(offs, counts, ns, c->d_aux, st);
         }
         check_flags(c, st);
         na = c->h_flags[kFlagAux];
@@ -1022,7 +1015,7 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         qoff = direct_or_scratch(c, "run_qoff", o->seq_offsets, o->seq_offsets ? o->amplicons_cap + 1 : 0, na + 1);
         if (na) {
             Stage sg(c, "pair", st, 1);
-            launch_pair_write(sites, ns, nullptr, filt, pd, counts, offs, amps, nullptr, na, nullptr, 0, st);
+            launch_pair_write(sites, ns, filt, pd, counts, offs, amps, na, st);
         }
         uint64_t *len = (uint64_t *)scratch(c, "fetch_len", (na + 1) * sizeof(uint64_t));
         size_t tb2 = scan_u64_temp_bytes(na + 1);
@@ -1045,7 +1038,7 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         }
     }
     // later one-synchronisation runs size their scratch for counts like these
-    c->fast_amps = std::min<uint64_t>(kSmallScan - 1, std::max<uint64_t>(c->fast_amps, na + na / 4 + 16));
+    c->fast_amps = std::min<uint64_t>(kFastAmps, std::max<uint64_t>(c->fast_amps, na + na / 4 + 16));
     c->fast_seq = std::min<uint64_t>(1ull << 30, std::max<uint64_t>(c->fast_seq, nq + nq / 4 + 4096));
     overflow |= !deliver(o->sites, o->sites_cap, sites, ns, st);
     if (o->tm)
@@ -1229,16 +1222,16 @@ void group_device(ah_ctx *c, const GenomeSet &gs, uint32_t pid, int k, const std
     void *temp = scratch(c, "scan_temp", tb);
     {
         Stage sg(c, "pair", st, 2 + scan_u64_launches(ns));
-        launch_pair_count(sites, ns, nullptr, nullptr, pd, counts, nullptr, st);
+        launch_pair_count(sites, ns, nullptr, pd, counts, nullptr, st);
         exclusive_scan_u64(temp, tb, counts, offs, ns, st);
-        launch_total(offs, counts, ns, nullptr, 0, c->d_aux, 0, nullptr, nullptr, 0, st);
+        launch_total(offs, counts, ns, c->d_aux, st);
     }
     check_flags(c, st);
     const uint64_t na = c->h_flags[kFlagAux];
     ah_amplicon *amps = (ah_amplicon *)scratch(c, "serve_amps", std::max<uint64_t>(na, 1) * sizeof(ah_amplicon));
     if (na) {
         Stage sg(c, "pair", st, 1);
-        launch_pair_write(sites, ns, nullptr, nullptr, pd, counts, offs, amps, nullptr, na, nullptr, 0, st);
+        launch_pair_write(sites, ns, nullptr, pd, counts, offs, amps, na, st);
     }
     // staging layout: sites, amplicons, pass flags
     const size_t sb = ns * sizeof(ah_site), ab = na * sizeof(ah_amplicon);
@@ -2596,9 +2589,9 @@ ah_status ah_pair(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t
         void *temp = scratch(c, "scan_temp", tb);
         {
             Stage sg(c, "pair", st, 2 + scan_u64_launches(n));
-            launch_pair_count(s, n, nullptr, ps, pd, counts, c->d_err, st);
+            launch_pair_count(s, n, ps, pd, counts, c->d_err, st);
             exclusive_scan_u64(temp, tb, counts, offs, n, st);
-            launch_total(offs, counts, n, nullptr, 0, c->d_aux, 0, nullptr, nullptr, 0, st);
+            launch_total(offs, counts, n, c->d_aux, st);
         }
         check_flags(c, st); // the records' check and the count
         const uint64_t total = c->h_flags[kFlagAux];
@@ -2611,7 +2604,7 @@ ah_status ah_pair(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t
         ah_amplicon *dst = out_buf(c, "amp_out", out, total);
         {
             Stage sg(c, "pair", st, 1);
-            launch_pair_write(s, n, nullptr, ps, pd, counts, offs, dst, nullptr, total, nullptr, 0, st);
+            launch_pair_write(s, n, ps, pd, counts, offs, dst, total, st);
         }
         out_finish(out, dst, total, st);
         AH_CUDA(cudaStreamSynchronize(st));

@@ -235,9 +235,9 @@ __device__ __forceinline__ uint64_t dev_count(uint64_t n, const uint64_t *n_dev)
 // or write anything that another kernel of the chain touches.  Every block of such
 // a kernel waits, so a kernel that is complete has all earlier ones complete.  What
 // the chain hands on is read with plain loads (no const __restrict__, no __ldg: it
-// is not constant over the kernel's lifetime).  Measured on a GB300, one 4.8 Mbp
+// is not constant over the kernel's lifetime).  Measured on a GB300, one 4.6 Mbp
 // genome at k = 2 from its scan's end to the last kernel's: ten launches, 57 us
-// -> seven chained ones, 37.
+// -> four chained ones, 32.
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -317,37 +317,29 @@ void launch_tm_sweep(const ah_site *sites, uint64_t n_sites, const ah_amplicon *
                      int *err, cudaStream_t s);
 
 // pair.cu
-// n_dev (here and below): optional device count, min(*n_dev, n) records.
 // err (may be null): a device error word; while it is set the kernel leaves the records alone.
-void launch_pair_count(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, uint64_t *counts, const int *err, cudaStream_t s);
-// *out = offs[m-1] + counts[m-1] (the total of an exclusive scan over m values,
-// m = n or min(*n_dev + add, n)).  With eff != nullptr also *eff = the total if it
-// is at most cap, else 0 with redo_bit set in *redo.
-void launch_total(const uint64_t *offs, const uint64_t *counts, uint64_t n, const uint64_t *n_dev, uint64_t add,
-                  uint64_t *out, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit, cudaStream_t s);
+void launch_pair_count(const ah_site *sites, uint64_t n, const uint8_t *pass, const PairDev *pairs_d, uint64_t *counts,
+                       const int *err, cudaStream_t s);
+// Amplicons and sequence offsets of min(*n_dev, n) sites (n <= kSmallSort) of a scan in one
+// launch: *n_amps and *n_seq are the counts.  More than amps_max amplicons: none is written,
+// both counts are 0 and kRedoAmps is set in *redo; more than seq_max bases: *n_seq is 0 with
+// kRedoSeq.  seq_offsets holds amps_max + 1 words.
+void launch_pair_run(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
+                     const PairDev *pairs_d, ah_amplicon *out, uint64_t *seq_offsets, uint64_t amps_max,
+                     uint64_t seq_max, uint64_t *n_amps, uint64_t *n_seq, uint64_t *redo, cudaStream_t s);
+// *out = offs[n-1] + counts[n-1] (the total of an exclusive scan over n values)
+void launch_total(const uint64_t *offs, const uint64_t *counts, uint64_t n, uint64_t *out, cudaStream_t s);
 size_t scan_u64_temp_bytes(uint64_t n);
 // Exclusive scan of n u64 values; one block (no temporary) for n <= kOneBlockScan, CUB above
 // (36,000 values on a GB300: one block 27 us, CUB's two launches 9).
 constexpr uint64_t kOneBlockScan = 8192;
-// Most values of a scan whose count is known on the device only (one block).
-constexpr uint64_t kSmallScan = 65536;
 // number of kernels exclusive_scan_u64 launches for n values
 int scan_u64_launches(uint64_t n);
 void exclusive_scan_u64(void *temp, size_t temp_bytes, const uint64_t *in, uint64_t *out, uint64_t n, cudaStream_t s);
-// One-block exclusive scan of min(*n_dev + add, n) values (n <= kSmallScan), the
-// last `add` of them zero whatever `in` holds there;
-// with tot also their sum, and with eff the capacity check of launch_total.
-void exclusive_scan_u64_dev(const uint64_t *in, uint64_t *out, uint64_t n, const uint64_t *n_dev, uint64_t add,
-                            uint64_t *tot, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit,
-                            cudaStream_t s);
-// skip: optional device word; the kernel writes nothing when (*skip & skip_bit) != 0.
 // counts, offsets: launch_pair_count's results and their exclusive scan.
-// len (may be null): the amplicons' lengths as launch_fetch_lengths gives them, for sites
-// that a scan found.
-void launch_pair_write(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, const uint64_t *counts, const uint64_t *offsets, ah_amplicon *out,
-                       uint64_t *len, uint64_t cap, const uint64_t *skip, uint64_t skip_bit, cudaStream_t s);
+void launch_pair_write(const ah_site *sites, uint64_t n, const uint8_t *pass, const PairDev *pairs_d,
+                       const uint64_t *counts, const uint64_t *offsets, ah_amplicon *out, uint64_t cap,
+                       cudaStream_t s);
 
 // amplitype.cu: sequence variants and amplitypes.  Two hash tables of `size`
 // slots: variants (and then amplitypes) with the first index seen, and

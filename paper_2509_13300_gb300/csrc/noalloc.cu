@@ -155,7 +155,7 @@ extern "C" ah_status ah_pair_noalloc(const int32_t *pair_windows, uint32_t n_pai
         AH_CUDA(cudaStreamSynchronize(st));
         if (bad)
             return AH_ERR_ARG;
-        ah::launch_pair_count(sites, n, nullptr, pass, pd, counts, nullptr, st);
+        ah::launch_pair_count(sites, n, pass, pd, counts, nullptr, st);
         ah::exclusive_scan_u64(cub_temp, cub_bytes, counts, offs, n, st);
         AH_CUDA(cudaMemcpyAsync(&last[0], offs + n - 1, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
         AH_CUDA(cudaMemcpyAsync(&last[1], counts + n - 1, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
@@ -167,7 +167,7 @@ extern "C" ah_status ah_pair_noalloc(const int32_t *pair_windows, uint32_t n_pai
         if (total > cap)
             return AH_ERR_OVERFLOW;
         if (total) {
-            ah::launch_pair_write(sites, n, nullptr, pass, pd, counts, offs, out, nullptr, total, nullptr, 0, st);
+            ah::launch_pair_write(sites, n, pass, pd, counts, offs, out, total, st);
             AH_CUDA(cudaStreamSynchronize(st));
         }
     } catch (const ah::Error &e) {

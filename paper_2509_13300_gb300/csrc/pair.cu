@@ -16,6 +16,7 @@
 // only at a shared position, and the write pass starts from the counts, as most
 // sites lead no amplicon.  Measured on a GB300: 0.94 M sites, count 20 -> 13 us,
 // write 28 -> 13; 3.3 M sites, write 68 -> 20.
+#include <cooperative_groups.h>
 #include <cub/device/device_scan.cuh>
 
 #include "ah_internal.h"
@@ -130,146 +131,239 @@ __device__ __forceinline__ bool in_window(const PairDev &pd, uint32_t s_pos, con
     return r.pos >= s_pos && len >= pd.min_len && len <= pd.max_len;
 }
 
-__global__ void pair_count_kernel(const ah_site *s, uint64_t n_arg, const uint64_t *n_dev, const uint8_t *pass,
-                                  const PairDev *__restrict__ pairs, uint64_t *counts, const int *err)
+__device__ __forceinline__ int orient_of(int x, int y) { return (x == 0 && y == 1) ? 0 : (x == 1 && y == 0) ? 1 : (x == 0 ? 2 : 3); }
+
+// Amplicons of the group that site a leads, and the sum of their lengths.
+__device__ __forceinline__ uint32_t count_group(const ah_site *s, uint64_t n, const uint8_t *pass,
+                                                const PairDev *__restrict__ pairs, uint64_t a, uint64_t *bases)
+{
+    uint32_t cnt = 0;
+    *bases = 0;
+    const Group g = make_group(s, n, pass, pairs, a);
+    if (!g.valid)
+        return 0;
+    const ah_site sa = s[a];
+    const PairDev &pd = pairs[sa.pair];
+    for (uint64_t b = g.first; b < n; ++b) {
+        const ah_site r = s[b];
+        if (r.pair != sa.pair || r.contig != sa.contig || r.pos > g.tmax)
+            break;
+        if (r.strand != 1 || (pass && !pass[b]))
+            continue;
+        uint32_t end;
+        if (in_window(pd, sa.pos, r, &end)) {
+            cnt += g.nl;
+            *bases += (uint64_t)g.nl * (end - sa.pos);
+        }
+    }
+    return cnt;
+}
+
+// Write them from out[o] on, those below cap; with qoff, also the sequence offset of each, the
+// first at base.
+__device__ __forceinline__ void write_group(const ah_site *s, uint64_t n, const uint8_t *pass,
+                                            const PairDev *__restrict__ pairs, uint64_t a, uint64_t o, uint64_t base,
+                                            ah_amplicon *out, uint64_t *qoff, uint64_t cap)
+{
+    const Group g = make_group(s, n, pass, pairs, a);
+    if (!g.valid)
+        return;
+    const ah_site sa = s[a];
+    const PairDev &pd = pairs[sa.pair];
+    // streams: (left index li, right primer y); cursor = next candidate index
+    uint64_t cur[4];
+    const int ns = g.nl * 2;
+    auto advance = [&](int st, uint64_t from) -> uint64_t {
+        const int y = st & 1;
+        for (uint64_t b = from; b < n; ++b) {
+            const ah_site r = s[b];
+            if (r.pair != sa.pair || r.contig != sa.contig || r.pos > g.tmax)
+                return n;
+            if (r.strand != 1 || r.primer != y || (pass && !pass[b]))
+                continue;
+            uint32_t end;
+            if (in_window(pd, sa.pos, r, &end))
+                return b;
+        }
+        return n;
+    };
+    for (int st = 0; st < ns; ++st)
+        cur[st] = advance(st, g.first);
+    for (;;) {
+        int best = -1;
+        uint32_t bend = 0;
+        int bor = 0;
+        for (int st = 0; st < ns; ++st) {
+            if (cur[st] >= n)
+                continue;
+            const ah_site r = s[cur[st]];
+            const uint32_t end = r.pos + pd.L[r.primer];
+            const int orr = orient_of(g.lx[st >> 1], r.primer);
+            if (best < 0 || end < bend || (end == bend && orr < bor)) {
+                best = st;
+                bend = end;
+                bor = orr;
+            }
+        }
+        if (best < 0)
+            break;
+        if (o < cap) {
+            ah_amplicon am;
+            am.genome = sa.genome;
+            am.contig = sa.contig;
+            am.start = sa.pos;
+            am.end = bend;
+            am.left = (uint32_t)g.li[best >> 1];
+            am.right = (uint32_t)cur[best];
+            am.orient = (uint8_t)bor;
+            am.pair = sa.pair;
+            am.pad0 = am.pad1 = 0;
+            out[o] = am;
+            if (qoff) {
+                qoff[o] = base;
+                base += bend - sa.pos;
+            }
+        }
+        ++o;
+        cur[best] = advance(best, cur[best] + 1);
+    }
+}
+
+__global__ void pair_count_kernel(const ah_site *s, uint64_t n, const uint8_t *pass, const PairDev *__restrict__ pairs,
+                                  uint64_t *counts, const int *err)
 {
     chain_start();
     chain_wait();
     if (err && *(volatile const int *)err) // the records' check failed: nothing is indexed with them
         return;
-    const uint64_t n = dev_count(n_arg, n_dev);
     for (uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t cnt = 0;
-        const Group g = make_group(s, n, pass, pairs, a);
-        if (g.valid) {
-            const ah_site sa = s[a];
-            const PairDev &pd = pairs[sa.pair];
-            for (uint64_t b = g.first; b < n; ++b) {
-                const ah_site r = s[b];
-                if (r.pair != sa.pair || r.contig != sa.contig || r.pos > g.tmax)
-                    break;
-                if (r.strand != 1 || (pass && !pass[b]))
-                    continue;
-                uint32_t end;
-                if (in_window(pd, sa.pos, r, &end))
-                    cnt += g.nl;
-            }
-        }
-        counts[a] = cnt;
+        uint64_t bases;
+        counts[a] = count_group(s, n, pass, pairs, a, &bases);
     }
 }
 
-__device__ __forceinline__ int orient_of(int x, int y) { return (x == 0 && y == 1) ? 0 : (x == 1 && y == 0) ? 1 : (x == 0 ? 2 : 3); }
-
-__global__ void pair_write_kernel(const ah_site *s, uint64_t n_arg, const uint64_t *n_dev, const uint8_t *pass,
-                                  const PairDev *__restrict__ pairs, const uint64_t *counts, const uint64_t *offsets,
-                                  ah_amplicon *out, uint64_t *len, uint64_t cap, const uint64_t *skip, uint64_t skip_bit)
+__global__ void pair_write_kernel(const ah_site *s, uint64_t n, const uint8_t *pass, const PairDev *__restrict__ pairs,
+                                  const uint64_t *counts, const uint64_t *offsets, ah_amplicon *out, uint64_t cap)
 {
     chain_start();
     chain_wait();
-    if (skip && (*(const volatile uint64_t *)skip & skip_bit))
+    for (uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (uint64_t)gridDim.x * blockDim.x)
+        if (counts[a]) // most sites lead no amplicon
+            write_group(s, n, pass, pairs, a, offsets[a], 0, out, nullptr, cap);
+}
+
+// Both passes and the scan between them in one launch, for at most kSmallSort sites whose count
+// is on the device: a cluster of kPairCtas CTAs, a thread per site.  Counts and lengths stay in
+// registers; they are scanned within the block, and the blocks' totals are read through
+// distributed shared memory.  The sequence offsets follow from the same scan.
+// Bound: latency, and the host's launches around it.  Measured on a GB300 from the end of the
+// Tm kernel to the sequence decode: four launches (count, scan, write, scan of the lengths)
+// 9.3 us for 14 sites, 15 for 6,000 -> 8.1 and 14.2; the run of a small resident set, which waits
+// for the host's launches too, 93 -> 88.  A cluster of eight with two sites per thread took 18
+// us for 10,000 sites against 15.
+constexpr int kPairCtas = 16, kPairThreads = 1024, kPairRounds = (int)(kSmallSort / (kPairCtas * kPairThreads));
+static_assert(kPairRounds * kPairCtas * kPairThreads == kSmallSort, "whole rounds");
+
+__global__ void __cluster_dims__(kPairCtas, 1, 1) __launch_bounds__(kPairThreads)
+    pair_run_kernel(const ah_site *s, uint64_t n_arg, const uint64_t *n_dev, const uint8_t *pass,
+                    const PairDev *__restrict__ pairs, ah_amplicon *out, uint64_t *qoff, uint64_t amps_max,
+                    uint64_t seq_max, uint64_t *n_amps, uint64_t *n_seq, uint64_t *redo)
+{
+    namespace cg = cooperative_groups;
+    __shared__ uint64_t wcnt[kPairRounds][32], wlen[kPairRounds][32]; // per warp
+    __shared__ uint64_t tot[kPairRounds][2];                          // the block's amplicons and bases per round
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_start();
+    chain_wait();
+    const uint64_t n = dev_count(n_arg, n_dev);
+    uint64_t cnt[kPairRounds], len[kPairRounds], icnt[kPairRounds], ilen[kPairRounds]; // own; inclusive in the warp
+#pragma unroll
+    for (int r = 0; r < kPairRounds; ++r) {
+        const uint64_t a = (uint64_t)(r * kPairCtas + rank) * kPairThreads + tid;
+        cnt[r] = len[r] = 0;
+        if (a < n)
+            cnt[r] = count_group(s, n, pass, pairs, a, &len[r]);
+        icnt[r] = cnt[r];
+        ilen[r] = len[r];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t c = __shfl_up_sync(0xffffffffu, icnt[r], d), l = __shfl_up_sync(0xffffffffu, ilen[r], d);
+            if (lane >= d) {
+                icnt[r] += c;
+                ilen[r] += l;
+            }
+        }
+        if (lane == 31) {
+            wcnt[r][warp] = icnt[r];
+            wlen[r][warp] = ilen[r];
+        }
+    }
+    __syncthreads();
+    if (warp < 2 * kPairRounds) { // inclusive over the warps: one warp per round and quantity
+        uint64_t *w = warp & 1 ? wlen[warp >> 1] : wcnt[warp >> 1];
+        uint64_t v = w[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xffffffffu, v, d);
+            if (lane >= d)
+                v += y;
+        }
+        w[lane] = v;
+        if (lane == 31)
+            tot[warp >> 1][warp & 1] = v;
+    }
+    cluster.sync(); // every block's totals
+    uint64_t total = 0, bases = 0, bcnt[kPairRounds], blen[kPairRounds]; // of all sites; before this block's round
+#pragma unroll
+    for (int r = 0; r < kPairRounds; ++r)
+        for (int q = 0; q < kPairCtas; ++q) {
+            const uint64_t *t = cluster.map_shared_rank(&tot[r][0], q);
+            if (q == rank) {
+                bcnt[r] = total;
+                blen[r] = bases;
+            }
+            total += t[0];
+            bases += t[1];
+        }
+    cluster.sync(); // no block leaves while its totals are read
+    const bool fits = total <= amps_max;
+    if (rank == 0 && tid == 0) {
+        *n_amps = fits ? total : 0;
+        const bool seq_fits = !fits || bases <= seq_max;
+        *n_seq = fits && seq_fits ? bases : 0;
+        qoff[fits ? total : 0] = fits ? bases : 0;
+        if (!fits || !seq_fits)
+            atomicOr((unsigned long long *)redo, (unsigned long long)(!fits ? kRedoAmps : kRedoSeq));
+    }
+    if (!fits)
         return;
-    const uint64_t n = dev_count(n_arg, n_dev);
-    for (uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (uint64_t)gridDim.x * blockDim.x) {
-        if (!counts[a]) // most sites lead no amplicon
-            continue;
-        const Group g = make_group(s, n, pass, pairs, a);
-        if (!g.valid)
-            continue;
-        const ah_site sa = s[a];
-        const PairDev &pd = pairs[sa.pair];
-        // streams: (left index li, right primer y); cursor = next candidate index
-        uint64_t cur[4];
-        const int ns = g.nl * 2;
-        auto advance = [&](int st, uint64_t from) -> uint64_t {
-            const int y = st & 1;
-            for (uint64_t b = from; b < n; ++b) {
-                const ah_site r = s[b];
-                if (r.pair != sa.pair || r.contig != sa.contig || r.pos > g.tmax)
-                    return n;
-                if (r.strand != 1 || r.primer != y || (pass && !pass[b]))
-                    continue;
-                uint32_t end;
-                if (in_window(pd, sa.pos, r, &end))
-                    return b;
-            }
-            return n;
-        };
-        for (int st = 0; st < ns; ++st)
-            cur[st] = advance(st, g.first);
-        uint64_t o = offsets[a];
-        for (;;) {
-            int best = -1;
-            uint32_t bend = 0;
-            int bor = 0;
-            for (int st = 0; st < ns; ++st) {
-                if (cur[st] >= n)
-                    continue;
-                const ah_site r = s[cur[st]];
-                const uint32_t end = r.pos + pd.L[r.primer];
-                const int orr = orient_of(g.lx[st >> 1], r.primer);
-                if (best < 0 || end < bend || (end == bend && orr < bor)) {
-                    best = st;
-                    bend = end;
-                    bor = orr;
-                }
-            }
-            if (best < 0)
-                break;
-            if (o < cap) {
-                ah_amplicon am;
-                am.genome = sa.genome;
-                am.contig = sa.contig;
-                am.start = sa.pos;
-                am.end = bend;
-                am.left = (uint32_t)g.li[best >> 1];
-                am.right = (uint32_t)cur[best];
-                am.orient = (uint8_t)bor;
-                am.pair = sa.pair;
-                am.pad0 = am.pad1 = 0;
-                out[o] = am;
-                if (len) // of sites from a scan: both ends lie in the contig
-                    len[o] = bend - sa.pos;
-            }
-            ++o;
-            cur[best] = advance(best, cur[best] + 1);
+#pragma unroll
+    for (int r = 0; r < kPairRounds; ++r)
+        if (cnt[r]) {
+            const uint64_t o = bcnt[r] + (warp ? wcnt[r][warp - 1] : 0) + icnt[r] - cnt[r];
+            const uint64_t l = blen[r] + (warp ? wlen[r][warp - 1] : 0) + ilen[r] - len[r];
+            write_group(s, n, pass, pairs, (uint64_t)(r * kPairCtas + rank) * kPairThreads + tid, o, l, out, qoff, amps_max);
         }
-    }
 }
 
-__global__ void total_kernel(const uint64_t *offs, const uint64_t *counts, uint64_t n_arg, const uint64_t *n_dev,
-                             uint64_t add, uint64_t *out, uint64_t cap, uint64_t *eff, uint64_t *redo,
-                             uint64_t redo_bit)
+__global__ void total_kernel(const uint64_t *offs, const uint64_t *counts, uint64_t n, uint64_t *out)
 {
     chain_start();
     chain_wait();
-    const uint64_t n = n_dev ? min(*n_dev + add, n_arg) : n_arg;
-    const uint64_t t = n ? offs[n - 1] + counts[n - 1] : 0;
-    *out = t;
-    if (eff) {
-        *eff = t <= cap ? t : 0;
-        if (t > cap)
-            atomicOr((unsigned long long *)redo, (unsigned long long)redo_bit);
-    }
+    *out = n ? offs[n - 1] + counts[n - 1] : 0;
 }
 
-// One-block exclusive scan of m u64 values (m = n, or min(*n_dev + add, n)),
-// 4096 at a time: coalesced loads (four per thread in flight) staged through
-// shared memory, each thread scans four consecutive values, warp shuffles and
-// one shared pass scan the 1024 thread sums, and the results leave through
-// shared memory as coalesced stores.  With tot it also writes the sum of all
-// m values; with eff, *eff = that sum if it is at most cap, else 0 with
-// redo_bit set in *redo.  The last `add` values count as zero (not read).
-__global__ void __launch_bounds__(1024) scan_small_kernel(const uint64_t *in, uint64_t *out, uint32_t n_arg,
-                                                          const uint64_t *n_dev, uint64_t add, uint64_t *tot,
-                                                          uint64_t cap, uint64_t *eff, uint64_t *redo,
-                                                          uint64_t redo_bit)
+// One-block exclusive scan of n u64 values, 4096 at a time: coalesced loads (four per thread in
+// flight) staged through shared memory, each thread scans four consecutive values, warp shuffles
+// and one shared pass scan the 1024 thread sums, and the results leave through shared memory as
+// coalesced stores.
+__global__ void __launch_bounds__(1024) scan_small_kernel(const uint64_t *in, uint64_t *out, uint32_t n)
 {
     chain_start();
     chain_wait();
     __shared__ uint64_t buf[4096];
     __shared__ uint64_t wsum[32];
-    const uint32_t n = n_dev ? (uint32_t)min(*(const volatile uint64_t *)n_dev + add, (uint64_t)n_arg) : n_arg;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint64_t carry = 0;
     for (uint32_t base = 0; base < n; base += 4096) {
@@ -277,7 +371,7 @@ __global__ void __launch_bounds__(1024) scan_small_kernel(const uint64_t *in, ui
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const uint32_t i = base + tid + 1024u * u;
-            v[u] = i + add < n ? in[i] : 0;
+            v[u] = i < n ? in[i] : 0;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -321,14 +415,6 @@ __global__ void __launch_bounds__(1024) scan_small_kernel(const uint64_t *in, ui
         }
         __syncthreads(); // buf and wsum are rewritten by the next chunk
     }
-    if (tid == 0 && tot) {
-        *tot = carry;
-        if (eff) {
-            *eff = carry <= cap ? carry : 0;
-            if (carry > cap)
-                atomicOr((unsigned long long *)redo, (unsigned long long)redo_bit);
-        }
-    }
 }
 
 unsigned grid_for(uint64_t n, int threads)
@@ -343,19 +429,34 @@ unsigned grid_for(uint64_t n, int threads)
 
 } // namespace
 
-void launch_pair_count(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, uint64_t *counts, const int *err, cudaStream_t s)
+void launch_pair_count(const ah_site *sites, uint64_t n, const uint8_t *pass, const PairDev *pairs_d, uint64_t *counts,
+                       const int *err, cudaStream_t s)
 {
     if (!n)
         return;
-    launch_chained(pair_count_kernel, grid_for(n, 128), 128, 0, s, sites, n, n_dev, pass, pairs_d,
-                   counts, err);
+    launch_chained(pair_count_kernel, grid_for(n, 128), 128, 0, s, sites, n, pass, pairs_d, counts, err);
 }
 
-void launch_total(const uint64_t *offs, const uint64_t *counts, uint64_t n, const uint64_t *n_dev, uint64_t add,
-                  uint64_t *out, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit, cudaStream_t s)
+void launch_pair_run(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
+                     const PairDev *pairs_d, ah_amplicon *out, uint64_t *seq_offsets, uint64_t amps_max,
+                     uint64_t seq_max, uint64_t *n_amps, uint64_t *n_seq, uint64_t *redo, cudaStream_t s)
 {
-    launch_chained(total_kernel, 1, 1, 0, s, offs, counts, n, n_dev, add, out, cap, eff, redo, redo_bit);
+    if (n == 0 || n > kSmallSort)
+        throw Error(AH_ERR_ARG, "pairing with a device count: size outside 1..16384");
+    static int attr_dev = -1; // a cluster of 16 is an opt-in, once per device
+    int dev = 0;
+    AH_CUDA(cudaGetDevice(&dev));
+    if (dev != attr_dev) {
+        AH_CUDA(cudaFuncSetAttribute(pair_run_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        attr_dev = dev;
+    }
+    launch_chained(pair_run_kernel, kPairCtas, kPairThreads, 0, s, sites, n, n_dev, pass, pairs_d, out, seq_offsets,
+                   amps_max, seq_max, n_amps, n_seq, redo);
+}
+
+void launch_total(const uint64_t *offs, const uint64_t *counts, uint64_t n, uint64_t *out, cudaStream_t s)
+{
+    launch_chained(total_kernel, 1, 1, 0, s, offs, counts, n, out);
 }
 
 size_t scan_u64_temp_bytes(uint64_t n)
@@ -370,33 +471,20 @@ void exclusive_scan_u64(void *temp, size_t temp_bytes, const uint64_t *in, uint6
     if (n == 0)
         return;
     if (n <= kOneBlockScan) {
-        launch_chained(scan_small_kernel, 1, 1024, 0, s, in, out, (uint32_t)n, nullptr, 0, nullptr, 0, nullptr, nullptr,
-                       0);
+        launch_chained(scan_small_kernel, 1, 1024, 0, s, in, out, (uint32_t)n);
         return;
     }
     AH_CUDA(cub::DeviceScan::ExclusiveSum(temp, temp_bytes, in, out, (int64_t)n, s));
 }
 
-void exclusive_scan_u64_dev(const uint64_t *in, uint64_t *out, uint64_t n, const uint64_t *n_dev, uint64_t add,
-                            uint64_t *tot, uint64_t cap, uint64_t *eff, uint64_t *redo, uint64_t redo_bit,
-                            cudaStream_t s)
-{
-    if (n == 0 || n > kSmallScan)
-        throw Error(AH_ERR_ARG, "device-count scan: size outside 1..65536");
-    launch_chained(scan_small_kernel, 1, 1024, 0, s, in, out, (uint32_t)n, n_dev, add, tot, cap, eff, redo,
-                   redo_bit);
-}
-
 int scan_u64_launches(uint64_t n) { return n == 0 ? 0 : n <= kOneBlockScan ? 1 : 2; }
 
-void launch_pair_write(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
-                       const PairDev *pairs_d, const uint64_t *counts, const uint64_t *offsets, ah_amplicon *out,
-                       uint64_t *len, uint64_t cap, const uint64_t *skip, uint64_t skip_bit, cudaStream_t s)
+void launch_pair_write(const ah_site *sites, uint64_t n, const uint8_t *pass, const PairDev *pairs_d,
+                       const uint64_t *counts, const uint64_t *offsets, ah_amplicon *out, uint64_t cap, cudaStream_t s)
 {
     if (!n)
         return;
-    launch_chained(pair_write_kernel, grid_for(n, 128), 128, 0, s, sites, n, n_dev, pass, pairs_d,
-                   counts, offsets, out, len, cap, skip, skip_bit);
+    launch_chained(pair_write_kernel, grid_for(n, 128), 128, 0, s, sites, n, pass, pairs_d, counts, offsets, out, cap);
 }
 
 } // namespace ah

@@ -1468,3 +1468,27 @@ def test_rank_sort_ranges(ctx, n_sites, spread):
 
 def oracle_reverse_complement(s):
     return s[::-1].translate(str.maketrans("ACGT", "TGCA"))
+
+
+@pytest.mark.parametrize("n_contigs,contig", [(1, 900), (40, 3000), (3, 1_200_000)])
+@pytest.mark.parametrize("tm_filter", [False, True])
+def test_run_pairs_in_one_launch_at_block_edges(ctx, n_contigs, contig, tm_filter):
+    """A run's amplicons and sequence offsets come from one launch that scans counts over its blocks: no site, sites
+    in one block and over many, with and without the Tm filter, first with outputs that are too small."""
+    w = synth.random_small(contig, n_bases=n_contigs * contig, n_contigs=n_contigs, L_f=9, L_r=8, k=1, min_len=20,
+                           max_len=400)
+    p = dict(w.pairs[0], tm_min=-10.0)
+    want = oracle.scan(w.seq, w.contig_off, w.contig_genome, [p])
+    _, passed = oracle.tm(w.seq, w.contig_off, want, [p])
+    amps = oracle.pair(want, [p], passed if tm_filter else None)
+    seqs, offs = oracle.fetch(w.seq, w.contig_off, amps)
+    sid = ctx.load(w.seq, w.contig_off, w.contig_genome)
+    try:
+        pid = ctx.ah_set_primers(p["fwd"], p["rev"], p)
+        for _ in range(2):
+            r = ctx.run(sid, [pid], tm_filter=tm_filter)
+            assert r["sites"].tobytes() == want.tobytes() and r["amps"].tobytes() == amps.tobytes()
+            assert r["seqs"] == seqs and np.array_equal(r["offs"], offs)
+    finally:
+        ctx.ah_unload_genomes(sid)
+    assert len(want) <= 16384 and (contig != 1_200_000 or len(want) > 4096)
