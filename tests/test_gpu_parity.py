@@ -1492,3 +1492,33 @@ def test_run_pairs_in_one_launch_at_block_edges(ctx, n_contigs, contig, tm_filte
     finally:
         ctx.ah_unload_genomes(sid)
     assert len(want) <= 16384 and (contig != 1_200_000 or len(want) > 4096)
+
+
+@pytest.mark.parametrize("parts", [1, 2, 15, 16, 17, 40])
+def test_mirrored_tiles_of_few_and_many_contigs(ctx, parts):
+    """Contig ends at every place in a word and next to tile ends, about `parts` per tile (tiles of few parts are
+    gathered part by part, others word by word), with runs of contigs of one to seven bases: the letters come back."""
+    import torch
+    rng = np.random.default_rng(parts)
+    T = 32 * 1024
+    for n in (37, T - 2, 3 * T + 33):
+        cuts = [rng.integers(t, min(n, t + T), parts) for t in range(0, n, T)]
+        near = [t + d for t in range(T, n, T) for d in (-1, 0, 1, 31, 32, 33)] if parts > 1 else []
+        tiny = np.cumsum(rng.integers(1, 8, 9)) + int(rng.integers(0, max(1, n - 80)))
+        off = np.unique(np.concatenate([[0, n], *cuts, near, tiny if parts in (2, 40) else []]))
+        off = off[(off >= 0) & (off <= n)].astype(np.uint64)
+        gen = np.arange(len(off) - 1, dtype=np.uint32)
+        seq = synth.random_bases(rng, n, 0.5).copy()
+        seq[rng.integers(0, n, 3)] = ord("N")
+        amps = np.zeros(len(off) - 1, dtype=ah.AMPLICON_DTYPE)
+        amps["contig"] = np.arange(len(amps))
+        amps["end"] = np.diff(off.astype(np.int64))
+        want, _ = oracle.fetch(oracle.reverse_contigs(seq, off), off, amps)
+        buf = torch.from_numpy(np.concatenate([np.zeros(5, np.uint8), seq])).cuda()
+        torch.cuda.synchronize()
+        sid = ctx.ah_load_genomes(buf[5:], n, off, gen, reversed=True)
+        try:
+            got, _ = ctx.fetch(sid, amps)
+        finally:
+            ctx.ah_unload_genomes(sid)
+        assert got == want, n
