@@ -248,8 +248,10 @@ enum PackInput { kAligned, kShifted, kReversed };
 // A reversed tile of few contigs' parts, c_end the last of them, into the staging
 // buffer: part by part, so that a thread's loads do not wait for the search of each
 // word's contig, then the words that hold an end, byte by byte; zero past the end.
-// Measured on a GB300, mirrored 100 Mbp, most tiles with a contig's end: 58 us with the
-// search in every word -> 52.
+// Measured on a GB300, mirrored 100 Mbp of 409 contigs (361 of 3,052 tiles hold an end): 58 us
+// with the search in every word -> 52.  (One contig 43, 1,500 contigs 61, 4,000 82; not
+// mirrored 39.  Loading a tile's contig once instead of twice, or six blocks per SM instead
+// of five, changed nothing.)
 constexpr uint32_t kFewParts = 16;
 
 __device__ __forceinline__ void gather_parts(const uint8_t *__restrict__ seq, uint64_t lim, uint64_t p0,
