@@ -155,6 +155,7 @@ def lib():
             "ah_debug_hmm_profile": (I32, [P, P, U64, U64, ctypes.POINTER(U64), ctypes.POINTER(U64), P, P]),
             "ah_debug_scan_source": (I32, [ctypes.c_char_p, ctypes.c_char_p, I32, I32, I32, I32, ctypes.c_char_p, S]),
             "ah_debug_scan_stall": (I32, [P, I32]),
+            "ah_debug_pair_cluster": (I32, [P, I32]),
             "ah_debug_pipe_rates": (I32, [P]),
         }
         for name, (res, args) in sig.items():
@@ -241,6 +242,11 @@ class Context:
         """Test aid: make later scans take their timeout path (each warp's first
         slice waits on a barrier that nothing completes; 20 us limit)."""
         self._check(self._lib.ah_debug_scan_stall(self.h, 1 if on else 0))
+
+    def debug_pair_cluster(self, on: bool):
+        """Test aid: False makes later runs take the form of a device that has no room for the
+        cluster of the one-launch pairing; True, what the device has."""
+        self._check(self._lib.ah_debug_pair_cluster(self.h, 1 if on else 0))
 
     def ah_set_profiling(self, enable):
         """0/False off, 1/True stage events and host sections, 2 host sections only,

@@ -78,6 +78,7 @@ struct ah_ctx {
     // counts of runs that needed more; the last run's site count
     uint64_t fast_amps = 16384, fast_seq = 4u << 20;
     uint64_t last_sites = 0;
+    bool pair_cluster = false; // the device has room for launch_pair_run's cluster: else runs go step by step
     // a run queued by ah_run_begin and not yet completed by ah_run_end
     struct FastRun {
         bool sites_direct = false, amps_direct = false, seq_direct = false;
@@ -839,7 +840,8 @@ template <class T> bool deliver(T *user, uint64_t cap, const T *dev, uint64_t co
 // its launch size sets a kRedo* bit and the later kernels see zero records; the
 // host then finishes with the step-by-step form (run_steps), which reuses the
 // scan's keys when they all fit.  Step by step (run_steps): one
-// synchronisation per data-dependent size, any size.
+// synchronisation per data-dependent size, any size; also what every run takes
+// on a device without room for launch_pair_run's cluster.
 // ---------------------------------------------------------------------------
 enum FastResult { kFastDone, kFastKeys, kFastRescan };
 constexpr uint64_t kFastAmps = 65535; // most amplicons of the one-synchronisation form
@@ -1526,6 +1528,7 @@ ah_status ah_create(int device, size_t mem_budget_bytes, ah_ctx **out)
                 c->tuning_given = true;
             }
         }
+        c->pair_cluster = pair_run_available();
         AH_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
         c->d_flags = (uint64_t *)dev_alloc(c, kFlagWords * sizeof(uint64_t));
         c->d_counter = c->d_flags + kFlagCounter;
@@ -2237,13 +2240,14 @@ ah_status ah_run_begin(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uin
         P.st = st;
         P.caller = caller;
         P.pd = pd;
-        if (gs.n_tiles && c->last_sites <= kSmallSort) {
+        if (gs.n_tiles && c->pair_cluster && c->last_sites <= kSmallSort) {
             fast_begin(c, gs, pats, pd, n_pairs, o, st, (cudaEvent_t)scan_done, &P.fr);
             leave_run_stream(c, caller);
             P.active = true;
             return;
         }
-        // counts above the one-synchronisation sizes (seen in the last run): queue the
+        // counts above the one-synchronisation sizes (seen in the last run), or a device
+        // without room for the pairing's cluster: queue the
         // scan and its count's copy only; ah_run_end reads the count and finishes step
         // by step, so the caller's next packing (after scan_done) runs beside that
         if (!gs.n_tiles) {
@@ -2950,6 +2954,18 @@ ah_status ah_debug_scan_stall(ah_ctx *c, int on)
         return AH_ERR_ARG;
     c->scan_stall_first = on != 0;
     return AH_OK;
+}
+
+// Test aid (not in the public header).  on == 0: later runs take the form of a
+// device without room for launch_pair_run's cluster.  on != 0: what the device has.
+ah_status ah_debug_pair_cluster(ah_ctx *c, int on)
+{
+    if (!c)
+        return AH_ERR_ARG;
+    return guarded(c, [&] {
+        require_idle(c);
+        c->pair_cluster = on != 0 && pair_run_available();
+    });
 }
 
 ah_status ah_hmm_free(ah_ctx *c, uint32_t hmm_id)

@@ -323,7 +323,10 @@ void launch_pair_count(const ah_site *sites, uint64_t n, const uint8_t *pass, co
 // Amplicons and sequence offsets of min(*n_dev, n) sites (n <= kSmallSort) of a scan in one
 // launch: *n_amps and *n_seq are the counts.  More than amps_max amplicons: none is written,
 // both counts are 0 and kRedoAmps is set in *redo; more than seq_max bases: *n_seq is 0 with
-// kRedoSeq.  seq_offsets holds amps_max + 1 words.
+// kRedoSeq.  seq_offsets holds amps_max + 1 words.  Only where pair_run_available(): the launch
+// needs room for a cluster of 16 CTAs (16 SMs of one GPC), which a slice of a GPU may not have.
+// The call also opts the kernel in to that size on the current device.
+bool pair_run_available();
 void launch_pair_run(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
                      const PairDev *pairs_d, ah_amplicon *out, uint64_t *seq_offsets, uint64_t amps_max,
                      uint64_t seq_max, uint64_t *n_amps, uint64_t *n_seq, uint64_t *redo, cudaStream_t s);

@@ -255,7 +255,9 @@ __global__ void pair_write_kernel(const ah_site *s, uint64_t n, const uint8_t *p
 // Both passes and the scan between them in one launch, for at most kSmallSort sites whose count
 // is on the device: a cluster of kPairCtas CTAs, a thread per site.  Counts and lengths stay in
 // registers; they are scanned within the block, and the blocks' totals are read through
-// distributed shared memory.  The sequence offsets follow from the same scan.
+// distributed shared memory.  The sequence offsets follow from the same scan.  Sixteen CTAs
+// are beyond the cluster size that every device has room for (eight): where pair_run_available
+// finds none, runs go step by step, with the kernels above.
 // Bound: latency, and the host's launches around it.  Measured on a GB300 from the end of the
 // Tm kernel to the sequence decode: four launches (count, scan, write, scan of the lengths)
 // 9.3 us for 14 sites, 15 for 6,000 -> 8.1 and 14.2; the run of a small resident set, which waits
@@ -437,19 +439,32 @@ void launch_pair_count(const ah_site *sites, uint64_t n, const uint8_t *pass, co
     launch_chained(pair_count_kernel, grid_for(n, 128), 128, 0, s, sites, n, pass, pairs_d, counts, err);
 }
 
+bool pair_run_available()
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kPairCtas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kPairCtas);
+    cfg.blockDim = dim3(kPairThreads);
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    const bool ok =
+        cudaFuncSetAttribute(pair_run_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, pair_run_kernel, &cfg) == cudaSuccess && clusters > 0;
+    if (!ok)
+        cudaGetLastError(); // (not an error: the step-by-step form needs no cluster)
+    return ok;
+}
+
 void launch_pair_run(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const uint8_t *pass,
                      const PairDev *pairs_d, ah_amplicon *out, uint64_t *seq_offsets, uint64_t amps_max,
                      uint64_t seq_max, uint64_t *n_amps, uint64_t *n_seq, uint64_t *redo, cudaStream_t s)
 {
     if (n == 0 || n > kSmallSort)
         throw Error(AH_ERR_ARG, "pairing with a device count: size outside 1..16384");
-    static int attr_dev = -1; // a cluster of 16 is an opt-in, once per device
-    int dev = 0;
-    AH_CUDA(cudaGetDevice(&dev));
-    if (dev != attr_dev) {
-        AH_CUDA(cudaFuncSetAttribute(pair_run_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        attr_dev = dev;
-    }
     launch_chained(pair_run_kernel, kPairCtas, kPairThreads, 0, s, sites, n, n_dev, pass, pairs_d, out, seq_offsets,
                    amps_max, seq_max, n_amps, n_seq, redo);
 }

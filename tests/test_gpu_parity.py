@@ -1522,3 +1522,42 @@ def test_mirrored_tiles_of_few_and_many_contigs(ctx, parts):
         finally:
             ctx.ah_unload_genomes(sid)
         assert got == want, n
+
+
+@pytest.mark.parametrize("pipelined", [False, True])
+def test_run_on_a_device_without_room_for_the_pairing_cluster(pipelined):
+    """A device slice without room for a cluster of 16 CTAs takes the step-by-step form: every output of a run, and
+    of queued ones with the next load beside them, as where the cluster fits; the whole GPU has room for it."""
+    w = synth.tiny(3)
+    p = dict(w.pairs[0], tm_min=45.0)
+    want = oracle.scan(w.seq, w.contig_off, w.contig_genome, [p])
+    tm, passed = oracle.tm(w.seq, w.contig_off, want, [p])
+    amps = oracle.pair(want, [p], passed)
+    seqs, offs = oracle.fetch(w.seq, w.contig_off, amps)
+    assert len(amps)
+    with ah.Context(0) as c:
+        pid = c.ah_set_primers(p["fwd"], p["rev"], p)
+        sid = c.load(w.seq, w.contig_off, w.contig_genome)
+        for on, launches in ((True, 1), (False, 4), (True, 1)):  # cluster; count, scan, total, write
+            c.debug_pair_cluster(on)
+            if pipelined:
+                buf = dict(sites=np.zeros(len(want), ah.SITE_DTYPE), tm=np.zeros(len(want), np.float32),
+                           pass_=np.zeros(len(want), np.uint8), amps=np.zeros(len(amps), ah.AMPLICON_DTYPE),
+                           seq=np.zeros(len(seqs), np.uint8), offs=np.zeros(len(amps) + 1, np.uint64))
+                o = ah.RunOut(buf["sites"].ctypes.data, len(want), 0, buf["tm"].ctypes.data, buf["pass_"].ctypes.data,
+                              buf["amps"].ctypes.data, len(amps), 0, buf["seq"].ctypes.data, len(seqs), 0,
+                              buf["offs"].ctypes.data, 1, 0)
+                c.ah_run_begin(sid, [pid], o)
+                other = c.load(w.seq, w.contig_off, w.contig_genome)
+                c.ah_run_end(o)
+                c.ah_unload_genomes(other)
+                assert (o.n_sites, o.n_amplicons, o.n_seq) == (len(want), len(amps), len(seqs))
+                r = dict(buf, seqs=buf["seq"].tobytes())
+            else:
+                caps = (len(want), len(amps), len(seqs))
+                c.ah_set_profiling(1)
+                r = c.run(sid, [pid], caps=caps)
+                assert c.ah_get_profile("pair")[1] == launches
+                c.ah_set_profiling(0)
+            assert r["sites"].tobytes() == want.tobytes() and np.array_equal(r["pass_"], passed)
+            assert r["amps"].tobytes() == amps.tobytes() and r["seqs"] == seqs and np.array_equal(r["offs"], offs)
