@@ -2851,6 +2851,24 @@ ah_status ah_hmm_tables(ah_ctx *c, uint32_t hmm_id, uint64_t *m_out, uint64_t *r
 
 namespace {
 
+// Device memory of one call: back in the allocator's cache when the call ends (its work done or,
+// on an error, waited for), so that it takes nothing from a memory budget between calls.
+struct CallBlock {
+    ah_ctx *c;
+    cudaStream_t st;
+    void *p = nullptr;
+    CallBlock(ah_ctx *c_, cudaStream_t st_) : c(c_), st(st_) {}
+    CallBlock(const CallBlock &) = delete;
+    CallBlock &operator=(const CallBlock &) = delete;
+    ~CallBlock()
+    {
+        if (!p)
+            return;
+        cudaStreamSynchronize(st);
+        dev_free(c, p, 0);
+    }
+};
+
 // ah_hmm_score (Viterbi) and ah_hmm_forward (Forward): the same checks, grouping and launch
 ah_status hmm_scores(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_amplicon *amplicons, uint64_t n,
                      float *score_out, void *stream, bool forward)
@@ -2898,15 +2916,16 @@ ah_status hmm_scores(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_ampli
         uint32_t *d_ord = (uint32_t *)scratch(c, "hmm_order", n * sizeof(uint32_t));
         AH_CUDA(cudaMemcpyAsync(d_ord, ord.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
         float *out = out_buf(c, "hmm_out", score_out, n);
-        // the wavefront's boundary buffers (at most 1/16 of a memory budget): fewer blocks where
-        // there is no room for them, and without room for one block's the kernel that needs none
+        // the wavefront's boundary buffers, a sixteenth of a memory budget where one block's fit
+        // in it: fewer blocks where there is no room for them, and without room for one block's
+        // the kernel that needs none
         uint64_t blocks = hmm_use_wave() ? hmm_wave_blocks(n, p.m, (int)max_len, c->sms) : 0;
         while (blocks > 1 && c->budget && hmm_scratch_bytes(blocks, p.m, (int)max_len) > c->budget / 16)
             blocks /= 2;
-        void *bnd = nullptr;
-        while (blocks && !bnd && hmm_scratch_bytes(blocks, p.m, (int)max_len)) {
+        CallBlock bnd(c, st);
+        while (blocks && !bnd.p && hmm_scratch_bytes(blocks, p.m, (int)max_len)) {
             try {
-                bnd = scratch(c, "hmm_bnd", hmm_scratch_bytes(blocks, p.m, (int)max_len));
+                bnd.p = dev_alloc(c, hmm_scratch_bytes(blocks, p.m, (int)max_len));
             } catch (const Error &e) {
                 if (e.status != AH_ERR_BUDGET && e.status != AH_ERR_OOM)
                     throw;
@@ -2915,7 +2934,7 @@ ah_status hmm_scores(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_ampli
         }
         if (blocks) {
             Stage sg(c, "hmm", st, 1);
-            launch_hmm_wave(a, d_ord, n, gs.planes, gs.contig_off, gs.n_contigs, p, (int)max_len, forward, bnd, blocks,
+            launch_hmm_wave(a, d_ord, n, gs.planes, gs.contig_off, gs.n_contigs, p, (int)max_len, forward, bnd.p, blocks,
                             out, c->d_err, c->sms, st);
         } else {
             Stage sg(c, "hmm", st, 1);

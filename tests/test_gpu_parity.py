@@ -1561,3 +1561,39 @@ def test_run_on_a_device_without_room_for_the_pairing_cluster(pipelined):
                 c.ah_set_profiling(0)
             assert r["sites"].tobytes() == want.tobytes() and np.array_equal(r["pass_"], passed)
             assert r["amps"].tobytes() == amps.tobytes() and r["seqs"] == seqs and np.array_equal(r["offs"], offs)
+
+
+def test_hmm_scores_leave_a_memory_budget_as_it_was():
+    """The wavefront's buffers are the call's own: after it, a set loads that fills what the budget leaves beside
+    everything the other kernel's call keeps."""
+    import torch
+    budget, m, n = 48 << 20, 300, 200
+    rng = np.random.default_rng(12)
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    ref = acgt[rng.integers(0, 4, m)].tobytes().decode()
+    seq = acgt[rng.integers(0, 4, n * m)]
+    amps = np.zeros(n, dtype=ah.AMPLICON_DTYPE)
+    amps["start"] = np.arange(n) * m
+    amps["end"] = amps["start"] + m
+    device = torch.from_numpy(seq).cuda()
+    torch.cuda.synchronize()
+    off, gen = np.array([0, len(seq)], np.uint64), np.zeros(1, np.uint32)
+    used = {}
+    for kernel in ("rows", "wave"):
+        with pytest.MonkeyPatch.context() as mp, ah.Context(0, budget) as c:
+            mp.setenv("AH_HMM_KERNEL", kernel)
+            sid = c.ah_load_genomes(device, len(seq), off, gen)
+            hid = c.hmm_build([ref, ref, ref[:-1]])
+            scores = c.hmm_score(sid, hid, amps)
+            assert np.isfinite(scores).all()
+            used[kernel] = c.device_bytes()
+            if kernel == "rows":
+                continue
+            tile = 4 * (1024 + 32) * 4
+            tiles = (budget - used["rows"] - 4096) // (tile + 8)
+            big = torch.full((tiles * 32768,), ord("A"), dtype=torch.uint8, device="cuda")
+            torch.cuda.synchronize()
+            sid2 = c.ah_load_genomes(big, len(big), np.array([0, len(big)], np.uint64), gen)
+            c.ah_unload_genomes(sid2)
+            assert c.hmm_score(sid, hid, amps).tobytes() == scores.tobytes()
+    assert used["wave"] > used["rows"] + (1 << 20)  # it did have buffers
