@@ -2895,11 +2895,13 @@ ah_status hmm_scores(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_ampli
             memcpy(h.data(), amplicons, n * sizeof(ah_amplicon));
         }
         uint32_t max_len = 1;
+        uint64_t letters = 0;
         for (const ah_amplicon &a : h) {
             require(a.contig < gs.n_contigs && a.start <= a.end &&
                         (uint64_t)a.end <= gs.contig_off_h[a.contig + 1] - gs.contig_off_h[a.contig],
                     AH_ERR_ARG, "ah_hmm_score: an amplicon lies outside its contig");
             max_len = std::max(max_len, a.end - a.start);
+            letters += a.end - a.start;
         }
         require(max_len <= kHmmMaxLetters / 4, AH_ERR_ARG,
                 "ah_hmm_score: amplicons longer than " + std::to_string(kHmmMaxLetters / 4) + " letters");
@@ -2919,7 +2921,8 @@ ah_status hmm_scores(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_ampli
         // the wavefront's boundary buffers, a sixteenth of a memory budget where one block's fit
         // in it: fewer blocks where there is no room for them, and without room for one block's
         // the kernel that needs none
-        uint64_t blocks = hmm_use_wave() ? hmm_wave_blocks(n, p.m, (int)max_len, c->sms) : 0;
+        const bool wave = hmm_use_wave(forward, n, letters, (int)max_len, p.m);
+        uint64_t blocks = wave ? hmm_wave_blocks(n, p.m, (int)max_len, c->sms) : 0;
         while (blocks > 1 && c->budget && hmm_scratch_bytes(blocks, p.m, (int)max_len) > c->budget / 16)
             blocks /= 2;
         CallBlock bnd(c, st);

@@ -21,7 +21,7 @@
 // the same recurrence with the maximum of the predecessors replaced by
 // log2(2^a + 2^b) (the log-sum semiring).  Two kernels compute the recurrence.
 //
-// hmm_wave_kernel (the default): a warp runs one stripe of 32 * K columns of one
+// hmm_wave_kernel (the default; hmm_use_wave): a warp runs one stripe of 32 * K columns of one
 // amplicon; lane l owns K consecutive columns with their nine move scores in
 // registers and, at step s, computes row i = s - l (an anti-diagonal
 // wavefront): M and I of its columns from its own previous row, the delete
@@ -44,8 +44,9 @@
 // 1,461 columns 22.8 -> 6.3 ms (1.36 T cells/s); Forward, 5,000 x 460 11.3 -> 1.0 ms
 // (1.05 T cells/s); one amplicon of 1,461 letters 1,577 -> 500 us (Viterbi).
 //
-// hmm_score_kernel (where a memory budget has no room for the wavefront's
-// buffers, and AH_HMM_KERNEL=rows): a block scores a group of amplicons of
+// hmm_score_kernel (Viterbi scores of amplicons much shorter than the profile,
+// both scores where a memory budget has no room for the wavefront's buffers, and
+// AH_HMM_KERNEL=rows): a block scores a group of amplicons of
 // similar length in lockstep, rows = sequence letters: each thread owns K
 // consecutive profile columns with their 13 scores in registers; M and I of a
 // row depend only on the previous row (the left neighbour's values come by
@@ -962,10 +963,24 @@ size_t hmm_scratch_bytes(uint64_t blocks, int m, int max_len)
     return wave_stripes(m) == 1 ? 0 : blocks * kWaveWarps * 2ull * (uint64_t)(max_len + 1) * sizeof(float4);
 }
 
-bool hmm_use_wave()
+// Viterbi scores of amplicons much shorter than the profile go to the kernel that walks rows: a
+// stripe of the wavefront takes 31 steps to fill and the stripes follow one another, while that
+// kernel has all columns at work from the first row.  The line, in letters of the mean amplicon
+// (of the longest where the call does not fill the GPU and its longest amplicon decides), is where
+// the two met on a GB300 or a little above; wavefront against rows, us: one amplicon,
+// 1,461 columns 20 letters 67, 34; 60 letters 102, 76; 150 letters 116, 188; 3,070 columns 100
+// letters 214, 127; 300 letters 262, 345; 5,000 amplicons, 3,070 columns 20 letters 1,214, 807;
+// 60 letters 1,954, 2,305.  (Forward scores stay with the wavefront: on odds they are more exact.)
+bool hmm_use_wave(bool forward, uint64_t n, uint64_t letters, int max_len, int m)
 {
-    const char *kern = getenv("AH_HMM_KERNEL");
-    return !(kern && strcmp(kern, "rows") == 0);
+    if (const char *kern = getenv("AH_HMM_KERNEL"))
+        if (!strcmp(kern, "rows") || !strcmp(kern, "wave"))
+            return kern[0] == 'w';
+    if (forward || n == 0)
+        return true;
+    constexpr uint64_t kFull = 608; // amplicons that fill the GPU: four blocks for each of 152 SMs
+    const uint64_t line = 20 * (uint64_t)wave_stripes(m) - 12;
+    return n <= kFull ? (uint64_t)max_len > line : letters > n * std::min<uint64_t>(line, 75);
 }
 
 void launch_hmm_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n, const uint32_t *planes,

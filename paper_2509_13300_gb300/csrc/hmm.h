@@ -7,8 +7,9 @@
 
 namespace ah {
 
-// False when AH_HMM_KERNEL=rows asks for the block-per-group kernel (a profiling aid).
-bool hmm_use_wave();
+// Whether the wavefront scores a call of n amplicons (their letters in all, the longest) against a
+// profile of m columns; AH_HMM_KERNEL=rows or wave decides instead (a profiling aid).
+bool hmm_use_wave(bool forward, uint64_t n, uint64_t letters, int max_len, int m);
 
 // Blocks the wavefront takes for n amplicons of at most max_len letters, and the
 // device scratch of `blocks` of them in bytes: two stripe-boundary buffers of

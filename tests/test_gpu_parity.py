@@ -1597,3 +1597,44 @@ def test_hmm_scores_leave_a_memory_budget_as_it_was():
             c.ah_unload_genomes(sid2)
             assert c.hmm_score(sid, hid, amps).tobytes() == scores.tobytes()
     assert used["wave"] > used["rows"] + (1 << 20)  # it did have buffers
+
+
+@pytest.mark.parametrize("m,n,line", [(300, 3, 28), (1100, 700, 75), (3000, 3, 228), (3000, 700, 75)])
+def test_viterbi_of_amplicons_shorter_than_the_profile(m, n, line, monkeypatch):
+    """Viterbi scores go by rows up to a line in letters (of the longest of few amplicons, of the mean of many) and by
+    the wavefront, which takes boundary buffers, above it; Forward always by the wavefront.  Scores at both sides of
+    the line against the oracle in fp64."""
+    rng = np.random.default_rng(m + n)
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    ref = acgt[rng.integers(0, 4, m)].tobytes().decode()
+    train = [ref, ref, ref[:-2]]
+    seq = acgt[rng.integers(0, 4, 100_000)]
+    seq[:m] = np.frombuffer(ref.encode(), np.uint8)
+    _, T, E = oracle.hmm_build(train)
+    fin = ~np.isinf(T)
+    pmean = float(np.concatenate([np.abs(T[fin]), np.abs(E[1:]).ravel()]).mean())
+    for L, wave in ((1, False), (line, False), (line + 1, True)):
+        amps = np.zeros(n, dtype=ah.AMPLICON_DTYPE)
+        amps["start"] = np.r_[7, rng.integers(0, len(seq) - L, n - 1)]
+        amps["end"] = amps["start"] + L
+        with ah.Context(0) as c:
+            sid = c.load(seq, np.array([0, len(seq)], np.uint64), np.zeros(1, np.uint32))
+            hid = c.hmm_build(train)
+            monkeypatch.setenv("AH_HMM_KERNEL", "rows")
+            c.hmm_score(sid, hid, amps)
+            monkeypatch.delenv("AH_HMM_KERNEL")
+            before = c.device_bytes()
+            got = c.hmm_score(sid, hid, amps).astype(np.float64)
+            assert (c.device_bytes() > before) == wave, L
+            before = c.device_bytes()
+            got_f = c.hmm_forward(sid, hid, amps).astype(np.float64)
+            assert wave or c.device_bytes() > before, L
+        some = [0, 1, n - 1]
+        seqs = [seq[amps["start"][i]:amps["end"][i]].tobytes().decode() for i in some]
+        want = np.array([oracle.hmm_viterbi(T, E, x) for x in seqs])
+        want_f = np.array([oracle.hmm_forward(T, E, x) for x in seqs])
+        # the bound of the parity test above: ten standard deviations of a walk of fp32 roundings
+        N = L + m
+        assert (np.abs(got[some] - want) <= 10.0 * np.sqrt(N) * 2.0 ** -24 * (np.abs(want) + N * pmean) + 1e-4).all()
+        assert (np.abs(got_f[some] - want_f) <=
+                10.0 * np.sqrt(N) * (2.0 ** -24 * (np.abs(want_f) + N * pmean) + 4 * 2.0 ** -23) + 1e-4).all()
