@@ -104,14 +104,14 @@ void launch_decode_keys(const uint64_t *keys, uint64_t n, int pbits, const uint6
 // [8, end_bit) -- (pair, flat position, primer, strand) names one site -- so
 // a key's place in canonical order is the number of keys below it.  Every block
 // sorts all keys into kRankBuckets ranges of equal width in shared memory (count,
-// scan, scatter; up to 1,024 keys stay one range), then ranks its own share of
-// them, a warp per key against the keys of its range, decodes them and writes each
-// record at its rank: no block waits for another, one launch.
+// scan, scatter; up to 1,024 keys stay one range; a range that holds too many is divided
+// into equal parts first), then ranks its own share of them, a warp per key against the
+// keys of its range or part, decodes them and writes each record at its rank: no block
+// waits for another, one launch.
 // Bound: latency (the count and the scatter are one shared-memory atomic per key
 // and thread).  Measured on a GB300, against the former n^2 compares of all keys
-// over the GPU: 6,000 sites 14 -> 7 us; 10,000 sites of 33 sort bits 25 -> 12; 14 sites 3.2 -> 3.4.
-// (All keys in one range: every key is compared with all, a third of the former
-// compares' instructions.)
+// over the GPU: 6,000 sites 14 -> 7 us; 10,000 sites of 33 sort bits 25 -> 12; 14 sites 3.2 -> 3.4;
+// 16,000 sites within 0.4 Mbp of a 400 Mbp set, all in one range, 44 -> 18 (undivided 71).
 // ---------------------------------------------------------------------------
 namespace ah {
 namespace {
@@ -119,6 +119,10 @@ namespace {
 constexpr int kRankThreads = 512;
 constexpr int kRankKeys = 16;    // keys of a thread held in registers; more are read twice
 constexpr int kRankBuckets = 1024;
+// A range of more keys is divided again (2,000 keys in one range: 10.0 us undivided, 11.6
+// divided; 6,000: 19 and 12); at most seven of the 16,384 keys' ranges are.
+constexpr uint32_t kRankCrowd = 2048;
+static_assert(kSmallSort / (kRankCrowd + 1) < 8, "a divided range has at least 128 parts");
 constexpr uint32_t kRankStageContigs = 4096; // contig offset tables up to this size are staged in shared memory
 
 // Shared memory: the keys by range, then the contig offsets when stage_contigs.
@@ -130,6 +134,11 @@ __global__ void __launch_bounds__(kRankThreads, 2)
     extern __shared__ __align__(16) uint64_t rank_smem[];
     __shared__ uint32_t end[kRankBuckets]; // keys of a range; then where it ends in cand
     __shared__ uint32_t wsum[kRankThreads / 32];
+    // divided ranges: their numbers (kNone: not divided), the keys of their parts, then where these end in cand
+    constexpr uint32_t kNone = 0xffu;
+    __shared__ uint8_t number[kRankBuckets];
+    __shared__ uint32_t part_end[kRankBuckets];
+    __shared__ uint32_t n_divided, part0[8]; // part0: a divided range's start in cand, less that of its parts
     __shared__ uint64_t query[kRankThreads];
     __shared__ uint32_t rank[kRankThreads];
     uint64_t *cand = rank_smem, *coff = rank_smem + n_arg;
@@ -159,6 +168,11 @@ __global__ void __launch_bounds__(kRankThreads, 2)
     if ((uint32_t)tid < q1 - q0) // the block's first queries
         query[tid] = keys[q0 + tid];
     const bool flat = n <= kRankBuckets; // few keys: one range
+    bool crowded = false;                // some range is divided
+    int part_bits = 0, part_shift = 0;   // parts of a divided range: 2^part_bits
+    auto part_of = [&](uint64_t key, uint32_t num) {
+        return num << part_bits | ((uint32_t)(key >> part_shift) & ((1u << part_bits) - 1u));
+    };
     if (flat) {
         for (uint32_t i = tid; i < n; i += kRankThreads)
             cand[i] = keys[i];
@@ -181,30 +195,89 @@ __global__ void __launch_bounds__(kRankThreads, 2)
         // exclusive scan: each thread its kRankBuckets / kRankThreads = 2 ranges
         static_assert(kRankBuckets == 2 * kRankThreads, "two ranges per thread");
         const uint32_t c0 = end[2 * tid], c1 = end[2 * tid + 1];
-        uint32_t incl = c0 + c1;
+        auto before_pair = [&](uint32_t sum) { // the threads' sums before this one's; whether a range is crowded
+            uint32_t incl = sum;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d)
-                incl += y;
-        }
-        if (lane == 31)
-            wsum[warp] = incl;
-        __syncthreads();
-        uint32_t before = incl - c0 - c1;
-        for (int w = 0; w < warp; ++w)
-            before += wsum[w];
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d)
+                    incl += y;
+            }
+            if (lane == 31)
+                wsum[warp] = incl;
+            crowded = __syncthreads_or(max(c0, c1) > kRankCrowd);
+            uint32_t before = incl - sum;
+            for (int w = 0; w < warp; ++w)
+                before += wsum[w];
+            return before;
+        };
+        const uint32_t before = before_pair(c0 + c1);
         end[2 * tid] = before;
         end[2 * tid + 1] = before + c0;
-        __syncthreads();
-        // scatter: `end` moves from a range's start to its end
+        if (!crowded) {
+            __syncthreads();
+            // scatter: `end` moves from a range's start to its end
 #pragma unroll
-        for (int u = 0; u < kRankKeys; ++u)
-            if (tid + u * kRankThreads < n)
-                cand[atomicAdd(&end[k[u] >> shift], 1u)] = k[u];
-        for (uint32_t i = tid + kRankKeys * kRankThreads; i < n; i += kRankThreads) {
-            const uint64_t key = keys[i];
-            cand[atomicAdd(&end[key >> shift], 1u)] = key;
+            for (int u = 0; u < kRankKeys; ++u)
+                if (tid + u * kRankThreads < n)
+                    cand[atomicAdd(&end[k[u] >> shift], 1u)] = k[u];
+            for (uint32_t i = tid + kRankKeys * kRankThreads; i < n; i += kRankThreads) {
+                const uint64_t key = keys[i];
+                cand[atomicAdd(&end[key >> shift], 1u)] = key;
+            }
+        } else {
+            // The crowded ranges share kRankBuckets parts.  (They hold more than 2^11 keys, which
+            // differ above bit 8, so a range spans more than 2^19 and a part is wider than a key.)
+            if (tid == 0)
+                n_divided = 0;
+            part_end[2 * tid] = part_end[2 * tid + 1] = 0;
+            __syncthreads();
+            auto divide = [&](uint32_t r, uint32_t start, uint32_t c) {
+                uint32_t num = kNone;
+                if (c > kRankCrowd) {
+                    num = atomicAdd(&n_divided, 1u);
+                    part0[num] = start;
+                    end[r] = start + c; // (its keys go by parts)
+                }
+                number[r] = (uint8_t)num;
+            };
+            divide(2 * tid, before, c0);
+            divide(2 * tid + 1, before + c0, c1);
+            __syncthreads();
+            part_bits = 10 - (32 - __clz(n_divided - 1)); // (one range: __clz(0) = 32)
+            part_shift = shift - part_bits;
+            auto count_part = [&](uint64_t key) {
+                const uint32_t num = number[key >> shift];
+                if (num != kNone)
+                    atomicAdd(&part_end[part_of(key, num)], 1u);
+            };
+#pragma unroll
+            for (int u = 0; u < kRankKeys; ++u)
+                if (tid + u * kRankThreads < n)
+                    count_part(k[u]);
+            for (uint32_t i = tid + kRankKeys * kRankThreads; i < n; i += kRankThreads)
+                count_part(keys[i]);
+            __syncthreads();
+            const uint32_t p0 = part_end[2 * tid], p1 = part_end[2 * tid + 1], at = before_pair(p0 + p1);
+            const uint32_t num = (2u * tid) >> part_bits; // (of both: a divided range has an even number of parts)
+            if ((2u * tid) == num << part_bits && num < n_divided)
+                part0[num] -= at;
+            __syncthreads();
+            if (num < n_divided) {
+                part_end[2 * tid] = part0[num] + at;
+                part_end[2 * tid + 1] = part0[num] + at + p0;
+            }
+            __syncthreads();
+            auto place = [&](uint64_t key) {
+                const uint32_t r = (uint32_t)(key >> shift), num = number[r];
+                cand[atomicAdd(num == kNone ? &end[r] : &part_end[part_of(key, num)], 1u)] = key;
+            };
+#pragma unroll
+            for (int u = 0; u < kRankKeys; ++u)
+                if (tid + u * kRankThreads < n)
+                    place(k[u]);
+            for (uint32_t i = tid + kRankKeys * kRankThreads; i < n; i += kRankThreads)
+                place(keys[i]);
         }
     }
     __syncthreads();
@@ -220,7 +293,13 @@ __global__ void __launch_bounds__(kRankThreads, 2)
         for (uint32_t j = warp; j < m; j += kRankThreads / 32) {
             const uint64_t key = query[j];
             const uint32_t b = (uint32_t)(key >> shift);
-            const uint32_t first = flat || !b ? 0u : end[b - 1], last = flat ? n : end[b];
+            uint32_t first = flat || !b ? 0u : end[b - 1], last = flat ? n : end[b];
+            if (crowded && number[b] != kNone) {
+                const uint32_t q = part_of(key, number[b]);
+                if (q & ((1u << part_bits) - 1u))
+                    first = part_end[q - 1];
+                last = part_end[q];
+            }
             uint32_t below = 0;
             for (uint32_t i = first + lane; i < last; i += 32)
                 below += cand[i] < key ? 1u : 0u;

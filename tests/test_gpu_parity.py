@@ -1638,3 +1638,45 @@ def test_viterbi_of_amplicons_shorter_than_the_profile(m, n, line, monkeypatch):
         assert (np.abs(got[some] - want) <= 10.0 * np.sqrt(N) * 2.0 ** -24 * (np.abs(want) + N * pmean) + 1e-4).all()
         assert (np.abs(got_f[some] - want_f) <=
                 10.0 * np.sqrt(N) * (2.0 ** -24 * (np.abs(want_f) + N * pmean) + 4 * 2.0 ** -23) + 1e-4).all()
+
+
+@pytest.mark.parametrize("n_sites", [1025, 3000, 8200, 16384])
+@pytest.mark.parametrize("where", ["first", "last", "two", "dozen", "mixed"])
+def test_rank_sort_of_sites_crowded_into_few_ranges(ctx, n_sites, where):
+    """Sites of a small run that lie in few of the 1,024 ranges of the key space: all in the first, all in the last
+    ones, in two places, in a dozen, and half in one place with the rest spread; a second pair has no site."""
+    rng = np.random.default_rng(n_sites)
+    fwd, rev = "ACGTTGCAAGCT", "GGATCCATTCAG"
+    n, room = 1 << 28, n_sites * 14 + 64
+    spans = {"first": [(0, 1.0)], "last": [(n - room, 1.0)], "two": [(1000, 0.5), (n // 3, 0.5)],
+             "dozen": [(n // 13 * j, 1 / 12) for j in range(12)], "mixed": [(n // 2, 0.5)]}[where]
+    at = [s0 + 13 * np.arange(int(round(n_sites * part))) for s0, part in spans]
+    if where == "mixed":
+        at.append(rng.choice(n // 64 - 2, n_sites // 2, replace=False) * 64)
+    at = np.unique(np.concatenate(at))[:n_sites]
+    words = np.stack([np.frombuffer(w.encode(), np.uint8) for w in
+                      (fwd, oracle_reverse_complement(fwd), rev, oracle_reverse_complement(rev))])
+    seq = np.full(n, ord("N"), np.uint8)
+    which = rng.integers(0, 4, len(at))
+    for p, w in zip(at, which):
+        seq[p:p + 12] = words[w]
+    whole = (seq[at[:, None] + np.arange(12)] == words[which]).all(axis=1)  # (a plant may lie over another)
+    off, gen = np.array([0, n // 5, n], np.uint64), np.array([0, 0], np.uint32)
+    pairs = [synth.pcr_params(f, r, k=0, min_len=30, max_len=200) for f, r in ((fwd, rev), ("TTTTTTTTTTTTT", "TTTTTTTTTTTTTT"))]
+    sid = ctx.load(seq, off, gen)
+    try:
+        pids = [ctx.ah_set_primers(p["fwd"], p["rev"], p) for p in pairs]
+        run = ctx.run(sid, pids, tm_filter=False, caps=(n_sites + 64, 8 * n_sites, 1 << 22))
+        alone = ctx.scan(sid, pids)
+    finally:
+        ctx.ah_unload_genomes(sid)
+    got = run["sites"]
+    contig = (at >= n // 5).astype(np.uint32)
+    end = np.where(contig, n, n // 5)
+    keep = (at + 12 <= end) & whole
+    order = np.array([(0, 0), (0, 1), (1, 0), (1, 1)])[which]  # a copy at p: primer and strand
+    assert keep.sum() > 1000 and len(got) == keep.sum()
+    assert np.array_equal(got["pos"], (at - np.where(contig, n // 5, 0))[keep]) and np.array_equal(got["contig"], contig[keep])
+    assert np.array_equal(got["primer"], order[keep, 0]) and np.array_equal(got["strand"], order[keep, 1])
+    assert not got["mm"].any() and not got["pair"].any() and not got["genome"].any()
+    assert alone.tobytes() == got.tobytes()
