@@ -254,17 +254,21 @@ __global__ void pair_write_kernel(const ah_site *s, uint64_t n, const uint8_t *p
 
 // Both passes and the scan between them in one launch, for at most kSmallSort sites whose count
 // is on the device: a cluster of kPairCtas CTAs, a thread per site.  Counts and lengths stay in
-// registers; they are scanned within the block, and the blocks' totals are read through
-// distributed shared memory.  The sequence offsets follow from the same scan.  Sixteen CTAs
-// are beyond the cluster size that every device has room for (eight): where pair_run_available
-// finds none, runs go step by step, with the kernels above.
+// registers; they are scanned within the warp, and every CTA scans the totals of all the cluster's
+// warps, read through distributed shared memory.  The sequence offsets follow from the same scan.
+// Groups of 32 sites go to the CTAs in turn: few sites, or the neighbouring sites of a hot spot
+// that lead many amplicons each, keep all 16 SMs at work (5,000 sites of 62,500 amplicons: 103
+// us with 1,024 neighbours per CTA, five SMs at work, 62 so; 6,000 sites 2 us less).  Sixteen CTAs are beyond the cluster size that
+// every device has room for (eight): where pair_run_available finds none, runs go step by step,
+// with the kernels above.
 // Bound: latency, and the host's launches around it.  Measured on a GB300 from the end of the
 // Tm kernel to the sequence decode: four launches (count, scan, write, scan of the lengths)
 // 9.3 us for 14 sites, 15 for 6,000 -> 8.1 and 14.2; the run of a small resident set, which waits
 // for the host's launches too, 93 -> 88.  A cluster of eight with two sites per thread took 18
 // us for 10,000 sites against 15.
-constexpr int kPairCtas = 16, kPairThreads = 1024, kPairRounds = (int)(kSmallSort / (kPairCtas * kPairThreads));
-static_assert(kPairRounds * kPairCtas * kPairThreads == kSmallSort, "whole rounds");
+constexpr int kPairCtas = 16, kPairThreads = 1024, kPairWarps = kPairThreads / 32;
+constexpr int kPairSets = kPairCtas * kPairWarps; // groups of 32 sites
+static_assert(kPairSets * 32 == kSmallSort && kPairSets <= kPairThreads && kPairCtas == 16, "a thread per site, and per set");
 
 __global__ void __cluster_dims__(kPairCtas, 1, 1) __launch_bounds__(kPairThreads)
     pair_run_kernel(const ah_site *s, uint64_t n_arg, const uint64_t *n_dev, const uint8_t *pass,
@@ -272,63 +276,58 @@ __global__ void __cluster_dims__(kPairCtas, 1, 1) __launch_bounds__(kPairThreads
                     uint64_t seq_max, uint64_t *n_amps, uint64_t *n_seq, uint64_t *redo)
 {
     namespace cg = cooperative_groups;
-    __shared__ uint64_t wcnt[kPairRounds][32], wlen[kPairRounds][32]; // per warp
-    __shared__ uint64_t tot[kPairRounds][2];                          // the block's amplicons and bases per round
+    __shared__ ulonglong2 warp_sum[kPairWarps];               // amplicons and bases of this CTA's warps
+    __shared__ ulonglong2 before_warp[kPairWarps];            // ... of all sites before them
+    __shared__ ulonglong2 set_sum[kPairSets / 32];            // ... of 32 sets
     const cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // inclusive over the lanes
+    auto scan2 = [&](uint64_t &c, uint64_t &l) {
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t x = __shfl_up_sync(0xffffffffu, c, d), y = __shfl_up_sync(0xffffffffu, l, d);
+            if (lane >= d) {
+                c += x;
+                l += y;
+            }
+        }
+    };
     chain_start();
     chain_wait();
     const uint64_t n = dev_count(n_arg, n_dev);
-    uint64_t cnt[kPairRounds], len[kPairRounds], icnt[kPairRounds], ilen[kPairRounds]; // own; inclusive in the warp
-#pragma unroll
-    for (int r = 0; r < kPairRounds; ++r) {
-        const uint64_t a = (uint64_t)(r * kPairCtas + rank) * kPairThreads + tid;
-        cnt[r] = len[r] = 0;
-        if (a < n)
-            cnt[r] = count_group(s, n, pass, pairs, a, &len[r]);
-        icnt[r] = cnt[r];
-        ilen[r] = len[r];
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint64_t c = __shfl_up_sync(0xffffffffu, icnt[r], d), l = __shfl_up_sync(0xffffffffu, ilen[r], d);
-            if (lane >= d) {
-                icnt[r] += c;
-                ilen[r] += l;
-            }
-        }
-        if (lane == 31) {
-            wcnt[r][warp] = icnt[r];
-            wlen[r][warp] = ilen[r];
-        }
+    const uint64_t a = (uint64_t)(warp * kPairCtas + rank) * 32 + lane; // set (warp, rank) of the sites
+    uint64_t cnt = 0, len = 0;
+    if (a < n)
+        cnt = count_group(s, n, pass, pairs, a, &len);
+    uint64_t icnt = cnt, ilen = len; // inclusive in the warp
+    scan2(icnt, ilen);
+    if (lane == 31)
+        warp_sum[warp] = make_ulonglong2(icnt, ilen);
+    cluster.sync(); // every warp's totals
+    uint64_t c = 0, l = 0;
+    ulonglong2 own = make_ulonglong2(0, 0); // of set tid, in the sites' order
+    if (tid < kPairSets) {
+        own = *cluster.map_shared_rank(&warp_sum[tid / kPairCtas], tid % kPairCtas);
+        c = own.x;
+        l = own.y;
+        scan2(c, l);
+        if (lane == 31)
+            set_sum[warp] = make_ulonglong2(c, l);
     }
     __syncthreads();
-    if (warp < 2 * kPairRounds) { // inclusive over the warps: one warp per round and quantity
-        uint64_t *w = warp & 1 ? wlen[warp >> 1] : wcnt[warp >> 1];
-        uint64_t v = w[lane];
+    uint64_t total = 0, bases = 0; // of all sites
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xffffffffu, v, d);
-            if (lane >= d)
-                v += y;
+    for (int w = 0; w < kPairSets / 32; ++w) {
+        if (w == warp) {
+            c += total;
+            l += bases;
         }
-        w[lane] = v;
-        if (lane == 31)
-            tot[warp >> 1][warp & 1] = v;
+        total += set_sum[w].x;
+        bases += set_sum[w].y;
     }
-    cluster.sync(); // every block's totals
-    uint64_t total = 0, bases = 0, bcnt[kPairRounds], blen[kPairRounds]; // of all sites; before this block's round
-#pragma unroll
-    for (int r = 0; r < kPairRounds; ++r)
-        for (int q = 0; q < kPairCtas; ++q) {
-            const uint64_t *t = cluster.map_shared_rank(&tot[r][0], q);
-            if (q == rank) {
-                bcnt[r] = total;
-                blen[r] = bases;
-            }
-            total += t[0];
-            bases += t[1];
-        }
-    cluster.sync(); // no block leaves while its totals are read
+    if (tid < kPairSets && tid % kPairCtas == rank)
+        before_warp[tid / kPairCtas] = make_ulonglong2(c - own.x, l - own.y);
+    cluster.sync(); // before_warp; and no block leaves while its totals are read
     const bool fits = total <= amps_max;
     if (rank == 0 && tid == 0) {
         *n_amps = fits ? total : 0;
@@ -338,15 +337,9 @@ __global__ void __cluster_dims__(kPairCtas, 1, 1) __launch_bounds__(kPairThreads
         if (!fits || !seq_fits)
             atomicOr((unsigned long long *)redo, (unsigned long long)(!fits ? kRedoAmps : kRedoSeq));
     }
-    if (!fits)
-        return;
-#pragma unroll
-    for (int r = 0; r < kPairRounds; ++r)
-        if (cnt[r]) {
-            const uint64_t o = bcnt[r] + (warp ? wcnt[r][warp - 1] : 0) + icnt[r] - cnt[r];
-            const uint64_t l = blen[r] + (warp ? wlen[r][warp - 1] : 0) + ilen[r] - len[r];
-            write_group(s, n, pass, pairs, (uint64_t)(r * kPairCtas + rank) * kPairThreads + tid, o, l, out, qoff, amps_max);
-        }
+    if (fits && cnt)
+        write_group(s, n, pass, pairs, a, before_warp[warp].x + icnt - cnt, before_warp[warp].y + ilen - len, out, qoff,
+                    amps_max);
 }
 
 __global__ void total_kernel(const uint64_t *offs, const uint64_t *counts, uint64_t n, uint64_t *out)

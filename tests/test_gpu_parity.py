@@ -1680,3 +1680,38 @@ def test_rank_sort_of_sites_crowded_into_few_ranges(ctx, n_sites, where):
     assert np.array_equal(got["primer"], order[keep, 0]) and np.array_equal(got["strand"], order[keep, 1])
     assert not got["mm"].any() and not got["pair"].any() and not got["genome"].any()
     assert alone.tobytes() == got.tobytes()
+
+
+@pytest.mark.parametrize("spots,left,right", [(1, 1, 1), (1, 31, 33), (16, 16, 16), (25, 25, 25), (63, 30, 34),
+                                              (512, 4, 4), (2048, 4, 4), (40, 90, 90)])
+def test_run_of_hot_spots_that_lead_many_amplicons(ctx, spots, left, right):
+    """Neighbouring sites that pair with one another, from one amplicon to more than the one-launch form holds: groups
+    of 32 sites lie over all CTAs of the pairing's cluster, up to its last site; amplicons, sequences and offsets as
+    the oracle gives them."""
+    rng = np.random.default_rng(spots)
+    fwd, rev = "ACGTTGCAAGCT", "GGATCCATTCAG"
+    step = 14 * (left + right) + 2200
+    n = spots * step + 500
+    seq = np.full(n, ord("T"), np.uint8)
+    words = [np.frombuffer(w.encode(), np.uint8) for w in (fwd, oracle_reverse_complement(rev))]
+    for j in range(spots):
+        for i in range(left + right):
+            at = j * step + 14 * i + (int(rng.integers(100, 300)) if i >= left else 0)
+            at = min(at, (j + 1) * step - 2000)
+            seq[at:at + 12] = words[i >= left]
+    off = np.array([0, n // step // 2 * step, n], np.uint64)
+    gen = np.zeros(2, np.uint32)
+    pair = synth.pcr_params(fwd, rev, k=0, min_len=30, max_len=14 * (left + right) + 400)
+    want = oracle.scan(seq, off, gen, [pair])
+    amps = oracle.pair(want, [pair])
+    seqs, offs = oracle.fetch(seq, off, amps)
+    assert len(want) and len(amps)
+    sid = ctx.load(seq, off, gen)
+    try:
+        pid = ctx.ah_set_primers(fwd, rev, pair)
+        for caps in ((len(want), len(amps), len(seqs)), (0, 0, 0)):
+            r = ctx.run(sid, [pid], tm_filter=False, caps=caps)
+            assert r["sites"].tobytes() == want.tobytes() and r["amps"].tobytes() == amps.tobytes()
+            assert r["seqs"] == seqs and np.array_equal(r["offs"], offs)
+    finally:
+        ctx.ah_unload_genomes(sid)
