@@ -1826,14 +1826,15 @@ static ah_status load_impl(ah_ctx *c, const uint8_t *seq, uint64_t n_bases, cons
                 ah_ctx::PinSlot &gsl = pin_slot(c, run_bytes + tab_bytes);
                 memcpy(gsl.p, two->gaps, run_bytes);
                 uint2 *tg = reinterpret_cast<uint2 *>(gsl.p + run_bytes);
-                uint64_t gi = 0, ge = 0; // the first run ending after the tile's start, the first starting past its reach
+                uint64_t gi = 0; // the first run that ends past the tile's start
                 for (uint64_t t = 0; t < gs->n_tiles; ++t) {
-                    const uint64_t p0 = t * kTileBases;
-                    while (gi < two->n_gaps && two->gaps[2 * gi] + two->gaps[2 * gi + 1] <= p0)
+                    const uint64_t p1 = (t + 1) * kTileBases, first = gi;
+                    while (gi < two->n_gaps && two->gaps[2 * gi] + two->gaps[2 * gi + 1] <= p1)
                         ++gi;
-                    while (ge < two->n_gaps && two->gaps[2 * ge] < p0 + kTileBases + 32)
+                    uint64_t ge = gi; // and of the runs past those, the ones that start in the tile or its extension
+                    while (ge < two->n_gaps && two->gaps[2 * ge] < p1 + 32)
                         ++ge;
-                    tg[t] = make_uint2((uint32_t)gi, (uint32_t)std::max(gi, ge));
+                    tg[t] = make_uint2((uint32_t)first, (uint32_t)ge);
                 }
                 launch_copy_words((const uint32_t *)gsl.dp, (uint32_t *)gaps_d, (run_bytes + tab_bytes) / 4, st);
                 AH_CUDA(cudaEventRecord(gsl.ev, st));
