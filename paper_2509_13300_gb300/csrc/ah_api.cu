@@ -893,7 +893,7 @@ void fast_begin(ah_ctx *c, const GenomeSet &gs, const std::vector<ScanPattern> &
                                 gs.n_contigs, gs.contig_genome, sites, F + kFlagSites, F + kFlagRedo, st);
     }
     {
-        Stage sg(c, "tm", st, 2);
+        Stage sg(c, "tm", st, tm_launches(ns_max, tm_few_exact(c)));
         launch_tm(sites, ns_max, F + kFlagSites, pd, (int)n_pairs, gs.planes, gs.contig_off, tm, pass, queue,
                   (uint32_t *)(F + kFlagTmQueue), tm_seg_max(c), tm_few_exact(c), c->d_err, st);
     }
@@ -993,7 +993,7 @@ void run_steps(ah_ctx *c, const GenomeSet &gs, const PairDev *pd, uint32_t n_pai
         // canonical sites, Tm, pair counts (synchronisation: the amplicon count)
         sort_decode(c, gs, n_pairs, keys, ns, sites, st);
         {
-            Stage sg(c, "tm", st, 2);
+            Stage sg(c, "tm", st, tm_launches(ns, tm_few_exact(c)));
             uint32_t *q = (uint32_t *)scratch(c, "tm_queue", 2 * ns * sizeof(uint32_t));
             launch_tm(sites, ns, nullptr, pd, (int)n_pairs, gs.planes, gs.contig_off, tm, pass, q,
                       (uint32_t *)(c->d_flags + kFlagTmQueue), tm_seg_max(c), tm_few_exact(c), c->d_err, st);
@@ -1214,7 +1214,7 @@ void group_device(ah_ctx *c, const GenomeSet &gs, uint32_t pid, int k, const std
     uint8_t *pass = (uint8_t *)scratch(c, "serve_pass", ns);
     uint32_t *q = (uint32_t *)scratch(c, "tm_queue", 2 * ns * sizeof(uint32_t));
     {
-        Stage sg(c, "tm", st, 2);
+        Stage sg(c, "tm", st, tm_launches(ns, tm_few_exact(c)));
         launch_tm(sites, ns, nullptr, pd, 1, gs.planes, gs.contig_off, tm, pass, q,
                   (uint32_t *)(c->d_flags + kFlagTmQueue), tm_seg_max(c), tm_few_exact(c), c->d_err, st);
     }
@@ -2376,7 +2376,7 @@ ah_status ah_tm_sweep(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint
         } // (the kernels below leave records that failed it alone; check_flags reports them)
         float *tm = (float *)scratch(c, "sweep_tm", std::max<uint64_t>(n_sites, 1) * sizeof(float));
         if (n_sites) {
-            Stage sg(c, "tm", st, 2);
+            Stage sg(c, "tm", st, tm_launches(n_sites, tm_few_exact(c)));
             uint32_t *q = (uint32_t *)scratch(c, "tm_queue", 2 * n_sites * sizeof(uint32_t));
             launch_tm(s, n_sites, nullptr, pd, (int)n_pairs, gs.planes, gs.contig_off, tm, nullptr, q,
                       (uint32_t *)(c->d_flags + kFlagTmQueue), tm_seg_max(c), tm_few_exact(c), c->d_err, st);
@@ -2550,7 +2550,7 @@ ah_status ah_tm(ah_ctx *c, uint32_t set_id, const uint32_t *pair_ids, uint32_t n
         float *tm = out_buf(c, "tm_out", tm_out, n);
         uint8_t *ps = pass_out ? out_buf(c, "pass_out", pass_out, n) : nullptr;
         {
-            Stage sg(c, "tm", st, 2);
+            Stage sg(c, "tm", st, tm_launches(n, tm_few_exact(c)));
             uint32_t *q = (uint32_t *)scratch(c, "tm_queue", 2 * n * sizeof(uint32_t));
             launch_tm(s, n, nullptr, pd, (int)n_pairs, gs.planes, gs.contig_off, tm, ps, q,
                       (uint32_t *)(c->d_flags + kFlagTmQueue), tm_seg_max(c),

@@ -302,6 +302,8 @@ struct PairDev {
 void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const PairDev *pairs_d, int n_pairs, const uint32_t *planes,
                const uint64_t *contig_off, float *tm_out, uint8_t *pass_out, uint32_t *queue, uint32_t *queue_n,
                int seg_max, bool few_exact, int *err, cudaStream_t s);
+// number of kernels launch_tm launches
+int tm_launches(uint64_t n, bool few_exact);
 
 // Tm-threshold sweep (tm.cu): per-site pass bits for n_thr <= 64 thresholds
 // (thr_d: deg C, device), then per threshold the amplicons whose two sites

@@ -1386,7 +1386,17 @@ __global__ void sweep_genomes_kernel(const unsigned long long *__restrict__ gmas
     add_counts(all, n_thr, lane, gcount);
 }
 
+// Whether one thread takes a site (tm_fast_kernel, then the four-lane kernel on the sites near the
+// threshold).  Few sites (a latency-bound launch): the four-lane kernel alone finishes first; many:
+// one thread per site has 6 times its rate on 3.2 M sites.  On a GB300, the four-lane kernel alone
+// against the two: 16,384 sites 22 us against 15 + 14 (15 + 2 when no site is deferred), 24,000 25
+// against 15 + 14, 32,767 44 against 15 + 14; the line lies where they meet with sites deferred.
+constexpr uint64_t kFastMinSites = 24576;
+bool tm_fast(uint64_t n, bool few_exact) { return few_exact && n >= kFastMinSites; }
+
 } // namespace
+
+int tm_launches(uint64_t n, bool few_exact) { return n == 0 ? 0 : few_exact && !tm_fast(n, few_exact) ? 1 : 2; }
 
 void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const PairDev *pairs_d, int n_pairs,
                const uint32_t *planes, const uint64_t *contig_off, float *tm_out, uint8_t *pass_out, uint32_t *queue,
@@ -1424,14 +1434,9 @@ void launch_tm(const ah_site *sites, uint64_t n, const uint64_t *n_dev, const Pa
                     b = std::min(b, atoi(e));
         cached_dev = dev;
     }
-    constexpr uint64_t kFastMinSites = 24576;
-    const bool fast = few_exact && n >= kFastMinSites;
+    const bool fast = tm_fast(n, few_exact);
     if (!n_dev && (fast || !few_exact)) // queue length, deferred sites
         AH_CUDA(cudaMemsetAsync(queue_n, 0, 2 * sizeof(uint64_t), s));
-    // Few sites (a latency-bound launch): the four-lane kernel alone finishes first; many
-    // sites: one thread per site (6x the four-lane rate on 3.2 M sites).  On a GB300:
-    // 16,384 sites 22 us against 15 + 14 for the two kernels below (2 when no site is
-    // deferred), 24,000 sites 25 against 15 + 14, 32,767 sites 44 against 15 + 14.
     if (fast) {
         // every site in one thread; those near tm_min go to the four-lane kernel below
         uint32_t *defer = queue + n;

@@ -1715,3 +1715,29 @@ def test_run_of_hot_spots_that_lead_many_amplicons(ctx, spots, left, right):
             assert r["seqs"] == seqs and np.array_equal(r["offs"], offs)
     finally:
         ctx.ah_unload_genomes(sid)
+
+
+def test_launch_counts_of_the_tm_stage_and_of_a_small_run():
+    """The profile counts the kernels that a call launches: a small run is five (scan, site sort, Tm, pairing,
+    sequences); the Tm stage one below the thread-per-site line, two from there on, and two under a table whose
+    entropies may reach the concentration term (where many sites may need every oligo)."""
+    w = synth.tiny(5)
+    p = dict(w.pairs[0], tm_min=40.0)
+    tables = {v: ah.NNTable() for v in (1.0, 10.0)}  # L - 1 stacks of 1 stay below it, of 10 do not
+    for v, t in tables.items():
+        t.stack_dS[:] = [v] * 256
+    with ah.Context(0) as c:
+        sid = c.load(w.seq, w.contig_off, w.contig_genome)
+        pid = c.ah_set_primers(p["fwd"], p["rev"], p)
+        c.ah_set_profiling(1)
+        c.run(sid, [pid], caps=(64, 64, 1 << 16))
+        assert c.ah_get_profile(None)[1] == 5
+        for n, entropy, want in ((1, None, 1), (24575, None, 1), (24576, None, 2), (7, 1.0, 1), (7, 10.0, 2)):
+            if entropy:
+                c.ah_set_nn_table(pid, tables[entropy])
+            sites = np.zeros(n, dtype=ah.SITE_DTYPE)
+            sites["pos"] = np.arange(n) % 1000
+            c.ah_set_profiling(1)
+            c.tm(sid, [pid], sites)
+            assert c.ah_get_profile("tm")[1] == want, n
+        c.ah_set_profiling(0)
