@@ -134,10 +134,10 @@ __device__ __forceinline__ bool in_window(const PairDev &pd, uint32_t s_pos, con
 __device__ __forceinline__ int orient_of(int x, int y) { return (x == 0 && y == 1) ? 0 : (x == 1 && y == 0) ? 1 : (x == 0 ? 2 : 3); }
 
 // Amplicons of the group that site a leads, and the sum of their lengths.
-__device__ __forceinline__ uint32_t count_group(const ah_site *s, uint64_t n, const uint8_t *pass,
+__device__ __forceinline__ uint64_t count_group(const ah_site *s, uint64_t n, const uint8_t *pass,
                                                 const PairDev *__restrict__ pairs, uint64_t a, uint64_t *bases)
 {
-    uint32_t cnt = 0;
+    uint64_t cnt = 0;
     *bases = 0;
     const Group g = make_group(s, n, pass, pairs, a);
     if (!g.valid)
