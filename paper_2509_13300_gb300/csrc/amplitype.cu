@@ -4,8 +4,9 @@
 //
 // Variants: each amplicon's sequence (as ah_fetch returns it: RF reverse-
 // complemented, N for any non-ACGT letter) is hashed straight from the packed
-// planes with two polynomial hashes modulo the Mersenne prime 2^61 - 1;
-// amplicons with equal hash pairs are one variant.  Variants, and then
+// planes with two polynomial hashes modulo the Mersenne prime 2^61 - 1 (the second
+// with the length's low three bits beside it); amplicons with equal pairs are one
+// variant.  Variants, and then
 // amplitypes, are numbered by first occurrence: every element enters a hash
 // table in device memory (open addressing) that keeps the smallest index seen
 // per key, so the elements that are their key's smallest are the first
@@ -15,12 +16,13 @@
 // words per (variant, copies) pair (two independent sums, order-free), the
 // copies counted in a second table keyed by (genome, variant).
 //
-// Bound: launches, memory latency and, in the hashing, the planes' reads from L2 (16
-// bytes per letter; a sixth fewer instructions per letter changed nothing).  Measured on a GB300, 65,000 amplicons of ~1,500 letters:
-// hashing 399 us (a lane per 1/32 of an amplicon, letter by letter) -> 122; the
-// rest of a call 3 x 16 radix-sort passes and ~60 small launches, 0.7 ms -> 15
-// launches, 0.13 ms.  (Fewer blocks for the kernels that enter a table, so that
-// common keys are entered before most elements look: 39 -> 58 us, not kept.)
+// Bound: launches, memory latency and, in the hashing, the planes' reads from L2
+// (16 bytes per letter; a sixth fewer instructions per letter changed nothing).
+// Measured on a GB300, 65,000 amplicons of ~1,500 letters: hashing 399 us (a lane per
+// 1/32 of an amplicon, letter by letter) -> 122; the rest of a call 3 x 16 radix-sort
+// passes and ~60 small launches, 0.7 ms -> 15 launches, 0.13 ms.  (Fewer blocks for the
+// kernels that enter a table, so that common keys are entered before most elements
+// look: 39 -> 58 us, not kept.)
 #include <algorithm>
 
 #include "ah_internal.h"
@@ -160,8 +162,9 @@ __device__ __forceinline__ uint64_t group_digit(const uint32_t *__restrict__ pla
 // letters is 32 digits of 60 bits, one per lane (four coalesced loads per 32
 // letters: consecutive positions lie in consecutive words), each times its
 // power of the base; hash = the groups in order (zeros beyond the end), then
-// the length.  A bad record sets *err.  Bound by the reads: 1.6 GB from L2 in 121 us
-// for 65,000 amplicons of ~1,500 letters.
+// the length.  (Neither word is ever the empty key: the low 61 bits are below 2^61 - 1.)
+// A bad record sets *err.  Bound by the reads: 1.6 GB from L2 in 121 us for 65,000
+// amplicons of ~1,500 letters.
 __global__ void amp_hash_kernel(const ah_amplicon *__restrict__ a, uint64_t n, const uint32_t *__restrict__ planes,
                                 const uint64_t *__restrict__ contig_off, const uint32_t *__restrict__ contig_genome,
                                 uint32_t n_contigs, uint64_t *__restrict__ hash1, uint64_t *__restrict__ hash2,
@@ -196,7 +199,7 @@ __global__ void amp_hash_kernel(const ah_amplicon *__restrict__ a, uint64_t n, c
         }
         if (lane == 0) {
             hash1[i] = mod61(mulmod61(h1, kB1) + len);
-            hash2[i] = mod61(mulmod61(h2, kB2) + len);
+            hash2[i] = mod61(mulmod61(h2, kB2) + len) | (uint64_t)len << 61; // its low three bits beside the hash
         }
     }
 }
