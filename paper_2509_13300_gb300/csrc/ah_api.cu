@@ -2922,7 +2922,7 @@ ah_status hmm_scores(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_ampli
         // the wavefront's boundary buffers, a sixteenth of a memory budget where one block's fit
         // in it: fewer blocks where there is no room for them, and without room for one block's
         // the kernel that needs none
-        const bool wave = hmm_use_wave(forward, n, letters, (int)max_len, p.m);
+        const bool wave = hmm_use_wave(p, forward, n, letters, (int)max_len);
         uint64_t blocks = wave ? hmm_wave_blocks(n, p.m, (int)max_len, c->sms) : 0;
         while (blocks > 1 && c->budget && hmm_scratch_bytes(blocks, p.m, (int)max_len) > c->budget / 16)
             blocks /= 2;

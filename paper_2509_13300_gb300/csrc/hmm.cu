@@ -35,7 +35,8 @@
 // idle for a whole amplicon.  Forward scores are computed as odds (sums and
 // products, no logarithms: the log-sum took an exp2 and a log2 per term, and
 // its roundings of scores of ~1,000 bits were the larger error) with a common
-// exponent per lane, brought up to date every fourth row.
+// exponent per lane, brought up to date every fourth row and wherever what comes
+// in from the left outweighs the lane by far.
 // Bound: issue slots, with latency next (three warps per scheduler by registers):
 // 143 instructions per step of 256 cells for Viterbi, 157 for Forward, issue 0.68
 // and 0.66.  K = 8 needs half the steps of K = 4 per profile; packed two-wide
@@ -189,6 +190,10 @@ void build_profile(const char *seqs, const uint64_t *off, uint64_t n, HmmProfile
                 p.e[(size_t)j * 4 + l] = (float)std::log2((ce[(size_t)j * 4 + l] + 1.0) / tot * 4.0);
         }
     }
+    p.rare = 0.0f;
+    for (float t : p.t)
+        if (std::isfinite(t))
+            p.rare = std::max(p.rare, -t);
 }
 
 namespace {
@@ -510,7 +515,8 @@ constexpr uint64_t kWaveWaitNs = 2000000000ull; // bound of a wait on another wa
 // extended by a move; acc(s, a, t): the sum of s and a extended by t; acc3: the
 // sum of three extended paths.
 struct WaveMax {
-    static constexpr bool kScaled = false;
+    static constexpr bool kScaled = false, kWatch = false;
+    static constexpr int kTop = 0;
     static constexpr float kZero = -INFINITY, kOne = 0.0f;
     __device__ static __forceinline__ float ext(float a, float t) { return a + t; }
     __device__ static __forceinline__ float acc(float s, float a, float t) { return fmaxf(s, a + t); }
@@ -519,8 +525,9 @@ struct WaveMax {
         return fmaxf(fmaxf(a + ta, b + tb), c + tc); // one three-input maximum
     }
 };
-struct WaveSum {
-    static constexpr bool kScaled = true;
+template <bool Watch> struct WaveSum {
+    static constexpr bool kScaled = true, kWatch = Watch;
+    static constexpr int kTop = Watch ? 80 : -24;
     static constexpr float kZero = 0.0f, kOne = 1.0f;
     __device__ static __forceinline__ float ext(float a, float t) { return a * t; }
     __device__ static __forceinline__ float acc(float s, float a, float t) { return fmaf(a, t, s); }
@@ -531,19 +538,32 @@ struct WaveSum {
 };
 
 // Exponents of the scaled odds: a value is mantissa * 2^E with one E per lane.
-// Every four rows a lane's largest mantissa is brought to 2^kTop.  A row grows
-// it by at most 2^2 (an emission is at most 4, the moves into a cell sum to at
-// most 1 per state left), and what comes in from the left lane is at most
-// 2^kFar above the lane's own level (beyond that the lane takes the left one's
-// exponent), so it stays below 2^128; the smallest normal float lies 156 bits
-// below it.  Within a lane's eight columns a cell more than ~75 bits below the
-// largest adds nothing a float could hold to any later cell (the larger one
-// reaches the same cells by at most eight deletions or insertions, whose
-// probabilities are at least 1 / (training sequences + 3)), so what underflows
-// is no loss.
-constexpr int kTop = 30, kFar = 80, kRise = 24;
+// Every four rows a lane's largest mantissa is brought to 2^kTop, and the factor
+// 2^(left lane's exponent - this one's) for what comes in from the left is renewed.
+// With p = 2^-c the rarest move's probability:
+//   - A lane's smallest cell that counts is the deletion state of its last column,
+//     through which a row's mass must go where no letters are left for it: up to
+//     eight moves below the largest cell, which itself may fall by a move a row until
+//     the next settling and lie one below what came in: 2^(kTop - 13 c).
+//   - Its largest: a lane holds at least what deletions bring it within a row, so
+//     its left neighbour lies at most 2^(11 c + 6) above it (eight columns, a lane of
+//     lag, a row of growth).  In four rows mass grows by four letters' 4^4 and a sum
+//     over the cells of two lanes, 2^15 in all, and by what four matches save against
+//     deletions, a move each for their columns and for those after them, 2^(8 c).
+// Without a look at what comes in (kWatch false), kTop + 19 c + 21 <= 127 and kTop -
+// 13 c >= -126: kTop = -24 holds for c <= kCalmBits (about 100 training sequences).
+// Only the first 32 steps of a stripe, in which mass reaches each lane for the first
+// time, need that look then.  Rarer moves: in every step (a tenth more instructions),
+// and a lane that is outweighed by more than 2^kRise, or whose left neighbour's
+// exponent lies kHot above its own, takes the level of what comes in: four rows end
+// below 2^(kTop + kRise + 13), and kTop = 80 leaves 13 c <= 206: c <= kRareBits.  Moves
+// rarer than that (some 32,000 training sequences) go by logarithms
+// (hmm_score_kernel).  (With kTop = 30 and the left lane's exponent taken over where
+// it lay 80 above, profiles with moves rarer than 2^-8 could lose mass or overflow.)
+constexpr int kRise = 24, kHot = 100;
+constexpr float kCalmBits = 6.8f, kRareBits = 15.0f;
 constexpr int kNoMass = -(1 << 20); // exponent of a lane that holds only zeros
-__device__ __forceinline__ int level_of(float x) { return (int)(__float_as_uint(x) >> 23) - 127 - kTop; }
+template <int Top> __device__ __forceinline__ int level_of(float x) { return (int)(__float_as_uint(x) >> 23) - 127 - Top; }
 __device__ __forceinline__ float power_of_two(int e) // 2^e for e <= 127; 0 below the normal range
 {
     return e < -126 ? 0.0f : __uint_as_float((uint32_t)(e + 127) << 23);
@@ -697,6 +717,8 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
             pM[k] = pI[k] = pD[k] = Op::kZero;
         float lM = Op::kZero, lI = Op::kZero, lD = Op::kZero;
         int E = kNoMass;
+        if (Op::kScaled && c0 == 0) // row 0 begins there
+            E = -Op::kTop;
         const int lane_m = (m - s * span) / K; // (last stripe) the lane of column m
         const int steps = len + 1 + (last_stripe ? lane_m : 31);
         // rows r0 + lane of the previous stripe's boundary, once they are written; each four rows
@@ -743,7 +765,20 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
         for (int c = 0; c < kVec; ++c)
             em[c] = emi_s[4 * letter_stride + c * 32];
         int x_next = seq[-lane];
-        float from_left = 1.0f; // 2^(left lane's exponent - this lane's)
+        // 2^(left lane's exponent - this lane's); with a look at what comes in, infinite where that is
+        // no number to go by (nothing ever comes into columns above m)
+        float from_left = 1.0f;
+        auto link = [&](int left_e, auto look) {
+            const int d = left_e - E;
+            if (decltype(look)::value && d > kHot)
+                from_left = c0 <= m ? INFINITY : 0.0f;
+            else
+                from_left = power_of_two(min(d, 127));
+        };
+        if constexpr (Op::kScaled) {
+            const int rE = __shfl_up_sync(0xffffffffu, E, 1);
+            link(lane > 0 ? rE : s > 0 ? __float_as_int(ring[0].w) : kNoMass, std::true_type());
+        }
         auto scale_own = [&](float f) {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
@@ -755,57 +790,61 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
             lI *= f;
             lD *= f;
         };
-        // One step.  kFirst: the first 32 steps of a stripe, in which mass reaches each lane for the
-        // first time: exponents are compared in every step.  (Rows below 0: every state is zero,
-        // and so is what the recurrence makes of them; rows above len: unused.)
+        // One step.  kFirst: among the first 32, which bring mass to each lane for the first time;
+        // they look at what comes in.  (Rows below 0: every state is zero, and so is what the
+        // recurrence makes of them; rows above len: unused.)
         auto step = [&](int st, auto first) {
-            constexpr bool kFirst = decltype(first)::value;
+            constexpr bool kFirst = decltype(first)::value, kLook = Op::kScaled && (kFirst || Op::kWatch);
             // column c0 - 1 at this row: the left lane's latest row, or the previous stripe's boundary
-            float rM = __shfl_up_sync(0xffffffffu, pM[K - 1], 1);
-            float rI = __shfl_up_sync(0xffffffffu, pI[K - 1], 1);
-            float rD = __shfl_up_sync(0xffffffffu, pD[K - 1], 1);
-            int rE = kNoMass;
-            if constexpr (Op::kScaled && kFirst)
-                rE = __shfl_up_sync(0xffffffffu, E, 1);
-            if (lane == 0) {
-                rM = rI = rD = Op::kZero;
-                rE = kNoMass;
-                if (s > 0) {
-                    const float4 v = ring[st & 63];
-                    rM = v.x;
-                    rI = v.y;
-                    rD = v.z;
-                    rE = __float_as_int(v.w);
+            float rM, rI, rD;
+            auto come = [&] {
+                rM = __shfl_up_sync(0xffffffffu, pM[K - 1], 1);
+                rI = __shfl_up_sync(0xffffffffu, pI[K - 1], 1);
+                rD = __shfl_up_sync(0xffffffffu, pD[K - 1], 1);
+                int rE = kNoMass;
+                if (lane == 0) {
+                    rM = rI = rD = Op::kZero;
+                    if (s > 0) {
+                        const float4 v = ring[st & 63];
+                        rM = v.x;
+                        rI = v.y;
+                        rD = v.z;
+                        rE = __float_as_int(v.w);
+                    }
                 }
-            }
+                return rE; // lane 0's
+            };
+            come();
             // the next row's emissions and the letter after it, for the next step
             float4 em_next[kVec];
 #pragma unroll
             for (int c = 0; c < kVec; ++c)
                 em_next[c] = emi_s[x_next * letter_stride + c * 32];
             x_next = seq[st + 1 - lane];
-            if constexpr (Op::kScaled && kFirst) {
-                const float big = fmaxf(fmaxf(rM, rI), rD);
-                const int level = rE + level_of(big);
-                int d = rE - E;
-                if (level - E > kRise || d > kFar) {
-                    if (level > E && big > 0.0f) { // it outweighs the lane: the lane takes its level
-                        scale_own(power_of_two(max(E - level, -127)));
-                        E = level;
-                        d = rE - E;
-                    }
-                    rM = ldexpf(rM, d);
-                    rI = ldexpf(rI, d);
-                    rD = ldexpf(rD, d);
-                    from_left = 1.0f;
-                } else {
-                    from_left = power_of_two(d);
-                }
-            }
             if constexpr (Op::kScaled) {
                 rM *= from_left;
                 rI *= from_left;
                 rD *= from_left;
+            }
+            if constexpr (kLook) {
+                // (an infinite factor leaves nothing that compares as less)
+                const bool over = !(fmaxf(fmaxf(rM, rI), rD) <= power_of_two(Op::kTop + kRise));
+                if (__any_sync(0xffffffffu, over)) {
+                    const int e0 = come(), e1 = __shfl_up_sync(0xffffffffu, E, 1), rE = lane == 0 ? e0 : e1;
+                    const float x = fmaxf(fmaxf(rM, rI), rD);
+                    const int level = rE + level_of<Op::kTop>(x);
+                    if (over && level > E && x > 0.0f) { // it outweighs the lane: the lane takes its level
+                        scale_own(power_of_two(E - level));
+                        E = level;
+                    }
+                    const int d = max(-252, min(rE - E, 254));
+                    const float f1 = power_of_two(d / 2), f2 = power_of_two(d - d / 2);
+                    rM = rM * f1 * f2;
+                    rI = rI * f1 * f2;
+                    rD = rD * f1 * f2;
+                    const int e2 = __shfl_up_sync(0xffffffffu, E, 1);
+                    link(lane == 0 ? e0 : e2, std::true_type());
+                }
             }
             float cM[K], cI[K];
 #pragma unroll
@@ -818,10 +857,8 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
                 cI[k] = Op::acc3(pM[k], toI[k][kM], pI[k], toI[k][kI], pD[k], toI[k][kD]);
             }
             if constexpr (kFirst)
-                if (st == 0 && s == 0 && lane == 0) { // B = M_0 at row 0
-                    cM[0] = Op::kScaled ? power_of_two(kTop) : Op::kOne;
-                    E = Op::kScaled ? -kTop : E;
-                }
+                if (st == 0 && s == 0 && lane == 0) // B = M_0 at row 0
+                    cM[0] = Op::kScaled ? power_of_two(Op::kTop) : Op::kOne;
             // the delete chain along the row
 #pragma unroll
             for (int k = 0; k < K; ++k)
@@ -847,8 +884,8 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
                     at_end[k] = make_float4(pM[k], pI[k], pD[k], __int_as_float(E));
             }
         };
-        // after every fourth step (its last: st)
-        auto settle = [&](int st) {
+        // after every fourth step (its last: st); look: those that follow look at what comes in
+        auto settle = [&](int st, auto look) {
             if ((st & 31) == 31) {
                 if (!last_stripe && lane == 31) { // rows .. st - 31 are written
                     __threadfence_block();
@@ -869,26 +906,25 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
                     big[2] = fmaxf(big[2], pD[k]);
                 }
                 const float b = fmaxf(fmaxf(big[0], big[1]), big[2]);
-                const int up = b > 0.0f ? max(level_of(b), -126) : 0;
+                const int up = b > 0.0f ? max(level_of<Op::kTop>(b), -126) : 0;
                 scale_own(power_of_two(-up));
                 E += up;
-                // the factor of what comes in during the next four steps
+                // what comes in during the next four steps
                 int rE = __shfl_up_sync(0xffffffffu, E, 1);
                 if (lane == 0)
                     rE = s > 0 ? __float_as_int(ring[(st + 1) & 63].w) : kNoMass;
-                if (rE - E > kFar) {
-                    scale_own(power_of_two(max(E - rE, -127)));
-                    E = rE;
-                }
-                from_left = power_of_two(rE - E);
+                link(rE, look);
             }
         };
         int st = 0;
+        const std::bool_constant<Op::kWatch> watch;
 #pragma unroll 1
         for (; st < 32 && st < steps; ++st) {
             step(st, std::true_type());
-            if ((st & 3) == 3)
-                settle(st);
+            if (st == 31)
+                settle(st, watch);
+            else if ((st & 3) == 3)
+                settle(st, std::true_type());
         }
 #pragma unroll 1
         for (; st < steps; st += 4) { // (up to three steps more than needed)
@@ -896,7 +932,7 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
             step(st + 1, std::false_type());
             step(st + 2, std::false_type());
             step(st + 3, std::false_type());
-            settle(st + 3);
+            settle(st + 3, watch);
         }
         if (!last_stripe) {
             if (lane == 31) { // every row is written
@@ -971,15 +1007,17 @@ size_t hmm_scratch_bytes(uint64_t blocks, int m, int max_len)
 // 1,461 columns 20 letters 67, 34; 60 letters 102, 76; 150 letters 116, 188; 3,070 columns 100
 // letters 214, 127; 300 letters 262, 345; 5,000 amplicons, 3,070 columns 20 letters 1,214, 807;
 // 60 letters 1,954, 2,305.  (Forward scores stay with the wavefront: on odds they are more exact.)
-bool hmm_use_wave(bool forward, uint64_t n, uint64_t letters, int max_len, int m)
+bool hmm_use_wave(const HmmProfile &p, bool forward, uint64_t n, uint64_t letters, int max_len)
 {
+    if (forward && p.rare > kRareBits)
+        return false;
     if (const char *kern = getenv("AH_HMM_KERNEL"))
         if (!strcmp(kern, "rows") || !strcmp(kern, "wave"))
             return kern[0] == 'w';
     if (forward || n == 0)
         return true;
     constexpr uint64_t kFull = 608; // amplicons that fill the GPU: four blocks for each of 152 SMs
-    const uint64_t line = 20 * (uint64_t)wave_stripes(m) - 12;
+    const uint64_t line = 20 * (uint64_t)wave_stripes(p.m) - 12;
     return n <= kFull ? (uint64_t)max_len > line : letters > n * std::min<uint64_t>(line, 75);
 }
 
@@ -996,8 +1034,10 @@ void launch_hmm_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n,
         launch(amps, order, n, planes, contig_off, n_contigs, forward ? p.d_t_odds : p.d_t,
                forward ? p.d_e_odds : p.d_e, p.m, max_len, (float4 *)bnd, blocks, score_out, err, sms, s);
     };
-    if (forward)
-        wave_narrow(p.m) ? go(launch_wave<WaveSum, 4>) : go(launch_wave<WaveSum, 8>);
+    if (forward && p.rare <= kCalmBits)
+        wave_narrow(p.m) ? go(launch_wave<WaveSum<false>, 4>) : go(launch_wave<WaveSum<false>, 8>);
+    else if (forward)
+        wave_narrow(p.m) ? go(launch_wave<WaveSum<true>, 4>) : go(launch_wave<WaveSum<true>, 8>);
     else
         wave_narrow(p.m) ? go(launch_wave<WaveMax, 4>) : go(launch_wave<WaveMax, 8>);
 }

@@ -8,8 +8,8 @@
 namespace ah {
 
 // Whether the wavefront scores a call of n amplicons (their letters in all, the longest) against a
-// profile of m columns; AH_HMM_KERNEL=rows or wave decides instead (a profiling aid).
-bool hmm_use_wave(bool forward, uint64_t n, uint64_t letters, int max_len, int m);
+// profile; AH_HMM_KERNEL=rows or wave decides instead (a profiling aid) where both can.
+bool hmm_use_wave(const HmmProfile &p, bool forward, uint64_t n, uint64_t letters, int max_len);
 
 // Blocks the wavefront takes for n amplicons of at most max_len letters, and the
 // device scratch of `blocks` of them in bytes: two stripe-boundary buffers of

@@ -1741,3 +1741,55 @@ def test_launch_counts_of_the_tm_stage_and_of_a_small_run():
             c.tm(sid, [pid], sites)
             assert c.ah_get_profile("tm")[1] == want, n
         c.ah_set_profiling(0)
+
+
+@pytest.mark.parametrize("kind", ["copies", "one deletion", "deletions by turns", "one insertion", "insertions by turns"])
+@pytest.mark.parametrize("m,n_train", [(40, 40_000), (60, 20_000), (300, 4000), (500, 100), (500, 3000), (700, 700)])
+def test_forward_on_odds_after_large_training_sets(ctx, m, n_train, kind):
+    """The range of the scaled odds: profiles whose rare moves and letters have probabilities down to 1 / (training
+    sequences + 4) and whose common ones include long deletions, single deletions in every other column, long and
+    scattered insertions; amplicons that agree, end early, start late, are turned about, lie apart by a few letters
+    or agree with nothing.  Forward (and Viterbi) against the oracle in fp64."""
+    rng = np.random.default_rng(m)
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    ref = acgt[rng.integers(0, 4, m)].tobytes().decode()
+
+    def random(n):
+        return acgt[rng.integers(0, 4, n)].tobytes().decode()
+
+    a, b = m // 5, m // 2  # the columns of the variants
+    ins = random(40)
+    variants = {"copies": [ref], "one deletion": [ref[:a] + ref[b:]],
+                "deletions by turns": [ref[:a] + ref[a:b:2] + ref[b:], ref[:a] + ref[a + 1:b:2] + ref[b:]],
+                "one insertion": [ref[:a] + ins + ref[a:]],
+                "insertions by turns": [ref[:a] + "".join(x + "A" for x in ref[a:b]) + ref[b:]]}[kind]
+    train = [ref] * (n_train // 2 + 1)
+    train += [variants[i % len(variants)] for i in range(n_train - len(train))]
+    seqs = [ref, "", ref[:1], ref[:m // 3], ref[m // 3:], ref[m // 2:] + ref[:m // 2], random(m), random(2 * m),
+            ref[:a] + random(30) + ref[a:], ref[:a] + ref[a + 6:], ref[:b] + random(3) + ref[b:], ref + random(50),
+            random(50) + ref, ref[:a] + random(b - a) + ref[b:], "A" * m, ref[:b] + "A" * 200 + ref[b:],
+            ref[::-1], ref + ref, ref[:a] + ref[a:b] * 2 + ref[b:], *variants]
+    seqs += [synth._mutate(rng, v, 0.1, 0.1) for v in variants for _ in range(4)]
+    seq = np.frombuffer(("".join(seqs) + "A").encode(), np.uint8).copy()
+    amps = np.zeros(len(seqs), dtype=ah.AMPLICON_DTYPE)
+    ends = np.cumsum([len(x) for x in seqs])
+    amps["end"], amps["start"] = ends, ends - [len(x) for x in seqs]
+    sid = ctx.load(seq, np.array([0, len(seq)], np.uint64), np.zeros(1, np.uint32))
+    try:
+        hid = ctx.hmm_build(train)
+        _, ref_i, T, E = ctx.hmm_tables(hid)
+        assert train[ref_i] == ref
+        got, got_f = ctx.hmm_score(sid, hid, amps).astype(np.float64), ctx.hmm_forward(sid, hid, amps).astype(np.float64)
+        ctx.hmm_free(hid)
+    finally:
+        ctx.ah_unload_genomes(sid)
+    T, E = T.astype(np.float64), E.astype(np.float64)  # (the tables' own roundings are the other tests')
+    want = np.array([oracle.hmm_viterbi(T, E, x) for x in seqs])
+    want_f = np.array([oracle.hmm_forward(T, E, x) for x in seqs])
+    fin = ~np.isinf(T)
+    pmean = float(np.concatenate([np.abs(T[fin]), np.abs(E[1:]).ravel()]).mean())
+    N = np.array([len(x) for x in seqs]) + m
+    # the bound of the parity test above: ten standard deviations of a walk of fp32 roundings
+    assert (np.abs(got - want) <= 10.0 * np.sqrt(N) * 2.0 ** -24 * (np.abs(want) + N * pmean) + 1e-4).all()
+    tol_f = 10.0 * np.sqrt(N) * (2.0 ** -24 * (np.abs(want_f) + N * pmean) + 4 * 2.0 ** -23) + 1e-4
+    assert (np.abs(got_f - want_f) <= tol_f).all(), (np.abs(got_f - want_f) / tol_f).max()
