@@ -693,7 +693,10 @@ __global__ void __launch_bounds__(32 * kWaveWarps, K <= 4 ? 4 : 3) hmm_wave_kern
         }
         float4 *out_rows = buffer_of(warp, task);
         const float4 *in_rows = buffer_of(before, task - 1); // (s > 0)
-        // the task that used this buffer before has been read
+        // The task that used this buffer before, eight back, has been read.  (Where that was a last
+        // stripe, which hands nothing on, the user before it is sixteen back: its reader, the
+        // next warp, has read task - 12 since, for which task - 4 waited here: neither of these
+        // is a last stripe unless this one is too, as then the stripes divide four.)
         if (!last_stripe && task >= 2 * kWaveWarps && (task - 2 * kWaveWarps) % n_stripes + 1 != n_stripes && !failed &&
             !wait_for(&used[warp], task - 2 * kWaveWarps + 1))
             failed = true;

@@ -1743,6 +1743,43 @@ def test_launch_counts_of_the_tm_stage_and_of_a_small_run():
         c.ah_set_profiling(0)
 
 
+@pytest.mark.parametrize("m", [600, 1100, 1400, 1700, 2300, 2500, 2800, 3000])
+def test_hmm_wavefront_uses_its_boundary_buffers_again(ctx, m):
+    """Blocks with many tasks (a memory budget leaves one or two blocks for 24 amplicons of 3, 5, 6, 7, 9, 10, 11 and
+    12 stripes), so that a buffer's turn comes round while a last stripe, which hands nothing on, lies between: the
+    same scores as with a block per amplicon, and the oracle's."""
+    rng = np.random.default_rng(m)
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    ref = acgt[rng.integers(0, 4, m)].tobytes().decode()
+    train = [ref, ref, ref[:-3], ref[5:]]
+    seqs = [synth._mutate(rng, ref[:int(m * rng.uniform(0.2, 1.0))], 0.05, 0.02) for _ in range(22)]
+    seqs += ["", ref + ref[:m // 4]]
+    seq = np.frombuffer(("".join(seqs) + "A").encode(), np.uint8).copy()
+    off = np.array([0, len(seq)], np.uint64)
+    amps = np.zeros(len(seqs), dtype=ah.AMPLICON_DTYPE)
+    ends = np.cumsum([len(x) for x in seqs])
+    amps["end"], amps["start"] = ends, ends - [len(x) for x in seqs]
+    got = []
+    with ah.Context(0, 8 << 20) as small:
+        for c in (ctx, small):
+            sid = c.load(seq, off, np.zeros(1, np.uint32))
+            hid = c.hmm_build(train)
+            got.append((c.hmm_score(sid, hid, amps), c.hmm_forward(sid, hid, amps)))
+            c.hmm_free(hid)
+            c.ah_unload_genomes(sid)
+    assert got[0][0].tobytes() == got[1][0].tobytes() and got[0][1].tobytes() == got[1][1].tobytes()
+    _, T, E = oracle.hmm_build(train)
+    fin = ~np.isinf(T)
+    pmean = float(np.concatenate([np.abs(T[fin]), np.abs(E[1:]).ravel()]).mean())
+    for i in (0, 22, 23):
+        N = len(seqs[i]) + m
+        # the bound of the parity test above: ten standard deviations of a walk of fp32 roundings
+        want, want_f = oracle.hmm_viterbi(T, E, seqs[i]), oracle.hmm_forward(T, E, seqs[i])
+        assert abs(float(got[0][0][i]) - want) <= 10.0 * np.sqrt(N) * 2.0 ** -24 * (abs(want) + N * pmean) + 1e-4
+        assert abs(float(got[0][1][i]) - want_f) <= \
+            10.0 * np.sqrt(N) * (2.0 ** -24 * (abs(want_f) + N * pmean) + 4 * 2.0 ** -23) + 1e-4
+
+
 @pytest.mark.parametrize("kind", ["copies", "one deletion", "deletions by turns", "one insertion", "insertions by turns"])
 @pytest.mark.parametrize("m,n_train", [(40, 40_000), (60, 20_000), (300, 4000), (500, 100), (500, 3000), (700, 700)])
 def test_forward_on_odds_after_large_training_sets(ctx, m, n_train, kind):
