@@ -1830,3 +1830,35 @@ def test_forward_on_odds_after_large_training_sets(ctx, m, n_train, kind):
     assert (np.abs(got - want) <= 10.0 * np.sqrt(N) * 2.0 ** -24 * (np.abs(want) + N * pmean) + 1e-4).all()
     tol_f = 10.0 * np.sqrt(N) * (2.0 ** -24 * (np.abs(want_f) + N * pmean) + 4 * 2.0 ** -23) + 1e-4
     assert (np.abs(got_f - want_f) <= tol_f).all(), (np.abs(got_f - want_f) / tol_f).max()
+
+
+@pytest.mark.parametrize("tiles,per_claim", [(7295, 1), (7297, 2), (10_950, 3), (29_191, 8)])
+def test_scan_tiles_claimed_several_at_a_time(tiles, per_claim, monkeypatch):
+    """Large sets hand out their tiles in claims of up to eight (n_tiles / (24 CTAs) of them; one CTA per SM here, so
+    that smaller sets do too), the last claim past the set's end: a site in every tile, at its edges and inside, is
+    found once, and again in a second scan."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms != 152:
+        pytest.skip("the sizes are for 152 SMs")
+    assert min(8, max(1, tiles // (sms * 24))) == per_claim
+    monkeypatch.setenv("AH_SCAN_TUNING", "4,0,0,4,2,1")
+    fwd, rev = "ACGTTGCAAGCT", "GGATCCATTCAG"
+    T = 32 * 1024
+    n = tiles * T - 17
+    rng = np.random.default_rng(tiles)
+    at = np.arange(tiles) * T + rng.choice([0, 1, 31, 1023, 1024, T // 2, T - 40, T - 13, T - 11, T - 1], tiles)
+    at[-1] = n - 12
+    word = np.frombuffer(fwd.encode(), np.uint8)
+    seq = torch.full((n,), ord("T"), dtype=torch.uint8, device="cuda")
+    seq[torch.from_numpy(at[:, None] + np.arange(12)).cuda()] = torch.from_numpy(np.tile(word, (tiles, 1))).cuda()
+    whole = np.r_[np.diff(at) >= 12, True] & np.r_[True, np.diff(at) >= 12]  # (a plant may lie over the next one)
+    torch.cuda.synchronize()
+    with ah.Context(0) as c:
+        sid = c.ah_load_genomes(seq, n, np.array([0, n], np.uint64), np.zeros(1, np.uint32))
+        pid = c.ah_set_primers(fwd, rev, synth.pcr_params(fwd, rev, k=0, min_len=30, max_len=200))
+        for _ in range(2):
+            got = c.scan(sid, [pid])
+            assert np.array_equal(np.sort(got["pos"]), got["pos"]) and len(np.unique(got["pos"])) == len(got)
+            assert np.isin(at[whole], got["pos"]).all() and np.isin(got["pos"], at).all()
+            assert not got["primer"].any() and not got["strand"].any() and not got["mm"].any()
