@@ -553,13 +553,9 @@ PairDev make_pair_dev(const PrimerPair &pp)
     d.min_len = pp.params.min_len;
     d.max_len = pp.params.max_len;
     memcpy(d.mask, pp.mask, sizeof(d.mask));
-    for (int x = 0; x < 2; ++x) { // Tm shortest-path keys: both ends and every degenerate position
-        int nk = 0;
+    for (int x = 0; x < 2; ++x)
         for (int q = 0; q < pp.L[x]; ++q)
-            if (q == 0 || q == pp.L[x] - 1 || __builtin_popcount(pp.mask[x][q]) > 1)
-                d.key[x][nk++] = (uint8_t)q;
-        d.nkey[x] = nk;
-    }
+            d.nkey[x] += q == 0 || q == pp.L[x] - 1 || __builtin_popcount(pp.mask[x][q]) > 1;
     d.tm_min = pp.params.tm_min;
     d.tm_min_f = (float)pp.params.tm_min;
     const double x = (pp.params.dnac1_nM - pp.params.dnac2_nM / 2.0) * 1e-9;

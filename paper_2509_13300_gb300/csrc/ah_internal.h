@@ -272,9 +272,7 @@ struct PairDev {
     int L[2];
     int min_len, max_len;
     uint8_t mask[2][AH_MAX_PRIMER_LEN];
-    // Tm shortest-path steps: positions 0 and L-1 and every degenerate position, ascending
-    int nkey[2];
-    uint8_t key[2][AH_MAX_PRIMER_LEN];
+    int nkey[2]; // key positions of the Tm's shortest path: 0, L-1 and every degenerate one
     // 1 when every duplex of either primer has dS + C < 0 (a bound from the table's
     // largest entries): only sites within ~1e-9 K of tm_min can need exhaustive fp64
     int few_exact;
