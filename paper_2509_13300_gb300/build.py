@@ -12,6 +12,7 @@ from __future__ import annotations
 import concurrent.futures as cf
 import glob
 import os
+import re
 import subprocess
 import sys
 
@@ -54,11 +55,22 @@ def source_digest() -> str:
 # the source files that define each profiled kernel (with the internal header)
 KERNEL_SOURCES = {"ah_scan_kernel": ["scan_jit.cu"], "pack_kernel": ["pack.cu"], "tm_kernel": ["tm.cu"],
                   "tm_fast_kernel": ["tm.cu"],
-                  "rank_sort_decode_kernel": ["sites.cu"], "hmm_score_kernel": ["hmm.cu"]}
+                  "rank_sort_decode_kernel": ["sites.cu"], "hmm_score_kernel": ["hmm.cu"],
+                  "hmm_wave_kernel": ["hmm.cu"]}
+
+
+# literals are kept as they are (the scan's source is one, comments included)
+_CODE = re.compile(r'R"(\w*)\(.*?\)\1"|"(?:\\.|[^"\\\n])*"|' + r"'(?:\\.|[^'\\\n])+'|//[^\n]*|/\*.*?\*/|\s+", re.S)
+
+
+def _code_only(src: str) -> str:
+    """C++ source without its comments, blanks and line breaks as one space."""
+    return _CODE.sub(lambda m: m[0] if m[0][0] in "R\"'" else " ", src)
 
 
 def kernel_digest(kernel: str) -> str | None:
-    """Hash of one kernel's sources: a profile of the kernel stays valid while it matches."""
+    """Hash of the code of one kernel's sources, comments left out: a profile of the kernel stays
+    valid while it matches."""
     import hashlib
     files = KERNEL_SOURCES.get(kernel)
     if not files:
@@ -66,7 +78,8 @@ def kernel_digest(kernel: str) -> str | None:
     h = hashlib.sha256()
     for f in files + ["ah_internal.h"]:
         h.update(f.encode())
-        h.update(open(os.path.join(CSRC, f), "rb").read())
+        with open(os.path.join(CSRC, f), encoding="utf-8") as fh:
+            h.update(re.sub(r" +", " ", _code_only(fh.read())).encode())
     return h.hexdigest()[:16]
 
 

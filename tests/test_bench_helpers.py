@@ -153,3 +153,24 @@ def test_form_keys_summarise_each_form_and_report_a_failing_one(monkeypatch):
     assert out["batched"]["plain"]["genomes"] == 400 and out["batched"]["wall_s"] >= 0.0
     assert out["served"] == {"error": "RuntimeError: no device"}
     assert args.steps == 20 and args.n_genomes == 123  # the caller's arguments are left alone
+
+
+def test_kernel_digest_follows_the_code_and_not_its_comments(tmp_path, monkeypatch):
+    """A kernel's committed profile stays current when only comments or line breaks of its sources change, and
+    not when code, a literal or a comment inside the generated scan's source does."""
+    from paper_2509_13300_gb300 import build
+    header = "// layout\nconstexpr int kTileW = 1024; /* words */\n"
+    source = 'const char *k = R"CUDA(\n a // b\n)CUDA";\nint f() { return 1; } // one\nos << "x // y\\n";\nchar c = \'"\';\n'
+    monkeypatch.setattr(build, "CSRC", str(tmp_path))
+
+    def digest(h, s):
+        (tmp_path / "ah_internal.h").write_text(h)
+        (tmp_path / "scan_jit.cu").write_text(s)
+        return build.kernel_digest("ah_scan_kernel")
+
+    first = digest(header, source)
+    assert digest(header.replace("layout", "the layout,\n// in words"), source) == first
+    assert digest(header.replace("/* words */", ""), source.replace("// one", "/* 1 */ // \"uno")) == first
+    for h, s in ((header.replace("1024", "2048"), source), (header, source.replace("return 1", "return 2")),
+                 (header, source.replace("a // b", "a // c")), (header, source.replace("x // y", "x // z"))):
+        assert digest(h, s) != first
