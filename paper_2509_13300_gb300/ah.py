@@ -239,8 +239,8 @@ class Context:
         return int(self._lib.ah_device_bytes(self.h))
 
     def debug_scan_stall(self, on: bool):
-        """Test aid: make later scans take their timeout path (each warp's first
-        slice waits on a barrier that nothing completes; 20 us limit)."""
+        """Test aid: make later scans take their timeout path (each CTA's first
+        tile waits on a barrier that nothing completes; 20 us limit)."""
         self._check(self._lib.ah_debug_scan_stall(self.h, 1 if on else 0))
 
     def debug_pair_cluster(self, on: bool):

@@ -48,8 +48,8 @@ struct ah_ctx {
     cudaEvent_t ev_load_start = nullptr; // a host load's copies start after the caller's earlier work
     cudaEvent_t ev_last_copy = nullptr;  // recorded after a host load's last copy
     uint64_t *h_flags = nullptr;     // pinned host mirror of the flag block
-    // test of the timeout path (ah_debug_scan_stall): each warp's first slice
-    // is armed without a copy and the per-slice wait limit drops to 20 us
+    // test of the timeout path (ah_debug_scan_stall): each CTA's first tile
+    // is armed without a copy and the limit of a wait for a tile drops to 20 us
     bool scan_stall_first = false;
     bool flags_dirty = false;        // work was queued that may set the error word, not read since
     std::vector<cudaEvent_t> set_events; // free "ready" events of genome sets
@@ -679,7 +679,7 @@ ScanTuning tuning_for(ah_ctx *c, const std::vector<ScanPattern> &pats)
 // Launch the generated scan kernel over tiles [0, n_tiles) of a set.
 // Scan n_tiles tiles: the first n_tiles of the set, or tile_list[0 .. n_tiles) (device) when given.
 // The caller resets the flag block (the work counter included) on the same stream first.
-// work: the launch's slice counter (a flag word zeroed by the caller's reset_flags).
+// work: the launch's counter of tile claims (a flag word zeroed by the caller's reset_flags).
 void launch_scan(ah_ctx *c, ScanKernel *k, const GenomeSet &gs, uint64_t n_tiles, uint64_t *keys, uint64_t cap,
                  int pbits, cudaStream_t st, const uint64_t *tile_list, uint64_t *work)
 {
@@ -2962,9 +2962,9 @@ ah_status ah_hmm_forward(ah_ctx *c, uint32_t set_id, uint32_t hmm_id, const ah_a
 }
 
 // Test aid (not in the public header).  on != 0: in later scans the first
-// slice of every warp is armed on its barrier with no copy behind it (a wait
-// that nothing will end) and the per-slice wait limit is 20 us, so the scan
-// takes its timeout path -- error word, bounded wait for the warp's copies
+// tile of every CTA is armed on its barrier with no copy behind it (a wait
+// that nothing will end) and the limit of a wait is 20 us, so the scan
+// takes its timeout path -- error word, bounded wait for the CTA's copies
 // still in flight, exit -- and the call returns AH_ERR_TIMEOUT.  Nothing
 // faults or hangs.  on == 0 restores normal scans.
 ah_status ah_debug_scan_stall(ah_ctx *c, int on)

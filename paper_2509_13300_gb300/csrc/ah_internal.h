@@ -218,7 +218,7 @@ enum FlagWord : int {
     kFlagAmps = 5,    // ... amplicons
     kFlagSeq = 6,     // ... sequence bytes
     kFlagRedo = 7,    // ... kRedo* bits: a count above what the launches were sized for
-    kFlagWork = 8,    // scan: slices claimed so far, one word per launch group (zeroed before a scan)
+    kFlagWork = 8,    // scan: claims of tiles so far, one word per launch group (zeroed before a scan)
     kFlagErr = kFlagWork + AH_MAX_PAIRS_PER_SCAN, // DeviceErr (low 32 bits)
     kFlagWords = kFlagErr + 1
 };

@@ -82,7 +82,9 @@ void launch_fetch(const ah_amplicon *a, uint64_t n, const uint64_t *n_dev, const
     // count, so its grid stays at the blocks that are resident together (four per SM
     // beside the chain's other kernels): with 2,048, most of them waiting for room only
     // to find no amplicon, the launch took 9.0 us for 7 amplicons against 3.3 (700: 10.0
-    // against 6.7; 3,600: 14.5 against 14.4; with two per SM 2.2, 6.3 and 25)
+    // against 6.7; 3,600: 14.5 against 14.4; with two per SM 2.2, 6.3 and 25).  Runs of very many
+    // would gain by more: 57,600 amplicons of 220 bases 82 us against 72 with 1,216 blocks and 64
+    // with 2,048; of 1,600 bases 250, 245, 228
     const uint64_t most = n_dev ? 608 : 8192;
     const uint64_t blocks = n < most ? n : most;
     launch_chained(fetch_kernel, (unsigned)blocks, 256, 0, s, a, n, n_dev, offsets, planes,

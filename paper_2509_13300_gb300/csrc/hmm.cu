@@ -1078,8 +1078,8 @@ void launch_hmm_score(const ah_amplicon *amps, const uint32_t *order, uint64_t n
         AH_HMM_TRY(8, 1, 256)
         vk = va = 0;
     }
-    // default (measured on 639 columns: 4 columns x 2 amplicons 398 GCUPS; 2 x 2 272; 4 x 1 315;
-    // 8 x 1 234, register-capped); longer profiles take 6 columns x 1 amplicon
+    // 4 columns x 2 amplicons (on 639 columns 398 GCUPS; 2 x 2 272; 4 x 1 315; 8 x 1 234,
+    // register-capped); longer profiles take 6 columns x 1 amplicon
     AH_HMM_TRY(4, 2, 512)
     AH_HMM_TRY(6, 1, 512)
 #undef AH_HMM_TRY

@@ -455,7 +455,7 @@ std::string scan_source(const std::vector<ScanPattern> &pats, const ScanTuning &
         span = std::max(span, pos[q].back() + 1);
     }
     const int R = t.R;
-    if (R != 4 && R != 8) // the loader reads 16-byte vectors at word lane * R of the slice
+    if (R != 4 && R != 8) // the loader reads 16-byte vectors at a warp's word lane * R
         throw Error(AH_ERR_ARG, "scan kernel: R must be 4 or 8");
     const int nwin = 4 * ((R + span - 1 + 3) / 4);
     Gen g;
