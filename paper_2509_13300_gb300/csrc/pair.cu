@@ -258,9 +258,9 @@ __global__ void pair_write_kernel(const ah_site *s, uint64_t n, const uint8_t *p
 // warps, read through distributed shared memory.  The sequence offsets follow from the same scan.
 // Groups of 32 sites go to the CTAs in turn: few sites, or the neighbouring sites of a hot spot
 // that lead many amplicons each, keep all 16 SMs at work (5,000 sites of 62,500 amplicons: 103
-// us with 1,024 neighbours per CTA, five SMs at work, 62 so; 6,000 sites 2 us less).  Sixteen CTAs are beyond the cluster size that
-// every device has room for (eight): where pair_run_available finds none, runs go step by step,
-// with the kernels above.
+// us with 1,024 neighbours per CTA, five SMs at work, 62 so; 6,000 sites 2 us less).  Sixteen
+// CTAs are beyond the cluster size that every device has room for (eight): where
+// pair_run_available finds none, runs go step by step, with the kernels above.
 // Bound: latency, and the host's launches around it.  Measured on a GB300 from the end of the
 // Tm kernel to the sequence decode: four launches (count, scan, write, scan of the lengths)
 // 9.3 us for 14 sites, 15 for 6,000 -> 8.1 and 14.2; the run of a small resident set, which waits
