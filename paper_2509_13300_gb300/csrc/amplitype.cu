@@ -16,8 +16,9 @@
 // words per (variant, copies) pair (two independent sums, order-free), the
 // copies counted in a second table keyed by (genome, variant).
 //
-// Bound: launches, memory latency and, in the hashing, the planes' reads from L2
-// (16 bytes per letter; a sixth fewer instructions per letter changed nothing).
+// Bound: launches, memory latency and, in the hashing, issue slots (ncu: issue 0.68,
+// ALU pipe 65 %, of the 16 bytes of planes per letter five in six from L1, 264 MB from
+// L2, 76 from DRAM; a sixth fewer instructions per letter changed nothing).
 // Measured on a GB300, 65,000 amplicons of ~1,500 letters: hashing 399 us (a lane per
 // 1/32 of an amplicon, letter by letter) -> 122; the rest of a call 3 x 16 radix-sort
 // passes and ~60 small launches, 0.7 ms -> 15 launches, 0.13 ms.  (Fewer blocks for the
@@ -163,8 +164,7 @@ __device__ __forceinline__ uint64_t group_digit(const uint32_t *__restrict__ pla
 // letters: consecutive positions lie in consecutive words), each times its
 // power of the base; hash = the groups in order (zeros beyond the end), then
 // the length.  (Neither word is ever the empty key: the low 61 bits are below 2^61 - 1.)
-// A bad record sets *err.  Bound by the reads: 1.6 GB from L2 in 121 us for 65,000
-// amplicons of ~1,500 letters.
+// A bad record sets *err.  65,000 amplicons of ~1,500 letters: 121 us.
 __global__ void amp_hash_kernel(const ah_amplicon *__restrict__ a, uint64_t n, const uint32_t *__restrict__ planes,
                                 const uint64_t *__restrict__ contig_off, const uint32_t *__restrict__ contig_genome,
                                 uint32_t n_contigs, uint64_t *__restrict__ hash1, uint64_t *__restrict__ hash2,
