@@ -93,7 +93,9 @@ struct HmmProfile {
     int m = 0;
     uint64_t reference = 0; // index of the training sequence used as the reference
     std::vector<float> t, e;
-    float rare = 0; // bits of the rarest move: its probability is 2^-rare
+    // how Forward scores are kept in range (hmm.cu): in logarithms, or as odds with a look at what comes
+    // into a lane at every step or only while its first mass arrives
+    enum Odds : uint8_t { kLogs, kWatched, kCalm } odds = kLogs;
     float *d_t = nullptr, *d_e = nullptr;           // device: the scores
     float *d_t_odds = nullptr, *d_e_odds = nullptr; // and 2^score, in the same block
 };

@@ -82,6 +82,8 @@ enum { kM = 0, kI = 1, kD = 2 };
 
 } // namespace
 
+static HmmProfile::Odds odds_form(const HmmProfile &p);
+
 void build_profile(const char *seqs, const uint64_t *off, uint64_t n, HmmProfile &p)
 {
     // the reference: most frequent sequence, first occurrence on ties (by hashing)
@@ -190,10 +192,7 @@ void build_profile(const char *seqs, const uint64_t *off, uint64_t n, HmmProfile
                 p.e[(size_t)j * 4 + l] = (float)std::log2((ce[(size_t)j * 4 + l] + 1.0) / tot * 4.0);
         }
     }
-    p.rare = 0.0f;
-    for (float t : p.t)
-        if (std::isfinite(t))
-            p.rare = std::max(p.rare, -t);
+    p.odds = odds_form(p);
 }
 
 namespace {
@@ -527,7 +526,7 @@ struct WaveMax {
 };
 template <bool Watch> struct WaveSum {
     static constexpr bool kScaled = true, kWatch = Watch;
-    static constexpr int kTop = Watch ? 80 : -24;
+    static constexpr int kTop = Watch ? 80 : 0;
     static constexpr float kZero = 0.0f, kOne = 1.0f;
     __device__ static __forceinline__ float ext(float a, float t) { return a * t; }
     __device__ static __forceinline__ float acc(float s, float a, float t) { return fmaf(a, t, s); }
@@ -540,28 +539,35 @@ template <bool Watch> struct WaveSum {
 // Exponents of the scaled odds: a value is mantissa * 2^E with one E per lane.
 // Every four rows a lane's largest mantissa is brought to 2^kTop, and the factor
 // 2^(left lane's exponent - this one's) for what comes in from the left is renewed.
-// With p = 2^-c the rarest move's probability:
-//   - A lane's smallest cell that counts is the deletion state of its last column,
-//     through which a row's mass must go where no letters are left for it: up to
-//     eight moves below the largest cell, which itself may fall by a move a row until
-//     the next settling and lie one below what came in: 2^(kTop - 13 c).
-//   - Its largest: a lane holds at least what deletions bring it within a row, so
-//     its left neighbour lies at most 2^(11 c + 6) above it (eight columns, a lane of
-//     lag, a row of growth).  In four rows mass grows by four letters' 4^4 and a sum
-//     over the cells of two lanes, 2^15 in all, and by what four matches save against
-//     deletions, a move each for their columns and for those after them, 2^(8 c).
-// Without a look at what comes in (kWatch false), kTop + 19 c + 21 <= 127 and kTop -
-// 13 c >= -126: kTop = -24 holds for c <= kCalmBits (about 100 training sequences).
-// Only the first 32 steps of a stripe, in which mass reaches each lane for the first
-// time, need that look then.  Rarer moves: in every step (a tenth more instructions),
-// and a lane that is outweighed by more than 2^kRise, or whose left neighbour's
-// exponent lies kHot above its own, takes the level of what comes in: four rows end
-// below 2^(kTop + kRise + 13), and kTop = 80 leaves 13 c <= 206: c <= kRareBits.  Moves
-// rarer than that (some 32,000 training sequences) go by logarithms
-// (hmm_score_kernel).  (With kTop = 30 and the left lane's exponent taken over where
-// it lay 80 above, profiles with moves rarer than 2^-8 could lose mass or overflow.)
+// Let a move into a deletion cost at most a bits, one into an insertion b, from a
+// deletion to the next d, from an insertion to itself i, any move c.
+//   fall: the smallest cell that counts is the deletion state of a lane's last column,
+//     through which a row's mass must go where no letters are left for it.  It is at
+//     least its lane's largest cell less a + 6 d; that one falls by b + 3 i at most in
+//     the rows between two settlings (by insertions, if nothing better) and lies at most a
+//     below what came in.  The other states of that column count down to c + 24 bits less.
+//     kTop - (c + 2 a + 6 d + b + 3 i) >= -125 keeps all of it among the floats.
+//   rise: a lane holds at least what deletions bring to it within a row.  A path that
+//     reaches it within the next four rows crosses the same columns with at most four
+//     matches, so it is at most a + 8 d bits above that: the columns of the matches and
+//     those after them.  Four letters give 4^4, and at most 2^13.2 cells add up.
+//     kTop + 22.2 + a + 8 d <= 127 keeps every mantissa finite.
+//   far: by the same counts the left lane's exponent lies at most 15.2 + 2 a + 10 d above
+//     this lane's (a row and a lane further), or a + 8 d + b + 3 i where a stripe's boundary
+//     rows share that of three rows ago; up to 127 the factor is a float.
+// Where all three hold (calm: kTop = 0), a look at what comes in is needed only while mass
+// reaches the lanes for the first time, the first 32 steps of a stripe.  Else (watched) each
+// step looks: a lane that is outweighed by more than 2^kRise, or whose left neighbour's
+// exponent lies kHot above its own, takes the level of what comes in, so four rows end below
+// 2^(kTop + kRise + 13), and kTop = 80 leaves fall 205 bits.  Beyond that the scores go by
+// logarithms (hmm_score_kernel).  With every move down to 2^-c, calm holds up to c = 9.3
+// (600 training sequences that each delete and insert everywhere), watched to 15.7; the 2,416
+// of an operon family, which seldom delete, are calm.  On a GB300, calm against watched: 5,000
+// amplicons x 460 columns 1,101 us and 1,270, 5,023 x 639 on that family's profile 2.02 ms and
+// 3.05.  (With kTop = 30 and the left lane's exponent taken over where it lay 80 above,
+// profiles lost mass or overflowed from c = 8 on.)
 constexpr int kRise = 24, kHot = 100;
-constexpr float kCalmBits = 6.8f, kRareBits = 15.0f;
+constexpr double kFallRoom = 125.0, kRiseRoom = 104.8, kFarRoom = 127.0; // at kTop = 0
 constexpr int kNoMass = -(1 << 20); // exponent of a lane that holds only zeros
 template <int Top> __device__ __forceinline__ int level_of(float x) { return (int)(__float_as_uint(x) >> 23) - 127 - Top; }
 __device__ __forceinline__ float power_of_two(int e) // 2^e for e <= 127; 0 below the normal range
@@ -986,6 +992,30 @@ void launch_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n, con
 
 } // namespace
 
+// The form of the odds that a profile's moves leave room for (see kTop).
+static HmmProfile::Odds odds_form(const HmmProfile &p)
+{
+    double a = 0, b = 0, c = 0, d = 0, i = 0;
+    for (int j = 0; j <= p.m; ++j)
+        for (int x = 0; x < 3; ++x) {
+            const float *t = &p.t[(size_t)j * 9 + x * 3];
+            for (int y = 0; y < 3; ++y) {
+                if (!std::isfinite(t[y])) // no such move
+                    continue;
+                double &most = y == kD ? a : y == kI ? b : c;
+                most = std::max(most, -(double)t[y]);
+                if (x == y && x != kM)
+                    (x == kD ? d : i) = std::max(x == kD ? d : i, -(double)t[y]);
+            }
+        }
+    c = std::max(c, std::max(a, b));
+    const double fall = c + 2 * a + 6 * d + b + 3 * i, rise = a + 8 * d;
+    const double far = std::max(15.2 + 2 * a + 10 * d, a + 8 * d + b + 3 * i);
+    if (fall <= kFallRoom && rise <= kRiseRoom && far <= kFarRoom)
+        return HmmProfile::kCalm;
+    return fall <= kFallRoom + WaveSum<true>::kTop ? HmmProfile::kWatched : HmmProfile::kLogs;
+}
+
 // One block per amplicon up to a full GPU; a profile of one stripe runs an amplicon per warp.
 uint64_t hmm_wave_blocks(uint64_t n, int m, int max_len, int sms)
 {
@@ -1012,7 +1042,7 @@ size_t hmm_scratch_bytes(uint64_t blocks, int m, int max_len)
 // 60 letters 1,954, 2,305.  (Forward scores stay with the wavefront: on odds they are more exact.)
 bool hmm_use_wave(const HmmProfile &p, bool forward, uint64_t n, uint64_t letters, int max_len)
 {
-    if (forward && p.rare > kRareBits)
+    if (forward && p.odds == HmmProfile::kLogs)
         return false;
     if (const char *kern = getenv("AH_HMM_KERNEL"))
         if (!strcmp(kern, "rows") || !strcmp(kern, "wave"))
@@ -1037,7 +1067,7 @@ void launch_hmm_wave(const ah_amplicon *amps, const uint32_t *order, uint64_t n,
         launch(amps, order, n, planes, contig_off, n_contigs, forward ? p.d_t_odds : p.d_t,
                forward ? p.d_e_odds : p.d_e, p.m, max_len, (float4 *)bnd, blocks, score_out, err, sms, s);
     };
-    if (forward && p.rare <= kCalmBits)
+    if (forward && p.odds == HmmProfile::kCalm)
         wave_narrow(p.m) ? go(launch_wave<WaveSum<false>, 4>) : go(launch_wave<WaveSum<false>, 8>);
     else if (forward)
         wave_narrow(p.m) ? go(launch_wave<WaveSum<true>, 4>) : go(launch_wave<WaveSum<true>, 8>);
