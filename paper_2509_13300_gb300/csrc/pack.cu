@@ -454,8 +454,8 @@ __global__ void __launch_bounds__(kPackThreads, In == kAligned ? 6 : 5) pack_ker
 // per column: the rows of column j that a run [a, b) covers are consecutive.
 // Bound: HBM (0.25 B read + 0.516 B written per base), then the latency of one
 // tile (its loads, a barrier, the matrix).  Measured, 1.5 Gbp with 0.1 % of no-base
-// runs on a GB300: 416 us with persistent blocks, a serial search of the tile's
-// runs and a bitmap read back row by row -> 266 us (4.3 TB/s).  (Packing pieces of a
+// bases on a GB300: 416 us with persistent blocks, a serial search of the tile's
+// runs and a bitmap read back row by row -> 205 us (5.6 TB/s).  (Packing pieces of a
 // host set while later pieces cross the link gains nothing: the copies stand
 // still for as long as the packing runs.)
 // ---------------------------------------------------------------------------

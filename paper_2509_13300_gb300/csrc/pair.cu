@@ -263,7 +263,7 @@ __global__ void pair_write_kernel(const ah_site *s, uint64_t n, const uint8_t *p
 // pair_run_available finds none, runs go step by step, with the kernels above.
 // Bound: latency, and the host's launches around it.  Measured on a GB300 from the end of the
 // Tm kernel to the sequence decode: four launches (count, scan, write, scan of the lengths)
-// 9.3 us for 14 sites, 15 for 6,000 -> 8.1 and 14.2; the run of a small resident set, which waits
+// 9.3 us for 14 sites, 15 for 6,000 -> 8 to 9 and 10; the run of a small resident set, which waits
 // for the host's launches too, 93 -> 88.  A cluster of eight with two sites per thread took
 // 18 us for 10,000 sites against 15.  Beside another stream's packing, whose blocks it waits for
 // (16 SMs of one GPC must have room at once), 28 us against 13 alone for 10,000 sites; the
