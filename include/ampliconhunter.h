@@ -356,8 +356,9 @@ typedef struct ah_run_out {
  * launches are sized for (at most 16384 sites and the sites capacity when the
  * site outputs are device memory; the amplicon and sequence capacities when
  * those outputs are device memory, else sizes the context grows from earlier
- * calls; fewer than 65536 amplicons), else the call continues step by step
- * with up to three more.  Device outputs are complete when the call returns
+ * calls; fewer than 65536 amplicons), else, and on a device slice without room
+ * for a cluster of 16 thread blocks, the call continues step by step with up
+ * to three more.  Device outputs are complete when the call returns
  * (copies to host outputs too).  An output whose capacity is too small is not
  * written, its count is still reported, the others are written, and the call
  * returns AH_ERR_OVERFLOW.
